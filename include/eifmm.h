@@ -74,11 +74,10 @@ typedef enum {
  *            tier 2: M2L on the FP32 SIMT pipes, each offset's sum in FP32
  *                    and the offsets added with compensated FP32 sums;
  *                    FP32 elsewhere with one Newton step on every 1/r;
- *            tier 3: far field in FP64 (its M2L in FP32 pairs, hi + lo,
- *                    with exact product splits: about 46 bits), near
- *                    field in FP32 (Kahan sums);
- *            tier 4: FP64 everywhere (near field too) but the M2L, which
- *                    runs in FP32 pairs as in tier 3.
+ *            tier 3: far field in FP64, near field in FP32 (Kahan sums);
+ *            tier 4: FP64 everywhere (near field too), as FP64.
+ *          The FP64 far field's M2L is summed exactly in integer residues
+ *          on the tensor cores and rounded once to FP64.
  *          In every tier the M2L applies K^delta Delta (built once with
  *          FP64 solves) to W, so step 3 needs no solve.
  */
@@ -167,8 +166,8 @@ eifmm_status eifmm_ops_error_estimate(const eifmm_ops* ops, int level,
 /* Arithmetic tier that EIFMM_PREC_MIXED uses with these operators:
  * 0 = BF16 hi+lo M2L and an FP32 far field, 1 = FP16 hi+lo M2L with per-offset
  * drains, 2 = FP32 SIMT M2L with compensated sums over the offsets,
- * 3 = FP64 far field (M2L in FP32 pairs), 4 = FP64 everywhere, the near
- * field too (M2L in FP32 pairs).  eifmm_ops_load sets it
+ * 3 = FP64 far field, 4 = FP64 everywhere, the near field too.
+ * eifmm_ops_load sets it
  * from the built-in error estimate; `tier_override` >= 0 (at most 4) forces
  * a tier.  Errors: EINVAL (null ops, tier above 4). */
 eifmm_status eifmm_ops_plan(eifmm_ops* ops, int tier_override, int* tier);
@@ -258,8 +257,8 @@ void eifmm_tree_destroy(eifmm_tree* tree);
  *   SINGLE_STREAM: 1 runs the whole evaluate on the caller's stream instead
  *     of the near field, far field and coarse M2L levels on streams of their
  *     own (the result is bitwise the same);
- *   M2L_FP64: 1 runs the FP64 M2L instead of the FP32-pair one in tiers 3
- *     and 4;
+ *   M2L_FP64: 1 runs the M2L of the FP64 far field (the FP64 path, tiers 3
+ *     and 4) on the FP64 pipes instead of in residues on the tensor cores;
  *   M2L_STREAM_K: 1 runs the leaf-level transposed M2L as one CTA per SM
  *     over equal shares of the (tile, offset) work, split tiles added by a
  *     fix-up kernel, instead of one CTA per tile (at 2^20 points the launch

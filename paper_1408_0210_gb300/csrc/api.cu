@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "m2l_crt.h"
 #include "solve.cuh"
 
 namespace eifmm {
@@ -71,6 +72,11 @@ void free_workspace(Workspace* ws) {
   dfree(ws->part64);
   ws->part64 = nullptr;
   ws->part64_cap = 0;
+  dfree(ws->crt_buf);
+  dfree(ws->crt_max);
+  ws->crt_buf = nullptr;
+  ws->crt_max = nullptr;
+  ws->crt_bytes = 0;
   dfree(ws->blas_ws);
   ws->blas_ws = nullptr;
   for (int k = 0; k <= kMaxLevel; ++k) ws->m2l_kind[k] = ws->m2l_gshift[k] = 0;
@@ -129,6 +135,57 @@ static void free_streams(Workspace* ws) {
 
 eifmm_status alloc_mixed_workspace(Tree* t, const Ops* ops, int R);  // fmm32.cu
 
+eifmm_status alloc_wait_error(Workspace* ws) {
+  if (ws->err) return EIFMM_OK;
+  EIFMM_CUDA(cudaMallocHost(&ws->err_host, sizeof(int)));
+  *ws->err_host = 0;
+  EIFMM_TRY(dalloc(&ws->err, 1));
+  EIFMM_CUDA(cudaMemset(ws->err, 0, sizeof(int)));
+  return EIFMM_OK;
+}
+
+// Residue images of the M2L operators of levels 2..depth, built once per
+// operator set and ready for every stream on return.  A level whose image does
+// not fit the device's memory stays without one (its M2L runs on the FP32 or
+// FP64 pipes).  Several trees of one operator set may come here at the same time.
+static std::mutex g_crt_mu;
+eifmm_status ensure_crt_images(Ops* ops, int depth, cudaStream_t s) {
+  std::lock_guard<std::mutex> lock(g_crt_mu);
+  for (int k = 2; k <= depth; ++k) {
+    LevelOps& v = ops->lv[k];
+    const bool c = ops->compressed && v.r > 0;
+    CrtImage& im = c ? v.crtc : v.crt;
+    const int d = c ? v.r : v.d;
+    if (im.img || d < kCrtMinRank) continue;
+    const eifmm_status rc = build_crt_image(c ? v.Ct : v.kdT, d, &im, s);
+    if (rc == EIFMM_ENOMEM) continue;
+    EIFMM_TRY(rc);
+    if (!c) EIFMM_TRY(crt_kappa((int)ops->kern, v, ops->L * ldexp(1.0, -(k + 1)), &im.kappa, s));
+  }
+  return EIFMM_OK;
+}
+
+// Images and scratch of the residue M2L for an evaluation with the FP64 far
+// field.  Without room for the scratch crt_bytes stays 0 and the M2L runs on
+// the FP32 or FP64 pipes.
+static eifmm_status ensure_crt(Tree* t, Ops* ops, int R, cudaStream_t s) {
+  Workspace& ws = t->ws;
+  EIFMM_TRY(ensure_crt_images(ops, t->depth, s));
+  const CrtImage* im[kMaxLevel + 1] = {};
+  for (int k = 2; k <= t->depth; ++k)
+    im[k] = ops->compressed && ops->lv[k].r > 0 ? &ops->lv[k].crtc : &ops->lv[k].crt;
+  const size_t need = crt_scratch_bytes(t->depth, im, R);
+  if (need > ws.crt_bytes) {
+    dfree(ws.crt_buf);
+    ws.crt_buf = nullptr;
+    ws.crt_bytes = 0;
+    const eifmm_status rc = dmalloc(&ws.crt_buf, need);
+    if (rc == EIFMM_OK) ws.crt_bytes = need;
+    else if (rc != EIFMM_ENOMEM) return rc;
+  }
+  return EIFMM_OK;
+}
+
 eifmm_status ensure_workspace(Tree* t, const Ops* ops, int R, int prec) {
   Workspace& ws = t->ws;
   if (!ws.side) {
@@ -176,6 +233,8 @@ eifmm_status ensure_workspace(Tree* t, const Ops* ops, int R, int prec) {
     }
     if (need) EIFMM_TRY(dalloc(&ws.part64, need));
     ws.part64_cap = need;
+    EIFMM_TRY(dalloc(&ws.crt_max, (size_t)(kMaxLevel + 1) * R));
+    EIFMM_TRY(alloc_wait_error(&ws));
   } else {
     EIFMM_TRY(alloc_mixed_workspace(t, ops, R));
   }
@@ -509,10 +568,20 @@ static eifmm_status evaluate_impl(eifmm_tree* tree, const eifmm_ops* ops, const 
                                   int prec, cudaStream_t s) {
   Tree& t = tree->t;
   EIFMM_TRY(ensure_workspace(&t, &ops->o, n_rhs, prec));
+  if ((prec == EIFMM_PREC_FP64 || ops->o.tier >= 3) && !t.opt[EIFMM_OPT_M2L_FP64])
+    EIFMM_TRY(ensure_crt(&t, const_cast<Ops*>(&ops->o), n_rhs, s));
+  if (t.ws.err_host && *t.ws.err_host != 0) {
+    const int code = *t.ws.err_host;
+    *t.ws.err_host = 0;
+    cudaMemsetAsync(t.ws.err, 0, sizeof(int), s);
+    set_error("eifmm_evaluate: a bounded device wait of the previous call timed out (code " +
+              std::to_string(code) + ")");
+    return EIFMM_ETIMEOUT;
+  }
   eifmm_status rc;
   if (prec == EIFMM_PREC_FP64)
     rc = eval_fp64(&t, &ops->o, sigma, ld_sigma, n_rhs, f, ld_f, s);
-  else if (ops->o.tier >= 4)  // FP64 everywhere, the M2L in FP32 pairs
+  else if (ops->o.tier >= 4)  // FP64 everywhere
     rc = eval_fp64(&t, &ops->o, sigma, ld_sigma, n_rhs, f, ld_f, s, false, true);
   else
     rc = eval_mixed(&t, &ops->o, sigma, ld_sigma, n_rhs, f, ld_f, s);
@@ -535,7 +604,7 @@ static eifmm_status evaluate_impl(eifmm_tree* tree, const eifmm_ops* ops, const 
 // evaluated at depth min(depth, 4) with the operators' own kernel in FP64
 // and in every mixed tier; the cheapest tier whose relative L2
 // difference to FP64 stays below eps/4 is kept (else tier 4: FP64
-// throughout, the M2L in FP32 pairs).
+// throughout).
 // ---------------------------------------------------------------------------
 extern "C" eifmm_status eifmm_ops_calibrate(eifmm_ops* ops, double eps, eifmm_stream stream,
                                             int* tier_out) {
@@ -577,7 +646,9 @@ extern "C" eifmm_status eifmm_ops_calibrate(eifmm_ops* ops, double eps, eifmm_st
     }
     const double lo[3] = {0.0, 0.0, 0.0};
     if ((rc = eifmm_tree_build(dx, n, dx, n, lo, L, depth, 1, stream, &tree)) != EIFMM_OK) break;
-    // a view of the operators restricted to the calibration depth
+    // a view of the operators restricted to the calibration depth (with the
+    // images of the FP64 reference, which then belong to the set itself)
+    if ((rc = ensure_crt_images(&ops->o, depth, s)) != EIFMM_OK) break;
     eifmm_ops view;
     view.o = ops->o;
     view.o.depth = depth;
@@ -632,6 +703,8 @@ extern "C" eifmm_status eifmm_ops_calibrate(eifmm_ops* ops, double eps, eifmm_st
   dfree(fm);
   if (rc != EIFMM_OK) return rc;
   EIFMM_TRY(eifmm_ops_plan(ops, best, nullptr));
+  if (best < 3)  // only an evaluation in FP64 would use them, and it builds them again
+    for (int k = 2; k <= depth; ++k) free_crt_image(&ops->o.lv[k].crt);
   ops->o.calib_tier = best;
   if (tier_out) *tier_out = best;
   return EIFMM_OK;

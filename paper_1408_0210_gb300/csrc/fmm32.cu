@@ -1366,12 +1366,7 @@ eifmm_status alloc_mixed_workspace(Tree* t, const Ops* ops, int R) {
     ws.m2l_part_leaf_cap = need_leaf;
   }
   if (!ws.wmax) EIFMM_TRY(dalloc(&ws.wmax, (size_t)kMaxLevel + 1));
-  if (!ws.err) {
-    EIFMM_TRY(dalloc(&ws.err, 1));
-    EIFMM_CUDA(cudaMemset(ws.err, 0, sizeof(int)));
-    EIFMM_CUDA(cudaMallocHost(&ws.err_host, sizeof(int)));
-    *ws.err_host = 0;
-  }
+  EIFMM_TRY(alloc_wait_error(&ws));
   return EIFMM_OK;
 }
 
@@ -1712,14 +1707,6 @@ eifmm_status eval_mixed(Tree* t, const Ops* ops, const double* sigma, int64_t ld
                         double* f, int64_t ld_f, cudaStream_t s) {
   if (ops->tier == 3) return eval_fp64(t, ops, sigma, ld_sigma, R, f, ld_f, s, true, true);
   Workspace& ws = t->ws;
-  if (*ws.err_host != 0) {
-    const int code = *ws.err_host;
-    *ws.err_host = 0;
-    cudaMemsetAsync(ws.err, 0, sizeof(int), s);
-    set_error("eifmm_evaluate: a bounded device wait of the previous call timed out (code " +
-              std::to_string(code) + ")");
-    return EIFMM_ETIMEOUT;
-  }
   // P2M and L2P: the approximate reciprocal square root alone in tier 0
   // (relative error below 2^-22), one Newton step above
   const bool acc = ops->tier >= 1;

@@ -7,6 +7,7 @@
 #include <cstdlib>
 
 #include "internal.h"
+#include "m2l_crt.h"
 #include "transfer.cuh"
 #include "solve.cuh"
 
@@ -163,8 +164,8 @@ k_m2l64(int level, int d, int R, const double* __restrict__ kdT,
 }
 
 
-// Step 4 of the mixed path's tier 3 (FP64 far field) with the FP64 numbers
-// carried as unevaluated sums of two FP32 numbers (hi + lo, about 46
+// Step 4 of tiers 3 and 4 for operators that amplify rounding
+// (kCrtMaxKappa in internal.h), with the FP64 numbers carried as unevaluated sums of two FP32 numbers (hi + lo, about 46
 // significant bits) on the FP32 pipes, which run 72 times faster than the
 // FP64 ones on this GPU.  Each product hi_a hi_b is split exactly with an
 // FMA (p + e), the cross terms hi_a lo_b + lo_a hi_b are added in FP32, and
@@ -592,19 +593,31 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   // K^delta Delta), so step 4 reads W; What itself is formed only when it is
   // exported
   record(ws, 3, s);
-  // step 4 (the compressed operators of Section 4.2 when they are built)
-  for (int k = 2; k <= kap; ++k) {
-    if (timing_enabled()) cudaEventRecord(ws.ev_m2l[k], s);
-    const bool pair = pair_m2l && !t->opt[EIFMM_OPT_M2L_FP64];  // tiers 3 and 4: FP32 pairs
-    if (ops->compressed && ops->lv[k].r > 0)
-      EIFMM_TRY(m2l_compressed(ws, ops, k, R, pair, s));
-    else if (pair)
-      EIFMM_TRY(launch_m2l_df(k, ops->lv[k].d, R, ops->lv[k].kdT, ops->d_slot_lists, ws.W[k], ws.g[k],
-                              ws.part64, ws.part64_cap, ws.nsm, s));
-    else
-      EIFMM_TRY(launch_m2l64(k, ops->lv[k].d, R, ops->lv[k].kdT, ops->d_slot_lists, ws.W[k], ws.g[k],
-                             ws.part64, ws.part64_cap, ws.nsm, s));
-    if (timing_enabled()) cudaEventRecord(ws.ev_m2le[k], s);
+  // step 4 (the compressed operators of Section 4.2 when they are built): the
+  // residue M2L on the tensor cores for all levels together; FP32 pairs in
+  // tiers 3 and 4 and the FP64 pipes otherwise where a level has no image, and
+  // where the tree option or the operators (kCrtMaxKappa) ask for them
+  {
+    const bool fp64 = t->opt[EIFMM_OPT_M2L_FP64] != 0, pair = pair_m2l && !fp64;
+    CrtJob jobs[kMaxLevel];
+    int nj = 0;
+    for (int k = 2; k <= kap; ++k) {
+      const LevelOps& v = ops->lv[k];
+      if (timing_enabled()) cudaEventRecord(ws.ev_m2l[k], s);
+      if (ops->compressed && v.r > 0)
+        EIFMM_TRY(m2l_compressed(ws, ops, k, R, fp64, pair, s));
+      else if (!fp64 && v.crt.img && ws.crt_bytes > 0 && !(pair && v.crt.kappa > kCrtMaxKappa))
+        jobs[nj++] = CrtJob{k, &v.crt, ws.W[k], ws.g[k]};
+      else if (pair)
+        EIFMM_TRY(launch_m2l_df(k, v.d, R, v.kdT, ops->d_slot_lists, ws.W[k], ws.g[k], ws.part64, ws.part64_cap,
+                                ws.nsm, s));
+      else
+        EIFMM_TRY(launch_m2l64(k, v.d, R, v.kdT, ops->d_slot_lists, ws.W[k], ws.g[k], ws.part64, ws.part64_cap,
+                               ws.nsm, s));
+      if (timing_enabled() && k < kap) cudaEventRecord(ws.ev_m2le[k], s);
+    }
+    if (nj > 0) EIFMM_TRY(launch_m2l_crt(nj, jobs, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
+    if (timing_enabled()) cudaEventRecord(ws.ev_m2le[kap], s);
   }
   record(ws, 4, s);
   // step 5 (l^2 = g^2)
@@ -641,6 +654,7 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
     EIFMM_CHECK_LAUNCH();
   }
   record(ws, 8, s);
+  EIFMM_CUDA(cudaMemcpyAsync(ws.err_host, ws.err, sizeof(int), cudaMemcpyDeviceToHost, s));
   return EIFMM_OK;
 }
 

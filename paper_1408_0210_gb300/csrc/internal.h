@@ -53,6 +53,15 @@ void dfree(void* p);
 __host__ __device__ inline double kern_f64(int kern, double z0, double z1, double z2);
 
 // ------------------------------------------------------------ operators --
+// Residues of an M2L operator stack for the FP64 M2L on the tensor cores
+// (m2l_crt.cu): [modulus][slot][column tile][k8][Nt columns m'][8 terms l].
+constexpr int kCrtMods = 14;
+struct CrtImage {
+  void* img = nullptr;         // BF16
+  double* colscale = nullptr;  // [d] scale of column m' in the reconstruction
+  double kappa = 0.0;          // amplification of rounding by the operators (crt_kappa)
+  int d = 0, K = 0, Nt = 0, NT = 0;  // rank, terms padded to 16, columns of a tile, tiles
+};
 struct LevelOps {
   int d = 0;          // EIM rank of the level
   int dp = 0;         // d padded to a multiple of 64 (tensor-core layouts)
@@ -91,6 +100,8 @@ struct LevelOps {
   double* Ct = nullptr;    // [343][l < r][m' < r]: C^delta_{m'l} = (U^t K^delta U)_{m'l}
   int r = 0, r_i = 0, r_ii = 0;     // kept rank and the counts of the two filters
   double s_kept = 0.0, s_next = 0.0;  // last kept and first dropped singular value / s_0
+  CrtImage crt;            // residues of kdT, built at the first use of the FP64 far field
+  CrtImage crtc;           // residues of Ct, with it
   int kd_img_fmt = -1;     // -1 none, else the PlaneFmt of the image
   float* kscale = nullptr; // [dp] power-of-two scale of row m' (FP16 image)
 };
@@ -176,6 +187,9 @@ struct Workspace {
   float* m2l_part = nullptr;    // partial M2L sums of the split offset lists
   double* part64 = nullptr;     // the same for the FP64 far field (FP64 and FP32-pair M2L)
   size_t part64_cap = 0;        // doubles in part64
+  void* crt_buf = nullptr;      // residue planes and sums of the FP64 M2L on the tensor cores
+  size_t crt_bytes = 0;
+  unsigned long long* crt_max = nullptr;  // [kMaxLevel + 1][R] bits of the largest |W|
   int nsm = 0;                  // SMs of the workspace's device
   uint32_t* wmax = nullptr;     // [kMaxLevel + 1] bits of max |W| per level (FP16 planes)
   SkPlanDev sk;                 // stream-K plan of the leaf level (tier 0), when it pays
@@ -257,9 +271,11 @@ eifmm_status eval_mixed(Tree* t, const Ops* ops, const double* sigma,
                         int64_t ld_sigma, int R, double* f, int64_t ld_f,
                         cudaStream_t s);
 eifmm_status ensure_workspace(Tree* t, const Ops* ops, int R, int prec);
-// Step 4 of level k with the compressed operators (sarcmp.cu) on the FP64
-// far field; pair: FP32-pair arithmetic, else FP64.
-// FP64 far-field M2L (fmm64.cu): offset groups split the offset list of a
+// Residue images of levels 2..depth (m2l_crt.cu), built once per operator
+// set; returns when they are ready for every stream.
+eifmm_status ensure_crt_images(Ops* ops, int depth, cudaStream_t s);
+eifmm_status alloc_wait_error(Workspace* ws);
+// FP64 far-field M2L on the FP64 pipes and in FP32 pairs (fmm64.cu): offset groups split the offset list of a
 // level with few blocks; `part` (part_cap doubles) holds their partial sums.
 int m2l64_groups(int64_t blocks, int nsm);
 int64_t m2l_df_blocks(int level, int d, int R);
@@ -268,7 +284,18 @@ eifmm_status launch_m2l_df(int level, int d, int R, const double* kdT, const int
                            double* g, double* part, size_t part_cap, int nsm, cudaStream_t s);
 eifmm_status launch_m2l64(int level, int d, int R, const double* kdT, const int* slot_lists, const double* W,
                           double* g, double* part, size_t part_cap, int nsm, cudaStream_t s);
-eifmm_status m2l_compressed(Workspace& ws, const Ops* ops, int k, int R, bool pair, cudaStream_t s);
+// Step 4 of level k with the compressed operators (sarcmp.cu) on the FP64 far
+// field; fp64: on the FP64 pipes; pair: FP32 pairs rather than those where
+// the residue M2L cannot run.
+eifmm_status m2l_compressed(Workspace& ws, const Ops* ops, int k, int R, bool fp64, bool pair, cudaStream_t s);
+// Smallest rank that runs on the tensor cores.
+constexpr int kCrtMinRank = 8;
+// Operators with a larger crt_kappa keep FP32 pairs in tiers 3 and 4: there the
+// pairs' own rounding shows in the result (measured 1.3e-14 kappa of f: 1e-8 for
+// the config-3 kernel at eps 1e-6, kappa 7.7e5, and 3.5e-12 for 1/r at 1e-7,
+// kappa 1.2e3), and those results stay what they were.  The FP64 path, whose
+// rounding is 1000 times smaller, takes the residues for all operators.
+constexpr double kCrtMaxKappa = 1e4;
 void free_workspace(Workspace* ws);
 bool timing_enabled();
 

@@ -1,0 +1,939 @@
+// m2l_crt.cu -- step 4 of Algorithm 3 (M2L, Eq. M2Lstep) in FP64 accuracy on
+// the tcgen05 tensor cores.
+//
+//   g^I_{m'} = sum_{J in I(I)} sum_l T^delta_{m'l} W^J_l
+//
+// The FP64 pipes of this GPU run at 1/72 of the FP32 rate, the tensor cores
+// 25 times above the latter.  The sum is therefore formed exactly in integers by
+// residues (K. Ozaki, Y. Uchino, T. Imamura, "Ozaki Scheme II", 2025): W is
+// rounded to 59-bit integers with one power-of-two scale per level and
+// right-hand side, row m' of every T^delta with one scale per row, chosen so
+// that the whole sum over offsets and l stays below M / 2 in magnitude, M the
+// product of 14 pairwise coprime moduli up to 513 (125.2 bits).  Modulo m_i
+// both operands are integers in [-256, 256], exact in BF16; a product is at
+// most 2^16, so 240 terms are summed exactly in the FP32 accumulator (below
+// 2^24, every partial sum an integer).  The running sums are kept modulo m_i
+// in FP32 registers, and the Chinese remainder theorem gives the exact integer
+// sum, rounded once to FP64.
+//
+// Accuracy: the sum of |T| over a row and all offsets has 66 bits, the largest
+// |W| of a level 58, and the sum itself adds no rounding.  Against quad
+// precision g errs by 1.0e-16 to 6e-16 (2-norm; 1/r at eps 1e-4 to 1e-7, levels
+// 2 to 4, uniform and clustered points), the FP64 sum on the FP64 pipes by
+// 1.2e-15 to 6.8e-15 and the FP32 pairs by about 2e-12; for the config-3 kernel
+// (eps 1e-6) 4.2e-13 against 6.6e-12 in FP64.
+//
+// Four launches cover all levels: largest |W| per level and column; the
+// residue planes of W; the residue GEMMs; the reconstruction.  At 2^20 points,
+// depth 5: eps 1e-6 (d = 193) 0.04 + 0.11 + 5.7 + 0.28 ms, where the FP32 pairs
+// took 144 ms; eps 1e-4 (d = 126) 3.9 ms, where the FP64 pipes took 195 ms; eps
+// 1e-7 (d = 256) 7.5 ms (202 ms in FP32 pairs).  The GEMM issues 14 / 1 of the
+// method's products, 13% of them zero (189 offsets for 165 pairs per box) and
+// is bound by the stream of operator residues: 86 KB per offset and 128 boxes,
+// 64 bytes per cycle and SM at the tensor cores' full rate.
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+#include <vector>
+
+#include "m2l_crt.h"
+#include "tc_ptx.cuh"
+
+namespace eifmm {
+namespace {
+
+constexpr int kMods = kCrtMods;
+__host__ __device__ constexpr int crt_mod(int i) {
+  return i == 0 ? 513 : i == 1 ? 512 : i == 2 ? 511 : i == 3 ? 509 : i == 4 ? 505 : i == 5 ? 503 : i == 6 ? 499
+       : i == 7 ? 491 : i == 8 ? 487 : i == 9 ? 481 : i == 10 ? 479 : i == 11 ? 473 : i == 12 ? 467 : 463;
+}
+static_assert(kMods == 14, "crt_mod lists 14 moduli");
+constexpr int kWBits = 58;     // |W| 2^b < 2^58
+constexpr int kRowBits = 66;   // sum over offsets and l of |T| 2^a < 2^66
+constexpr int kEntryBits = 60; // |T| 2^a < 2^60
+constexpr int kMaxSteps = 15;  // k-steps of 16 terms in one accumulation: 240 terms
+
+// Target tile of a CTA: 8 x 4 x 4 boxes of one parity class (128 rows of the
+// MMA).  The sources of class c' for one y-shift and all x- and z-shifts lie
+// in a window of 10 x 4 x 6 boxes of that class's grid, kept in shared memory
+// as [k8][z][y][x][8 terms]: the canonical K-major layout without swizzle,
+// where a shift by one box is a shift of the start address by 16 bytes (x) or
+// 640 bytes (z), and the 8-row groups (y, z) lie 160 bytes apart.  One window
+// serves the 5 to 9 offsets of its class and y-shift, so that W is read from
+// L2 3.6 times less often than with one tile per offset.
+constexpr int kTX = 8, kTY = 4, kTZ = 4;
+constexpr int kWinRows = (kTX + 2) * kTY * (kTZ + 2);       // 240
+constexpr uint32_t kWinStep = 2u * kWinRows * 16u;          // bytes of one k-step of a window
+constexpr int kWins = 2;
+constexpr int kMaxStages = 8;
+constexpr int kDrainWarps = 8;
+constexpr int kThreads = 32 * (kDrainWarps + 3);
+constexpr uint32_t kSmemMax = 227u * 1024u;
+constexpr uint32_t kSmemBars = 512;
+
+// One level (or one slab and column range of it) of a launch.
+struct CrtLv {
+  int level, d, K, Nt, NT;   // rank, padded terms, columns per tile, column tiles
+  int h;                     // boxes per axis of a parity class
+  int z0, nz, sz0, snz;      // planes of target boxes, planes of source boxes held
+  int r0, Rc, R, G;          // columns r0 .. r0 + Rc of R, offset groups
+  int nchunk, n0, ks0, ks1;  // chunks of K: n0 of ks0 k-steps, then ks1 k-steps each
+  unsigned item0, pl0, rc0, mx0;  // first block of this level in each of the launches
+  const double* W;
+  double* g;
+  __nv_bfloat16* planes;     // [mod][r][class][k8][z][y][x][8]
+  int16_t* res;              // [mod][group][r][class][z][y][x][NT Nt]
+  const __nv_bfloat16* img;  // [mod][slot][column tile][k8][Nt][8]
+  const double* colscale;    // per column m': M 2^(-96 - a)
+  unsigned long long* wmax;  // [R] bits of the largest |W|
+};
+constexpr int kMaxLv = kMaxLevel - 1;
+struct CrtArgs {
+  int nlev, stages;
+  uint32_t stage_b, win_b;
+  int* err;
+  CrtLv lv[kMaxLv];
+};
+struct CrtMaps {
+  CUtensorMap m[kMaxLv];
+};
+struct CrtK {
+  uint32_t k[kMods][3];  // 2^96 y_i / m_i, y_i the inverse of M / m_i modulo m_i
+};
+
+// K / 16 k-steps in chunks of five and three: three chunks of five or five of
+// three fill an accumulation (kMaxSteps), and a chunk of five keeps the MMAs of
+// a step (5 x 104 cycles at N = 208) above the cost of its wait and commit.
+void split_chunks(CrtLv* v) {
+  const int n = v->K / 16;
+  int a = n / 5;
+  if (n < 8) {
+    v->ks0 = n <= 5 ? n : n - 3;
+    v->ks1 = 3;
+    v->n0 = 1;
+    v->nchunk = n <= 5 ? 1 : 2;
+    return;
+  }
+  while ((n - 5 * a) % 3) --a;  // reaches a = 2 n mod 3 at the latest, and 10 <= n where that is 2
+  v->ks0 = 5;
+  v->ks1 = 3;
+  v->n0 = a;
+  v->nchunk = a + (n - 5 * a) / 3;
+}
+__device__ __forceinline__ int chunk_ksteps(const CrtLv& v, int c) { return c < v.n0 ? v.ks0 : v.ks1; }
+
+// bits of shifts s + 1 in {0, 1, 2} along one axis whose child offset
+// 2 s + cs - ct is at most one box (the near field)
+__device__ __forceinline__ int near_bits(int cs, int ct) { return cs == ct ? 2 : (cs > ct ? 3 : 6); }
+
+// The (sz, sx) shifts of class cs and y-shift sy + 1 that belong to the
+// interaction list of class ct: bit 3 (sz + 1) + sx + 1.
+__device__ __forceinline__ int combo_mask(int ct, int cs, int sy1) {
+  if (!((near_bits((cs >> 1) & 1, (ct >> 1) & 1) >> sy1) & 1)) return 0x1ff;
+  const int nx = near_bits(cs & 1, ct & 1), nz = near_bits((cs >> 2) & 1, (ct >> 2) & 1);
+  const int m = ((nz & 1) ? nx : 0) | ((nz & 2) ? nx << 3 : 0) | ((nz & 4) ? nx << 6 : 0);
+  return 0x1ff & ~m;
+}
+
+// scale exponent of a column from the bits of its largest |W|
+__device__ __forceinline__ bool w_finite(unsigned long long bits) { return bits < 0x7ff0000000000000ull; }
+__device__ __forceinline__ int w_exp(unsigned long long bits) {
+  const int b = kWBits - ((int)(bits >> 52) - 1022);
+  return b > 1020 ? 1020 : b;
+}
+__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+
+// v modulo crt_mod(i), in [-m/2, m/2]; |v| <= 2^60
+__device__ __forceinline__ int residue(long long v, int i) {
+  const int m = crt_mod(i);
+  const int c20 = (1 << 20) % m, c40 = (int)((1ll << 40) % m);
+  const int v2 = (int)(v >> 40), v1 = (int)(v >> 20) & 0xfffff, v0 = (int)v & 0xfffff;
+  // |v2 c40| < 2^29 and v1 c20 + v0 < 2^29 + 2^20: the offset keeps it positive
+  const unsigned u = (unsigned)(v2 * c40 + v1 * c20 + v0) + (unsigned)m * (unsigned)((1u << 30) / m);
+  int r = (int)(u % (unsigned)m);
+  return r > m / 2 ? r - m : r;
+}
+
+__device__ __forceinline__ int find_level(const CrtArgs& a, unsigned CrtLv::*first, unsigned b) {
+  int q = 0;
+  while (q + 1 < a.nlev && b >= a.lv[q + 1].*first) ++q;
+  return q;
+}
+
+// ---------------------------------------------------------- largest |W| --
+constexpr int kMaxPer = 16384;  // entries per block
+__global__ void __launch_bounds__(256) k_crt_max(const __grid_constant__ CrtArgs a) {
+  const CrtLv& v = a.lv[find_level(a, &CrtLv::mx0, blockIdx.x)];
+  const unsigned b = blockIdx.x - v.mx0;
+  const int r = v.r0 + (int)(b % v.Rc);
+  const int64_t n = ((int64_t)1 << (3 * v.level)) * v.d;
+  const int64_t beg = (int64_t)(b / v.Rc) * kMaxPer, end = min(n, beg + kMaxPer);
+  unsigned long long mx = 0;
+  for (int64_t i = beg + threadIdx.x; i < end; i += 256) {
+    const int64_t box = v.R == 1 ? 0 : i / v.d;
+    const double w = v.R == 1 ? v.W[i] : v.W[(box * v.R + r) * v.d + (i - box * v.d)];
+    const unsigned long long x = (unsigned long long)__double_as_longlong(w) & 0x7fffffffffffffffull;
+    mx = x > mx ? x : mx;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = x > mx ? x : mx;
+  }
+  __shared__ unsigned long long sm[8];
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) mx = sm[w] > mx ? sm[w] : mx;
+    atomicMax(v.wmax + r, mx);
+  }
+}
+
+// ------------------------------------------------------- residue planes --
+// A block takes 8 boxes along x of one class, z, y and column: their W is
+// rounded to integers once, and every thread writes 8 terms of one box for
+// the 14 moduli (16-byte stores, 128 contiguous bytes per 8 threads).
+__global__ void __launch_bounds__(256) k_crt_planes(const __grid_constant__ CrtArgs a) {
+  extern __shared__ long long s_w[];  // [8][K + 1]
+  const CrtLv& v = a.lv[find_level(a, &CrtLv::pl0, blockIdx.x)];
+  unsigned b = blockIdx.x - v.pl0;
+  const int h = v.h, nxs = (h + 7) / 8;
+  const int xs = (int)(b % nxs);
+  b /= nxs;
+  const int y = (int)(b % h);
+  b /= h;
+  const int zs = (int)(b % v.snz);
+  b /= v.snz;
+  const int cls = (int)(b & 7), r = (int)(b >> 3);
+  const int z = v.sz0 + zs, K = v.K, ld = K + 1;
+  const unsigned long long bits = v.wmax[v.r0 + r];
+  const bool fin = w_finite(bits);
+  const double sc = pow2(w_exp(fin ? bits : 0));
+  for (int i = threadIdx.x; i < 8 * K; i += 256) {
+    const int bx = i / K, l = i - bx * K, x = 8 * xs + bx;
+    long long q = 0;
+    if (l < v.d && x < h && fin) {
+      const int64_t I = morton_encode(2 * x + (cls & 1), 2 * y + ((cls >> 1) & 1), 2 * z + (cls >> 2), v.level);
+      q = __double2ll_rn(v.W[(I * v.R + v.r0 + r) * v.d + l] * sc);
+    }
+    s_w[bx * ld + l] = q;
+  }
+  __syncthreads();
+  const int64_t plane = (int64_t)(K / 8) * v.snz * h * h * 8;  // elements of one (mod, r, class)
+  for (int u = threadIdx.x; u < K; u += 256) {
+    const int bx = u & 7, k8 = u >> 3, x = 8 * xs + bx;
+    if (x >= h) continue;
+    const long long* q = s_w + bx * ld + 8 * k8;
+    long long w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w[j] = q[j];
+    __nv_bfloat16* dst = v.planes + (int64_t)(r * 8 + cls) * plane + ((((int64_t)k8 * v.snz + zs) * h + y) * h + x) * 8;
+#pragma unroll
+    for (int i = 0; i < kMods; ++i) {
+      __nv_bfloat162 o[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        o[j] = __floats2bfloat162_rn((float)residue(w[2 * j], i), (float)residue(w[2 * j + 1], i));
+      *reinterpret_cast<uint4*>(dst + (int64_t)i * v.Rc * 8 * plane) = *reinterpret_cast<uint4*>(o);
+    }
+  }
+}
+
+// -------------------------------------------------------- residue GEMMs --
+// Shared-memory descriptor: K-major, no swizzle, version 1.  lbo: bytes from
+// the first 8 terms of a k-step to the next 8; sbo: bytes between 8-row groups.
+__device__ __forceinline__ uint64_t desc_k(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
+         ((uint64_t)1 << 46);
+}
+// D = F32, A and B BF16, both K-major, M = 128
+__device__ __forceinline__ uint32_t idesc_bf16(uint32_t n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
+}
+// the KS k-steps of one offset's chunk; n2: descriptor units between k-steps of B
+template <int KS>
+__device__ __forceinline__ void mma_steps(uint32_t dst, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                          uint32_t n2, uint32_t id, uint32_t acc, uint32_t el) {
+#pragma unroll
+  for (int kk = 0; kk < KS; ++kk)
+    mma_f16_el(dst, alo + kk * (kWinStep >> 4), ahi, blo + kk * n2, bhi, id, kk ? 1u : acc, el);
+}
+
+// One CTA: one modulus, one target tile (128 boxes of a class), one column
+// tile, one right-hand side, one group of (source class, y-shift) windows.
+// Warps 0-7 drain the accumulators, warp 8 streams the operator residues
+// (K-chunk of one offset per stage), warp 9 issues the MMAs, warp 10 loads the
+// windows.  M = 128 boxes, N = Nt columns m', K in chunks of at most 64 terms.
+// Two TMEM accumulators of Nt columns: while one is filled (15 k-steps at
+// most), the other is added to the register sums modulo m.
+__global__ void __launch_bounds__(kThreads, 1)
+k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs a) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int wu = __shfl_sync(0xffffffffu, warp, 0);  // uniform: the roles of warps 8 to 10 run converged
+  const int S = a.stages;
+  const uint32_t sbase = smem_u32(smem);
+  const uint32_t s_stage = sbase + kWins * a.win_b;
+  uint64_t* bars = (uint64_t*)(smem + kWins * a.win_b + (uint32_t)S * a.stage_b);
+  // bfull[8] bempty[8] wfull[2] wempty[2] afull[2] aempty[2]
+  auto bfull = [&](int i) { return smem_u32(&bars[i]); };
+  auto bempty = [&](int i) { return smem_u32(&bars[kMaxStages + i]); };
+  auto wfull = [&](int i) { return smem_u32(&bars[2 * kMaxStages + i]); };
+  auto wempty = [&](int i) { return smem_u32(&bars[2 * kMaxStages + 2 + i]); };
+  auto afull = [&](int i) { return smem_u32(&bars[2 * kMaxStages + 4 + i]); };
+  auto aempty = [&](int i) { return smem_u32(&bars[2 * kMaxStages + 6 + i]); };
+  uint32_t* tslot = (uint32_t*)(bars + 2 * kMaxStages + 8);
+  volatile int* abort = (volatile int*)(tslot + 1);
+
+  const int q = find_level(a, &CrtLv::item0, blockIdx.x);
+  const CrtLv& v = a.lv[q];
+  const int h = v.h, K = v.K, Nt = v.Nt, nchunk = v.nchunk;
+  unsigned b = blockIdx.x - v.item0;
+  const int ntx = (h + kTX - 1) / kTX, nty = (h + kTY - 1) / kTY, ntz = (v.nz + kTZ - 1) / kTZ;
+  const int x0 = kTX * (int)(b % ntx);
+  b /= ntx;
+  const int y0 = kTY * (int)(b % nty);
+  b /= nty;
+  const int z0 = v.z0 + kTZ * (int)(b % ntz);
+  b /= ntz;
+  const int ct = (int)(b & 7);
+  b >>= 3;
+  const int nt = (int)(b % v.NT);
+  b /= v.NT;
+  const int r = (int)(b % v.Rc);
+  b /= v.Rc;
+  const int grp = (int)(b % v.G), mod = (int)(b / v.G);
+  const int w_beg = grp * 24 / v.G, w_end = (grp + 1) * 24 / v.G;  // window = 3 class + y-shift
+
+  if (tid == 0) {
+    for (int i = 0; i < kMaxStages; ++i) {
+      mbar_init(bfull(i), 1);
+      mbar_init(bempty(i), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(wfull(i), 1);
+      mbar_init(wempty(i), 1);
+      mbar_init(afull(i), 1);
+      mbar_init(aempty(i), kDrainWarps);
+    }
+    *abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 8) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                 "r"(512u));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
+
+  if (wu == 8) {
+    // ----------------------------------------- operator residues (B) --
+    const uint32_t el = elect_one();
+    const int64_t tile_b = (int64_t)K * Nt * 2, slot_b = v.NT * tile_b;  // bytes of a column tile, of a slot
+    const char* img = (const char*)v.img + (int64_t)mod * kNumSlots * slot_b + nt * tile_b;
+    const int n0 = v.n0, ks0 = v.ks0, ks1 = v.ks1;
+    const uint32_t stage_b = a.stage_b;
+    int it = 0, st = 0;
+    uint32_t ph = 0, dst = s_stage;
+    bool ok = true;
+    for (int w = w_beg; w < w_end && ok; ++w) {
+      const int cs = w / 3, sy1 = w - 3 * cs;
+      const int mask = combo_mask(ct, cs, sy1);
+      // slot of the shift sx = sz = 0
+      const int sl0 = (2 * (sy1 - 1) + ((cs >> 1) & 1) - ((ct >> 1) & 1) + 3) * 7 + (cs & 1) - (ct & 1) + 3 +
+                      ((cs >> 2) - (ct >> 2) + 3) * 49;
+      const char* src = img + sl0 * slot_b;
+      for (int c = 0; c < nchunk && ok; ++c) {
+        const uint32_t bytes = (uint32_t)(c < n0 ? ks0 : ks1) * 32u * Nt;
+#pragma unroll
+        for (int m = 0; m < 9; ++m)
+          if (((mask >> m) & 1) && ok) {
+            if (it >= S) ok = mbar_wait_ab(bempty(st), ph ^ 1u, a.err, 11, abort);
+            if (ok) {
+              if (el) {
+                mbar_expect_tx(bfull(st), bytes);
+                bulk_g2s(dst, src + (2 * (m % 3 - 1) + 98 * (m / 3 - 1)) * slot_b, bytes, bfull(st));
+              }
+              __syncwarp();
+              ++it;
+              dst += stage_b;
+              if (++st == S) st = 0, ph ^= 1u, dst = s_stage;
+            }
+          }
+        src += bytes;
+      }
+    }
+    drain_fills(it, S, bars, a.err);
+  } else if (wu == 10) {
+    // ------------------------------------------------- windows of W (A) --
+    const uint32_t el = elect_one();
+    int wi = 0;
+    bool ok = true;
+    for (int w = w_beg; w < w_end && ok; ++w) {
+      const int cs = w / 3, sy1 = w - 3 * cs;
+      int k0 = 0;
+      for (int c = 0; c < nchunk; ++c, ++wi) {
+        const int ks = chunk_ksteps(v, c);
+        const int s = wi & 1;
+        if (wi >= kWins && !mbar_wait_ab(wempty(s), ((wi >> 1) - 1) & 1, a.err, 12, abort)) {
+          ok = false;
+          break;
+        }
+        if (el) {
+          mbar_expect_tx(wfull(s), (uint32_t)ks * kWinStep);
+          for (int kk = 0; kk < ks; ++kk)
+            tma_load_5d(sbase + (uint32_t)s * a.win_b + (uint32_t)kk * kWinStep, &maps.m[q], 8 * (x0 - 1),
+                        y0 + sy1 - 1, z0 - 1 - v.sz0, 2 * (k0 + kk), (mod * v.Rc + r) * 8 + cs, wfull(s));
+        }
+        __syncwarp();
+        k0 += ks;
+      }
+    }
+    drain_fills(wi, kWins, bars + 2 * kMaxStages, a.err);
+  } else if (wu == 9) {
+    // ----------------------------------------------------- MMA issuer --
+    const uint32_t el = elect_one();
+    const uint32_t id = idesc_bf16((uint32_t)Nt);
+    const uint64_t dA = desc_k(sbase, kWinRows * 16u, (kTX + 2) * 16u);
+    const uint64_t dB = desc_k(s_stage, (uint32_t)Nt * 16u, 128u);
+    const uint32_t ahi = (uint32_t)(dA >> 32), bhi = (uint32_t)(dB >> 32), n2 = 2u * (uint32_t)Nt;
+    const uint32_t stage16 = a.stage_b >> 4, win16 = a.win_b >> 4;
+    const int n0 = v.n0, ks0 = v.ks0, ks1 = v.ks1;
+    int st = 0, wi = 0, g = 0, acc = 0;
+    uint32_t ph = 0, blo = (uint32_t)dB, dst = tmem;
+    bool ok = true;
+    // the steps of one window whose chunk has KS k-steps, unrolled over its
+    // nine shifts: the start address of each is a constant offset
+    auto window = [&](auto ksc, int mask, uint32_t awin) {
+      constexpr int KS = decltype(ksc)::value;
+#pragma unroll
+      for (int m = 0; m < 9; ++m)
+        if ((mask >> m) & 1) {
+          if (acc + KS > kMaxSteps) {  // this accumulator is full
+            mma_commit_el(afull(g & 1), el);
+            ++g;
+            acc = 0;
+            dst = tmem + (uint32_t)((g & 1) * Nt);
+            if (g >= 2) ok = ok && mbar_wait_ab(aempty(g & 1), ((g >> 1) - 1) & 1, a.err, 14, abort);
+          }
+          ok = ok && mbar_wait_ab(bfull(st), ph, a.err, 15, abort);
+          if (!ok) return;
+          tc_fence_after();
+          mma_steps<KS>(dst, awin + (uint32_t)((m / 3) * (kTX + 2) * kTY + m % 3), ahi, blo, bhi, n2, id,
+                        acc > 0 ? 1u : 0u, el);
+          acc += KS;
+          mma_commit_el(bempty(st), el);
+          blo += stage16;
+          if (++st == S) st = 0, ph ^= 1u, blo = (uint32_t)dB;
+        }
+    };
+    for (int w = w_beg; w < w_end && ok; ++w) {
+      const int mask = combo_mask(ct, w / 3, w % 3);
+      for (int c = 0; c < nchunk && ok; ++c, ++wi) {
+        const int ks = c < n0 ? ks0 : ks1;
+        const int s = wi & 1;
+        ok = mbar_wait_ab(wfull(s), (wi >> 1) & 1, a.err, 13, abort);
+        if (!ok) break;
+        const uint32_t awin = (uint32_t)dA + (s ? win16 : 0u);
+        if (ks == 5) window(std::integral_constant<int, 5>(), mask, awin);
+        else if (ks == 4) window(std::integral_constant<int, 4>(), mask, awin);
+        else if (ks == 3) window(std::integral_constant<int, 3>(), mask, awin);
+        else if (ks == 2) window(std::integral_constant<int, 2>(), mask, awin);
+        else window(std::integral_constant<int, 1>(), mask, awin);
+        if (ok) mma_commit_el(wempty(s), el);
+      }
+    }
+    if (ok) mma_commit_el(afull(g & 1), el);
+  } else if (warp < kDrainWarps) {
+    // -------------------------------------------------- residue sums --
+    // warp w reads TMEM lanes 32 (w % 4) .. and half w / 4 of the columns
+    int ng = 1;
+    {
+      int acc = 0;
+      for (int w = w_beg; w < w_end; ++w) {
+        const int n = __popc(combo_mask(ct, w / 3, w % 3));
+        for (int c = 0; c < nchunk; ++c) {
+          const int ks = chunk_ksteps(v, c);
+          for (int i = 0; i < n; ++i) {
+            if (acc + ks > kMaxSteps) ++ng, acc = 0;
+            acc += ks;
+          }
+        }
+      }
+    }
+    const int quad = warp & 3, half = warp >> 2, nh = Nt / 2;
+    const float fm = (float)crt_mod(mod);
+    const float2 inv2 = make_float2(1.0f / fm, 1.0f / fm), m2 = make_float2(-fm, -fm);
+    const float2 mg = make_float2(12582912.0f, 12582912.0f), ng2 = make_float2(-12582912.0f, -12582912.0f);
+    float2 sum[64];
+#pragma unroll
+    for (int j = 0; j < 64; ++j) sum[j] = make_float2(0.f, 0.f);
+    for (int g = 0; g < ng; ++g) {
+      bool have = mbar_wait_ab(afull(g & 1), (g >> 1) & 1, a.err, 16, abort);
+      have = __all_sync(0xffffffffu, have);
+      if (!have) break;
+      tc_fence_after();
+      const uint32_t t0 = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)((g & 1) * Nt + half * nh);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (16 * j < nh) {
+          float x[16];
+          tmem_ld16(t0 + 16u * j, x);
+          // |x| <= 240 2^16 and |sum| < 2^9: x + sum is an exact integer
+          // below 2^24; minus the nearest multiple of m (1.5 2^23 rounds to
+          // the nearest integer), again exact
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float2 u = __fadd2_rn(make_float2(x[2 * i], x[2 * i + 1]), sum[8 * j + i]);
+            const float2 k = __fadd2_rn(__ffma2_rn(u, inv2, mg), ng2);
+            sum[8 * j + i] = __ffma2_rn(k, m2, u);
+          }
+        }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(aempty(g & 1)) : "memory");
+    }
+    // row = (z, y, x) of the tile: TMEM lane 32 quad + lane
+    const int row = 32 * quad + lane;
+    const int x = x0 + (row & 7), y = y0 + ((row >> 3) & 3), z = z0 + (row >> 5);
+    if (x < h && y < h && z < v.z0 + v.nz) {
+      const int N = v.NT * Nt;
+      int16_t* out = v.res +
+                     ((((((int64_t)mod * v.G + grp) * v.Rc + r) * 8 + ct) * v.nz + (z - v.z0)) * h + y) * (int64_t)h * N +
+                     (int64_t)x * N + nt * Nt + half * nh;
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        if (8 * j < nh) {
+          uint32_t p[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            p[i] = ((uint32_t)(int)sum[4 * j + i].x & 0xffffu) | ((uint32_t)(int)sum[4 * j + i].y << 16);
+          *reinterpret_cast<uint4*>(out + 8 * j) = make_uint4(p[0], p[1], p[2], p[3]);
+        }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 8)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
+}
+
+// -------------------------------------------------------- reconstruction --
+// G / M modulo 1 = sum_i s_i y_i / m_i modulo 1, in 96-bit fixed point (the
+// constants' rounding adds at most 2^-82 of M, G itself is about 2^-10 of M).
+// A warp takes one (column, box) row, a lane two coefficients.
+__global__ void __launch_bounds__(128) k_crt_rebuild(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK kc) {
+  const CrtLv& v = a.lv[find_level(a, &CrtLv::rc0, blockIdx.x)];
+  const int lane = threadIdx.x & 31;
+  const int64_t cells = (int64_t)v.nz * v.h * v.h, rows = cells * 8 * v.Rc;
+  const int64_t row = (int64_t)(blockIdx.x - v.rc0) * 4 + (threadIdx.x >> 5);
+  if (row >= rows) return;
+  const int64_t cell = row % cells;
+  const int cls = (int)((row / cells) & 7), r = v.r0 + (int)(row / (cells * 8));
+  const int x = (int)(cell % v.h), y = (int)((cell / v.h) % v.h), z = v.z0 + (int)(cell / ((int64_t)v.h * v.h));
+  const int64_t I = morton_encode(2 * x + (cls & 1), 2 * y + ((cls >> 1) & 1), 2 * z + (cls >> 2), v.level);
+  const int N = v.NT * v.Nt;
+  const int16_t* res = v.res + row * N;
+  double* g = v.g + (I * v.R + r) * v.d;
+  const unsigned long long bits = v.wmax[r];
+  const bool fin = w_finite(bits);
+  const double ws = fin ? pow2(-w_exp(bits)) : __longlong_as_double(0x7ff8000000000000ll);
+  for (int c = 2 * lane; c < v.d; c += 64) {
+    unsigned long long p[2][3] = {};
+#pragma unroll
+    for (int i = 0; i < kMods; ++i) {
+      const int m = crt_mod(i);
+      const short2 t = *reinterpret_cast<const short2*>(res + (int64_t)i * v.G * rows * N + c);
+      int s0 = t.x, s1 = t.y;
+      if (v.G > 1) {
+        for (int k = 1; k < v.G; ++k) {
+          const short2 u = *reinterpret_cast<const short2*>(res + ((int64_t)i * v.G + k) * rows * N + c);
+          s0 += u.x;
+          s1 += u.y;
+        }
+        s0 %= m;
+        s1 %= m;
+      }
+      // non-negative, and zero for zero: a sum of nothing is exactly 0
+      s0 += s0 < 0 ? m : 0;
+      s1 += s1 < 0 ? m : 0;
+#pragma unroll
+      for (int w = 0; w < 3; ++w) {
+        p[0][w] += (unsigned long long)(unsigned)s0 * kc.k[i][w];
+        p[1][w] += (unsigned long long)(unsigned)s1 * kc.k[i][w];
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      if (c + e >= v.d) break;
+      const unsigned long long p1 = p[e][1] + (p[e][0] >> 32), p2 = p[e][2] + (p1 >> 32);
+      const long long hi = (long long)((p2 << 32) | (p1 & 0xffffffffull));
+      const double G = fma((double)hi, 4294967296.0, (double)(unsigned)p[e][0]);
+      g[c + e] = G * v.colscale[c + e] * ws;
+    }
+  }
+}
+
+// ---------------------------------------------------------- the images --
+// Largest entry and sum of |T| over slots and l for 32 rows m' per block.
+__global__ void __launch_bounds__(1024) k_crt_rowsum(const double* __restrict__ kdT, int d, double* __restrict__ mx,
+                                                     double* __restrict__ l1) {
+  const int mp = blockIdx.x * 32 + threadIdx.x;
+  double s = 0.0, m = 0.0;
+  if (mp < d)
+    for (int64_t i = threadIdx.y; i < (int64_t)kNumSlots * d; i += 32) {
+      const int slot = (int)(i / d);
+      const int dx = slot % 7 - 3, dy = (slot / 7) % 7 - 3, dz = slot / 49 - 3;
+      if (abs(dx) <= 1 && abs(dy) <= 1 && abs(dz) <= 1) continue;
+      const double t = fabs(kdT[i * d + mp]);
+      s += t;
+      m = fmax(m, t);
+    }
+  __shared__ double ss[32][33], sm[32][33];
+  ss[threadIdx.y][threadIdx.x] = s;
+  sm[threadIdx.y][threadIdx.x] = m;
+  __syncthreads();
+  if (threadIdx.y == 0 && mp < d) {
+    for (int k = 1; k < 32; ++k) {
+      s += ss[k][threadIdx.x];
+      m = fmax(m, sm[k][threadIdx.x]);
+    }
+    l1[mp] = s;
+    mx[mp] = m;
+  }
+}
+
+// Exponents a of the rows: l1 2^a < 2^kRowBits and mx 2^a < 2^kEntryBits.
+__global__ void k_crt_rowscale(const double* __restrict__ mx, const double* __restrict__ l1, int d, double mscale,
+                               double* __restrict__ up, double* __restrict__ colscale) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= d) return;
+  int e = 0, e1 = 0;
+  // the sum itself carries rounding; 2^-40 relative covers it
+  frexp(l1[m] * (1.0 + 0x1p-40), &e);
+  frexp(mx[m], &e1);
+  int s = min(kRowBits - e, kEntryBits - e1);
+  s = l1[m] > 0.0 ? max(-900, min(900, s)) : 0;
+  up[m] = pow2(s);
+  colscale[m] = ldexp(mscale, -s);
+}
+
+// One thread per (slot, column tile, k8, n): 8 terms of one row for every modulus.
+__global__ void __launch_bounds__(256) k_crt_image(const double* __restrict__ kdT, int d, int K, int Nt, int NT,
+                                                   const double* __restrict__ up, __nv_bfloat16* __restrict__ img) {
+  const int slot = blockIdx.y;
+  const int64_t tile_e = (int64_t)K * Nt;
+  const int units = NT * (K / 8) * Nt;
+  for (int u = blockIdx.x * 256 + threadIdx.x; u < units; u += gridDim.x * 256) {
+    const int n = u % Nt, k8 = (u / Nt) % (K / 8), nt = u / (Nt * (K / 8));
+    const int mp = nt * Nt + n;
+    long long w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int l = 8 * k8 + j;
+      w[j] = (mp < d && l < d) ? __double2ll_rn(kdT[((int64_t)slot * d + l) * d + mp] * up[mp]) : 0;
+    }
+    __nv_bfloat16* dst = img + ((int64_t)slot * NT + nt) * tile_e + ((int64_t)k8 * Nt + n) * 8;
+#pragma unroll
+    for (int i = 0; i < kMods; ++i) {
+      __nv_bfloat162 o[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        o[j] = __floats2bfloat162_rn((float)residue(w[2 * j], i), (float)residue(w[2 * j + 1], i));
+      *reinterpret_cast<uint4*>(dst + (int64_t)i * kNumSlots * NT * tile_e) = *reinterpret_cast<uint4*>(o);
+    }
+  }
+}
+
+// out[slot]: the ratio of crt_kappa for one offset (0 in the near field).
+__global__ void __launch_bounds__(128) k_crt_kappa(int kern, int d, double lk, const double* __restrict__ X,
+                                                   const double* __restrict__ Y, const double* __restrict__ kdT,
+                                                   double* __restrict__ out) {
+  __shared__ double w[kMaxD];
+  __shared__ double red[2][4];
+  const int slot = blockIdx.x;
+  const int dx = slot % 7 - 3, dy = (slot / 7) % 7 - 3, dz = slot / 49 - 3;
+  for (int l = threadIdx.x; l < d; l += 128)
+    w[l] = fabs(kern_f64(kern, X[3 * l] - Y[0], X[3 * l + 1] - Y[1], X[3 * l + 2] - Y[2]));
+  __syncthreads();
+  double num = 0.0, den = 0.0;
+  const bool far = abs(dx) > 1 || abs(dy) > 1 || abs(dz) > 1;
+  for (int m = threadIdx.x; far && m < d; m += 128) {
+    double s = 0.0;
+    for (int l = 0; l < d; ++l) s += fabs(kdT[((int64_t)slot * d + l) * d + m]) * w[l];
+    num = fmax(num, s);
+    den = fmax(den, fabs(kern_f64(kern, Y[3 * m] - (Y[0] + 2.0 * dx * lk), Y[3 * m + 1] - (Y[1] + 2.0 * dy * lk),
+                                  Y[3 * m + 2] - (Y[2] + 2.0 * dz * lk))));
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    num = fmax(num, __shfl_xor_sync(0xffffffffu, num, o));
+    den = fmax(den, __shfl_xor_sync(0xffffffffu, den, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = num;
+    red[1][threadIdx.x >> 5] = den;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < 4; ++i) {
+      num = fmax(num, red[0][i]);
+      den = fmax(den, red[1][i]);
+    }
+    out[slot] = num > 0.0 ? num / den : 0.0;
+  }
+}
+
+unsigned __int128 crt_product() {
+  unsigned __int128 M = 1;
+  for (int i = 0; i < kMods; ++i) M *= (unsigned)crt_mod(i);
+  return M;
+}
+
+CrtK crt_constants() {
+  CrtK c;
+  for (int i = 0; i < kMods; ++i) {
+    const int m = crt_mod(i);
+    int p = 1;  // M / m_i modulo m_i
+    for (int j = 0; j < kMods; ++j)
+      if (j != i) p = (int)((int64_t)p * crt_mod(j) % m);
+    int y = 1;
+    while ((int64_t)p * y % m != 1) ++y;
+    const unsigned __int128 k = (((unsigned __int128)y << 96) + m / 2) / m;
+    for (int w = 0; w < 3; ++w) c.k[i][w] = (uint32_t)(k >> (32 * w));
+  }
+  return c;
+}
+
+// The scratch of a level is split into columns and slabs of planes beyond this.
+constexpr size_t kScratchLimit = (size_t)4 << 30;
+
+size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
+size_t planes_bytes(const CrtImage& im, int h, int snz, int Rc) {
+  return align256((size_t)kMods * Rc * 8 * snz * h * h * im.K * 2);
+}
+size_t res_bytes(const CrtImage& im, int h, int nz, int Rc, int G) {
+  return align256((size_t)kMods * G * Rc * 8 * nz * h * h * im.NT * im.Nt * 2);
+}
+constexpr int kMaxGroups = 8;
+// offset groups are used only by launches of few tiles: levels below this one
+constexpr int kGroupLevel = 4;
+size_t job_bytes(const CrtImage& im, int level, int nz, int Rc) {
+  const int h = 1 << (level - 1);
+  const int snz = std::min(h, nz + 2);
+  return planes_bytes(im, h, snz, Rc) + res_bytes(im, h, nz, Rc, level < kGroupLevel ? kMaxGroups : 1);
+}
+// columns and planes of one slab of a level within `limit` bytes
+void slab_shape(const CrtImage& im, int level, int R, size_t limit, int* Rc, int* nz) {
+  const int h = 1 << (level - 1);
+  *Rc = R;
+  *nz = h;
+  while (*Rc > 1 && job_bytes(im, level, *nz, *Rc) > limit) *Rc = (*Rc + 1) / 2;
+  while (*nz > kTZ && job_bytes(im, level, *nz, *Rc) > limit) *nz = std::max(kTZ, (*nz / 2 + kTZ - 1) / kTZ * kTZ);
+}
+
+}  // namespace
+
+size_t crt_scratch_bytes(int depth, const CrtImage* const* img, int R) {
+  size_t total = 0, most = 0;
+  for (int k = 2; k <= depth; ++k) {
+    if (!img[k] || !img[k]->img) continue;
+    int Rc, nz;
+    slab_shape(*img[k], k, R, kScratchLimit, &Rc, &nz);
+    const size_t n = job_bytes(*img[k], k, nz, Rc);
+    total += n;
+    most = std::max(most, n);
+  }
+  return std::max(most, std::min(total, kScratchLimit));
+}
+
+void free_crt_image(CrtImage* im) {
+  dfree(im->img);
+  dfree(im->colscale);
+  *im = CrtImage();
+}
+
+eifmm_status build_crt_image(const double* kdT, int d, CrtImage* im, cudaStream_t s) {
+  im->d = d;
+  im->K = (d + 15) / 16 * 16;
+  im->NT = (im->K + 255) / 256;
+  im->Nt = ((im->K / 16 + im->NT - 1) / im->NT) * 16;
+  double* tmp = nullptr;  // largest entry, sum and 2^a of each row
+  eifmm_status rc = dalloc(&tmp, (size_t)3 * d);
+  if (rc == EIFMM_OK) rc = dalloc(&im->colscale, d);
+  const size_t e = (size_t)kMods * kNumSlots * im->NT * im->K * im->Nt;
+  if (rc == EIFMM_OK) rc = dmalloc(&im->img, e * sizeof(__nv_bfloat16));
+  if (rc == EIFMM_OK) {
+    k_crt_rowsum<<<(d + 31) / 32, dim3(32, 32), 0, s>>>(kdT, d, tmp, tmp + d);
+    count_launch();
+    const double mscale = std::ldexp((double)crt_product(), -96);
+    k_crt_rowscale<<<(d + 127) / 128, 128, 0, s>>>(tmp, tmp + d, d, mscale, tmp + 2 * d, im->colscale);
+    count_launch();
+    const int units = im->NT * (im->K / 8) * im->Nt;
+    k_crt_image<<<dim3((units + 255) / 256, kNumSlots), 256, 0, s>>>(kdT, d, im->K, im->Nt, im->NT, tmp + 2 * d,
+                                                                     (__nv_bfloat16*)im->img);
+    count_launch();
+    // other streams may read the image as soon as this returns
+    if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
+      set_error("building the residue images of the M2L operators failed");
+      rc = EIFMM_ECUDA;
+    }
+  }
+  dfree(tmp);
+  if (rc != EIFMM_OK) free_crt_image(im);
+  return rc;
+}
+
+eifmm_status crt_kappa(int kern, const LevelOps& v, double lk, double* kappa, cudaStream_t s) {
+  double* out = nullptr;
+  EIFMM_TRY(dalloc(&out, kNumSlots));
+  k_crt_kappa<<<kNumSlots, 128, 0, s>>>(kern, v.d, lk, v.X, v.Y, v.kdT, out);
+  count_launch();
+  double h[kNumSlots];
+  const bool ok = cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
+                  cudaStreamSynchronize(s) == cudaSuccess;
+  dfree(out);
+  if (!ok) {
+    set_error("the amplification of the M2L operators could not be computed");
+    return EIFMM_ECUDA;
+  }
+  *kappa = *std::max_element(h, h + kNumSlots);
+  return EIFMM_OK;
+}
+
+eifmm_status launch_m2l_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t buf_bytes,
+                            unsigned long long* wmax, int nsm, int* err, cudaStream_t s) {
+  auto encode = encode_fn();
+  if (!encode) {
+    set_error("cuTensorMapEncodeTiled is not available from the driver");
+    return EIFMM_ECUDA;
+  }
+  static const CrtK kc = crt_constants();
+  static bool attr[64] = {};
+  int dev = 0;
+  EIFMM_CUDA(cudaGetDevice(&dev));
+  if (dev >= 64 || !attr[dev]) {
+    EIFMM_CUDA(cudaFuncSetAttribute(k_crt_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
+    if (dev < 64) attr[dev] = true;
+  }
+  EIFMM_CUDA(cudaMemsetAsync(wmax, 0, sizeof(unsigned long long) * (kMaxLevel + 1) * R, s));
+  // slabs of all jobs, largest levels first; consecutive ones that fit the
+  // scratch together share their launches
+  std::vector<CrtLv> todo;
+  for (int j = njobs - 1; j >= 0; --j) {
+    const CrtJob& b = jobs[j];
+    int Rc, nz;
+    slab_shape(*b.img, b.level, R, kScratchLimit, &Rc, &nz);
+    const int h = 1 << (b.level - 1);
+    for (int r0 = 0; r0 < R; r0 += Rc)
+      for (int z0 = 0; z0 < h; z0 += nz) {
+        CrtLv v = {};
+        v.level = b.level;
+        v.d = b.img->d;
+        v.K = b.img->K;
+        v.Nt = b.img->Nt;
+        v.NT = b.img->NT;
+        v.h = h;
+        v.z0 = z0;
+        v.nz = std::min(nz, h - z0);
+        v.sz0 = std::max(0, z0 - 1);
+        v.snz = std::min(h, z0 + v.nz + 1) - v.sz0;
+        v.r0 = r0;
+        v.Rc = std::min(Rc, R - r0);
+        v.R = R;
+        split_chunks(&v);
+        v.W = b.W;
+        v.g = b.g;
+        v.img = (const __nv_bfloat16*)b.img->img;
+        v.colscale = b.img->colscale;
+        v.wmax = wmax + (size_t)b.level * R;
+        todo.push_back(v);
+      }
+  }
+  for (size_t i0 = 0; i0 < todo.size();) {
+    CrtArgs a = {};
+    CrtMaps maps = {};
+    a.err = err;
+    size_t off = 0, i1 = i0;
+    int64_t items = 0;
+    auto tiles = [](const CrtLv& v) {
+      return (int64_t)((v.h + kTX - 1) / kTX) * ((v.h + kTY - 1) / kTY) * ((v.nz + kTZ - 1) / kTZ) * 8 * v.NT * v.Rc *
+             kMods;
+    };
+    for (; i1 < todo.size() && a.nlev < kMaxLv; ++i1) {
+      const CrtLv& v = todo[i1];
+      const size_t need = planes_bytes(CrtImage{nullptr, nullptr, 0.0, v.d, v.K, v.Nt, v.NT}, v.h, v.snz, v.Rc) +
+                          res_bytes(CrtImage{nullptr, nullptr, 0.0, v.d, v.K, v.Nt, v.NT}, v.h, v.nz, v.Rc,
+                                    v.level < kGroupLevel ? kMaxGroups : 1);
+      if (a.nlev > 0 && off + need > buf_bytes) break;
+      if (need > buf_bytes) {
+        set_error("residue M2L: scratch too small");
+        return EIFMM_EINVAL;
+      }
+      off += need;
+      items += tiles(v);
+      a.lv[a.nlev++] = v;
+    }
+    off = 0;
+    unsigned it = 0, pl = 0, rb = 0, mx = 0;
+    uint32_t stage = 0, win = 0;
+    size_t pl_smem = 0;
+    for (int q = 0; q < a.nlev; ++q) {
+      CrtLv& v = a.lv[q];
+      const CrtImage im{nullptr, nullptr, 0.0, v.d, v.K, v.Nt, v.NT};
+      // a launch of few tiles: the windows of the coarse levels' tiles are
+      // split into groups until the CTAs cover four waves
+      v.G = 1;
+      if (v.level < kGroupLevel)
+        while (v.G < kMaxGroups && items * v.G < 4 * (int64_t)nsm) v.G *= 2;
+      v.planes = (__nv_bfloat16*)((char*)buf + off);
+      off += planes_bytes(im, v.h, v.snz, v.Rc);
+      v.res = (int16_t*)((char*)buf + off);
+      off += res_bytes(im, v.h, v.nz, v.Rc, v.G);
+      v.item0 = it;
+      v.pl0 = pl;
+      v.rc0 = rb;
+      v.mx0 = mx;
+      it += (unsigned)(tiles(v) * v.G);
+      pl += (unsigned)((int64_t)((v.h + 7) / 8) * v.h * v.snz * 8 * v.Rc);
+      rb += (unsigned)(((int64_t)v.nz * v.h * v.h * 8 * v.Rc + 3) / 4);
+      mx += (unsigned)((((int64_t)1 << (3 * v.level)) * v.d + kMaxPer - 1) / kMaxPer * v.Rc);
+      const uint32_t ks = (uint32_t)std::max(v.ks0, v.nchunk > v.n0 ? v.ks1 : 0);
+      stage = std::max(stage, ks * 32u * (uint32_t)v.Nt);
+      win = std::max(win, ks * kWinStep);
+      pl_smem = std::max(pl_smem, (size_t)8 * (v.K + 1) * sizeof(long long));
+      const cuuint64_t hh = (cuuint64_t)v.h;
+      cuuint64_t dims[5] = {8 * hh, hh, (cuuint64_t)v.snz, (cuuint64_t)v.K / 8, (cuuint64_t)kMods * v.Rc * 8};
+      cuuint64_t strides[4] = {16 * hh, 16 * hh * hh, 16 * hh * hh * v.snz, 16 * hh * hh * v.snz * (v.K / 8)};
+      cuuint32_t box[5] = {8 * (kTX + 2), kTY, kTZ + 2, 2, 1};
+      cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+      const CUresult r = encode(&maps.m[q], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, v.planes, dims, strides, box, estr,
+                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+      if (r != CUDA_SUCCESS) {
+        set_error("cuTensorMapEncodeTiled failed with code " + std::to_string((int)r));
+        return EIFMM_ECUDA;
+      }
+    }
+    a.stage_b = stage;
+    a.win_b = win;
+    a.stages = (int)std::min<uint32_t>(kMaxStages, (kSmemMax - 1024 - kSmemBars - kWins * win) / stage);
+    const uint32_t smem = 1024 + kSmemBars + kWins * win + (uint32_t)a.stages * stage;
+    // a level that runs in several slabs needs its maximum once; repeating it
+    // per slab gives the same value
+    k_crt_max<<<mx, 256, 0, s>>>(a);
+    EIFMM_CHECK_LAUNCH();
+    k_crt_planes<<<pl, 256, pl_smem, s>>>(a);
+    EIFMM_CHECK_LAUNCH();
+    k_crt_gemm<<<it, kThreads, smem, s>>>(maps, a);
+    EIFMM_CHECK_LAUNCH();
+    k_crt_rebuild<<<rb, 128, 0, s>>>(a, kc);
+    EIFMM_CHECK_LAUNCH();
+    i0 = i1;
+  }
+  return EIFMM_OK;
+}
+
+}  // namespace eifmm

@@ -29,65 +29,12 @@
 
 #include "internal.h"
 #include "m2l_tc.h"
+#include "tc_ptx.cuh"
 
 namespace eifmm {
 namespace {
 
 constexpr int kRows = 128;
-constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t a, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(a), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ uint32_t mbar_try(uint32_t a, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(a), "r"(parity)
-      : "memory");
-  return ok;
-}
-// Bounded wait; returns false (and records `code`) after `limit` cycles.
-__device__ __forceinline__ bool mbar_wait_lim(uint32_t a, uint32_t parity, int* err, int code, long long limit) {
-  const long long t0 = clock64();
-  while (!mbar_try(a, parity)) {
-    if (clock64() - t0 > limit) {
-      atomicExch(err, code);
-      return false;
-    }
-  }
-  return true;
-}
-__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, int* err, int code) {
-  return mbar_wait_lim(a, parity, err, code, kWaitCycles);
-}
-
-// The producer's last act: every copy it issued has landed (each stage's
-// last fill completed its phase) before the CTA may exit, also after an
-// abort.  it = fills issued so far, ring of `stages`.  Bounded like every
-// wait.
-__device__ __forceinline__ void drain_fills(int it, int stages, const uint64_t* bars_full, int* err) {
-  for (int k = 0; k < stages && k < it; ++k) {
-    const int i = it - 1 - k;  // a recent fill
-    mbar_wait(smem_u32(&bars_full[i % stages]), (uint32_t)((i / stages) & 1), err, 5);
-  }
-}
-
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(mbar)
-      : "memory");
-}
 __device__ __forceinline__ void cp16(uint32_t dst, const void* src, uint32_t src_bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
@@ -97,13 +44,6 @@ __device__ __forceinline__ void cp_wait0() { asm volatile("cp.async.wait_group 0
 __device__ __forceinline__ void fence_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row atoms of
 // 1024 bytes stacked along M/N (SBO = 1024), version 1 (sm_100 family).
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
@@ -155,23 +95,6 @@ __device__ __forceinline__ void issue_chunk(uint32_t dacc, uint64_t da, uint64_t
       mma<TF32>(dacc, ad, bd, id_lo, acc);
       if (wide) mma<TF32>(dacc + 256, ad, bd + 2048u, id_hi, acc);
     }
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t mbar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-               : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // Template parameter TF32 selects kind::tf32 (4-byte elements) instead of
@@ -367,15 +290,6 @@ k_m2l_tc(M2LTcArgs a) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)a.tmem_cols));
 }
 
-__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2,
-                                            int c3, int c4, uint32_t mbar) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(mbar)
-      : "memory");
-}
-
 // TMA variant.  What is stored per parity class on a grid,
 // [plane][class][Z][Y][X*R + r][dp] with (X, Y, Z) = box coordinates / 2, so
 // the 128 source rows of a tile for one offset form a regular box of that
@@ -564,21 +478,6 @@ constexpr int kT2Rows = 256;
 constexpr int kT2Stages = 2;
 constexpr int kSegOffsets = 4;
 constexpr int kT2Threads = 320;
-
-// Bounded wait that also gives up when another role has set *abort.
-__device__ __forceinline__ bool mbar_wait_ab(uint32_t a, uint32_t parity, int* err, int code,
-                                             volatile int* abort) {
-  const long long t0 = clock64();
-  while (!mbar_try(a, parity)) {
-    if (*abort) return false;
-    if (clock64() - t0 > kWaitCycles) {
-      atomicExch(err, code);
-      *abort = 1;
-      return false;
-    }
-  }
-  return true;
-}
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   uint32_t r[32];
@@ -1367,11 +1266,7 @@ bool m2l_tma_block(int R, int* bx, int* by, int* bz) {
   return true;
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn encode_fn() {
+EncodeTiledFn encode_fn() {
   static EncodeTiledFn fn = nullptr;
   if (!fn) {
     void* p = nullptr;

@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "m2l_crt.h"
 #include "solve.cuh"
 
 namespace eifmm {
@@ -279,6 +280,8 @@ void free_ops(Ops* ops) {
     dfree(v.X32);
     dfree(v.kd_img);
     dfree(v.kscale);
+    free_crt_image(&v.crt);
+    free_crt_image(&v.crtc);
     dfree(v.U);
     dfree(v.Ct);
     dfree(v.kd32);

@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "m2l_crt.h"
 #include "solve.cuh"
 
 namespace eifmm {
@@ -228,6 +229,7 @@ int sarcmp_rank(const std::vector<double>& s, double eps, int* r_i, int* r_ii) {
 void free_compression(LevelOps& v) {
   dfree(v.U);
   dfree(v.Ct);
+  free_crt_image(&v.crtc);
   v.U = nullptr;
   v.Ct = nullptr;
   v.r = 0;
@@ -309,10 +311,11 @@ eifmm_status compress_ops(Ops* ops, double eps, cudaStream_t s) {
 
 // Step 4 at level k with the compressed operators, on the FP64 arrays of
 // the FP64 far field: What = Delta W into Wh[k], w~ = What U into tmp,
-// g~ = sum C^delta w~ into Wh[k] (FP32-pair arithmetic or FP64, as the
-// uncompressed M2L of the same path), g = g~ U^t.
+// g~ = sum C^delta w~ into Wh[k] (residues on the tensor cores, FP32 pairs or
+// FP64, as the uncompressed M2L), g = g~ U^t.
 
-eifmm_status m2l_compressed(Workspace& ws, const Ops* ops, int k, int R, bool pair, cudaStream_t s) {
+eifmm_status m2l_compressed(Workspace& ws, const Ops* ops, int k, int R, bool fp64, bool pair,
+                            cudaStream_t s) {
   const LevelOps& v = ops->lv[k];
   const int d = v.d, r = v.r;
   const int64_t rows = ((int64_t)1 << (3 * k)) * R;
@@ -322,10 +325,14 @@ eifmm_status m2l_compressed(Workspace& ws, const Ops* ops, int k, int R, bool pa
   EIFMM_TRY((launch_delta_batch<double, double, double, 0>(b, false, s)));
   double* wt = (double*)ws.tmp;  // rows x r
   EIFMM_TRY(gemm64(false, rows, r, d, ws.Wh[k], d, v.U, r, wt, r, s));
-  if (pair)
+  if (!fp64 && v.crtc.img && ws.crt_bytes > 0) {
+    const CrtJob job{k, &v.crtc, wt, ws.Wh[k]};
+    EIFMM_TRY(launch_m2l_crt(1, &job, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
+  } else if (pair) {
     EIFMM_TRY(launch_m2l_df(k, r, R, v.Ct, ops->d_slot_lists, wt, ws.Wh[k], ws.part64, ws.part64_cap, ws.nsm, s));
-  else
+  } else {
     EIFMM_TRY(launch_m2l64(k, r, R, v.Ct, ops->d_slot_lists, wt, ws.Wh[k], ws.part64, ws.part64_cap, ws.nsm, s));
+  }
   EIFMM_TRY(gemm64(true, rows, d, r, ws.Wh[k], r, v.U, r, ws.g[k], d, s));
   return EIFMM_OK;
 }
