@@ -72,6 +72,9 @@ void free_workspace(Workspace* ws) {
   dfree(ws->part64);
   ws->part64 = nullptr;
   ws->part64_cap = 0;
+  dfree(ws->fx_src);
+  dfree(ws->fx_tgt);
+  ws->fx_src = ws->fx_tgt = nullptr;
   dfree(ws->crt_buf);
   dfree(ws->crt_max);
   ws->crt_buf = nullptr;
@@ -235,6 +238,10 @@ eifmm_status ensure_workspace(Tree* t, const Ops* ops, int R, int prec) {
     ws.part64_cap = need;
     EIFMM_TRY(dalloc(&ws.crt_max, (size_t)(kMaxLevel + 1) * R));
     EIFMM_TRY(alloc_wait_error(&ws));
+    if (fx_usable((int)ops->kern, t->L)) {
+      EIFMM_TRY(dalloc(&ws.fx_src, (size_t)3 * std::max<int64_t>(t->src.n, 1)));
+      if (!t->same) EIFMM_TRY(dalloc(&ws.fx_tgt, (size_t)3 * std::max<int64_t>(t->tgt.n, 1)));
+    }
   } else {
     EIFMM_TRY(alloc_mixed_workspace(t, ops, R));
   }

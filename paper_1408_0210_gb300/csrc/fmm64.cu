@@ -41,14 +41,12 @@ __global__ void k_gather_sigma(const double* __restrict__ sigma, int64_t ld,
 }
 
 // Step 1: W_m^I = sum_{y_j in I} sigma_j K(x_m^{I_0}, y_j - c_I).
-template <int KERN>
 __global__ void __launch_bounds__(TPB)
-k_p2m64(int kern_rt, const int32_t* __restrict__ leaves, const int32_t* __restrict__ off,
+k_p2m64(int kern, const int32_t* __restrict__ leaves, const int32_t* __restrict__ off,
         const double* __restrict__ px, const double* __restrict__ py,
         const double* __restrict__ pz, const double* __restrict__ sig, int64_t n,
         int R, int depth, double lo0, double lo1, double lo2, double lk,
         const double* __restrict__ X, int d, double* __restrict__ W) {
-  const int kern = KERN >= 0 ? KERN : kern_rt;
   __shared__ double sz[3][TPB];
   __shared__ double ss[RC][TPB];
   const int b = leaves[blockIdx.x];
@@ -307,16 +305,14 @@ k_m2l_df(int level, int d, int R, const double* __restrict__ kdT, const int* __r
 
 // Step 7 + sum + un-permute: f(x_i) = sum_l' K(x_i - c_I, y_l'^{I_0}) lhat_l'
 // + f_N(x_i), written to the caller's original order.
-template <int KERN>
 __global__ void __launch_bounds__(TPB)
-k_l2p64(int kern_rt, const int32_t* __restrict__ leaves, const int32_t* __restrict__ off,
+k_l2p64(int kern, const int32_t* __restrict__ leaves, const int32_t* __restrict__ off,
         const int32_t* __restrict__ perm, const double* __restrict__ px,
         const double* __restrict__ py, const double* __restrict__ pz, int64_t n,
         int R, int depth, double lo0, double lo1, double lo2, double lk,
         const double* __restrict__ X, int d, const double* __restrict__ lh,
         const double* __restrict__ fnear, double* __restrict__ ffar,
         double* __restrict__ f, int64_t ld_f) {
-  const int kern = KERN >= 0 ? KERN : kern_rt;
   extern __shared__ double sm[];  // X (3d) then lhat (RC * d)
   double* sX = sm;
   double* sl = sm + 3 * d;
@@ -351,15 +347,13 @@ k_l2p64(int kern_rt, const int32_t* __restrict__ leaves, const int32_t* __restri
 }
 
 // Near field f_N(x_i) = sum over the 27 neighbouring leaves, FP64.
-template <int KERN>
 __global__ void __launch_bounds__(TPB)
-k_p2p64(int kern_rt, const int32_t* __restrict__ leaves, const int32_t* __restrict__ toff,
+k_p2p64(int kern, const int32_t* __restrict__ leaves, const int32_t* __restrict__ toff,
         const double* __restrict__ tx, const double* __restrict__ ty,
         const double* __restrict__ tz, int64_t nt, const int32_t* __restrict__ soff,
         const double* __restrict__ sx, const double* __restrict__ sy,
         const double* __restrict__ sz, const double* __restrict__ sig, int64_t ns,
         int R, int depth, int exclude_self, double* __restrict__ fnear) {
-  const int kern = KERN >= 0 ? KERN : kern_rt;
   __shared__ double s[3][TPB];
   __shared__ double ssg[RC][TPB];
   const int b = leaves[blockIdx.x];
@@ -463,14 +457,9 @@ eifmm_status launch_p2p64(const Tree* t, int kern, const double* sig, int R, dou
   const PointSet& T = t->tgt;
   const PointSet& S = t->src;
   if (T.n_nonempty == 0) return EIFMM_OK;
-  if (kern == EIFMM_KERNEL_INV_R)
-    k_p2p64<EIFMM_KERNEL_INV_R><<<T.n_nonempty, TPB, 0, s>>>(
-        kern, T.nonempty, T.leaf_off, T.x, T.y, T.z, T.n, S.leaf_off, S.x, S.y, S.z, sig, S.n, R,
-        t->depth, t->exclude_self, fnear);
-  else
-    k_p2p64<-1><<<T.n_nonempty, TPB, 0, s>>>(kern, T.nonempty, T.leaf_off, T.x, T.y, T.z, T.n,
-                                             S.leaf_off, S.x, S.y, S.z, sig, S.n, R, t->depth,
-                                             t->exclude_self, fnear);
+  if (t->ws.fx_src) return launch_p2p_fx(t, R, fnear, s);
+  k_p2p64<<<T.n_nonempty, TPB, 0, s>>>(kern, T.nonempty, T.leaf_off, T.x, T.y, T.z, T.n, S.leaf_off, S.x, S.y, S.z,
+                                       sig, S.n, R, t->depth, t->exclude_self, fnear);
   EIFMM_CHECK_LAUNCH();
   return EIFMM_OK;
 }
@@ -481,7 +470,7 @@ static void record(Workspace& ws, int i, cudaStream_t s) {
 }
 
 // Step 4 of level k on FP64 arrays [box R + r][d]: the operator stack kdT
-// ([343][l][m'], d x d) applied by FP32-pair arithmetic or in FP64.
+// ([343][l][m'], d x d) applied by FP32-pair arithmetic or on the FP64 pipes.
 // Offset groups of the FP64 and pair-arithmetic M2L: a coarse level has few
 // blocks (8 to 64 at levels 2 and 3), each walking all 189 offsets, so the
 // offset list is split until the blocks cover two waves of the SMs (at most
@@ -554,6 +543,7 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   const double lk = t->L * ldexp(1.0, -(kap + 1));
   record(ws, 0, s);
   EIFMM_TRY(launch_gather_sigma(sigma, ld_sigma, S, R, ws.sig, near32 ? ws.sig32 : nullptr, s));
+  if (ws.fx_src) EIFMM_TRY(launch_fx_points(t, s));
   // near field on the side stream, concurrent with the far field (on the
   // caller's stream, before it, with the single-stream option)
   EIFMM_CUDA(cudaEventRecord(ws.ev_fork, s));
@@ -568,15 +558,11 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   // step 1
   const LevelOps& vl = ops->lv[kap];
   EIFMM_CUDA(cudaMemsetAsync(ws.W[kap], 0, sizeof(double) * ((size_t)1 << (3 * kap)) * R * vl.d, s));
-  if (S.n_nonempty > 0) {
-    if (kern == EIFMM_KERNEL_INV_R)
-      k_p2m64<EIFMM_KERNEL_INV_R><<<S.n_nonempty, TPB, 0, s>>>(
-          kern, S.nonempty, S.leaf_off, S.x, S.y, S.z, ws.sig, S.n, R, kap, t->lo[0], t->lo[1],
-          t->lo[2], lk, vl.X, vl.d, ws.W[kap]);
-    else
-      k_p2m64<-1><<<S.n_nonempty, TPB, 0, s>>>(kern, S.nonempty, S.leaf_off, S.x, S.y, S.z, ws.sig,
-                                               S.n, R, kap, t->lo[0], t->lo[1], t->lo[2], lk, vl.X,
-                                               vl.d, ws.W[kap]);
+  if (ws.fx_src) {
+    EIFMM_TRY(launch_p2m_fx(t, vl, R, ws.W[kap], s));
+  } else if (S.n_nonempty > 0) {
+    k_p2m64<<<S.n_nonempty, TPB, 0, s>>>(kern, S.nonempty, S.leaf_off, S.x, S.y, S.z, ws.sig, S.n, R, kap, t->lo[0],
+                                         t->lo[1], t->lo[2], lk, vl.X, vl.d, ws.W[kap]);
     EIFMM_CHECK_LAUNCH();
   }
   record(ws, 1, s);
@@ -641,16 +627,12 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   // step 7 + near field + un-permute
   EIFMM_CUDA(cudaStreamWaitEvent(s, ws.ev_join, 0));
   record(ws, 7, s);
-  if (T.n_nonempty > 0) {
+  if (ws.fx_src) {
+    EIFMM_TRY(launch_l2p_fx(t, vl, R, f, ld_f, s));
+  } else if (T.n_nonempty > 0) {
     const size_t sm = (size_t)(3 * vl.d + RC * vl.d) * sizeof(double);
-    if (kern == EIFMM_KERNEL_INV_R)
-      k_l2p64<EIFMM_KERNEL_INV_R><<<T.n_nonempty, TPB, sm, s>>>(
-          kern, T.nonempty, T.leaf_off, T.perm, T.x, T.y, T.z, T.n, R, kap, t->lo[0], t->lo[1],
-          t->lo[2], lk, vl.X, vl.d, ws.lh, ws.fnear, ws.ffar, f, ld_f);
-    else
-      k_l2p64<-1><<<T.n_nonempty, TPB, sm, s>>>(kern, T.nonempty, T.leaf_off, T.perm, T.x, T.y, T.z,
-                                                T.n, R, kap, t->lo[0], t->lo[1], t->lo[2], lk, vl.X,
-                                                vl.d, ws.lh, ws.fnear, ws.ffar, f, ld_f);
+    k_l2p64<<<T.n_nonempty, TPB, sm, s>>>(kern, T.nonempty, T.leaf_off, T.perm, T.x, T.y, T.z, T.n, R, kap, t->lo[0],
+                                          t->lo[1], t->lo[2], lk, vl.X, vl.d, ws.lh, ws.fnear, ws.ffar, f, ld_f);
     EIFMM_CHECK_LAUNCH();
   }
   record(ws, 8, s);

@@ -68,6 +68,7 @@ struct LevelOps {
   double eps_est = 0;
   double* X = nullptr;     // d x 3, x_m^{I_0^k}
   double* Y = nullptr;     // d x 3, y_l^{J_0^k}
+  long long* Xq = nullptr; // X in units of 2^-fx_box_exponent(L) (inv_fx.cuh)
   double* G_rm = nullptr;  // Gamma row-major
   double* B_rm = nullptr;  // B row-major
   double* m2mT = nullptr;  // [8][q < d_{k+1}][m < d]: (K_M2M^i)^t, levels 2..depth-1
@@ -199,6 +200,8 @@ struct Workspace {
   void* blas_ws = nullptr;      // the library GEMMs' workspace of this tree (kXferBlasWorkspace bytes)
   double* sig = nullptr;        // sorted sigma, n_src x R (col-major, ld n_src)
   float* sig32 = nullptr;
+  long long* fx_src = nullptr;  // integer coordinates of the sources (x, y, z), FP64 far field of 1/r
+  long long* fx_tgt = nullptr;  // and of the targets where they are another set
   double* fnear = nullptr;      // n_tgt x R, sorted order
   double* ffar = nullptr;       // n_tgt x R, sorted order (debug only)
   float* gsym = nullptr;        // 13 x n: pair-symmetric near-field partials (R = 1, targets = sources)
@@ -248,6 +251,15 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma,
                        int64_t ld_sigma, int R, double* f, int64_t ld_f,
                        cudaStream_t s, bool near32 = false,
                        bool pair_m2l = false);
+// Point kernels of 1/r in FP64 on integer coordinates (point64.cu)
+bool fx_usable(int kern, double L);
+int fx_point_exponent(double L, int depth);
+int fx_box_exponent(double L);
+eifmm_status launch_to_fx(const double* x, int64_t n, int K, long long* q, cudaStream_t s);
+eifmm_status launch_fx_points(const Tree* t, cudaStream_t s);
+eifmm_status launch_p2m_fx(const Tree* t, const LevelOps& v, int R, double* W, cudaStream_t s);
+eifmm_status launch_l2p_fx(const Tree* t, const LevelOps& v, int R, double* f, int64_t ld_f, cudaStream_t s);
+eifmm_status launch_p2p_fx(const Tree* t, int R, double* fnear, cudaStream_t s);
 eifmm_status launch_p2p32(const Tree* t, int kern, const float* sig32, int R,
                           double* fnear, cudaStream_t s, bool accurate, float* gsym = nullptr);
 // Element format of the tensor-core M2L operand planes.

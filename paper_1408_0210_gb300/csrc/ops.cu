@@ -205,6 +205,10 @@ eifmm_status assemble_ops(Ops* ops, cudaStream_t s) {
         kern, v.d, lk, v.Y, v.kdT);
     EIFMM_CHECK_LAUNCH();
     EIFMM_TRY(to_f32(v.X, &v.X32, (int64_t)3 * v.d, s));
+    if (fx_usable(kern, ops->L)) {
+      EIFMM_TRY(dalloc(&v.Xq, (size_t)3 * v.d));
+      EIFMM_TRY(launch_to_fx(v.X, 3 * v.d, fx_box_exponent(ops->L), v.Xq, s));
+    }
     // Delta: Gamma then B^t; Delta^t: B then Gamma^t (reversed order)
     const int nb = (v.d + 31) / 32;
     const int64_t nt = delta_tiles_elems(v.d);
@@ -272,7 +276,7 @@ eifmm_status assemble_ops(Ops* ops, cudaStream_t s) {
 void free_ops(Ops* ops) {
   for (int k = 0; k <= kMaxLevel; ++k) {
     LevelOps& v = ops->lv[k];
-    dfree(v.X); dfree(v.Y); dfree(v.G_rm); dfree(v.B_rm);
+    dfree(v.X); dfree(v.Y); dfree(v.Xq); dfree(v.G_rm); dfree(v.B_rm);
     dfree(v.m2mT); dfree(v.l2lT); dfree(v.kdT); dfree(v.m2mT32); dfree(v.l2lT32);
     dfree(v.m2m); dfree(v.l2l); dfree(v.m2m32); dfree(v.l2l32); dfree(v.m2m_cb); dfree(v.l2l_cb);
     for (int o = 0; o < 4; ++o) { dfree(v.dt64[o]); dfree(v.dt32[o]); }
