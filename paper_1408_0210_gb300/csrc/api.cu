@@ -147,37 +147,56 @@ eifmm_status alloc_wait_error(Workspace* ws) {
   return EIFMM_OK;
 }
 
-// Residue images of the M2L operators of levels 2..depth, built once per
-// operator set and ready for every stream on return.  A level whose image does
-// not fit the device's memory stays without one (its M2L runs on the FP32 or
-// FP64 pipes).  Several trees of one operator set may come here at the same time.
+// Residue images of the operators of levels 2..depth, built once per
+// operator set and ready for every stream on return.  An operator whose
+// image does not fit the device's memory stays without one (the step runs on
+// the FP32 or FP64 pipes).  Several trees of one operator set may come here at the same time.
 static std::mutex g_crt_mu;
-eifmm_status ensure_crt_images(Ops* ops, int depth, cudaStream_t s) {
+eifmm_status ensure_crt_images(Ops* ops, int depth, bool m2l, cudaStream_t s) {
   std::lock_guard<std::mutex> lock(g_crt_mu);
+  auto build = [&](CrtImage* im, const double* T, int nslots, int dl, int d) {
+    if (im->img || dl < kCrtMinRank || d < kCrtMinRank) return EIFMM_OK;
+    const eifmm_status rc = build_crt_image(T, nslots, dl, d, im, s);
+    return rc == EIFMM_ENOMEM ? EIFMM_OK : rc;
+  };
   for (int k = 2; k <= depth; ++k) {
     LevelOps& v = ops->lv[k];
-    const bool c = ops->compressed && v.r > 0;
-    CrtImage& im = c ? v.crtc : v.crt;
-    const int d = c ? v.r : v.d;
-    if (im.img || d < kCrtMinRank) continue;
-    const eifmm_status rc = build_crt_image(c ? v.Ct : v.kdT, d, &im, s);
-    if (rc == EIFMM_ENOMEM) continue;
-    EIFMM_TRY(rc);
-    if (!c) EIFMM_TRY(crt_kappa((int)ops->kern, v, ops->L * ldexp(1.0, -(k + 1)), &im.kappa, s));
+    if (k < depth) EIFMM_TRY(build(&v.crt_m2m, v.m2mT, 8, ops->lv[k + 1].d, v.d));
+    if (k > 2) EIFMM_TRY(build(&v.crt_l2l, v.l2lT, 8, ops->lv[k - 1].d, v.d));
+    if (k == depth && v.d >= kCrtMinRank && !v.crt_dt.img && !v.crt_dt.refused) {
+      const eifmm_status rc = build_crt_delta_image(v, &v.crt_dt, s);
+      if (rc != EIFMM_OK && rc != EIFMM_ENOMEM) return rc;
+    }
+    if (!m2l) continue;
+    if (ops->compressed && v.r > 0) {
+      EIFMM_TRY(build(&v.crtc, v.Ct, kNumSlots, v.r, v.r));
+    } else if (!v.crt.img) {
+      EIFMM_TRY(build(&v.crt, v.kdT, kNumSlots, v.d, v.d));
+      if (v.crt.img) EIFMM_TRY(crt_kappa((int)ops->kern, v, ops->L * ldexp(1.0, -(k + 1)), &v.crt.kappa, s));
+    }
   }
   return EIFMM_OK;
 }
 
-// Images and scratch of the residue M2L for an evaluation with the FP64 far
-// field.  Without room for the scratch crt_bytes stays 0 and the M2L runs on
-// the FP32 or FP64 pipes.
+// Images and scratch of the residue products for an evaluation with the FP64
+// far field.  Without room for the scratch crt_bytes stays 0 and those steps
+// run on the FP32 or FP64 pipes.
 static eifmm_status ensure_crt(Tree* t, Ops* ops, int R, cudaStream_t s) {
   Workspace& ws = t->ws;
-  EIFMM_TRY(ensure_crt_images(ops, t->depth, s));
-  const CrtImage* im[kMaxLevel + 1] = {};
-  for (int k = 2; k <= t->depth; ++k)
-    im[k] = ops->compressed && ops->lv[k].r > 0 ? &ops->lv[k].crtc : &ops->lv[k].crt;
-  const size_t need = crt_scratch_bytes(t->depth, im, R);
+  EIFMM_TRY(ensure_crt_images(ops, t->depth, !t->opt[EIFMM_OPT_M2L_FP64], s));
+  CrtJob jobs[3 * kMaxLevel];
+  int n = 0;
+  auto add = [&](CrtMode m, int k, const CrtImage& im) {
+    if (im.img) jobs[n++] = CrtJob{m, k, &im, nullptr, nullptr, nullptr};
+  };
+  for (int k = 2; k <= t->depth; ++k) {
+    const LevelOps& v = ops->lv[k];
+    add(kCrtM2L, k, ops->compressed && v.r > 0 ? v.crtc : v.crt);
+    if (k < t->depth) add(kCrtM2M, k, v.crt_m2m);
+    if (k > 2) add(kCrtL2L, k, v.crt_l2l);
+    if (k == t->depth) add(kCrtBox, k, v.crt_dt);
+  }
+  const size_t need = n > 0 ? crt_scratch_bytes(n, jobs, R) : 0;
   if (need > ws.crt_bytes) {
     dfree(ws.crt_buf);
     ws.crt_buf = nullptr;
@@ -575,7 +594,7 @@ static eifmm_status evaluate_impl(eifmm_tree* tree, const eifmm_ops* ops, const 
                                   int prec, cudaStream_t s) {
   Tree& t = tree->t;
   EIFMM_TRY(ensure_workspace(&t, &ops->o, n_rhs, prec));
-  if ((prec == EIFMM_PREC_FP64 || ops->o.tier >= 3) && !t.opt[EIFMM_OPT_M2L_FP64])
+  if (prec == EIFMM_PREC_FP64 || ops->o.tier >= 3)
     EIFMM_TRY(ensure_crt(&t, const_cast<Ops*>(&ops->o), n_rhs, s));
   if (t.ws.err_host && *t.ws.err_host != 0) {
     const int code = *t.ws.err_host;
@@ -655,7 +674,7 @@ extern "C" eifmm_status eifmm_ops_calibrate(eifmm_ops* ops, double eps, eifmm_st
     if ((rc = eifmm_tree_build(dx, n, dx, n, lo, L, depth, 1, stream, &tree)) != EIFMM_OK) break;
     // a view of the operators restricted to the calibration depth (with the
     // images of the FP64 reference, which then belong to the set itself)
-    if ((rc = ensure_crt_images(&ops->o, depth, s)) != EIFMM_OK) break;
+    if ((rc = ensure_crt_images(&ops->o, depth, true, s)) != EIFMM_OK) break;
     eifmm_ops view;
     view.o = ops->o;
     view.o.depth = depth;
@@ -711,7 +730,8 @@ extern "C" eifmm_status eifmm_ops_calibrate(eifmm_ops* ops, double eps, eifmm_st
   if (rc != EIFMM_OK) return rc;
   EIFMM_TRY(eifmm_ops_plan(ops, best, nullptr));
   if (best < 3)  // only an evaluation in FP64 would use them, and it builds them again
-    for (int k = 2; k <= depth; ++k) free_crt_image(&ops->o.lv[k].crt);
+    for (int k = 2; k <= depth; ++k)
+      for (CrtImage* im : {&ops->o.lv[k].crt, &ops->o.lv[k].crt_m2m, &ops->o.lv[k].crt_l2l, &ops->o.lv[k].crt_dt}) free_crt_image(im);
   ops->o.calib_tier = best;
   if (tier_out) *tier_out = best;
   return EIFMM_OK;

@@ -533,6 +533,13 @@ eifmm_status launch_m2l64(int level, int d, int R, const double* kdT, const int*
   return G > 1 ? sum_groups64(part, G, n, g, s) : EIFMM_OK;
 }
 
+// M2M and L2L of np parents by residues on the tensor cores: four launches of
+// about 30 us together at least, which the warp kernels on the FP64 pipes take
+// at 4e6 products per column (64 parents at d = 90; d = 193: 52 us).
+static bool crt_transfer(const Workspace& ws, const CrtImage& im, int64_t np, int R) {
+  return im.img && ws.crt_bytes > 0 && (double)np * R * 8.0 * im.d * im.dl >= 4e6;
+}
+
 eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_sigma, int R,
                        double* f, int64_t ld_f, cudaStream_t s, bool near32, bool pair_m2l) {
   Workspace& ws = t->ws;
@@ -570,6 +577,11 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   for (int k = kap - 1; k >= 2; --k) {
     const int dk = ops->lv[k].d, dc = ops->lv[k + 1].d;
     const int64_t np = (int64_t)1 << (3 * k);
+    if (crt_transfer(ws, ops->lv[k].crt_m2m, np, R)) {
+      const CrtJob job{kCrtM2M, k, &ops->lv[k].crt_m2m, ws.W[k + 1], ws.W[k], nullptr};
+      EIFMM_TRY(launch_crt(1, &job, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
+      continue;
+    }
     k_m2m_warp<double><<<xfer_blocks(np, R, dk), 128, 0, s>>>(dk, dc, dk, dc, R, ops->lv[k].m2m,
                                                              ws.W[k + 1], ws.W[k], np);
     EIFMM_CHECK_LAUNCH();
@@ -593,7 +605,7 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
       if (ops->compressed && v.r > 0)
         EIFMM_TRY(m2l_compressed(ws, ops, k, R, fp64, pair, s));
       else if (!fp64 && v.crt.img && ws.crt_bytes > 0 && !(pair && v.crt.kappa > kCrtMaxKappa))
-        jobs[nj++] = CrtJob{k, &v.crt, ws.W[k], ws.g[k]};
+        jobs[nj++] = CrtJob{kCrtM2L, k, &v.crt, ws.W[k], ws.g[k], nullptr};
       else if (pair)
         EIFMM_TRY(launch_m2l_df(k, v.d, R, v.kdT, ops->d_slot_lists, ws.W[k], ws.g[k], ws.part64, ws.part64_cap,
                                 ws.nsm, s));
@@ -602,7 +614,7 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
                                ws.nsm, s));
       if (timing_enabled() && k < kap) cudaEventRecord(ws.ev_m2le[k], s);
     }
-    if (nj > 0) EIFMM_TRY(launch_m2l_crt(nj, jobs, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
+    if (nj > 0) EIFMM_TRY(launch_crt(nj, jobs, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
     if (timing_enabled()) cudaEventRecord(ws.ev_m2le[kap], s);
   }
   record(ws, 4, s);
@@ -610,13 +622,21 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   for (int k = 3; k <= kap; ++k) {
     const int dk = ops->lv[k].d, dp = ops->lv[k - 1].d;
     const int64_t nb = (int64_t)1 << (3 * k);
+    if (crt_transfer(ws, ops->lv[k].crt_l2l, nb / 8, R)) {
+      const CrtJob job{kCrtL2L, k, &ops->lv[k].crt_l2l, ws.l[k - 1], ws.l[k], ws.g[k]};
+      EIFMM_TRY(launch_crt(1, &job, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
+      continue;
+    }
     k_l2l_warp<double><<<xfer_blocks(nb, R, dk), 128, 0, s>>>(dk, dp, dk, dp, R, ops->lv[k].l2l,
                                                              ws.l[k - 1], ws.g[k], ws.l[k], nb);
     EIFMM_CHECK_LAUNCH();
   }
   record(ws, 5, s);
-  // step 6
-  {
+  // step 6: the explicit Delta^t in residues, or the triangular solves
+  if (vl.crt_dt.img && ws.crt_bytes > 0) {
+    const CrtJob job{kCrtBox, kap, &vl.crt_dt, ws.l[kap], ws.lh, nullptr};
+    EIFMM_TRY(launch_crt(1, &job, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
+  } else {
     DeltaBatch b;
     b.nlev = 1;
     b.lv[0] = delta_level(vl.d, delta_ops64(vl), true, ws.l[kap], vl.d, ws.lh, vl.d, nullptr,

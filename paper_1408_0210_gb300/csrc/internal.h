@@ -53,14 +53,15 @@ void dfree(void* p);
 __host__ __device__ inline double kern_f64(int kern, double z0, double z1, double z2);
 
 // ------------------------------------------------------------ operators --
-// Residues of an M2L operator stack for the FP64 M2L on the tensor cores
+// Residues of a stack of operators for the FP64 products on the tensor cores
 // (m2l_crt.cu): [modulus][slot][column tile][k8][Nt columns m'][8 terms l].
-constexpr int kCrtMods = 14;
 struct CrtImage {
   void* img = nullptr;         // BF16
   double* colscale = nullptr;  // [d] scale of column m' in the reconstruction
   double kappa = 0.0;          // amplification of rounding by the operators (crt_kappa)
-  int d = 0, K = 0, Nt = 0, NT = 0;  // rank, terms padded to 16, columns of a tile, tiles
+  bool refused = false;        // the operators cannot be represented
+  int nslots = 0, dl = 0, d = 0;     // operators, rank of the source and of the target
+  int K = 0, Nt = 0, NT = 0;         // terms padded to 16, columns of a tile, tiles
 };
 struct LevelOps {
   int d = 0;          // EIM rank of the level
@@ -103,6 +104,8 @@ struct LevelOps {
   double s_kept = 0.0, s_next = 0.0;  // last kept and first dropped singular value / s_0
   CrtImage crt;            // residues of kdT, built at the first use of the FP64 far field
   CrtImage crtc;           // residues of Ct, with it
+  CrtImage crt_m2m, crt_l2l;  // residues of m2mT and l2lT
+  CrtImage crt_dt;         // residues of Delta^t (where this is a tree's leaf level)
   int kd_img_fmt = -1;     // -1 none, else the PlaneFmt of the image
   float* kscale = nullptr; // [dp] power-of-two scale of row m' (FP16 image)
 };
@@ -284,8 +287,8 @@ eifmm_status eval_mixed(Tree* t, const Ops* ops, const double* sigma,
                         cudaStream_t s);
 eifmm_status ensure_workspace(Tree* t, const Ops* ops, int R, int prec);
 // Residue images of levels 2..depth (m2l_crt.cu), built once per operator
-// set; returns when they are ready for every stream.
-eifmm_status ensure_crt_images(Ops* ops, int depth, cudaStream_t s);
+// set; returns when they are ready for every stream.  m2l: the M2L's too.
+eifmm_status ensure_crt_images(Ops* ops, int depth, bool m2l, cudaStream_t s);
 eifmm_status alloc_wait_error(Workspace* ws);
 // FP64 far-field M2L on the FP64 pipes and in FP32 pairs (fmm64.cu): offset groups split the offset list of a
 // level with few blocks; `part` (part_cap doubles) holds their partial sums.

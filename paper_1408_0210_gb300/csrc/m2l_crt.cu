@@ -1,5 +1,5 @@
-// m2l_crt.cu -- step 4 of Algorithm 3 (M2L, Eq. M2Lstep) in FP64 accuracy on
-// the tcgen05 tensor cores.
+// m2l_crt.cu -- the dense products of Algorithm 3 (M2M, M2L, L2L and the Delta^t
+// of step 6) in FP64 accuracy on the tcgen05 tensor cores.  The M2L (step 4):
 //
 //   g^I_{m'} = sum_{J in I(I)} sum_l T^delta_{m'l} W^J_l
 //
@@ -31,6 +31,16 @@
 // method's products, 13% of them zero (189 offsets for 165 pairs per box) and
 // is bound by the stream of operator residues: 86 KB per offset and 128 boxes,
 // 64 bytes per cycle and SM at the tensor cores' full rate.
+//
+// M2M, L2L and Delta^t are the same sums over the 8 children, the parent and the
+// box itself, without shifts.  Delta^t is formed explicitly in double-double
+// and takes 18 moduli (160.5 bits): its entries reach 2^34 / |A| at eps 1e-7, and
+// the product cancels by as much.  K(x, X) Delta^t l then errs by 1.6e-16 to 9e-16
+// (1/r, eps 1e-4 to 1e-7) where the FP64 triangular solves err by 2.3e-16 to 2.7e-15
+// (config-3 at 1e-6: 1.4e-12 and 7.2e-12).  At 2^20 points, depth 5, d = 193, on
+// the FP64 pipes before: M2M 3.0 -> 0.44 ms, L2L 5.1 -> 0.61 ms, Delta^t 3.5 -> 0.70
+// ms; 512 leaves: Delta^t 1.73 -> 0.075 ms.  They are bound by their passes over
+// the residues (28 bytes an entry) and, for small levels, by their launches.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -42,15 +52,17 @@
 namespace eifmm {
 namespace {
 
-constexpr int kMods = kCrtMods;
+constexpr int kMods = 14;     // M2L, M2M, L2L: 125.2 bits
+constexpr int kBoxMods = 18;  // Delta^t: 160.5 bits
 __host__ __device__ constexpr int crt_mod(int i) {
   return i == 0 ? 513 : i == 1 ? 512 : i == 2 ? 511 : i == 3 ? 509 : i == 4 ? 505 : i == 5 ? 503 : i == 6 ? 499
-       : i == 7 ? 491 : i == 8 ? 487 : i == 9 ? 481 : i == 10 ? 479 : i == 11 ? 473 : i == 12 ? 467 : 463;
+       : i == 7 ? 491 : i == 8 ? 487 : i == 9 ? 481 : i == 10 ? 479 : i == 11 ? 473 : i == 12 ? 467 : i == 13 ? 463
+       : i == 14 ? 461 : i == 15 ? 457 : i == 16 ? 449 : 443;
 }
-static_assert(kMods == 14, "crt_mod lists 14 moduli");
-constexpr int kWBits = 58;     // |W| 2^b < 2^58
-constexpr int kRowBits = 66;   // sum over offsets and l of |T| 2^a < 2^66
-constexpr int kEntryBits = 60; // |T| 2^a < 2^60
+// |W| 2^b < 2^wbits; sum over offsets and l of |T| 2^a < 2^rowbits; wbits +
+// rowbits + 1 (the sign) is the size of the product of the moduli.
+constexpr int kWBits = 58, kRowBits = 66, kEntryBits = 60;  // |T| 2^a < 2^60
+constexpr int kBoxWBits = 55, kBoxRowBits = 104;
 constexpr int kMaxSteps = 15;  // k-steps of 16 terms in one accumulation: 240 terms
 
 // Target tile of a CTA: 8 x 4 x 4 boxes of one parity class (128 rows of the
@@ -73,14 +85,20 @@ constexpr uint32_t kSmemBars = 512;
 
 // One level (or one slab and column range of it) of a launch.
 struct CrtLv {
-  int level, d, K, Nt, NT;   // rank, padded terms, columns per tile, column tiles
-  int h;                     // boxes per axis of a parity class
+  CrtMode mode;
+  int slevel, ds, ncs;       // source boxes: level, rank, parity classes (8, or 1: the whole grid)
+  int tlevel, d, nct;        // target boxes: level, rank, classes
+  int K, Nt, NT;             // padded terms, columns per tile, column tiles
+  int nw, nslots;            // windows per target class, operators of the stack
+  int wbits;                 // size of the integers of W
+  int h;                     // boxes per axis of a class (of source and target alike)
   int z0, nz, sz0, snz;      // planes of target boxes, planes of source boxes held
   int r0, Rc, R, G;          // columns r0 .. r0 + Rc of R, offset groups
   int nchunk, n0, ks0, ks1;  // chunks of K: n0 of ks0 k-steps, then ks1 k-steps each
   unsigned item0, pl0, rc0, mx0;  // first block of this level in each of the launches
   const double* W;
   double* g;
+  const double* add;         // added to the sum, same layout as g (may be null)
   __nv_bfloat16* planes;     // [mod][r][class][k8][z][y][x][8]
   int16_t* res;              // [mod][group][r][class][z][y][x][NT Nt]
   const __nv_bfloat16* img;  // [mod][slot][column tile][k8][Nt][8]
@@ -97,8 +115,10 @@ struct CrtArgs {
 struct CrtMaps {
   CUtensorMap m[kMaxLv];
 };
+// 2^(32 NW) y_i / m_i, y_i the inverse of M / m_i modulo m_i, for NM moduli
+template <int NM, int NW>
 struct CrtK {
-  uint32_t k[kMods][3];  // 2^96 y_i / m_i, y_i the inverse of M / m_i modulo m_i
+  uint32_t k[NM][NW];
 };
 
 // K / 16 k-steps in chunks of five and three: three chunks of five or five of
@@ -135,10 +155,38 @@ __device__ __forceinline__ int combo_mask(int ct, int cs, int sy1) {
   return 0x1ff & ~m;
 }
 
+// Window w of target class ct: source class, y-shift + 1, mask of (sz, sx)
+// shifts (bit 3 (sz + 1) + sx + 1) and the operator of the shift (0, 0).
+struct Win {
+  int cs, sy1, mask, slot;
+};
+__device__ __forceinline__ Win window_of(const CrtLv& v, int ct, int w) {
+  Win o;
+  if (v.mode == kCrtM2L) {
+    o.cs = w / 3;
+    o.sy1 = w - 3 * o.cs;
+    o.mask = combo_mask(ct, o.cs, o.sy1);
+    o.slot = (2 * (o.sy1 - 1) + ((o.cs >> 1) & 1) - ((ct >> 1) & 1) + 3) * 7 + (o.cs & 1) - (ct & 1) + 3 +
+             ((o.cs >> 2) - (ct >> 2) + 3) * 49;
+  } else {  // no shift: the 8 children of a box (M2M), its parent (L2L), itself (box)
+    o.cs = v.mode == kCrtM2M ? w : (v.mode == kCrtL2L ? 0 : ct);
+    o.slot = v.mode == kCrtM2M ? w : (v.mode == kCrtL2L ? ct : 0);
+    o.sy1 = 1;
+    o.mask = 0x10;
+  }
+  return o;
+}
+
+// Morton key of box (x, y, z) of class c of nc
+__device__ __forceinline__ int64_t class_box(int nc, int c, int x, int y, int z, int level) {
+  if (nc == 1) return morton_encode(x, y, z, level);
+  return morton_encode(2 * x + (c & 1), 2 * y + ((c >> 1) & 1), 2 * z + (c >> 2), level);
+}
+
 // scale exponent of a column from the bits of its largest |W|
 __device__ __forceinline__ bool w_finite(unsigned long long bits) { return bits < 0x7ff0000000000000ull; }
-__device__ __forceinline__ int w_exp(unsigned long long bits) {
-  const int b = kWBits - ((int)(bits >> 52) - 1022);
+__device__ __forceinline__ int w_exp(unsigned long long bits, int wbits) {
+  const int b = wbits - ((int)(bits >> 52) - 1022);
   return b > 1020 ? 1020 : b;
 }
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
@@ -166,12 +214,12 @@ __global__ void __launch_bounds__(256) k_crt_max(const __grid_constant__ CrtArgs
   const CrtLv& v = a.lv[find_level(a, &CrtLv::mx0, blockIdx.x)];
   const unsigned b = blockIdx.x - v.mx0;
   const int r = v.r0 + (int)(b % v.Rc);
-  const int64_t n = ((int64_t)1 << (3 * v.level)) * v.d;
+  const int64_t n = ((int64_t)1 << (3 * v.slevel)) * v.ds;
   const int64_t beg = (int64_t)(b / v.Rc) * kMaxPer, end = min(n, beg + kMaxPer);
   unsigned long long mx = 0;
   for (int64_t i = beg + threadIdx.x; i < end; i += 256) {
-    const int64_t box = v.R == 1 ? 0 : i / v.d;
-    const double w = v.R == 1 ? v.W[i] : v.W[(box * v.R + r) * v.d + (i - box * v.d)];
+    const int64_t box = v.R == 1 ? 0 : i / v.ds;
+    const double w = v.R == 1 ? v.W[i] : v.W[(box * v.R + r) * v.ds + (i - box * v.ds)];
     const unsigned long long x = (unsigned long long)__double_as_longlong(w) & 0x7fffffffffffffffull;
     mx = x > mx ? x : mx;
   }
@@ -192,6 +240,7 @@ __global__ void __launch_bounds__(256) k_crt_max(const __grid_constant__ CrtArgs
 // A block takes 8 boxes along x of one class, z, y and column: their W is
 // rounded to integers once, and every thread writes 8 terms of one box for
 // the 14 moduli (16-byte stores, 128 contiguous bytes per 8 threads).
+template <int NM>
 __global__ void __launch_bounds__(256) k_crt_planes(const __grid_constant__ CrtArgs a) {
   extern __shared__ long long s_w[];  // [8][K + 1]
   const CrtLv& v = a.lv[find_level(a, &CrtLv::pl0, blockIdx.x)];
@@ -203,17 +252,17 @@ __global__ void __launch_bounds__(256) k_crt_planes(const __grid_constant__ CrtA
   b /= h;
   const int zs = (int)(b % v.snz);
   b /= v.snz;
-  const int cls = (int)(b & 7), r = (int)(b >> 3);
+  const int cls = (int)(b % v.ncs), r = (int)(b / v.ncs);
   const int z = v.sz0 + zs, K = v.K, ld = K + 1;
   const unsigned long long bits = v.wmax[v.r0 + r];
   const bool fin = w_finite(bits);
-  const double sc = pow2(w_exp(fin ? bits : 0));
+  const double sc = pow2(w_exp(fin ? bits : 0, v.wbits));
   for (int i = threadIdx.x; i < 8 * K; i += 256) {
     const int bx = i / K, l = i - bx * K, x = 8 * xs + bx;
     long long q = 0;
-    if (l < v.d && x < h && fin) {
-      const int64_t I = morton_encode(2 * x + (cls & 1), 2 * y + ((cls >> 1) & 1), 2 * z + (cls >> 2), v.level);
-      q = __double2ll_rn(v.W[(I * v.R + v.r0 + r) * v.d + l] * sc);
+    if (l < v.ds && x < h && fin) {
+      const int64_t I = class_box(v.ncs, cls, x, y, z, v.slevel);
+      q = __double2ll_rn(v.W[(I * v.R + v.r0 + r) * v.ds + l] * sc);
     }
     s_w[bx * ld + l] = q;
   }
@@ -226,14 +275,14 @@ __global__ void __launch_bounds__(256) k_crt_planes(const __grid_constant__ CrtA
     long long w[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) w[j] = q[j];
-    __nv_bfloat16* dst = v.planes + (int64_t)(r * 8 + cls) * plane + ((((int64_t)k8 * v.snz + zs) * h + y) * h + x) * 8;
+    __nv_bfloat16* dst = v.planes + (int64_t)(r * v.ncs + cls) * plane + ((((int64_t)k8 * v.snz + zs) * h + y) * h + x) * 8;
 #pragma unroll
-    for (int i = 0; i < kMods; ++i) {
+    for (int i = 0; i < NM; ++i) {
       __nv_bfloat162 o[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j)
         o[j] = __floats2bfloat162_rn((float)residue(w[2 * j], i), (float)residue(w[2 * j + 1], i));
-      *reinterpret_cast<uint4*>(dst + (int64_t)i * v.Rc * 8 * plane) = *reinterpret_cast<uint4*>(o);
+      *reinterpret_cast<uint4*>(dst + (int64_t)i * v.Rc * v.ncs * plane) = *reinterpret_cast<uint4*>(o);
     }
   }
 }
@@ -296,14 +345,14 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
   b /= nty;
   const int z0 = v.z0 + kTZ * (int)(b % ntz);
   b /= ntz;
-  const int ct = (int)(b & 7);
-  b >>= 3;
+  const int ct = (int)(b % v.nct);
+  b /= v.nct;
   const int nt = (int)(b % v.NT);
   b /= v.NT;
   const int r = (int)(b % v.Rc);
   b /= v.Rc;
   const int grp = (int)(b % v.G), mod = (int)(b / v.G);
-  const int w_beg = grp * 24 / v.G, w_end = (grp + 1) * 24 / v.G;  // window = 3 class + y-shift
+  const int w_beg = grp * v.nw / v.G, w_end = (grp + 1) * v.nw / v.G;
 
   if (tid == 0) {
     for (int i = 0; i < kMaxStages; ++i) {
@@ -333,19 +382,16 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     // ----------------------------------------- operator residues (B) --
     const uint32_t el = elect_one();
     const int64_t tile_b = (int64_t)K * Nt * 2, slot_b = v.NT * tile_b;  // bytes of a column tile, of a slot
-    const char* img = (const char*)v.img + (int64_t)mod * kNumSlots * slot_b + nt * tile_b;
+    const char* img = (const char*)v.img + (int64_t)mod * v.nslots * slot_b + nt * tile_b;
     const int n0 = v.n0, ks0 = v.ks0, ks1 = v.ks1;
     const uint32_t stage_b = a.stage_b;
     int it = 0, st = 0;
     uint32_t ph = 0, dst = s_stage;
     bool ok = true;
     for (int w = w_beg; w < w_end && ok; ++w) {
-      const int cs = w / 3, sy1 = w - 3 * cs;
-      const int mask = combo_mask(ct, cs, sy1);
-      // slot of the shift sx = sz = 0
-      const int sl0 = (2 * (sy1 - 1) + ((cs >> 1) & 1) - ((ct >> 1) & 1) + 3) * 7 + (cs & 1) - (ct & 1) + 3 +
-                      ((cs >> 2) - (ct >> 2) + 3) * 49;
-      const char* src = img + sl0 * slot_b;
+      const Win wn = window_of(v, ct, w);
+      const int mask = wn.mask;
+      const char* src = img + wn.slot * slot_b;
       for (int c = 0; c < nchunk && ok; ++c) {
         const uint32_t bytes = (uint32_t)(c < n0 ? ks0 : ks1) * 32u * Nt;
 #pragma unroll
@@ -373,7 +419,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     int wi = 0;
     bool ok = true;
     for (int w = w_beg; w < w_end && ok; ++w) {
-      const int cs = w / 3, sy1 = w - 3 * cs;
+      const Win wn = window_of(v, ct, w);
       int k0 = 0;
       for (int c = 0; c < nchunk; ++c, ++wi) {
         const int ks = chunk_ksteps(v, c);
@@ -386,7 +432,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
           mbar_expect_tx(wfull(s), (uint32_t)ks * kWinStep);
           for (int kk = 0; kk < ks; ++kk)
             tma_load_5d(sbase + (uint32_t)s * a.win_b + (uint32_t)kk * kWinStep, &maps.m[q], 8 * (x0 - 1),
-                        y0 + sy1 - 1, z0 - 1 - v.sz0, 2 * (k0 + kk), (mod * v.Rc + r) * 8 + cs, wfull(s));
+                        y0 + wn.sy1 - 1, z0 - 1 - v.sz0, 2 * (k0 + kk), (mod * v.Rc + r) * v.ncs + wn.cs, wfull(s));
         }
         __syncwarp();
         k0 += ks;
@@ -431,7 +477,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
         }
     };
     for (int w = w_beg; w < w_end && ok; ++w) {
-      const int mask = combo_mask(ct, w / 3, w % 3);
+      const int mask = window_of(v, ct, w).mask;
       for (int c = 0; c < nchunk && ok; ++c, ++wi) {
         const int ks = c < n0 ? ks0 : ks1;
         const int s = wi & 1;
@@ -454,7 +500,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     {
       int acc = 0;
       for (int w = w_beg; w < w_end; ++w) {
-        const int n = __popc(combo_mask(ct, w / 3, w % 3));
+        const int n = __popc(window_of(v, ct, w).mask);
         for (int c = 0; c < nchunk; ++c) {
           const int ks = chunk_ksteps(v, c);
           for (int i = 0; i < n; ++i) {
@@ -502,7 +548,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     if (x < h && y < h && z < v.z0 + v.nz) {
       const int N = v.NT * Nt;
       int16_t* out = v.res +
-                     ((((((int64_t)mod * v.G + grp) * v.Rc + r) * 8 + ct) * v.nz + (z - v.z0)) * h + y) * (int64_t)h * N +
+                     ((((((int64_t)mod * v.G + grp) * v.Rc + r) * v.nct + ct) * v.nz + (z - v.z0)) * h + y) * (int64_t)h * N +
                      (int64_t)x * N + nt * Nt + half * nh;
 #pragma unroll
       for (int j = 0; j < 16; ++j)
@@ -522,29 +568,33 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
 }
 
 // -------------------------------------------------------- reconstruction --
-// G / M modulo 1 = sum_i s_i y_i / m_i modulo 1, in 96-bit fixed point (the
-// constants' rounding adds at most 2^-82 of M, G itself is about 2^-10 of M).
+// G / M modulo 1 = sum_i s_i y_i / m_i modulo 1, in fixed point of NW words (the
+// constants' rounding adds at most 2^(14 - 32 NW) of M; G itself is about 2^-10
+// of M, 2^-40 for Delta^t, whose terms cancel, with one word more).
 // A warp takes one (column, box) row, a lane two coefficients.
-__global__ void __launch_bounds__(128) k_crt_rebuild(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK kc) {
+template <int NM, int NW>
+__global__ void __launch_bounds__(128)
+k_crt_rebuild(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK<NM, NW> kc) {
   const CrtLv& v = a.lv[find_level(a, &CrtLv::rc0, blockIdx.x)];
   const int lane = threadIdx.x & 31;
-  const int64_t cells = (int64_t)v.nz * v.h * v.h, rows = cells * 8 * v.Rc;
+  const int64_t cells = (int64_t)v.nz * v.h * v.h, rows = cells * v.nct * v.Rc;
   const int64_t row = (int64_t)(blockIdx.x - v.rc0) * 4 + (threadIdx.x >> 5);
   if (row >= rows) return;
   const int64_t cell = row % cells;
-  const int cls = (int)((row / cells) & 7), r = v.r0 + (int)(row / (cells * 8));
+  const int cls = (int)((row / cells) % v.nct), r = v.r0 + (int)(row / (cells * v.nct));
   const int x = (int)(cell % v.h), y = (int)((cell / v.h) % v.h), z = v.z0 + (int)(cell / ((int64_t)v.h * v.h));
-  const int64_t I = morton_encode(2 * x + (cls & 1), 2 * y + ((cls >> 1) & 1), 2 * z + (cls >> 2), v.level);
+  const int64_t I = class_box(v.nct, cls, x, y, z, v.tlevel);
   const int N = v.NT * v.Nt;
   const int16_t* res = v.res + row * N;
   double* g = v.g + (I * v.R + r) * v.d;
+  const double* add = v.add ? v.add + (I * v.R + r) * v.d : nullptr;
   const unsigned long long bits = v.wmax[r];
   const bool fin = w_finite(bits);
-  const double ws = fin ? pow2(-w_exp(bits)) : __longlong_as_double(0x7ff8000000000000ll);
+  const double ws = fin ? pow2(-w_exp(bits, v.wbits)) : __longlong_as_double(0x7ff8000000000000ll);
   for (int c = 2 * lane; c < v.d; c += 64) {
-    unsigned long long p[2][3] = {};
+    unsigned long long p[2][NW] = {};
 #pragma unroll
-    for (int i = 0; i < kMods; ++i) {
+    for (int i = 0; i < NM; ++i) {
       const int m = crt_mod(i);
       const short2 t = *reinterpret_cast<const short2*>(res + (int64_t)i * v.G * rows * N + c);
       int s0 = t.x, s1 = t.y;
@@ -561,7 +611,7 @@ __global__ void __launch_bounds__(128) k_crt_rebuild(const __grid_constant__ Crt
       s0 += s0 < 0 ? m : 0;
       s1 += s1 < 0 ? m : 0;
 #pragma unroll
-      for (int w = 0; w < 3; ++w) {
+      for (int w = 0; w < NW; ++w) {
         p[0][w] += (unsigned long long)(unsigned)s0 * kc.k[i][w];
         p[1][w] += (unsigned long long)(unsigned)s1 * kc.k[i][w];
       }
@@ -569,25 +619,34 @@ __global__ void __launch_bounds__(128) k_crt_rebuild(const __grid_constant__ Crt
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       if (c + e >= v.d) break;
-      const unsigned long long p1 = p[e][1] + (p[e][0] >> 32), p2 = p[e][2] + (p1 >> 32);
-      const long long hi = (long long)((p2 << 32) | (p1 & 0xffffffffull));
-      const double G = fma((double)hi, 4294967296.0, (double)(unsigned)p[e][0]);
-      g[c + e] = G * v.colscale[c + e] * ws;
+#pragma unroll
+      for (int w = 1; w < NW; ++w) p[e][w] += p[e][w - 1] >> 32;
+      // the signed top 64 bits and the words below
+      const long long hi = (long long)((p[e][NW - 1] << 32) | (p[e][NW - 2] & 0xffffffffull));
+      double G = fma((double)hi, 4294967296.0, (double)(unsigned)p[e][NW - 3]);
+      if (NW == 4) {
+        // the top words may hold little but the sign: add the last word exactly
+        // where the upper three fit a double, where they do not it is below
+        // its rounding
+        G = fma(G, 4294967296.0, (double)(unsigned)p[e][0]);
+      }
+      const double y = G * v.colscale[c + e] * ws;
+      g[c + e] = add ? add[c + e] + y : y;
     }
   }
 }
 
 // ---------------------------------------------------------- the images --
 // Largest entry and sum of |T| over slots and l for 32 rows m' per block.
-__global__ void __launch_bounds__(1024) k_crt_rowsum(const double* __restrict__ kdT, int d, double* __restrict__ mx,
-                                                     double* __restrict__ l1) {
+__global__ void __launch_bounds__(1024) k_crt_rowsum(const double* __restrict__ kdT, int nslots, int dl, int d,
+                                                     double* __restrict__ mx, double* __restrict__ l1) {
   const int mp = blockIdx.x * 32 + threadIdx.x;
   double s = 0.0, m = 0.0;
   if (mp < d)
-    for (int64_t i = threadIdx.y; i < (int64_t)kNumSlots * d; i += 32) {
-      const int slot = (int)(i / d);
+    for (int64_t i = threadIdx.y; i < (int64_t)nslots * dl; i += 32) {
+      const int slot = (int)(i / dl);
       const int dx = slot % 7 - 3, dy = (slot / 7) % 7 - 3, dz = slot / 49 - 3;
-      if (abs(dx) <= 1 && abs(dy) <= 1 && abs(dz) <= 1) continue;
+      if (nslots == kNumSlots && abs(dx) <= 1 && abs(dy) <= 1 && abs(dz) <= 1) continue;  // the near field
       const double t = fabs(kdT[i * d + mp]);
       s += t;
       m = fmax(m, t);
@@ -606,24 +665,25 @@ __global__ void __launch_bounds__(1024) k_crt_rowsum(const double* __restrict__ 
   }
 }
 
-// Exponents a of the rows: l1 2^a < 2^kRowBits and mx 2^a < 2^kEntryBits.
+// Exponents a of the rows: l1 2^a < 2^rowbits and mx 2^a < 2^entrybits.
 __global__ void k_crt_rowscale(const double* __restrict__ mx, const double* __restrict__ l1, int d, double mscale,
-                               double* __restrict__ up, double* __restrict__ colscale) {
+                               int rowbits, int entrybits, double* __restrict__ up, double* __restrict__ colscale) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= d) return;
   int e = 0, e1 = 0;
   // the sum itself carries rounding; 2^-40 relative covers it
   frexp(l1[m] * (1.0 + 0x1p-40), &e);
   frexp(mx[m], &e1);
-  int s = min(kRowBits - e, kEntryBits - e1);
+  int s = min(rowbits - e, entrybits - e1);
   s = l1[m] > 0.0 ? max(-900, min(900, s)) : 0;
   up[m] = pow2(s);
   colscale[m] = ldexp(mscale, -s);
 }
 
 // One thread per (slot, column tile, k8, n): 8 terms of one row for every modulus.
-__global__ void __launch_bounds__(256) k_crt_image(const double* __restrict__ kdT, int d, int K, int Nt, int NT,
-                                                   const double* __restrict__ up, __nv_bfloat16* __restrict__ img) {
+__global__ void __launch_bounds__(256) k_crt_image(const double* __restrict__ kdT, int nslots, int dl, int d, int K,
+                                                   int Nt, int NT, const double* __restrict__ up,
+                                                   __nv_bfloat16* __restrict__ img) {
   const int slot = blockIdx.y;
   const int64_t tile_e = (int64_t)K * Nt;
   const int units = NT * (K / 8) * Nt;
@@ -634,7 +694,7 @@ __global__ void __launch_bounds__(256) k_crt_image(const double* __restrict__ kd
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int l = 8 * k8 + j;
-      w[j] = (mp < d && l < d) ? __double2ll_rn(kdT[((int64_t)slot * d + l) * d + mp] * up[mp]) : 0;
+      w[j] = (mp < d && l < dl) ? __double2ll_rn(kdT[((int64_t)slot * dl + l) * d + mp] * up[mp]) : 0;
     }
     __nv_bfloat16* dst = img + ((int64_t)slot * NT + nt) * tile_e + ((int64_t)k8 * Nt + n) * 8;
 #pragma unroll
@@ -643,8 +703,110 @@ __global__ void __launch_bounds__(256) k_crt_image(const double* __restrict__ kd
 #pragma unroll
       for (int j = 0; j < 4; ++j)
         o[j] = __floats2bfloat162_rn((float)residue(w[2 * j], i), (float)residue(w[2 * j + 1], i));
-      *reinterpret_cast<uint4*>(dst + (int64_t)i * kNumSlots * NT * tile_e) = *reinterpret_cast<uint4*>(o);
+      *reinterpret_cast<uint4*>(dst + (int64_t)i * nslots * NT * tile_e) = *reinterpret_cast<uint4*>(o);
     }
+  }
+}
+
+// ------------------------------------------------- Delta^t, explicitly --
+// Delta^t = Gamma^-t B^-1 in double-double (106 bits), a warp per column j: B z
+// = e_j forward, Gamma^t w = z backward, the dot products over the lanes.
+struct Dd {
+  double h, l;
+};
+__device__ __forceinline__ Dd dd_norm(double a, double b) {  // |a| >= |b| or a = 0
+  const double s = __dadd_rn(a, b);
+  return {s, __dadd_rn(b, -__dadd_rn(s, -a))};
+}
+__device__ __forceinline__ Dd dd_add(Dd a, Dd b) {
+  const double s = __dadd_rn(a.h, b.h), sb = __dadd_rn(s, -a.h);
+  const double e = __dadd_rn(__dadd_rn(a.h, -__dadd_rn(s, -sb)), __dadd_rn(b.h, -sb));
+  const double t = __dadd_rn(a.l, b.l), tb = __dadd_rn(t, -a.l);
+  const double f = __dadd_rn(__dadd_rn(a.l, -__dadd_rn(t, -tb)), __dadd_rn(b.l, -tb));
+  const Dd x = dd_norm(s, __dadd_rn(e, t));
+  return dd_norm(x.h, __dadd_rn(x.l, f));
+}
+__device__ __forceinline__ Dd dd_mul(Dd a, double b) {
+  const double p = __dmul_rn(a.h, b), e = __fma_rn(a.h, b, -p);
+  return dd_norm(p, __fma_rn(a.l, b, e));
+}
+__device__ __forceinline__ Dd dd_div(Dd a, double b) {
+  const double q1 = __ddiv_rn(a.h, b);
+  const Dd r1 = dd_add(a, dd_mul({b, 0.0}, -q1));
+  const double q2 = __ddiv_rn(r1.h, b);
+  const Dd r2 = dd_add(r1, dd_mul({b, 0.0}, -q2));
+  return dd_add(dd_norm(q1, q2), {__ddiv_rn(r2.h, b), 0.0});
+}
+__device__ __forceinline__ Dd dd_warp_sum(Dd v) {
+  for (int o = 16; o > 0; o >>= 1)
+    v = dd_add(v, {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)});
+  return v;
+}
+// hi, lo: [j][i] = Delta^t_{ij}
+__global__ void __launch_bounds__(32) k_delta_t_dd(int d, const double* __restrict__ G, const double* __restrict__ B,
+                                                   double* __restrict__ hi, double* __restrict__ lo) {
+  __shared__ double zh[kMaxD], zl[kMaxD];
+  const int j = blockIdx.x, lane = threadIdx.x;
+  for (int i = lane; i < d; i += 32) zh[i] = zl[i] = 0.0;
+  for (int i = j; i < d; ++i) {
+    __syncwarp();
+    Dd s = {0.0, 0.0};
+    for (int m = j + lane; m < i; m += 32) s = dd_add(s, dd_mul({zh[m], zl[m]}, -B[(int64_t)i * d + m]));
+    s = dd_warp_sum(s);
+    if (lane == 0) {
+      if (i == j) s = {1.0, 0.0};  // the sum is empty
+      zh[i] = s.h;
+      zl[i] = s.l;
+    }
+  }
+  for (int i = d - 1; i >= 0; --i) {
+    __syncwarp();
+    Dd s = {0.0, 0.0};
+    for (int m = i + 1 + lane; m < d; m += 32) s = dd_add(s, dd_mul({zh[m], zl[m]}, -G[(int64_t)m * d + i]));
+    s = dd_warp_sum(s);
+    if (lane == 0) {
+      s = dd_div(dd_add({zh[i], zl[i]}, s), G[(int64_t)i * d + i]);
+      zh[i] = s.h;
+      zl[i] = s.l;
+    }
+  }
+  __syncwarp();
+  for (int i = lane; i < d; i += 32) {
+    hi[(int64_t)j * d + i] = zh[i];
+    lo[(int64_t)j * d + i] = zl[i];
+  }
+}
+
+// x 2^s toward zero, for |x| 2^s < 2^126.
+__device__ __int128 scaled_int(double x, int s) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff);
+  if (e == 0) return 0;
+  const __int128 m = (__int128)((b & 0xfffffffffffffull) | (1ull << 52));
+  const int t = e - 1075 + s;
+  const __int128 q = t >= 0 ? (t < 74 ? m << t : 0) : (t > -64 ? m >> -t : 0);
+  return b >> 63 ? -q : q;
+}
+// As k_crt_image for one operator given as hi + lo; up: 2^a of the rows.
+__global__ void __launch_bounds__(256) k_crt_image_dd(const double* __restrict__ hi, const double* __restrict__ lo,
+                                                      int d, int K, int Nt, int NT, const double* __restrict__ up,
+                                                      __nv_bfloat16* __restrict__ img) {
+  const int64_t tile_e = (int64_t)K * Nt;
+  const int u = blockIdx.x * 256 + threadIdx.x;
+  if (u >= NT * K * Nt) return;
+  const int n = u % Nt, l = (u / Nt) % K, nt = u / (Nt * K), mp = nt * Nt + n;
+  __int128 w = 0;
+  if (mp < d && l < d) {
+    const int s = (int)(((unsigned long long)__double_as_longlong(up[mp]) >> 52) & 0x7ff) - 1023;
+    w = scaled_int(hi[(int64_t)l * d + mp], s) + scaled_int(lo[(int64_t)l * d + mp], s);
+  }
+  __nv_bfloat16* dst = img + (int64_t)nt * tile_e + ((int64_t)(l / 8) * Nt + n) * 8 + (l & 7);
+  for (int i = 0; i < kBoxMods; ++i) {
+    const int m = crt_mod(i);
+    int r = (int)(w % m);
+    if (2 * r > m) r -= m;
+    if (2 * r < -m) r += m;
+    dst[(int64_t)i * NT * tile_e] = __float2bfloat16_rn((float)r);
   }
 }
 
@@ -686,23 +848,37 @@ __global__ void __launch_bounds__(128) k_crt_kappa(int kern, int d, double lk, c
   }
 }
 
-unsigned __int128 crt_product() {
-  unsigned __int128 M = 1;
-  for (int i = 0; i < kMods; ++i) M *= (unsigned)crt_mod(i);
-  return M;
+// Product of the first n moduli times 2^-shift.
+double crt_product_scaled(int n, int shift) {
+  unsigned __int128 m = 1;  // exact to 125 bits, then the moduli beyond in FP64
+  double rest = 1.0;
+  for (int i = 0; i < n; ++i) {
+    if (i < kMods) m *= (unsigned)crt_mod(i);
+    else rest *= crt_mod(i);
+  }
+  return std::ldexp((double)m * rest, -shift);
 }
 
-CrtK crt_constants() {
-  CrtK c;
-  for (int i = 0; i < kMods; ++i) {
-    const int m = crt_mod(i);
-    int p = 1;  // M / m_i modulo m_i
-    for (int j = 0; j < kMods; ++j)
-      if (j != i) p = (int)((int64_t)p * crt_mod(j) % m);
-    int y = 1;
-    while ((int64_t)p * y % m != 1) ++y;
-    const unsigned __int128 k = (((unsigned __int128)y << 96) + m / 2) / m;
-    for (int w = 0; w < 3; ++w) c.k[i][w] = (uint32_t)(k >> (32 * w));
+template <int NM, int NW>
+CrtK<NM, NW> crt_constants() {
+  CrtK<NM, NW> c;
+  for (int i = 0; i < NM; ++i) {
+    const uint64_t m = (uint64_t)crt_mod(i);
+    uint64_t p = 1;  // M / m_i modulo m_i
+    for (int j = 0; j < NM; ++j)
+      if (j != i) p = p * (uint64_t)crt_mod(j) % m;
+    uint64_t y = 1;
+    while (p * y % m != 1) ++y;
+    // y / m to NW words by long division, rounded to nearest
+    uint64_t r = y;
+    for (int w = NW - 1; w >= 0; --w) {
+      r <<= 32;
+      c.k[i][w] = (uint32_t)(r / m);
+      r %= m;
+    }
+    if (2 * r >= m)
+      for (int w = 0; w < NW && ++c.k[i][w] == 0; ++w) {
+      }
   }
   return c;
 }
@@ -711,39 +887,43 @@ CrtK crt_constants() {
 constexpr size_t kScratchLimit = (size_t)4 << 30;
 
 size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
-size_t planes_bytes(const CrtImage& im, int h, int snz, int Rc) {
-  return align256((size_t)kMods * Rc * 8 * snz * h * h * im.K * 2);
+// Class grid of a job whose target boxes have level `level`.
+int mode_mods(CrtMode m) { return m == kCrtBox ? kBoxMods : kMods; }
+int mode_ncs(CrtMode m) { return m == kCrtL2L ? 1 : 8; }
+int mode_nct(CrtMode m) { return m == kCrtM2M ? 1 : 8; }
+int mode_h(CrtMode m, int level) { return m == kCrtM2M ? 1 << level : 1 << (level - 1); }
+size_t planes_bytes(CrtMode m, int K, int h, int snz, int Rc) {
+  return align256((size_t)mode_mods(m) * Rc * mode_ncs(m) * snz * h * h * K * 2);
 }
-size_t res_bytes(const CrtImage& im, int h, int nz, int Rc, int G) {
-  return align256((size_t)kMods * G * Rc * 8 * nz * h * h * im.NT * im.Nt * 2);
+size_t res_bytes(CrtMode m, int N, int h, int nz, int Rc, int G) {
+  return align256((size_t)mode_mods(m) * G * Rc * mode_nct(m) * nz * h * h * N * 2);
 }
 constexpr int kMaxGroups = 8;
-// offset groups are used only by launches of few tiles: levels below this one
+// offset groups are used only by M2L launches of few tiles: levels below this one
 constexpr int kGroupLevel = 4;
-size_t job_bytes(const CrtImage& im, int level, int nz, int Rc) {
-  const int h = 1 << (level - 1);
+int max_groups(CrtMode m, int level) { return m == kCrtM2L && level < kGroupLevel ? kMaxGroups : 1; }
+size_t job_bytes(CrtMode m, const CrtImage& im, int level, int nz, int Rc) {
+  const int h = mode_h(m, level);
   const int snz = std::min(h, nz + 2);
-  return planes_bytes(im, h, snz, Rc) + res_bytes(im, h, nz, Rc, level < kGroupLevel ? kMaxGroups : 1);
+  return planes_bytes(m, im.K, h, snz, Rc) + res_bytes(m, im.NT * im.Nt, h, nz, Rc, max_groups(m, level));
 }
 // columns and planes of one slab of a level within `limit` bytes
-void slab_shape(const CrtImage& im, int level, int R, size_t limit, int* Rc, int* nz) {
-  const int h = 1 << (level - 1);
+void slab_shape(CrtMode m, const CrtImage& im, int level, int R, size_t limit, int* Rc, int* nz) {
   *Rc = R;
-  *nz = h;
-  while (*Rc > 1 && job_bytes(im, level, *nz, *Rc) > limit) *Rc = (*Rc + 1) / 2;
-  while (*nz > kTZ && job_bytes(im, level, *nz, *Rc) > limit) *nz = std::max(kTZ, (*nz / 2 + kTZ - 1) / kTZ * kTZ);
+  *nz = mode_h(m, level);
+  while (*Rc > 1 && job_bytes(m, im, level, *nz, *Rc) > limit) *Rc = (*Rc + 1) / 2;
+  while (*nz > kTZ && job_bytes(m, im, level, *nz, *Rc) > limit) *nz = std::max(kTZ, (*nz / 2 + kTZ - 1) / kTZ * kTZ);
 }
 
 }  // namespace
 
-size_t crt_scratch_bytes(int depth, const CrtImage* const* img, int R) {
+size_t crt_scratch_bytes(int njobs, const CrtJob* jobs, int R) {
   size_t total = 0, most = 0;
-  for (int k = 2; k <= depth; ++k) {
-    if (!img[k] || !img[k]->img) continue;
+  for (int j = 0; j < njobs; ++j) {
     int Rc, nz;
-    slab_shape(*img[k], k, R, kScratchLimit, &Rc, &nz);
-    const size_t n = job_bytes(*img[k], k, nz, Rc);
-    total += n;
+    slab_shape(jobs[j].mode, *jobs[j].img, jobs[j].level, R, kScratchLimit, &Rc, &nz);
+    const size_t n = job_bytes(jobs[j].mode, *jobs[j].img, jobs[j].level, nz, Rc);
+    if (jobs[j].mode == kCrtM2L) total += n;  // the levels of the M2L share a launch
     most = std::max(most, n);
   }
   return std::max(most, std::min(total, kScratchLimit));
@@ -755,25 +935,27 @@ void free_crt_image(CrtImage* im) {
   *im = CrtImage();
 }
 
-eifmm_status build_crt_image(const double* kdT, int d, CrtImage* im, cudaStream_t s) {
+eifmm_status build_crt_image(const double* kdT, int nslots, int dl, int d, CrtImage* im, cudaStream_t s) {
   im->d = d;
-  im->K = (d + 15) / 16 * 16;
-  im->NT = (im->K + 255) / 256;
-  im->Nt = ((im->K / 16 + im->NT - 1) / im->NT) * 16;
+  im->dl = dl;
+  im->nslots = nslots;
+  im->K = (dl + 15) / 16 * 16;
+  im->NT = (d + 255) / 256;
+  im->Nt = (((d + 15) / 16 + im->NT - 1) / im->NT) * 16;
   double* tmp = nullptr;  // largest entry, sum and 2^a of each row
   eifmm_status rc = dalloc(&tmp, (size_t)3 * d);
   if (rc == EIFMM_OK) rc = dalloc(&im->colscale, d);
-  const size_t e = (size_t)kMods * kNumSlots * im->NT * im->K * im->Nt;
+  const size_t e = (size_t)kMods * nslots * im->NT * im->K * im->Nt;
   if (rc == EIFMM_OK) rc = dmalloc(&im->img, e * sizeof(__nv_bfloat16));
   if (rc == EIFMM_OK) {
-    k_crt_rowsum<<<(d + 31) / 32, dim3(32, 32), 0, s>>>(kdT, d, tmp, tmp + d);
+    k_crt_rowsum<<<(d + 31) / 32, dim3(32, 32), 0, s>>>(kdT, nslots, dl, d, tmp, tmp + d);
     count_launch();
-    const double mscale = std::ldexp((double)crt_product(), -96);
-    k_crt_rowscale<<<(d + 127) / 128, 128, 0, s>>>(tmp, tmp + d, d, mscale, tmp + 2 * d, im->colscale);
+    const double mscale = crt_product_scaled(kMods, 96);
+    k_crt_rowscale<<<(d + 127) / 128, 128, 0, s>>>(tmp, tmp + d, d, mscale, kRowBits, kEntryBits, tmp + 2 * d, im->colscale);
     count_launch();
     const int units = im->NT * (im->K / 8) * im->Nt;
-    k_crt_image<<<dim3((units + 255) / 256, kNumSlots), 256, 0, s>>>(kdT, d, im->K, im->Nt, im->NT, tmp + 2 * d,
-                                                                     (__nv_bfloat16*)im->img);
+    k_crt_image<<<dim3((units + 255) / 256, nslots), 256, 0, s>>>(kdT, nslots, dl, d, im->K, im->Nt, im->NT,
+                                                                  tmp + 2 * d, (__nv_bfloat16*)im->img);
     count_launch();
     // other streams may read the image as soon as this returns
     if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
@@ -783,6 +965,55 @@ eifmm_status build_crt_image(const double* kdT, int d, CrtImage* im, cudaStream_
   }
   dfree(tmp);
   if (rc != EIFMM_OK) free_crt_image(im);
+  return rc;
+}
+
+eifmm_status build_crt_delta_image(const LevelOps& v, CrtImage* im, cudaStream_t s) {
+  const int d = v.d;
+  im->d = im->dl = d;
+  im->nslots = 1;
+  im->K = (d + 15) / 16 * 16;
+  im->NT = (d + 255) / 256;
+  im->Nt = (((d + 15) / 16 + im->NT - 1) / im->NT) * 16;
+  double* tmp = nullptr;  // Delta^t hi and lo, then per row: largest entry, sum, 2^a
+  const size_t dd = (size_t)d * d;
+  eifmm_status rc = dalloc(&tmp, 2 * dd + 3 * d);
+  if (rc == EIFMM_OK) rc = dalloc(&im->colscale, d);
+  if (rc == EIFMM_OK) rc = dmalloc(&im->img, (size_t)kBoxMods * im->NT * im->K * im->Nt * sizeof(__nv_bfloat16));
+  bool fine = false;
+  if (rc == EIFMM_OK) {
+    double *hi = tmp, *lo = tmp + dd, *row = tmp + 2 * dd;
+    k_delta_t_dd<<<d, 32, 0, s>>>(d, v.G_rm, v.B_rm, hi, lo);
+    count_launch();
+    k_crt_rowsum<<<(d + 31) / 32, dim3(32, 32), 0, s>>>(hi, 1, d, d, row, row + d);
+    count_launch();
+    k_crt_rowscale<<<(d + 127) / 128, 128, 0, s>>>(row, row + d, d, crt_product_scaled(kBoxMods, 128), kBoxRowBits,
+                                                   kBoxRowBits, row + 2 * d, im->colscale);
+    count_launch();
+    k_crt_image_dd<<<(im->NT * im->K * im->Nt + 255) / 256, 256, 0, s>>>(hi, lo, d, im->K, im->Nt, im->NT, row + 2 * d,
+                                                                         (__nv_bfloat16*)im->img);
+    count_launch();
+    std::vector<double> up(d);
+    double g11 = 0.0;
+    if (cudaMemcpyAsync(up.data(), row + 2 * d, d * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaMemcpyAsync(&g11, v.G_rm, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
+      set_error("building the residue image of Delta^t failed");
+      rc = EIFMM_ECUDA;
+    } else {
+      // the entries are rounded to 2^-a: times |A| <= |Gamma_11| and d terms
+      // that is the backward error of the product, which stays below 2^-52 as
+      // the triangular solves' does (1/r at eps 1e-7: 2^-55)
+      double q = 0.0;
+      for (double u : up) q = std::max(q, 1.0 / u);
+      fine = q * std::fabs(g11) * d <= 0x1p-52;
+    }
+  }
+  dfree(tmp);
+  if (rc != EIFMM_OK || !fine) {
+    free_crt_image(im);
+    im->refused = rc == EIFMM_OK;
+  }
   return rc;
 }
 
@@ -803,14 +1034,15 @@ eifmm_status crt_kappa(int kern, const LevelOps& v, double lk, double* kappa, cu
   return EIFMM_OK;
 }
 
-eifmm_status launch_m2l_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t buf_bytes,
+eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t buf_bytes,
                             unsigned long long* wmax, int nsm, int* err, cudaStream_t s) {
   auto encode = encode_fn();
   if (!encode) {
     set_error("cuTensorMapEncodeTiled is not available from the driver");
     return EIFMM_ECUDA;
   }
-  static const CrtK kc = crt_constants();
+  static const CrtK<kMods, 3> kc = crt_constants<kMods, 3>();
+  static const CrtK<kBoxMods, 4> kcb = crt_constants<kBoxMods, 4>();
   static bool attr[64] = {};
   int dev = 0;
   EIFMM_CUDA(cudaGetDevice(&dev));
@@ -825,13 +1057,21 @@ eifmm_status launch_m2l_crt(int njobs, const CrtJob* jobs, int R, void* buf, siz
   for (int j = njobs - 1; j >= 0; --j) {
     const CrtJob& b = jobs[j];
     int Rc, nz;
-    slab_shape(*b.img, b.level, R, kScratchLimit, &Rc, &nz);
-    const int h = 1 << (b.level - 1);
+    slab_shape(b.mode, *b.img, b.level, R, kScratchLimit, &Rc, &nz);
+    const int h = mode_h(b.mode, b.level);
     for (int r0 = 0; r0 < R; r0 += Rc)
       for (int z0 = 0; z0 < h; z0 += nz) {
         CrtLv v = {};
-        v.level = b.level;
+        v.mode = b.mode;
+        v.tlevel = b.level;
+        v.slevel = b.mode == kCrtM2M ? b.level + 1 : b.mode == kCrtL2L ? b.level - 1 : b.level;
+        v.ncs = mode_ncs(b.mode);
+        v.nct = mode_nct(b.mode);
+        v.nw = b.mode == kCrtM2L ? 24 : b.mode == kCrtM2M ? 8 : 1;
+        v.nslots = b.img->nslots;
+        v.wbits = b.mode == kCrtBox ? kBoxWBits : kWBits;
         v.d = b.img->d;
+        v.ds = b.img->dl;
         v.K = b.img->K;
         v.Nt = b.img->Nt;
         v.NT = b.img->NT;
@@ -846,6 +1086,7 @@ eifmm_status launch_m2l_crt(int njobs, const CrtJob* jobs, int R, void* buf, siz
         split_chunks(&v);
         v.W = b.W;
         v.g = b.g;
+        v.add = b.add;
         v.img = (const __nv_bfloat16*)b.img->img;
         v.colscale = b.img->colscale;
         v.wmax = wmax + (size_t)b.level * R;
@@ -859,15 +1100,14 @@ eifmm_status launch_m2l_crt(int njobs, const CrtJob* jobs, int R, void* buf, siz
     size_t off = 0, i1 = i0;
     int64_t items = 0;
     auto tiles = [](const CrtLv& v) {
-      return (int64_t)((v.h + kTX - 1) / kTX) * ((v.h + kTY - 1) / kTY) * ((v.nz + kTZ - 1) / kTZ) * 8 * v.NT * v.Rc *
-             kMods;
+      return (int64_t)((v.h + kTX - 1) / kTX) * ((v.h + kTY - 1) / kTY) * ((v.nz + kTZ - 1) / kTZ) * v.nct * v.NT * v.Rc *
+             mode_mods(v.mode);
     };
     for (; i1 < todo.size() && a.nlev < kMaxLv; ++i1) {
       const CrtLv& v = todo[i1];
-      const size_t need = planes_bytes(CrtImage{nullptr, nullptr, 0.0, v.d, v.K, v.Nt, v.NT}, v.h, v.snz, v.Rc) +
-                          res_bytes(CrtImage{nullptr, nullptr, 0.0, v.d, v.K, v.Nt, v.NT}, v.h, v.nz, v.Rc,
-                                    v.level < kGroupLevel ? kMaxGroups : 1);
-      if (a.nlev > 0 && off + need > buf_bytes) break;
+      const size_t need = planes_bytes(v.mode, v.K, v.h, v.snz, v.Rc) +
+                          res_bytes(v.mode, v.NT * v.Nt, v.h, v.nz, v.Rc, max_groups(v.mode, v.tlevel));
+      if (a.nlev > 0 && (off + need > buf_bytes || mode_mods(v.mode) != mode_mods(a.lv[0].mode))) break;
       if (need > buf_bytes) {
         set_error("residue M2L: scratch too small");
         return EIFMM_EINVAL;
@@ -882,30 +1122,28 @@ eifmm_status launch_m2l_crt(int njobs, const CrtJob* jobs, int R, void* buf, siz
     size_t pl_smem = 0;
     for (int q = 0; q < a.nlev; ++q) {
       CrtLv& v = a.lv[q];
-      const CrtImage im{nullptr, nullptr, 0.0, v.d, v.K, v.Nt, v.NT};
       // a launch of few tiles: the windows of the coarse levels' tiles are
       // split into groups until the CTAs cover four waves
       v.G = 1;
-      if (v.level < kGroupLevel)
-        while (v.G < kMaxGroups && items * v.G < 4 * (int64_t)nsm) v.G *= 2;
+      while (v.G < max_groups(v.mode, v.tlevel) && items * v.G < 4 * (int64_t)nsm) v.G *= 2;
       v.planes = (__nv_bfloat16*)((char*)buf + off);
-      off += planes_bytes(im, v.h, v.snz, v.Rc);
+      off += planes_bytes(v.mode, v.K, v.h, v.snz, v.Rc);
       v.res = (int16_t*)((char*)buf + off);
-      off += res_bytes(im, v.h, v.nz, v.Rc, v.G);
+      off += res_bytes(v.mode, v.NT * v.Nt, v.h, v.nz, v.Rc, v.G);
       v.item0 = it;
       v.pl0 = pl;
       v.rc0 = rb;
       v.mx0 = mx;
       it += (unsigned)(tiles(v) * v.G);
-      pl += (unsigned)((int64_t)((v.h + 7) / 8) * v.h * v.snz * 8 * v.Rc);
-      rb += (unsigned)(((int64_t)v.nz * v.h * v.h * 8 * v.Rc + 3) / 4);
-      mx += (unsigned)((((int64_t)1 << (3 * v.level)) * v.d + kMaxPer - 1) / kMaxPer * v.Rc);
+      pl += (unsigned)((int64_t)((v.h + 7) / 8) * v.h * v.snz * v.ncs * v.Rc);
+      rb += (unsigned)(((int64_t)v.nz * v.h * v.h * v.nct * v.Rc + 3) / 4);
+      mx += (unsigned)((((int64_t)1 << (3 * v.slevel)) * v.ds + kMaxPer - 1) / kMaxPer * v.Rc);
       const uint32_t ks = (uint32_t)std::max(v.ks0, v.nchunk > v.n0 ? v.ks1 : 0);
       stage = std::max(stage, ks * 32u * (uint32_t)v.Nt);
       win = std::max(win, ks * kWinStep);
       pl_smem = std::max(pl_smem, (size_t)8 * (v.K + 1) * sizeof(long long));
       const cuuint64_t hh = (cuuint64_t)v.h;
-      cuuint64_t dims[5] = {8 * hh, hh, (cuuint64_t)v.snz, (cuuint64_t)v.K / 8, (cuuint64_t)kMods * v.Rc * 8};
+      cuuint64_t dims[5] = {8 * hh, hh, (cuuint64_t)v.snz, (cuuint64_t)v.K / 8, (cuuint64_t)mode_mods(v.mode) * v.Rc * v.ncs};
       cuuint64_t strides[4] = {16 * hh, 16 * hh * hh, 16 * hh * hh * v.snz, 16 * hh * hh * v.snz * (v.K / 8)};
       cuuint32_t box[5] = {8 * (kTX + 2), kTY, kTZ + 2, 2, 1};
       cuuint32_t estr[5] = {1, 1, 1, 1, 1};
@@ -925,11 +1163,14 @@ eifmm_status launch_m2l_crt(int njobs, const CrtJob* jobs, int R, void* buf, siz
     // per slab gives the same value
     k_crt_max<<<mx, 256, 0, s>>>(a);
     EIFMM_CHECK_LAUNCH();
-    k_crt_planes<<<pl, 256, pl_smem, s>>>(a);
+    const bool box = a.lv[0].mode == kCrtBox;
+    if (box) k_crt_planes<kBoxMods><<<pl, 256, pl_smem, s>>>(a);
+    else k_crt_planes<kMods><<<pl, 256, pl_smem, s>>>(a);
     EIFMM_CHECK_LAUNCH();
     k_crt_gemm<<<it, kThreads, smem, s>>>(maps, a);
     EIFMM_CHECK_LAUNCH();
-    k_crt_rebuild<<<rb, 128, 0, s>>>(a, kc);
+    if (box) k_crt_rebuild<kBoxMods, 4><<<rb, 128, 0, s>>>(a, kcb);
+    else k_crt_rebuild<kMods, 3><<<rb, 128, 0, s>>>(a, kc);
     EIFMM_CHECK_LAUNCH();
     i0 = i1;
   }

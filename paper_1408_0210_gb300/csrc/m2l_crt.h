@@ -1,26 +1,37 @@
-// m2l_crt.h -- launcher of the FP64 M2L on the tensor cores (m2l_crt.cu).
+// m2l_crt.h -- launcher of the FP64 products on the tensor cores (m2l_crt.cu).
 #pragma once
 #include "internal.h"
 
 namespace eifmm {
 
-// Step 4 of one level: g[I][r] = sum_J K^delta W[J][r] on FP64 arrays
-// [box (Morton)][R][d].
+// One level of a product g[I][r] = add[I][r] + sum_J T^{IJ} W[J][r] on FP64
+// arrays [box (Morton)][R][rank], `level` the level of the target boxes I.
+enum CrtMode {
+  kCrtM2L = 0,  // J in the interaction list, 343 operators by offset
+  kCrtM2M = 1,  // J the 8 children, 8 operators by octant
+  kCrtL2L = 2,  // J the parent, 8 operators by octant
+  kCrtBox = 3,  // J = I, one operator (Delta^t at the leaf level)
+};
 struct CrtJob {
+  CrtMode mode;
   int level;
   const CrtImage* img;
   const double* W;
   double* g;
+  const double* add;
 };
-// Bytes of scratch the jobs of levels 2..depth use at most (img: per level);
-// levels whose planes exceed the library's limit run in slabs and columns.
-size_t crt_scratch_bytes(int depth, const CrtImage* const* img, int R);
+// Scratch for the jobs of one call (M2L jobs run together, others one by one);
+// jobs beyond the library's limit run in slabs and columns.
+size_t crt_scratch_bytes(int njobs, const CrtJob* jobs, int R);
 // All jobs on stream s, in `buf` (buf_bytes from crt_scratch_bytes); wmax:
 // [kMaxLevel + 1][R] words; err: error word of the bounded waits.
-eifmm_status launch_m2l_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t buf_bytes,
-                            unsigned long long* wmax, int nsm, int* err, cudaStream_t s);
-// The residue image of an operator stack kdT ([343][l][m'], d x d).
-eifmm_status build_crt_image(const double* kdT, int d, CrtImage* img, cudaStream_t s);
+eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t buf_bytes, unsigned long long* wmax,
+                        int nsm, int* err, cudaStream_t s);
+// The residue image of an operator stack [nslots][l < dl][m' < d].
+eifmm_status build_crt_image(const double* kdT, int nslots, int dl, int d, CrtImage* img, cudaStream_t s);
+// The residue image of Delta^t of a level, from Gamma and B in double-double.
+// An operator set too ill conditioned for its 104 bits sets img->refused.
+eifmm_status build_crt_delta_image(const LevelOps& v, CrtImage* img, cudaStream_t s);
 // How much the operators of a level amplify rounding: the largest, over the
 // offsets, of max_{m'} sum_l |T_{m'l}| |K(x_l, y)| over max_{m'} |K(y_{m'}, y +
 // delta)| for a unit charge at the first node y of the box, whose W is K(x_l, y)

@@ -286,6 +286,9 @@ void free_ops(Ops* ops) {
     dfree(v.kscale);
     free_crt_image(&v.crt);
     free_crt_image(&v.crtc);
+    free_crt_image(&v.crt_m2m);
+    free_crt_image(&v.crt_l2l);
+    free_crt_image(&v.crt_dt);
     dfree(v.U);
     dfree(v.Ct);
     dfree(v.kd32);

@@ -326,8 +326,8 @@ eifmm_status m2l_compressed(Workspace& ws, const Ops* ops, int k, int R, bool fp
   double* wt = (double*)ws.tmp;  // rows x r
   EIFMM_TRY(gemm64(false, rows, r, d, ws.Wh[k], d, v.U, r, wt, r, s));
   if (!fp64 && v.crtc.img && ws.crt_bytes > 0) {
-    const CrtJob job{k, &v.crtc, wt, ws.Wh[k]};
-    EIFMM_TRY(launch_m2l_crt(1, &job, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
+    const CrtJob job{kCrtM2L, k, &v.crtc, wt, ws.Wh[k], nullptr};
+    EIFMM_TRY(launch_crt(1, &job, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
   } else if (pair) {
     EIFMM_TRY(launch_m2l_df(k, r, R, v.Ct, ops->d_slot_lists, wt, ws.Wh[k], ws.part64, ws.part64_cap, ws.nsm, s));
   } else {

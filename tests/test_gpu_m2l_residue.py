@@ -1,4 +1,4 @@
-"""The FP64 M2L by residues on the tensor cores against the FP64 M2L on the
+"""The FP64 products by residues on the tensor cores: the M2L against the one on the
 FP64 pipes (option m2l_fp64), at the edges of its tiles.
 
 Tolerance: both sum n = 189 d products.  The FP64 kernel's rounding is at most
@@ -73,3 +73,40 @@ def test_residue_m2l_extreme_scales(E):
     assert not out[0.0].any()
     for scale in (2.0 ** 900, 2.0 ** -900):  # a power of two changes no mantissa
         assert np.array_equal(out[scale], out[1.0] * scale)
+
+
+# M2M, L2L and Delta^t by residues: ranks that differ from level to level, with
+# remainders of a k-step and of a column tile, one and two column tiles, several
+# columns.  Against the CPU EIFMM of the same levels: both carry FP64 rounding
+# through the chain (1e-12, as for the whole FP64 path; at eps 1e-8 the sums of
+# 189 d products of operators with kappa 7e3 add 189 d 2^-53 10 = 6e-11).
+@pytest.mark.parametrize("eps,ranks,R,tol", [(1e-6, (70, 129, 193), 1, 1e-12), (1e-6, (193, 65, 8), 3, 1e-12),
+                                             (1e-8, (270, 300, 265), 1, 1e-10)])
+def test_residue_transfers_match_the_oracle(E, eps, ranks, R, tol):
+    import oracle as orc
+    depth, n = 4, 5000
+    x = wl.uniform_cube(n, 41)
+    s = wl.sigma_uniform(n, R, 42)
+    lv = {}
+    for k, d in zip(range(2, depth + 1), ranks):
+        e = orc.eim("inv_r", orc.train_x(k), orc.train_y(k), eps)
+        d = min(d, e["d"])
+        lv[k] = dict(d=d, X=e["X"][:d], Y=e["Y"][:d], Gamma=np.ascontiguousarray(e["Gamma"][:d, :d]),
+                     B=np.ascontiguousarray(e["B"][:d, :d]), eps_est=eps)
+    f2, dm = orc.eifmm("inv_r", 1.0, [0, 0, 0], depth, lv, x, x, s, dump=True)
+    ops = E.eifmm_ops_load("inv_r", 1.0, depth, lv)
+    tree = E.eifmm_tree_build(dev(x), None, (0, 0, 0), 1.0, depth, True)
+    f = torch.zeros(R, n, dtype=torch.float64, device="cuda").T
+    E.eifmm_evaluate(tree, ops, dev(s.T).T, f, "fp64")
+    torch.cuda.synchronize()
+    rel = lambda a, b: float(np.abs(a - np.asarray(b).reshape(a.shape)).max() / np.abs(b).max())  # noqa: E731
+    for k in range(2, depth + 1):
+        assert rel(E.eifmm_debug_export(tree, 0, k, lv[k]["d"], R), dm["W"][k]) <= tol, k
+        assert rel(E.eifmm_debug_export(tree, 3, k, lv[k]["d"], R), dm["l"][k]) <= tol, k
+    # Delta^t l: backward error, A^t lhat = l
+    A = 1.0 / np.linalg.norm(lv[depth]["X"][:, None] - lv[depth]["Y"][None], axis=-1)
+    lh = E.eifmm_debug_export(tree, 4, depth, lv[depth]["d"], R)
+    ll = E.eifmm_debug_export(tree, 3, depth, lv[depth]["d"], R)
+    assert np.abs(lh @ A - ll).max() <= 1e-12 * (np.abs(lh) @ A).max()
+    assert rel(E.eifmm_debug_export(tree, 5, depth, 0, R), dm["f_far"]) <= tol
+    assert rel(f.cpu().numpy(), f2) <= tol
