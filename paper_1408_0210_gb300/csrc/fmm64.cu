@@ -565,7 +565,12 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   // step 1
   const LevelOps& vl = ops->lv[kap];
   EIFMM_CUDA(cudaMemsetAsync(ws.W[kap], 0, sizeof(double) * ((size_t)1 << (3 * kap)) * R * vl.d, s));
-  if (ws.fx_src) {
+  // Where the M2L keeps FP32 pairs (kCrtMaxKappa), their rounding depends on the
+  // last bits of W: there W comes from the FP64 pipes as before.
+  bool pairs = false;
+  for (int k = 2; k <= kap; ++k)
+    pairs = pairs || (pair_m2l && !t->opt[EIFMM_OPT_M2L_FP64] && !ops->compressed && ops->lv[k].crt.kappa > kCrtMaxKappa);
+  if (ws.fx_src && !pairs) {
     EIFMM_TRY(launch_p2m_fx(t, vl, R, ws.W[kap], s));
   } else if (S.n_nonempty > 0) {
     k_p2m64<<<S.n_nonempty, TPB, 0, s>>>(kern, S.nonempty, S.leaf_off, S.x, S.y, S.z, ws.sig, S.n, R, kap, t->lo[0],
@@ -577,7 +582,7 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   for (int k = kap - 1; k >= 2; --k) {
     const int dk = ops->lv[k].d, dc = ops->lv[k + 1].d;
     const int64_t np = (int64_t)1 << (3 * k);
-    if (crt_transfer(ws, ops->lv[k].crt_m2m, np, R)) {
+    if (!pairs && crt_transfer(ws, ops->lv[k].crt_m2m, np, R)) {
       const CrtJob job{kCrtM2M, k, &ops->lv[k].crt_m2m, ws.W[k + 1], ws.W[k], nullptr};
       EIFMM_TRY(launch_crt(1, &job, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
       continue;

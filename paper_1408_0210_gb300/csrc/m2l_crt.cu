@@ -637,13 +637,16 @@ k_crt_rebuild(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK<NM
 }
 
 // ---------------------------------------------------------- the images --
-// Largest entry and sum of |T| over slots and l for 32 rows m' per block.
-__global__ void __launch_bounds__(1024) k_crt_rowsum(const double* __restrict__ kdT, int nslots, int dl, int d,
-                                                     double* __restrict__ mx, double* __restrict__ l1) {
-  const int mp = blockIdx.x * 32 + threadIdx.x;
+// Largest entry and sum of |T| over slots and l for 32 rows m' and one of the
+// kRowParts shares of the (slot, l) per block: part[share][0 or 1][m'].
+constexpr int kRowParts = 64;
+__global__ void __launch_bounds__(256) k_crt_rowsum(const double* __restrict__ kdT, int nslots, int dl, int d,
+                                                    double* __restrict__ part) {
+  const int mp = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y;
+  const int64_t n = (int64_t)nslots * dl, i0 = n * y / kRowParts, i1 = n * (y + 1) / kRowParts;
   double s = 0.0, m = 0.0;
   if (mp < d)
-    for (int64_t i = threadIdx.y; i < (int64_t)nslots * dl; i += 32) {
+    for (int64_t i = i0 + threadIdx.y; i < i1; i += 8) {
       const int slot = (int)(i / dl);
       const int dx = slot % 7 - 3, dy = (slot / 7) % 7 - 3, dz = slot / 49 - 3;
       if (nslots == kNumSlots && abs(dx) <= 1 && abs(dy) <= 1 && abs(dz) <= 1) continue;  // the near field
@@ -651,31 +654,36 @@ __global__ void __launch_bounds__(1024) k_crt_rowsum(const double* __restrict__ 
       s += t;
       m = fmax(m, t);
     }
-  __shared__ double ss[32][33], sm[32][33];
+  __shared__ double ss[8][33], sm[8][33];
   ss[threadIdx.y][threadIdx.x] = s;
   sm[threadIdx.y][threadIdx.x] = m;
   __syncthreads();
   if (threadIdx.y == 0 && mp < d) {
-    for (int k = 1; k < 32; ++k) {
+    for (int k = 1; k < 8; ++k) {
       s += ss[k][threadIdx.x];
       m = fmax(m, sm[k][threadIdx.x]);
     }
-    l1[mp] = s;
-    mx[mp] = m;
+    part[(int64_t)(2 * y) * d + mp] = m;
+    part[(int64_t)(2 * y + 1) * d + mp] = s;
   }
 }
 
 // Exponents a of the rows: l1 2^a < 2^rowbits and mx 2^a < 2^entrybits.
-__global__ void k_crt_rowscale(const double* __restrict__ mx, const double* __restrict__ l1, int d, double mscale,
-                               int rowbits, int entrybits, double* __restrict__ up, double* __restrict__ colscale) {
+__global__ void k_crt_rowscale(const double* __restrict__ part, int d, double mscale, int rowbits, int entrybits,
+                               double* __restrict__ up, double* __restrict__ colscale) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= d) return;
+  double mx = 0.0, l1 = 0.0;
+  for (int y = 0; y < kRowParts; ++y) {
+    mx = fmax(mx, part[(int64_t)(2 * y) * d + m]);
+    l1 += part[(int64_t)(2 * y + 1) * d + m];
+  }
   int e = 0, e1 = 0;
   // the sum itself carries rounding; 2^-40 relative covers it
-  frexp(l1[m] * (1.0 + 0x1p-40), &e);
-  frexp(mx[m], &e1);
+  frexp(l1 * (1.0 + 0x1p-40), &e);
+  frexp(mx, &e1);
   int s = min(rowbits - e, entrybits - e1);
-  s = l1[m] > 0.0 ? max(-900, min(900, s)) : 0;
+  s = l1 > 0.0 ? max(-900, min(900, s)) : 0;
   up[m] = pow2(s);
   colscale[m] = ldexp(mscale, -s);
 }
@@ -942,20 +950,20 @@ eifmm_status build_crt_image(const double* kdT, int nslots, int dl, int d, CrtIm
   im->K = (dl + 15) / 16 * 16;
   im->NT = (d + 255) / 256;
   im->Nt = (((d + 15) / 16 + im->NT - 1) / im->NT) * 16;
-  double* tmp = nullptr;  // largest entry, sum and 2^a of each row
-  eifmm_status rc = dalloc(&tmp, (size_t)3 * d);
+  double* tmp = nullptr;  // 2^a of each row, then the shares of its largest entry and sum
+  eifmm_status rc = dalloc(&tmp, (size_t)(2 * kRowParts + 1) * d);
   if (rc == EIFMM_OK) rc = dalloc(&im->colscale, d);
   const size_t e = (size_t)kMods * nslots * im->NT * im->K * im->Nt;
   if (rc == EIFMM_OK) rc = dmalloc(&im->img, e * sizeof(__nv_bfloat16));
   if (rc == EIFMM_OK) {
-    k_crt_rowsum<<<(d + 31) / 32, dim3(32, 32), 0, s>>>(kdT, nslots, dl, d, tmp, tmp + d);
+    k_crt_rowsum<<<dim3((d + 31) / 32, kRowParts), dim3(32, 8), 0, s>>>(kdT, nslots, dl, d, tmp + d);
     count_launch();
     const double mscale = crt_product_scaled(kMods, 96);
-    k_crt_rowscale<<<(d + 127) / 128, 128, 0, s>>>(tmp, tmp + d, d, mscale, kRowBits, kEntryBits, tmp + 2 * d, im->colscale);
+    k_crt_rowscale<<<(d + 127) / 128, 128, 0, s>>>(tmp + d, d, mscale, kRowBits, kEntryBits, tmp, im->colscale);
     count_launch();
     const int units = im->NT * (im->K / 8) * im->Nt;
     k_crt_image<<<dim3((units + 255) / 256, nslots), 256, 0, s>>>(kdT, nslots, dl, d, im->K, im->Nt, im->NT,
-                                                                  tmp + 2 * d, (__nv_bfloat16*)im->img);
+                                                                  tmp, (__nv_bfloat16*)im->img);
     count_launch();
     // other streams may read the image as soon as this returns
     if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
@@ -975,9 +983,9 @@ eifmm_status build_crt_delta_image(const LevelOps& v, CrtImage* im, cudaStream_t
   im->K = (d + 15) / 16 * 16;
   im->NT = (d + 255) / 256;
   im->Nt = (((d + 15) / 16 + im->NT - 1) / im->NT) * 16;
-  double* tmp = nullptr;  // Delta^t hi and lo, then per row: largest entry, sum, 2^a
+  double* tmp = nullptr;  // Delta^t hi and lo, then as in build_crt_image
   const size_t dd = (size_t)d * d;
-  eifmm_status rc = dalloc(&tmp, 2 * dd + 3 * d);
+  eifmm_status rc = dalloc(&tmp, 2 * dd + (size_t)(2 * kRowParts + 1) * d);
   if (rc == EIFMM_OK) rc = dalloc(&im->colscale, d);
   if (rc == EIFMM_OK) rc = dmalloc(&im->img, (size_t)kBoxMods * im->NT * im->K * im->Nt * sizeof(__nv_bfloat16));
   bool fine = false;
@@ -985,17 +993,17 @@ eifmm_status build_crt_delta_image(const LevelOps& v, CrtImage* im, cudaStream_t
     double *hi = tmp, *lo = tmp + dd, *row = tmp + 2 * dd;
     k_delta_t_dd<<<d, 32, 0, s>>>(d, v.G_rm, v.B_rm, hi, lo);
     count_launch();
-    k_crt_rowsum<<<(d + 31) / 32, dim3(32, 32), 0, s>>>(hi, 1, d, d, row, row + d);
+    k_crt_rowsum<<<dim3((d + 31) / 32, kRowParts), dim3(32, 8), 0, s>>>(hi, 1, d, d, row + d);
     count_launch();
-    k_crt_rowscale<<<(d + 127) / 128, 128, 0, s>>>(row, row + d, d, crt_product_scaled(kBoxMods, 128), kBoxRowBits,
-                                                   kBoxRowBits, row + 2 * d, im->colscale);
+    k_crt_rowscale<<<(d + 127) / 128, 128, 0, s>>>(row + d, d, crt_product_scaled(kBoxMods, 128), kBoxRowBits,
+                                                   kBoxRowBits, row, im->colscale);
     count_launch();
-    k_crt_image_dd<<<(im->NT * im->K * im->Nt + 255) / 256, 256, 0, s>>>(hi, lo, d, im->K, im->Nt, im->NT, row + 2 * d,
+    k_crt_image_dd<<<(im->NT * im->K * im->Nt + 255) / 256, 256, 0, s>>>(hi, lo, d, im->K, im->Nt, im->NT, row,
                                                                          (__nv_bfloat16*)im->img);
     count_launch();
     std::vector<double> up(d);
     double g11 = 0.0;
-    if (cudaMemcpyAsync(up.data(), row + 2 * d, d * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    if (cudaMemcpyAsync(up.data(), row, d * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaMemcpyAsync(&g11, v.G_rm, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
       set_error("building the residue image of Delta^t failed");
