@@ -1659,6 +1659,7 @@ eifmm_status launch_m2l_level(Tree* t, const Ops* ops, int k, int R, int kind, i
   a.nbox = nboxes(k);
   a.R = R;
   a.rows = a.nbox * R;
+  a.d = v.d;
   a.dp = v.dp;
   a.tmem_cols = v.dp <= 128 ? 128 : (v.dp <= 256 ? 256 : 512);
   a.wa = ws.wa[k];

@@ -62,38 +62,26 @@ __host__ __device__ constexpr uint32_t idesc(uint32_t fmt, uint32_t n) {
   return (1u << 4) | (fmt << 7) | (fmt << 10) | ((n >> 3) << 17) | ((uint32_t)(kRows >> 4) << 24);
 }
 
-template <bool TF32>
-__device__ __forceinline__ void mma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
-  if (TF32)
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(id), "r"(acc));
-  else
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(id), "r"(acc));
-}
-
-// The 4 k-steps x 3 split products of one 128-byte chunk of l:
-//   D (+)= A_hi B_hi^t + A_hi B_lo^t + A_lo B_hi^t.
+// The KS k-steps x 3 split products of one 128-byte chunk of l:
+//   D (+)= A_hi B_hi^t + A_hi B_lo^t + A_lo B_hi^t,
+// issued by the elected lane of a converged warp (tc_ptx.cuh).
 // da / db: descriptors of plane 0 of the stage's A and B; plane 1 sits
 // pa16 / pb16 descriptor units (16 bytes) further and k-step kk at 2 kk (32
 // bytes), which never carries out of the 14-bit address field.  `wide`: a
 // second MMA covers accumulator columns 256.. (dp > 256).
-template <bool TF32>
+template <int KS = 4>
 __device__ __forceinline__ void issue_chunk(uint32_t dacc, uint64_t da, uint64_t db, uint32_t pa16, uint32_t pb16,
-                                            uint32_t id_lo, uint32_t id_hi, bool wide, bool first) {
+                                            uint32_t id_lo, uint32_t id_hi, bool wide, bool first, uint32_t el) {
+  const uint32_t ahi = (uint32_t)(da >> 32), bhi = (uint32_t)(db >> 32);
 #pragma unroll
-  for (int kk = 0; kk < 4; ++kk)
+  for (int kk = 0; kk < KS; ++kk)
 #pragma unroll
     for (int pr = 0; pr < 3; ++pr) {
-      const uint64_t ad = da + (pr == 2 ? pa16 : 0u) + 2u * kk;
-      const uint64_t bd = db + (pr == 1 ? pb16 : 0u) + 2u * kk;
+      const uint32_t ad = (uint32_t)da + (pr == 2 ? pa16 : 0u) + 2u * kk;
+      const uint32_t bd = (uint32_t)db + (pr == 1 ? pb16 : 0u) + 2u * kk;
       const uint32_t acc = (first && kk == 0 && pr == 0) ? 0u : 1u;
-      mma<TF32>(dacc, ad, bd, id_lo, acc);
-      if (wide) mma<TF32>(dacc + 256, ad, bd + 2048u, id_hi, acc);
+      mma_f16_el(dacc, ad, ahi, bd, bhi, id_lo, acc, el);
+      if (wide) mma_f16_el(dacc + 256, ad, ahi, bd + 2048u, bhi, id_hi, acc, el);
     }
 }
 
@@ -114,6 +102,7 @@ k_m2l_tc(M2LTcArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x;
+  const int wu = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp, uniform
   const int esz = TF32 ? 4 : 2;
   const int dp = a.dp;
   const int S = a.stages;
@@ -223,8 +212,9 @@ k_m2l_tc(M2LTcArgs a) {
       fence_async_smem();
       asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(full((nit - 1) % S)) : "memory");
     }
-  } else if (tid == kRows) {
+  } else if (wu == kRows / 32) {
     // ----------------------------------------------------- MMA issuer --
+    const uint32_t el = elect_one();
     const uint32_t id_lo = idesc(TF32 ? 2u : 1u, dp > 256 ? 256u : (uint32_t)dp);
     const uint32_t id_hi = idesc(TF32 ? 2u : 1u, dp > 256 ? (uint32_t)(dp - 256) : 16u);
     // descriptors of the stages' A and B plane 0 (S <= 3), counters instead
@@ -245,8 +235,8 @@ k_m2l_tc(M2LTcArgs a) {
       const bool first = e < a.chains && c == 0;
       const uint64_t da = st == 0 ? dA0 : (st == 1 ? dA1 : dA2);
       const uint64_t db = st == 0 ? dB0 : (st == 1 ? dB1 : dB2);
-      issue_chunk<TF32>(dacc, da, db, a_bytes >> 4, b_bytes >> 4, id_lo, id_hi, dp > 256, first);
-      mma_commit(empty(st));
+      issue_chunk(dacc, da, db, a_bytes >> 4, b_bytes >> 4, id_lo, id_hi, dp > 256, first, el);
+      mma_commit_el(empty(st), el);
       if (++st == S) st = 0, ph ^= 1u;
       if (++c == nchunk) {
         c = 0;
@@ -254,7 +244,7 @@ k_m2l_tc(M2LTcArgs a) {
         if (++ch == a.chains) ch = 0;
       }
     }
-    if (ok && nit >= 1) mma_commit(done_bar);
+    if (ok && nit >= 1) mma_commit_el(done_bar, el);
   }
   // ---------------------------------------------------------- epilogue --
   if (tid < kRows) {
@@ -303,6 +293,7 @@ k_m2l_tma(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUten
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x;
+  const int wu = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp, uniform
   const int esz = TF32 ? 4 : 2;
   const int E = 128 / esz;
   const int dp = a.dp;
@@ -392,8 +383,9 @@ k_m2l_tma(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUten
       }
     }
     drain_fills(it, S, bars, a.err);
-  } else if (tid == 160) {
+  } else if (wu == 5) {
     // ----------------------------------------------------- MMA issuer --
+    const uint32_t el = elect_one();
     const uint32_t id_lo = idesc(TF32 ? 2u : 1u, dp > 256 ? 256u : (uint32_t)dp);
     const uint32_t id_hi = idesc(TF32 ? 2u : 1u, dp > 256 ? (uint32_t)(dp - 256) : 16u);
     // descriptors of the stages' A and B plane 0 (S <= 3), counters instead
@@ -412,8 +404,8 @@ k_m2l_tma(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUten
       const bool first = e < a.chains && c == 0;
       const uint64_t da = st == 0 ? dA0 : (st == 1 ? dA1 : dA2);
       const uint64_t db = st == 0 ? dB0 : (st == 1 ? dB1 : dB2);
-      issue_chunk<TF32>(dacc, da, db, a_bytes >> 4, b_bytes >> 4, id_lo, id_hi, dp > 256, first);
-      mma_commit(empty(st));
+      issue_chunk(dacc, da, db, a_bytes >> 4, b_bytes >> 4, id_lo, id_hi, dp > 256, first, el);
+      mma_commit_el(empty(st), el);
       if (++st == S) st = 0, ph ^= 1u;
       if (++c == nchunk) {
         c = 0;
@@ -421,7 +413,7 @@ k_m2l_tma(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUten
         if (++ch == a.chains) ch = 0;
       }
     }
-    if (ok && nit >= 1) mma_commit(done_bar);
+    if (ok && nit >= 1) mma_commit_el(done_bar, el);
   } else if (tid < 128) {
     // --------------------------------------------------------- epilogue --
     const int xr = xr0 + tid % bxr;
@@ -500,6 +492,7 @@ k_m2l_t256(const __grid_constant__ CUtensorMap tW0, const __grid_constant__ CUte
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int wu = __shfl_sync(0xffffffffu, warp, 0);  // uniform
   const int esz = TF32 ? 4 : 2;
   const int E = 128 / esz;
   const int dp = a.dp;  // 128
@@ -591,8 +584,9 @@ k_m2l_t256(const __grid_constant__ CUtensorMap tW0, const __grid_constant__ CUte
       }
     }
     drain_fills(it, kT2Stages, bars, a.err);
-  } else if (tid == 288) {
+  } else if (wu == 9) {
     // ----------------------------------------------------- MMA issuer --
+    const uint32_t el = elect_one();
     const uint32_t id = idesc(TF32 ? 2u : 1u, (uint32_t)kT2Rows);
     const uint64_t dK0 = sdesc(sbase), dK1 = sdesc(sbase + stage);
     const uint64_t dW0 = dK0 + (2 * k_bytes >> 4), dW1 = dK1 + (2 * k_bytes >> 4);
@@ -612,13 +606,13 @@ k_m2l_t256(const __grid_constant__ CUtensorMap tW0, const __grid_constant__ CUte
         }
         tc_fence_after();
         // A = K^delta planes (M), B = What planes (N): hi*hi, hi*lo, lo*hi
-        issue_chunk<TF32>(dacc, st == 0 ? dK0 : dK1, st == 0 ? dW0 : dW1, k_bytes >> 4, w_bytes >> 4, id, id,
-                          false, i == 0);
-        mma_commit(empty(st));
+        issue_chunk(dacc, st == 0 ? dK0 : dK1, st == 0 ? dW0 : dW1, k_bytes >> 4, w_bytes >> 4, id, id, false,
+                    i == 0, el);
+        mma_commit_el(empty(st), el);
         if (++st == kT2Stages) st = 0, ph ^= 1u;
       }
       done += kSegOffsets;
-      if (ok) mma_commit(sfull(b));
+      if (ok) mma_commit_el(sfull(b), el);
     }
   } else if (warp < 8) {
     // ------------------------------------------------------ epilogue --
@@ -701,6 +695,7 @@ k_m2l_t256s(const __grid_constant__ CUtensorMap tW0, const __grid_constant__ CUt
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int wu = __shfl_sync(0xffffffffu, warp, 0);  // uniform
   const int esz = TF32 ? 4 : 2;
   const int E = 128 / esz;
   const int dp = a.dp;  // 128
@@ -813,8 +808,9 @@ k_m2l_t256s(const __grid_constant__ CUtensorMap tW0, const __grid_constant__ CUt
       }
     }
     drain_fills(it, kT2Stages, bars, a.err);
-  } else if (tid == 288) {
+  } else if (wu == 9) {
     // ----------------------------------------------------- MMA issuer --
+    const uint32_t el = elect_one();
     const uint32_t id = idesc(TF32 ? 2u : 1u, (uint32_t)kT2Rows);
     const uint64_t dK0 = sdesc(sbase), dK1 = sdesc(sbase + stage);
     const uint64_t dW0 = dK0 + (2 * k_bytes >> 4), dW1 = dK1 + (2 * k_bytes >> 4);
@@ -838,12 +834,12 @@ k_m2l_t256s(const __grid_constant__ CUtensorMap tW0, const __grid_constant__ CUt
             break;
           }
           tc_fence_after();
-          issue_chunk<TF32>(dacc, st == 0 ? dK0 : dK1, st == 0 ? dW0 : dW1, k_bytes >> 4, w_bytes >> 4, id, id,
-                            false, i == 0);
-          mma_commit(empty(st));
+          issue_chunk(dacc, st == 0 ? dK0 : dK1, st == 0 ? dW0 : dW1, k_bytes >> 4, w_bytes >> 4, id, id,
+                      false, i == 0, el);
+          mma_commit_el(empty(st), el);
           if (++st == kT2Stages) st = 0, ph ^= 1u;
         }
-        if (ok) mma_commit(sfull(b));
+        if (ok) mma_commit_el(sfull(b), el);
       }
     }
   } else if (warp < 8) {
@@ -994,12 +990,16 @@ k_m2l_h16(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUten
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int wu = __shfl_sync(0xffffffffu, warp, 0);  // uniform
   constexpr int E = 64;                 // FP16 elements per 128-byte chunk
   constexpr int NCH = DP / E;           // chunks of l per offset
   constexpr int HALF = DP / 2;          // columns per drain warp
   constexpr uint32_t a_bytes = 16384u;  // 128 rows x 128 B per plane
   constexpr uint32_t b_bytes = DP * 128u;
   constexpr uint32_t stage = 2 * a_bytes + 2 * b_bytes;
+  // rows m' and k-steps beyond d are neither loaded (rows) nor multiplied
+  const int Nn = (a.d + 15) & ~15;
+  const uint32_t n_bytes = (uint32_t)Nn * 128u;
   constexpr uint32_t tcols = 2 * DP <= 128 ? 128 : (2 * DP <= 256 ? 256 : 512);
   uint64_t* bars = (uint64_t*)(smem + kH16Stages * stage);  // full[2] empty[2] afull[2] aempty[2]
   uint32_t* tslot = (uint32_t*)(bars + 8);
@@ -1078,18 +1078,21 @@ k_m2l_h16(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUten
           break;
         }
         const uint32_t sA = sbase + st * stage;
-        mbar_expect_tx(full(st), 2 * a_bytes + 2 * b_bytes);
+        const char* src = (const char*)a.kd_img + (((size_t)slot * NCH + c) * 2) * b_bytes;
+        mbar_expect_tx(full(st), 2 * a_bytes + 2 * n_bytes);
         tma_load_5d(sA, &tA0, c * E, sxr, sy, sz, sc, full(st));
         tma_load_5d(sA + a_bytes, &tA1, c * E, sxr, sy, sz, sc, full(st));
-        bulk_g2s(sA + 2 * a_bytes, (const char*)a.kd_img + (((size_t)slot * NCH + c) * 2) * b_bytes,
-                 2 * b_bytes, full(st));
+        bulk_g2s(sA + 2 * a_bytes, src, n_bytes, full(st));
+        bulk_g2s(sA + 2 * a_bytes + b_bytes, src + b_bytes, n_bytes, full(st));
         if (++st == kH16Stages) st = 0, ph ^= 1u;
       }
     }
     drain_fills(it, kH16Stages, bars, a.err);
-  } else if (tid == 288) {
+  } else if (wu == 9) {
     // ----------------------------------------------------- MMA issuer --
-    const uint32_t id = idesc(0u /* F16 */, (uint32_t)DP);
+    const uint32_t el = elect_one();
+    const uint32_t id = idesc(0u /* F16 */, (uint32_t)Nn);
+    const int klast = (a.d + 15) / 16 - 4 * (NCH - 1);  // k-steps of the last chunk that hold terms
     const uint64_t dA0 = sdesc(sbase), dA1 = sdesc(sbase + stage);
     const uint64_t dB0 = dA0 + (2 * a_bytes >> 4), dB1 = dA1 + (2 * a_bytes >> 4);
     int st = 0;
@@ -1106,12 +1109,16 @@ k_m2l_h16(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUten
           break;
         }
         tc_fence_after();
-        issue_chunk<false>(dacc, st == 0 ? dA0 : dA1, st == 0 ? dB0 : dB1, a_bytes >> 4, b_bytes >> 4, id, id,
-                           false, c == 0);
-        mma_commit(empty(st));
+        const uint64_t da = st == 0 ? dA0 : dA1, db = st == 0 ? dB0 : dB1;
+        const int ks = c == NCH - 1 ? klast : 4;
+        if (ks == 4) issue_chunk(dacc, da, db, a_bytes >> 4, b_bytes >> 4, id, id, false, c == 0, el);
+        else if (ks == 3) issue_chunk<3>(dacc, da, db, a_bytes >> 4, b_bytes >> 4, id, id, false, c == 0, el);
+        else if (ks == 2) issue_chunk<2>(dacc, da, db, a_bytes >> 4, b_bytes >> 4, id, id, false, c == 0, el);
+        else issue_chunk<1>(dacc, da, db, a_bytes >> 4, b_bytes >> 4, id, id, false, c == 0, el);
+        mma_commit_el(empty(st), el);
         if (++st == kH16Stages) st = 0, ph ^= 1u;
       }
-      if (ok) mma_commit(afull(b));
+      if (ok) mma_commit_el(afull(b), el);
     }
   } else if (warp < 8) {
     // ------------------------------------------------------- drains --
@@ -1148,9 +1155,11 @@ k_m2l_h16(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUten
       float* out = a.out + (size_t)grp * a.part_stride + (size_t)(I * R + r) * DP + HALF * hf;
       const float* inv = s_inv + HALF * hf;
 #pragma unroll
-      for (int j = 0; j < HALF; j += 4)
+      for (int j = 0; j < HALF; j += 4)  // Nn is a multiple of 16; the columns beyond hold nothing
         *reinterpret_cast<float4*>(out + j) =
-            make_float4(acc[j] * inv[j], acc[j + 1] * inv[j + 1], acc[j + 2] * inv[j + 2], acc[j + 3] * inv[j + 3]);
+            HALF * hf + j < Nn ? make_float4(acc[j] * inv[j], acc[j + 1] * inv[j + 1], acc[j + 2] * inv[j + 2],
+                                             acc[j + 3] * inv[j + 3])
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
   tc_fence_before();

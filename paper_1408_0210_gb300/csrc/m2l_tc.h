@@ -11,6 +11,7 @@ struct M2LTcArgs {
   int64_t nbox;          // 8^level
   int R;                 // right-hand sides; rows = nbox * R
   int64_t rows;
+  int d = 0;             // rank (FP16 kernel)
   int dp;                // padded rank (multiple of 64), <= kMaxDpTc
   int tmem_cols;         // power of two >= dp
   const void* wa;        // A planes [2][rows][dp] (BF16 or TF32 bit patterns)
