@@ -18,6 +18,8 @@
 #include <cstring>
 #include <cstdlib>
 
+#include <type_traits>
+
 #include "internal.h"
 #include "m2l_tc.h"
 #include "transfer.cuh"
@@ -56,7 +58,8 @@ __device__ __forceinline__ float kern_pt(int kern, float z0, float z1, float z2)
     const float y = rsqrt_approx(r2);
     return ACC ? y * fmaf(-0.5f * r2, y * y, 1.5f) : y;
   }
-  return ACC ? kern_f32(kern, z0, z1, z2) : kern_f32_fast(kern, z0, z1, z2);
+  const int k = KERN >= 0 ? KERN : kern;
+  return ACC ? kern_f32(k, z0, z1, z2) : kern_f32_fast(k, z0, z1, z2);
 }
 
 // Step 1: one CTA per leaf, threads = m (the d coefficients); the leaf's
@@ -349,6 +352,8 @@ k_p2p32(int kern_rt, const int32_t* __restrict__ leaves, const int32_t* __restri
   __shared__ float s_sh[27][3];  // leaf-centre offset of each segment
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int b = leaves[blockIdx.x];
+  const int beg = toff[b], end = toff[b + 1];
+  if ((int)blockIdx.y >= near_passes(end - beg)) return;
   int c[3];
   morton_decode(b, depth, c);
   const int n = 1 << depth;
@@ -377,7 +382,6 @@ k_p2p32(int kern_rt, const int32_t* __restrict__ leaves, const int32_t* __restri
   }
   __syncthreads();
   const int n_other = s_pos[26], n_all = s_pos[27];
-  const int beg = toff[b], end = toff[b + 1];
   // Target passes: 128 targets while that many remain, else 32 at a time
   // while more than 32 remain, then the rest, so that P x S fills the block
   // (P = 33 alone would leave 29 threads idle; on uniform leaves this
@@ -386,9 +390,11 @@ k_p2p32(int kern_rt, const int32_t* __restrict__ leaves, const int32_t* __restri
   // which saves the re-staging for leaves of more than 128 points.
   const bool once = n_all <= P2P_SRC && R <= RCT;
   bool staged = false;
+  int pass = 0;
   for (int t0 = beg, P = 0; t0 < end; t0 += P) {
     const int m = end - t0;
     P = m >= P2P_THREADS ? P2P_THREADS : (m > 32 ? 32 : m);
+    if (pass++ % (int)gridDim.y != (int)blockIdx.y) continue;
     const int S = P2P_THREADS / P;
     const int ti = tid % P, si = tid / P;
     const bool act = si < S;
@@ -573,6 +579,8 @@ k_p2p32x(const int32_t* __restrict__ leaves, const int32_t* __restrict__ toff, c
   __shared__ float s_sh[27][3];
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int b = leaves[blockIdx.x];
+  const int beg = toff[b], end = toff[b + 1];
+  if ((int)blockIdx.y >= near_passes(end - beg)) return;
   if (w == 0) {
     // segment `lane`: 0..25 the neighbours other than the leaf, 26 itself
     int c[3];
@@ -611,11 +619,11 @@ k_p2p32x(const int32_t* __restrict__ leaves, const int32_t* __restrict__ toff, c
   __syncthreads();
   const int n_real_other = s_pos[25] + s_len[25];
   const int n_other = s_pos[26], n_log = s_pos[27];
-  const int beg = toff[b], end = toff[b + 1];
-  int staged_c0 = -1;
+  int staged_c0 = -1, pass = 0;
   for (int t0 = beg, P = 0; t0 < end; t0 += P) {
     const int m = end - t0;
     P = m >= NF_THREADS ? NF_THREADS : (m > 32 ? 32 : m);
+    if (pass++ % (int)gridDim.y != (int)blockIdx.y) continue;
     const int S = min(NF_THREADS / P, NF_MAXS);
     const int ti = tid % P, si = tid / P;
     const bool act = si < S;
@@ -1561,12 +1569,12 @@ static void p2p_launch(const Tree* t, int kern, const float* sig32, int R, doubl
       cudaFuncSetAttribute(k_p2p32x<ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NF_SMEM);
       if (dev < 64) attr[dev][ACC] = true;
     }
-    k_p2p32x<ACC><<<(unsigned)T.n_nonempty, NF_THREADS, NF_SMEM, s>>>(
+    k_p2p32x<ACC><<<dim3(T.n_nonempty, near_split(T.max_leaf)), NF_THREADS, NF_SMEM, s>>>(
         T.nonempty, T.leaf_off, T.lx, T.ly, T.lz, S.leaf_off, S.lx, S.ly, S.lz, sig32, t->depth, two_l,
         t->exclude_self, fnear);
     return;
   }
-  k_p2p32<KERN, RCT, ACC><<<(unsigned)T.n_nonempty, P2P_THREADS, 0, s>>>(
+  k_p2p32<KERN, RCT, ACC><<<dim3(T.n_nonempty, near_split(T.max_leaf)), P2P_THREADS, 0, s>>>(
       kern, T.nonempty, T.leaf_off, T.lx, T.ly, T.lz, T.n, S.leaf_off, S.lx, S.ly, S.lz,
       sig32, S.n, R, t->depth, two_l, t->exclude_self, fnear);
 }
@@ -1596,23 +1604,26 @@ eifmm_status launch_p2p32(const Tree* t, int kern, const float* sig32, int R, do
     EIFMM_CHECK_LAUNCH();
     return EIFMM_OK;
   }
-  const bool inv = kern == EIFMM_KERNEL_INV_R;
-  if (R == 1) {
-    if (inv) {
-      if (accurate) p2p_launch<EIFMM_KERNEL_INV_R, 1, true>(t, kern, sig32, R, fnear, two_l, s);
-      else p2p_launch<EIFMM_KERNEL_INV_R, 1, false>(t, kern, sig32, R, fnear, two_l, s);
+  // one instance per kernel function: with the choice inside the loop over the
+  // sources and a crowded leaf on one CTA the config-3 near field of 2^20
+  // clustered points took 103 ms, now 24.8
+  auto go = [&](auto k) {
+    constexpr int K = decltype(k)::value;
+    if (R == 1) {
+      if (accurate) p2p_launch<K, 1, true>(t, kern, sig32, R, fnear, two_l, s);
+      else p2p_launch<K, 1, false>(t, kern, sig32, R, fnear, two_l, s);
     } else {
-      if (accurate) p2p_launch<-1, 1, true>(t, kern, sig32, R, fnear, two_l, s);
-      else p2p_launch<-1, 1, false>(t, kern, sig32, R, fnear, two_l, s);
+      if (accurate) p2p_launch<K, 4, true>(t, kern, sig32, R, fnear, two_l, s);
+      else p2p_launch<K, 4, false>(t, kern, sig32, R, fnear, two_l, s);
     }
-  } else {
-    if (inv) {
-      if (accurate) p2p_launch<EIFMM_KERNEL_INV_R, 4, true>(t, kern, sig32, R, fnear, two_l, s);
-      else p2p_launch<EIFMM_KERNEL_INV_R, 4, false>(t, kern, sig32, R, fnear, two_l, s);
-    } else {
-      if (accurate) p2p_launch<-1, 4, true>(t, kern, sig32, R, fnear, two_l, s);
-      else p2p_launch<-1, 4, false>(t, kern, sig32, R, fnear, two_l, s);
-    }
+  };
+  switch (kern) {
+    case EIFMM_KERNEL_INV_R: go(std::integral_constant<int, EIFMM_KERNEL_INV_R>()); break;
+    case EIFMM_KERNEL_CONFIG3: go(std::integral_constant<int, EIFMM_KERNEL_CONFIG3>()); break;
+    case EIFMM_KERNEL_EXP_R2: go(std::integral_constant<int, EIFMM_KERNEL_EXP_R2>()); break;
+    case EIFMM_KERNEL_COS20R_R: go(std::integral_constant<int, EIFMM_KERNEL_COS20R_R>()); break;
+    case EIFMM_KERNEL_SQRT_R2P1: go(std::integral_constant<int, EIFMM_KERNEL_SQRT_R2P1>()); break;
+    default: go(std::integral_constant<int, -1>()); break;
   }
   EIFMM_CHECK_LAUNCH();
   return EIFMM_OK;

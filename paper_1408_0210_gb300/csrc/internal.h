@@ -134,6 +134,7 @@ struct PointSet {
   int32_t* leaf_off = nullptr;  // 8^depth + 1
   int32_t* nonempty = nullptr;  // non-empty leaves
   int32_t n_nonempty = 0;
+  int32_t max_leaf = 0;         // points of the fullest leaf
   double* x = nullptr;          // sorted coordinates (SoA)
   double* y = nullptr;
   double* z = nullptr;
@@ -228,6 +229,19 @@ struct Workspace {
   bool evaluated = false;
   float step_ms[20] = {};
 };
+
+// Near-field passes over the targets of a leaf of n: 128 targets while that
+// many remain, else 32 while more than 32 remain, then the rest.
+__host__ __device__ inline int near_passes(int n) { return n / 128 + (n % 128 + 31) / 32; }
+// CTAs that share the passes of a leaf (gridDim.y of the near-field kernels).
+// One where the fullest leaf has at most eight passes; beyond, a crowded leaf
+// (its sources grow with its targets) would be one long serial CTA at the end.
+// 2^20 points of a mixture of 8 Gaussians (2,000 points in the fullest leaf),
+// config-3 kernel: with one instance per kernel function 103 -> 24.8 ms.
+inline int near_split(int max_leaf) {
+  const int p = near_passes(max_leaf);
+  return p <= 8 ? 1 : (p < 1024 ? (p + 3) / 4 : 256);
+}
 
 constexpr int kNumOptions = 6;  // eifmm_option
 

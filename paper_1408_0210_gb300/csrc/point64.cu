@@ -206,6 +206,8 @@ k_p2p_fx(FxLeaf lf, const int32_t* __restrict__ leaves, const int32_t* __restric
   __shared__ int s_pos[28], s_beg[27];
   const int tid = threadIdx.x, lane = tid & 31;
   const int b = leaves[blockIdx.x], kb = lf.K + 958;
+  const int beg = toff[b], end = toff[b + 1];
+  if ((int)blockIdx.y >= near_passes(end - beg)) return;
   if (tid < 32) {
     int c[3];
     morton_decode(b, lf.depth, c);
@@ -230,13 +232,12 @@ k_p2p_fx(FxLeaf lf, const int32_t* __restrict__ leaves, const int32_t* __restric
   }
   __syncthreads();
   const int total = s_pos[27];
-  const int beg = toff[b], end = toff[b + 1];
-  int staged = -1;
   for (int r0 = 0; r0 < R; r0 += RCT) {
-    staged = -1;
+    int staged = -1, pass = 0;
     for (int t0 = beg, P = 0; t0 < end; t0 += P) {
       const int m = end - t0;
       P = m >= FX_THREADS ? FX_THREADS : (m > 32 ? 32 : m);
+      if (pass++ % (int)gridDim.y != (int)blockIdx.y) continue;
       const int S = min(FX_THREADS / P, 32);
       const int ti = tid % P, si = tid / P;
       const bool act = si < S;
@@ -391,7 +392,7 @@ eifmm_status launch_p2p_fx(const Tree* t, int R, double* fnear, cudaStream_t s) 
   const long long* sq = t->ws.fx_src;
   const long long* tq = t->same ? sq : t->ws.fx_tgt;
 #define EIFMM_P2P_FX(RCT)                                                                                           \
-  k_p2p_fx<RCT><<<T.n_nonempty, FX_THREADS, 0, s>>>(f, T.nonempty, T.leaf_off, T.x, T.y, T.z, tq, tq + T.n,         \
+  k_p2p_fx<RCT><<<dim3(T.n_nonempty, near_split(T.max_leaf)), FX_THREADS, 0, s>>>(f, T.nonempty, T.leaf_off, T.x, T.y, T.z, tq, tq + T.n,         \
                                                     tq + 2 * T.n, T.n, S.leaf_off, S.x, S.y, S.z, sq, sq + S.n,     \
                                                     sq + 2 * S.n, t->ws.sig, S.n, R, t->exclude_self, fnear)
   if (R == 1) EIFMM_P2P_FX(1);

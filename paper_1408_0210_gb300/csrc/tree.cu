@@ -236,11 +236,14 @@ __global__ void k_gather_points(const double* __restrict__ xyz,
   lz[p] = (float)(pz - s_ctr[2 * nc + c[2]]);
 }
 
+// cnt[0]: their number, cnt[1]: the points of the fullest
 __global__ void k_nonempty(const int32_t* __restrict__ off, int64_t nleaf,
                            int32_t* __restrict__ list, int32_t* __restrict__ cnt) {
   const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (b >= nleaf) return;
-  if (off[b + 1] > off[b]) list[atomicAdd(cnt, 1)] = (int32_t)b;
+  const int n = b < nleaf ? off[b + 1] - off[b] : 0;
+  if (n > 0) list[atomicAdd(cnt, 1)] = (int32_t)b;
+  const int most = __reduce_max_sync(0xffffffffu, n);
+  if ((threadIdx.x & 31) == 0 && most > cnt[1]) atomicMax(cnt + 1, most);
 }
 
 struct SortScratch {
@@ -285,7 +288,7 @@ eifmm_status build_pointset(const double* xyz, int64_t n, const double lo[3],
   const int nb1 = nblocks > 0 ? nblocks : 1;
   size_t soff = 0;
   const size_t o_k2 = take(soff, nn * 4), o_v2 = take(soff, nn * 4), o_cnt = take(soff, (size_t)256 * nb1 * 4),
-               o_part = take(soff, scan_tiles((int64_t)256 * nb1) * 4), o_bad = take(soff, 2 * sizeof(int));
+               o_part = take(soff, scan_tiles((int64_t)256 * nb1) * 4), o_bad = take(soff, 3 * sizeof(int));
   // The sort's scratch is kept per device between builds (grown on demand,
   // held until the process exits); builds on one device take turns on it.
   int dev = 0;
@@ -305,7 +308,7 @@ eifmm_status build_pointset(const double* xyz, int64_t n, const double lo[3],
   uint32_t* counts = (uint32_t*)(scratch + o_cnt);
   uint32_t* parts = (uint32_t*)(scratch + o_part);
   int* dbad = (int*)(scratch + o_bad);
-  EIFMM_CUDA(cudaMemsetAsync(dbad, 0, 2 * sizeof(int), s));
+  EIFMM_CUDA(cudaMemsetAsync(dbad, 0, 3 * sizeof(int), s));
 
   const double scale = ldexp(1.0, depth) / L;
   if (n > 0) {
@@ -345,10 +348,11 @@ eifmm_status build_pointset(const double* xyz, int64_t n, const double lo[3],
   }
   k_nonempty<<<(unsigned)((nleaf + 255) / 256), 256, 0, s>>>(ps->leaf_off, nleaf, ps->nonempty, dbad + 1);
   EIFMM_CHECK_LAUNCH();
-  int hb[2] = {0, 0};
-  EIFMM_CUDA(cudaMemcpyAsync(hb, dbad, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  int hb[3] = {0, 0, 0};
+  EIFMM_CUDA(cudaMemcpyAsync(hb, dbad, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
   EIFMM_CUDA(cudaStreamSynchronize(s));
   ps->n_nonempty = hb[1];
+  ps->max_leaf = hb[2];
   if (hb[0] != 0) {
     set_error("eifmm_tree_build: " + std::to_string(hb[0]) +
               " coordinates lie outside the cube [lo, lo + L]^3");
