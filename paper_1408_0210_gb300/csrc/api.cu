@@ -85,6 +85,11 @@ void free_workspace(Workspace* ws) {
   for (int k = 0; k <= kMaxLevel; ++k) ws->m2l_kind[k] = ws->m2l_gshift[k] = 0;
   ws->p2p_sym = 0;
   free_sk_plan(&ws->sk);
+  for (M2LSparse& sp : ws->sparse) {
+    dfree(sp.list);
+    sp = M2LSparse();
+  }
+  ws->p2m_sparse = false;
   dfree(ws->fnear); dfree(ws->ffar); dfree(ws->tmp); dfree(ws->gsym); dfree(ws->wmax);
   ws->gsym = nullptr;
   ws->wmax = nullptr;

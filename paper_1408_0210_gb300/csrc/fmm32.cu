@@ -762,7 +762,8 @@ __device__ __forceinline__ float2 pt_r2(float2 ax, float2 ay, float2 az, float2 
 // broadcast 16-byte words (-x, -x | -y, -y) and (-z, -z | sigma, sigma).
 template <bool ACC>
 __global__ void __launch_bounds__(32 * PT_WARPS, 4)
-k_p2m32x(const int32_t* __restrict__ off, int64_t nleaf, const float* __restrict__ lx,
+k_p2m32x(const int32_t* __restrict__ leaves, int64_t nlist, const int32_t* __restrict__ off, int64_t nleaf,
+         const float* __restrict__ lx,
          const float* __restrict__ ly, const float* __restrict__ lz, const float* __restrict__ sig,
          const float* __restrict__ X, int d, int dp, float* __restrict__ W,
          __nv_bfloat16* __restrict__ planes, int grid_level, const double* __restrict__ sig64,
@@ -775,8 +776,9 @@ k_p2m32x(const int32_t* __restrict__ off, int64_t nleaf, const float* __restrict
   pt_stage_x(X, d, nq, s_xy, s_z);
   __syncthreads();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t b = (int64_t)blockIdx.x * PT_WARPS + w;
-  if (b >= nleaf) return;
+  const int64_t bi = (int64_t)blockIdx.x * PT_WARPS + w;
+  if (bi >= nlist) return;
+  const int64_t b = leaves ? leaves[bi] : bi;
   float2 ax[NI], ay[NI], az[NI], acc[NI];
 #pragma unroll
   for (int i = 0; i < NI; ++i) {
@@ -1314,6 +1316,9 @@ static eifmm_status launch_m2l_simt(const Tree* t, const Ops* ops, int k, int R,
   return EIFMM_OK;
 }
 
+// fewer than a quarter of the leaves hold points
+static bool sparse_set(const PointSet& p, int depth) { return 4 * (int64_t)p.n_nonempty < nboxes(depth); }
+
 eifmm_status alloc_mixed_workspace(Tree* t, const Ops* ops, int R) {
   Workspace& ws = t->ws;
   const int kap = t->depth;
@@ -1375,6 +1380,35 @@ eifmm_status alloc_mixed_workspace(Tree* t, const Ops* ops, int R) {
   }
   if (!ws.wmax) EIFMM_TRY(dalloc(&ws.wmax, (size_t)kMaxLevel + 1));
   EIFMM_TRY(alloc_wait_error(&ws));
+  // Trees most of whose boxes are empty, one right-hand side: the P2M writes the
+  // rows of non-empty leaves only, the M2L of tier 0 runs over the active target
+  // boxes and step 6 over the non-empty leaves.  Rows that no kernel writes are
+  // zero from here on.
+  if (R == 1) {
+    const size_t rowb = (size_t)ops->lv[kap].dp * 4, leaves = (size_t)nboxes(kap);
+    if (sparse_set(t->src, kap)) {
+      EIFMM_CUDA(cudaMemset(ws.W32[kap], 0, leaves * rowb));
+      EIFMM_CUDA(cudaMemset(ws.wa[kap], 0, 2 * leaves * rowb));
+      ws.p2m_sparse = true;
+    }
+    if (sparse_set(t->tgt, kap)) {
+      EIFMM_CUDA(cudaMemset(ws.lh32, 0, leaves * rowb));
+      for (int k = 5; ops->tier == 0 && k <= kap; ++k) {
+        if (!ws.wa_t256[k]) continue;
+        M2LSparse sp;
+        EIFMM_TRY(build_m2l_sparse(t->tgt.leaf_off, k, kap, &sp, nullptr));
+        int64_t n = 0;
+        for (int c : sp.cnt) n += c;
+        if (4 * n > nboxes(k)) {  // the dense tiles are cheaper to load
+          dfree(sp.list);
+          continue;
+        }
+        ws.sparse[k] = sp;
+        EIFMM_CUDA(cudaMemset(ws.g32[k], 0, (size_t)nboxes(k) * ops->lv[k].dp * 4));
+      }
+    }
+    EIFMM_CUDA(cudaStreamSynchronize(nullptr));  // the streams of the evaluation do not wait for the legacy one
+  }
   return EIFMM_OK;
 }
 
@@ -1689,6 +1723,7 @@ eifmm_status launch_m2l_level(Tree* t, const Ops* ops, int k, int R, int kind, i
     return launch_m2l_h16(a, ws.tmap[k][0], ws.tmap[k][1], ws.wmax, v.kscale, s);
   }
   const bool rule = kind == 0;
+  if (rule && ws.sparse[k].list && !t->opt[EIFMM_OPT_M2L_128ROW]) return launch_m2l_t256g(a, ws.sparse[k], s);
   if (rule) {
     // the transposed kernel where a parity class fills at least one of its
     // 256-row tiles; the 128-row kernel at the coarse levels
@@ -1713,6 +1748,18 @@ eifmm_status launch_m2l_level(Tree* t, const Ops* ops, int k, int R, int kind, i
   if (kind == 1) return launch_m2l_t256(a, ws.tmap2[k][0], ws.tmap2[k][1], tf32, s);
   if (kind == 2) return launch_m2l_tma(a, ws.tmap[k][0], ws.tmap[k][1], tf32, s);
   return launch_m2l_tc(a, tf32, s);
+}
+
+// Step 5 of level k for the SIMT transfer kernel
+static XferGemm l2l_gemm(const Ops& ops, int k, int R, const Workspace& ws) {
+  const LevelOps &v = ops.lv[k], &pv = ops.lv[k - 1];
+  XferGemm x;
+  x.mode = 1;
+  x.dk = v.d; x.ldk = v.dp; x.dc = pv.d; x.ldc = pv.dp; x.R = R;
+  x.ncol = nboxes(k - 1) * R;
+  x.A = v.l2l32; x.B = ws.l32[k - 1]; x.G = ws.g32[k]; x.C = ws.l32[k];
+  x.P8 = nullptr;
+  return x;
 }
 
 eifmm_status eval_mixed(Tree* t, const Ops* ops, const double* sigma, int64_t ld_sigma, int R,
@@ -1787,14 +1834,18 @@ eifmm_status eval_mixed(Tree* t, const Ops* ops, const double* sigma, int64_t ld
   k_p2m32<K, RC_, A><<<nb, TPB, 0, s>>>(kern, S.leaf_off, S.lx, S.ly, S.lz, ws.sig32, S.n, R, vl.X32, \
                                         vl.d, vl.dp, ws.W32[kap])
     if (p2m_x) {
-      const unsigned g = (unsigned)((nboxes(kap) + PT_WARPS - 1) / PT_WARPS);
+      const int32_t* list = ws.p2m_sparse ? S.nonempty : nullptr;
+      const int64_t nl = list ? S.n_nonempty : nboxes(kap);
+      const unsigned g = (unsigned)((nl + PT_WARPS - 1) / PT_WARPS);
       __nv_bfloat16* lp = leaf_planes_in_p2m ? (__nv_bfloat16*)ws.wa[kap] : nullptr;
       const int gl = ws.wa_grid[kap] ? kap : -1;
-      if (acc)
-        k_p2m32x<true><<<g, 32 * PT_WARPS, 0, s>>>(S.leaf_off, nboxes(kap), S.lx, S.ly, S.lz, ws.sig32, vl.X32,
+      if (g == 0) {
+        // no sources: every row is zero
+      } else if (acc)
+        k_p2m32x<true><<<g, 32 * PT_WARPS, 0, s>>>(list, nl, S.leaf_off, nboxes(kap), S.lx, S.ly, S.lz, ws.sig32, vl.X32,
                                                    vl.d, vl.dp, ws.W32[kap], lp, gl, sigma, S.perm);
       else
-        k_p2m32x<false><<<g, 32 * PT_WARPS, 0, s>>>(S.leaf_off, nboxes(kap), S.lx, S.ly, S.lz, ws.sig32, vl.X32,
+        k_p2m32x<false><<<g, 32 * PT_WARPS, 0, s>>>(list, nl, S.leaf_off, nboxes(kap), S.lx, S.ly, S.lz, ws.sig32, vl.X32,
                                                     vl.d, vl.dp, ws.W32[kap], lp, gl, sigma, S.perm);
     } else {
       EIFMM_POINT_DISPATCH(EIFMM_P2M);
@@ -1891,12 +1942,7 @@ eifmm_status eval_mixed(Tree* t, const Ops* ops, const double* sigma, int64_t ld
   for (int k = 3; k <= kap; ++k) {
     const LevelOps& v = ops->lv[k];
     const LevelOps& pv = ops->lv[k - 1];
-    XferGemm x;
-    x.mode = 1;
-    x.dk = v.d; x.ldk = v.dp; x.dc = pv.d; x.ldc = pv.dp; x.R = R;
-    x.ncol = nboxes(k - 1) * R;
-    x.A = v.l2l32; x.B = ws.l32[k - 1]; x.G = ws.g32[k]; x.C = ws.l32[k];
-    x.P8 = nullptr;
+    XferGemm x = l2l_gemm(*ops, k, R, ws);
     if (!xfer_blas(false, v, pv, nboxes(k - 1), R, ws.l32[k - 1], ws.g32[k], ws.l32[k], ws.blas_ws, s))
       EIFMM_TRY(launch_xfer_gemm(x, s));
   }
@@ -1907,6 +1953,10 @@ eifmm_status eval_mixed(Tree* t, const Ops* ops, const double* sigma, int64_t ld
     b.nlev = 1;
     b.lv[0] = delta_level(vl.d, delta_ops32(vl), true, ws.l32[kap], vl.dp, ws.lh32, vl.dp, nullptr,
                           nboxes(kap) * R);
+    if (R == 1 && sparse_set(T, kap)) {
+      b.lv[0].list = T.nonempty;
+      b.lv[0].nvec = T.n_nonempty;
+    }
     EIFMM_TRY((launch_delta_batch<float, float, float, 0>(b, true, s)));
   }
   record(ws, 6, s);
@@ -1958,8 +2008,36 @@ eifmm_status eval_mixed(Tree* t, const Ops* ops, const double* sigma, int64_t ld
   return EIFMM_OK;
 }
 
+// Steps 4 to 6 of the last evaluation again over all boxes, up to `level`, where
+// the evaluation left out boxes without targets (the values of the others stay
+// what they were, to the bit).
+static eifmm_status complete_sparse(Tree* t, const Ops* o, int level, bool lhat) {
+  Workspace& ws = t->ws;
+  bool any = false;
+  for (int k = 5; k <= level; ++k)
+    if (ws.sparse[k].list) {
+      any = true;
+      EIFMM_TRY(launch_m2l_level(t, o, k, 1, 1, 0, nullptr));
+    }
+  for (int k = 3; any && k <= level; ++k)
+    if (!xfer_blas(false, o->lv[k], o->lv[k - 1], nboxes(k - 1), 1, ws.l32[k - 1], ws.g32[k], ws.l32[k], ws.blas_ws,
+                   nullptr)) {
+      XferGemm x = l2l_gemm(*o, k, 1, ws);
+      EIFMM_TRY(launch_xfer_gemm(x, nullptr));
+    }
+  if (lhat && ws.nrhs == 1 && sparse_set(t->tgt, t->depth)) {
+    const LevelOps& v = o->lv[t->depth];
+    DeltaBatch b;
+    b.nlev = 1;
+    b.lv[0] = delta_level(v.d, delta_ops32(v), true, ws.l32[t->depth], v.dp, ws.lh32, v.dp, nullptr, nboxes(t->depth));
+    EIFMM_TRY((launch_delta_batch<float, float, float, 0>(b, true, nullptr)));
+  }
+  return EIFMM_OK;
+}
+
 eifmm_status export_mixed(const Tree& t, const Ops& o, int what, int level, double* out, int64_t n) {
   const Workspace& ws = t.ws;
+  if (what >= 2) EIFMM_TRY(complete_sparse(const_cast<Tree*>(&t), &o, level, what == 4));
   const LevelOps& v = o.lv[level];
   const int64_t nvec = nboxes(level) * ws.nrhs;
   const int64_t cnt = nvec * v.d;

@@ -153,6 +153,12 @@ struct SkPlanDev {
   int ntiles = 0, tpc = 0, nctas = 0, nfix = 0;
 };
 void free_sk_plan(SkPlanDev* p);
+// Active target boxes of one level for the sparse tensor-core M2L: class c has
+// cnt[c] of them at list + c 8^level / 8, in tiles tile0[c] .. tile0[c + 1].
+struct M2LSparse {
+  int* list = nullptr;
+  int cnt[8] = {}, tile0[9] = {};
+};
 eifmm_status wait_selftest(long long limit, int* code);  // m2l_tc.cu
 
 struct Workspace {
@@ -197,6 +203,8 @@ struct Workspace {
   unsigned long long* crt_max = nullptr;  // [kMaxLevel + 1][R] bits of the largest |W|
   int nsm = 0;                  // SMs of the workspace's device
   uint32_t* wmax = nullptr;     // [kMaxLevel + 1] bits of max |W| per level (FP16 planes)
+  M2LSparse sparse[kMaxLevel + 1];  // levels most of whose boxes hold no targets (tier 0, one right-hand side)
+  bool p2m_sparse = false;      // few leaves hold sources: rows of the others are zero from the start
   SkPlanDev sk;                 // stream-K plan of the leaf level (tier 0), when it pays
   int* err = nullptr;           // device error word of bounded waits
   int* err_host = nullptr;      // pinned copy, read at the next call

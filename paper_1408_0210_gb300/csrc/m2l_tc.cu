@@ -670,6 +670,236 @@ k_m2l_t256(const __grid_constant__ CUtensorMap tW0, const __grid_constant__ CUte
 }
 
 // ---------------------------------------------------------------------------
+// Sparse form of the transposed M2L (one right-hand side): a tile is 256 active
+// target boxes of one parity class from a list, wherever they lie, and two
+// warps gather their source rows of the W planes with cp.async (zeros outside
+// the cube) into the layout that the TMA box of k_m2l_t256 would have.  Every
+// row runs the same offsets in the same segments as there, so its sum is the
+// same to the bit.  On a surface the dense form multiplies mostly zeros:
+// 992,046 points on a sphere, depth 7, 4% of the leaves hold points: level 7 19.1 ->
+// 2.4 ms, level 6 2.5 -> 1.2 ms, the evaluation 28.8 -> 6.4 ms (with the sparse P2M
+// and step 6).  The gather of a stage is not overlapped with the next one's: a
+// tile takes about 1.6 times the dense one, so the list is used below a quarter.
+// ---------------------------------------------------------------------------
+constexpr int kGatherWarps = 2;
+constexpr int kT2gThreads = kT2Threads + 32 * kGatherWarps;
+
+__global__ void __launch_bounds__(kT2gThreads, 1) k_m2l_t256g(M2LTcArgs a, M2LSparse sp) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int wu = __shfl_sync(0xffffffffu, warp, 0);  // uniform
+  constexpr int nchunk = 2;                    // dp = 128
+  constexpr uint32_t k_bytes = 128u * 128u;    // one K^delta plane
+  constexpr uint32_t w_bytes = kT2Rows * 128u;  // one W plane
+  constexpr uint32_t stage = 2 * k_bytes + 2 * w_bytes;
+  uint64_t* bars = (uint64_t*)(smem + kT2Stages * stage);  // full[2] empty[2] sfull[2] sempty[2]
+  uint32_t* tslot = (uint32_t*)(bars + 8);
+  volatile int* abort = (volatile int*)(tslot + 1);
+  int* s_box = (int*)(bars + 9);                // [256] target boxes (Morton), -1 past the list
+  uint32_t* s_xyz = (uint32_t*)(s_box + kT2Rows);  // their class coordinates x | y << 10 | z << 20
+  const uint32_t sbase = smem_u32(smem);
+  auto full = [&](int st) { return smem_u32(&bars[st]); };
+  auto empty = [&](int st) { return smem_u32(&bars[2 + st]); };
+  auto sfull = [&](int b) { return smem_u32(&bars[4 + b]); };
+  auto sempty = [&](int b) { return smem_u32(&bars[6 + b]); };
+
+  const int h = a.h;
+  int oct = 0;
+  while (oct < 7 && (int)blockIdx.x >= sp.tile0[oct + 1]) ++oct;
+  const int n0 = ((int)blockIdx.x - sp.tile0[oct]) * kT2Rows;
+  const int cx = oct & 1, cy = (oct >> 1) & 1, cz = (oct >> 2) & 1;
+  const int* lst = a.slot_lists + oct * kListLen;
+  if (tid < kT2Rows) {
+    const int I = n0 + tid < sp.cnt[oct] ? sp.list[(int64_t)oct * (a.nbox / 8) + n0 + tid] : -1;
+    int c[3] = {0, 0, 0};
+    if (I >= 0) morton_decode(I, a.level, c);
+    s_box[tid] = I;
+    s_xyz[tid] = (uint32_t)(c[0] >> 1) | (uint32_t)(c[1] >> 1) << 10 | (uint32_t)(c[2] >> 1) << 20;
+  }
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(full(i), 1 + 32 * kGatherWarps);
+      mbar_init(empty(i), 1);
+      mbar_init(sfull(i), 1);
+      mbar_init(sempty(i), 8);  // one arrival per epilogue warp
+    }
+    *abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 8) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                 "r"(512u));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tslot;
+  constexpr int nseg = (kListLen + kSegOffsets - 1) / kSegOffsets;
+
+  if (tid == 256) {
+    // ------------------------------------------- operator images (bulk) --
+    int st = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    int it = 0;
+    for (int s = 0; s < kListLen && ok; ++s)
+      for (int c = 0; c < nchunk; ++c, ++it) {
+        if (it >= kT2Stages && !mbar_wait_ab(empty(st), ph ^ 1u, a.err, 1, abort)) {
+          ok = false;
+          break;
+        }
+        mbar_expect_tx(full(st), 2 * k_bytes);
+        bulk_g2s(sbase + st * stage, (const char*)a.kd_img + (((size_t)lst[s] * nchunk + c) * 2) * k_bytes, 2 * k_bytes,
+                 full(st));
+        if (++st == kT2Stages) st = 0, ph ^= 1u;
+      }
+    drain_fills(it, kT2Stages, bars, a.err);
+  } else if (wu >= 10) {
+    // ------------------------------------------------ gather of W rows --
+    // eight lanes copy the 128 bytes of a row, a warp four rows at a time
+    const int gw = wu - 10, sub = lane >> 3, pc = lane & 7;
+    const char* w0 = (const char*)a.wa + pc * 16;
+    const int64_t plane = a.rows * 256;  // bytes of one plane
+    int st = 0;
+    uint32_t ph = 0;
+    int it = 0;
+    bool ok = true;
+    for (int s = 0; s < kListLen && ok; ++s) {
+      const int slot = lst[s];
+      const int dx = slot % 7 - 3, dy = (slot / 7) % 7 - 3, dz = slot / 49 - 3;
+      const int sc = ((cx + dx) & 1) | (((cy + dy) & 1) << 1) | (((cz + dz) & 1) << 2);
+      const int sx = (cx + dx) >> 1, sy = (cy + dy) >> 1, sz = (cz + dz) >> 1;
+      for (int c = 0; c < nchunk; ++c, ++it) {
+        if (it >= kT2Stages) ok = ok && mbar_wait_ab(empty(st), ph ^ 1u, a.err, 6, abort);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        const uint32_t sW = sbase + st * stage + 2 * k_bytes;
+#pragma unroll 4
+        for (int i = 0; i < kT2Rows / (4 * kGatherWarps); ++i) {
+          const int row = gw * (kT2Rows / kGatherWarps) + 4 * i + sub;
+          const uint32_t p = s_xyz[row];
+          const int x = (int)(p & 1023u) + sx, y = (int)((p >> 10) & 1023u) + sy, z = (int)(p >> 20) + sz;
+          const bool in = s_box[row] >= 0 && x >= 0 && y >= 0 && z >= 0 && x < h && y < h && z < h;
+          const int64_t r = in ? (((int64_t)sc * h + z) * h + y) * h + x : 0;
+          const uint32_t dst = sW + (uint32_t)(row >> 3) * 1024u + (uint32_t)(row & 7) * 128u +
+                               (uint32_t)((pc ^ (row & 7)) << 4);
+          const char* src = w0 + r * 256 + c * 128;
+          const uint32_t nb = in ? 16u : 0u;
+          cp16(dst, src, nb);
+          cp16(dst + w_bytes, src + plane, nb);
+        }
+        cp_commit();
+        cp_wait0();
+        fence_async_smem();
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(full(st)) : "memory");
+        if (++st == kT2Stages) st = 0, ph ^= 1u;
+      }
+    }
+  } else if (wu == 9) {
+    // ----------------------------------------------------- MMA issuer --
+    const uint32_t el = elect_one();
+    const uint32_t id = idesc(1u, (uint32_t)kT2Rows);
+    const uint64_t dK0 = sdesc(sbase), dK1 = sdesc(sbase + stage);
+    const uint64_t dW0 = dK0 + (2 * k_bytes >> 4), dW1 = dK1 + (2 * k_bytes >> 4);
+    int st = 0, done = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int seg = 0; seg < nseg && ok; ++seg) {
+      const int b = seg & 1;
+      if (seg >= 2 && !mbar_wait_ab(sempty(b), ((seg >> 1) - 1) & 1, a.err, 4, abort)) break;
+      tc_fence_after();
+      const uint32_t dacc = tmem + (uint32_t)(b * kT2Rows);
+      const int nit = min(kSegOffsets, kListLen - done) * nchunk;
+      for (int i = 0; i < nit; ++i) {
+        if (!mbar_wait_ab(full(st), ph, a.err, 2, abort)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        issue_chunk(dacc, st == 0 ? dK0 : dK1, st == 0 ? dW0 : dW1, k_bytes >> 4, w_bytes >> 4, id, id, false,
+                    i == 0, el);
+        mma_commit_el(empty(st), el);
+        if (++st == kT2Stages) st = 0, ph ^= 1u;
+      }
+      done += kSegOffsets;
+      if (ok) mma_commit_el(sfull(b), el);
+    }
+  } else if (warp < 8) {
+    // ------------------------------------------------------ epilogue --
+    const int q = warp & 3, half = warp >> 2;
+    float acc[128];
+#pragma unroll
+    for (int j = 0; j < 128; ++j) acc[j] = 0.f;
+    for (int seg = 0; seg < nseg; ++seg) {
+      const int b = seg & 1;
+      bool have = mbar_wait_ab(sfull(b), (seg >> 1) & 1, a.err, 3, abort);
+      have = __all_sync(0xffffffffu, have);
+      if (!have) break;
+      tc_fence_after();
+      const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * kT2Rows + 128 * half);
+#pragma unroll
+      for (int j0 = 0; j0 < 128; j0 += 32) {
+        float v[32];
+        tmem_ld32(taddr + j0, v);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) acc[j0 + i] += v[i];
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sempty(b)) : "memory");
+    }
+    float* outg = a.g + 32 * q + lane;  // m'
+#pragma unroll
+    for (int j = 0; j < 128; ++j) {
+      const int I = s_box[128 * half + j];
+      if (I >= 0) outg[(int64_t)I * 128] = acc[j];
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 8)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
+}
+
+// Active target boxes of a level, by parity class: box I is active when leaves
+// below it hold targets (leaf_off at leaf level, I's leaves are contiguous).  A
+// block takes 2,048 consecutive boxes of one class; within it the Morton order
+// is kept, so that neighbours stay together in a tile.
+__global__ void __launch_bounds__(256) k_active_boxes(const int32_t* __restrict__ leaf_off, int64_t nbox, int shift,
+                                                      int* __restrict__ list, int* __restrict__ cnt) {
+  const int cls = blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t p0 = (int64_t)blockIdx.x * 2048 + threadIdx.x * 8, np = nbox / 8;
+  uint32_t m = 0;
+  for (int i = 0; i < 8; ++i) {
+    const int64_t I = 8 * (p0 + i) + cls;
+    if (p0 + i < np && leaf_off[(I + 1) << shift] > leaf_off[I << shift]) m |= 1u << i;
+  }
+  int n = __popc(m), x = n;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  __shared__ int s_w[9];
+  if (lane == 31) s_w[w] = x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int t = 0;
+    for (int i = 0; i < 8; ++i) {
+      const int v = s_w[i];
+      s_w[i] = t;
+      t += v;
+    }
+    s_w[8] = atomicAdd(cnt + cls, t);
+  }
+  __syncthreads();
+  int pos = s_w[8] + s_w[w] + x - n;
+  for (int i = 0; i < 8; ++i)
+    if ((m >> i) & 1) list[(int64_t)cls * np + pos++] = (int)(8 * (p0 + i) + cls);
+}
+
+// ---------------------------------------------------------------------------
 // Stream-K form of the transposed M2L for one level: exactly one CTA per SM.
 // The work is the sequence of (tile, active offset) units over all tiles
 // (tile t: parity class t / tpc, tile t % tpc of that class; tu[t] = units
@@ -1415,6 +1645,45 @@ eifmm_status launch_m2l_t256(const M2LTcArgs& a0, const void* map0, const void* 
         (const float4*)a.part, a.groups, n4, a.part_stride / 4, (float4*)a.g);
     EIFMM_CHECK_LAUNCH();
   }
+  return EIFMM_OK;
+}
+
+eifmm_status launch_m2l_t256g(const M2LTcArgs& a0, const M2LSparse& sp, cudaStream_t s) {
+  M2LTcArgs a = a0;
+  a.h = 1 << (a.level - 1);
+  static bool attr[kMaxDevices] = {};
+  const int dev = current_device();
+  if (dev >= kMaxDevices || !attr[dev]) {
+    EIFMM_CUDA(cudaFuncSetAttribute(k_m2l_t256g, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    if (dev < kMaxDevices) attr[dev] = true;
+  }
+  if (sp.tile0[8] == 0) return EIFMM_OK;
+  k_m2l_t256g<<<(unsigned)sp.tile0[8], kT2gThreads, m2l_t256_smem_bytes(), s>>>(a, sp);
+  EIFMM_CHECK_LAUNCH();
+  return EIFMM_OK;
+}
+
+eifmm_status build_m2l_sparse(const int32_t* leaf_off, int level, int depth, M2LSparse* sp, cudaStream_t s) {
+  const int64_t nbox = (int64_t)1 << (3 * level);
+  int* buf = nullptr;  // the list, then the counts
+  EIFMM_TRY(dalloc(&buf, (size_t)nbox + 8));
+  int* cnt = buf + nbox;
+  eifmm_status rc = EIFMM_OK;
+  if (cudaMemsetAsync(cnt, 0, 8 * sizeof(int), s) != cudaSuccess) rc = EIFMM_ECUDA;
+  k_active_boxes<<<dim3((unsigned)((nbox / 8 + 2047) / 2048), 8), 256, 0, s>>>(leaf_off, nbox, 3 * (depth - level), buf,
+                                                                              cnt);
+  count_launch();
+  if (cudaMemcpyAsync(sp->cnt, cnt, 8 * sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    rc = EIFMM_ECUDA;
+  if (rc != EIFMM_OK) {
+    dfree(buf);
+    set_error("the list of active boxes could not be built");
+    return rc;
+  }
+  sp->list = buf;
+  sp->tile0[0] = 0;
+  for (int c = 0; c < 8; ++c) sp->tile0[c + 1] = sp->tile0[c] + (sp->cnt[c] + kT2Rows - 1) / kT2Rows;
   return EIFMM_OK;
 }
 

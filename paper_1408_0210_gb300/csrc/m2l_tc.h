@@ -76,4 +76,11 @@ __host__ __device__ inline float f16_plane_scale(float maxabs) {
 eifmm_status launch_m2l_t256(const M2LTcArgs& a, const void* map0, const void* map1, bool tf32,
                              cudaStream_t s);
 
+// Sparse form (one right-hand side, dp = 128, no offset groups): the active
+// target boxes of a level as M2LSparse lists them.
+eifmm_status launch_m2l_t256g(const M2LTcArgs& a, const M2LSparse& sp, cudaStream_t s);
+// Lists the boxes of `level` whose leaves (of level `depth`) hold targets;
+// synchronises s.  sp->list is freed by the caller (dfree).
+eifmm_status build_m2l_sparse(const int32_t* leaf_off, int level, int depth, M2LSparse* sp, cudaStream_t s);
+
 }  // namespace eifmm

@@ -153,6 +153,7 @@ struct DeltaLevel {
   const void* in = nullptr;
   void* out = nullptr;
   void* planes = nullptr;
+  const int32_t* list = nullptr;  // rows of `in` and `out` (all of 0 .. nvec - 1 when null)
   int64_t nvec = 0;
   int d = 0, nb = 0, ldi = 0, ldo = 0, grid_level = -1, R = 1;
   int block0 = 0;
@@ -197,7 +198,8 @@ k_delta(const __grid_constant__ DeltaBatch b) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int64_t v = v0 + vv0 + u;
-          x[u] = (v < nvec && j < d) ? (T)__ldg(in + v * L.ldi + j) : (T)0;
+          const int64_t row = L.list && v < nvec ? L.list[v] : v;
+          x[u] = (v < nvec && j < d) ? (T)__ldg(in + row * L.ldi + j) : (T)0;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) sz[j * kDeltaLd + vv0 + u] = x[u];
@@ -229,7 +231,8 @@ k_delta(const __grid_constant__ DeltaBatch b) {
     const int64_t v = v0 + vv;
     if (v >= nvec) break;
     if (PLANES == 0) {
-      for (int j = lane; j < ldo; j += 32) out[v * ldo + j] = j < d ? (To)sz[j * kDeltaLd + vv] : (To)0;
+      const int64_t row = L.list ? L.list[v] : v;
+      for (int j = lane; j < ldo; j += 32) out[row * ldo + j] = j < d ? (To)sz[j * kDeltaLd + vv] : (To)0;
     } else {
       const int64_t prow = plane_row(v, L.grid_level, L.R);
       for (int j = lane; j < ldo; j += 32) {
