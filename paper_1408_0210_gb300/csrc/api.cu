@@ -262,7 +262,7 @@ eifmm_status ensure_workspace(Tree* t, const Ops* ops, int R, int prec) {
     ws.part64_cap = need;
     EIFMM_TRY(dalloc(&ws.crt_max, (size_t)(kMaxLevel + 1) * R));
     EIFMM_TRY(alloc_wait_error(&ws));
-    if (fx_usable((int)ops->kern, t->L)) {
+    if (fx_usable((int)ops->kern, t->L, t->depth)) {
       EIFMM_TRY(dalloc(&ws.fx_src, (size_t)3 * std::max<int64_t>(t->src.n, 1)));
       if (!t->same) EIFMM_TRY(dalloc(&ws.fx_tgt, (size_t)3 * std::max<int64_t>(t->tgt.n, 1)));
     }

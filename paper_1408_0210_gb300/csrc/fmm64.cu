@@ -457,7 +457,7 @@ eifmm_status launch_p2p64(const Tree* t, int kern, const double* sig, int R, dou
   const PointSet& T = t->tgt;
   const PointSet& S = t->src;
   if (T.n_nonempty == 0) return EIFMM_OK;
-  if (t->ws.fx_src) return launch_p2p_fx(t, R, fnear, s);
+  if (t->ws.fx_src) return launch_p2p_fx(t, kern, R, fnear, s);
   k_p2p64<<<T.n_nonempty, TPB, 0, s>>>(kern, T.nonempty, T.leaf_off, T.x, T.y, T.z, T.n, S.leaf_off, S.x, S.y, S.z,
                                        sig, S.n, R, t->depth, t->exclude_self, fnear);
   EIFMM_CHECK_LAUNCH();
@@ -571,7 +571,7 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   for (int k = 2; k <= kap; ++k)
     pairs = pairs || (pair_m2l && !t->opt[EIFMM_OPT_M2L_FP64] && !ops->compressed && ops->lv[k].crt.kappa > kCrtMaxKappa);
   if (ws.fx_src && !pairs) {
-    EIFMM_TRY(launch_p2m_fx(t, vl, R, ws.W[kap], s));
+    EIFMM_TRY(launch_p2m_fx(t, kern, vl, R, ws.W[kap], s));
   } else if (S.n_nonempty > 0) {
     k_p2m64<<<S.n_nonempty, TPB, 0, s>>>(kern, S.nonempty, S.leaf_off, S.x, S.y, S.z, ws.sig, S.n, R, kap, t->lo[0],
                                          t->lo[1], t->lo[2], lk, vl.X, vl.d, ws.W[kap]);
@@ -653,7 +653,7 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   EIFMM_CUDA(cudaStreamWaitEvent(s, ws.ev_join, 0));
   record(ws, 7, s);
   if (ws.fx_src) {
-    EIFMM_TRY(launch_l2p_fx(t, vl, R, f, ld_f, s));
+    EIFMM_TRY(launch_l2p_fx(t, kern, vl, R, f, ld_f, s));
   } else if (T.n_nonempty > 0) {
     const size_t sm = (size_t)(3 * vl.d + RC * vl.d) * sizeof(double);
     k_l2p64<<<T.n_nonempty, TPB, sm, s>>>(kern, T.nonempty, T.leaf_off, T.perm, T.x, T.y, T.z, T.n, R, kap, t->lo[0],

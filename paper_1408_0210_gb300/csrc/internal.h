@@ -276,15 +276,15 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma,
                        int64_t ld_sigma, int R, double* f, int64_t ld_f,
                        cudaStream_t s, bool near32 = false,
                        bool pair_m2l = false);
-// Point kernels of 1/r in FP64 on integer coordinates (point64.cu)
-bool fx_usable(int kern, double L);
+// Point kernels of 1/r and config-3 in FP64 on integer coordinates (point64.cu)
+bool fx_usable(int kern, double L, int depth);
 int fx_point_exponent(double L, int depth);
 int fx_box_exponent(double L);
 eifmm_status launch_to_fx(const double* x, int64_t n, int K, long long* q, cudaStream_t s);
 eifmm_status launch_fx_points(const Tree* t, cudaStream_t s);
-eifmm_status launch_p2m_fx(const Tree* t, const LevelOps& v, int R, double* W, cudaStream_t s);
-eifmm_status launch_l2p_fx(const Tree* t, const LevelOps& v, int R, double* f, int64_t ld_f, cudaStream_t s);
-eifmm_status launch_p2p_fx(const Tree* t, int R, double* fnear, cudaStream_t s);
+eifmm_status launch_p2m_fx(const Tree* t, int kern, const LevelOps& v, int R, double* W, cudaStream_t s);
+eifmm_status launch_l2p_fx(const Tree* t, int kern, const LevelOps& v, int R, double* f, int64_t ld_f, cudaStream_t s);
+eifmm_status launch_p2p_fx(const Tree* t, int kern, int R, double* fnear, cudaStream_t s);
 eifmm_status launch_p2p32(const Tree* t, int kern, const float* sig32, int R,
                           double* fnear, cudaStream_t s, bool accurate, float* gsym = nullptr);
 // Element format of the tensor-core M2L operand planes.

@@ -205,7 +205,7 @@ eifmm_status assemble_ops(Ops* ops, cudaStream_t s) {
         kern, v.d, lk, v.Y, v.kdT);
     EIFMM_CHECK_LAUNCH();
     EIFMM_TRY(to_f32(v.X, &v.X32, (int64_t)3 * v.d, s));
-    if (fx_usable(kern, ops->L)) {
+    if (fx_usable(kern, ops->L, 0)) {
       EIFMM_TRY(dalloc(&v.Xq, (size_t)3 * v.d));
       EIFMM_TRY(launch_to_fx(v.X, 3 * v.d, fx_box_exponent(ops->L), v.Xq, s));
     }

@@ -1,7 +1,7 @@
 // point64.cu -- the point kernels of the FP64 far field and near field for
-// K = 1/r: P2M (step 1), L2P (step 7 with the sum and the un-permute) and the
-// direct sum over the 27 neighbouring leaves, with 1/r from integer coordinate
-// differences (inv_fx.cuh) and the sums in FP64.
+// K = 1/r and the config-3 kernel: P2M (step 1), L2P (step 7 with the sum and the un-permute) and the
+// direct sum over the 27 neighbouring leaves, with the kernel from integer
+// coordinate differences (inv_fx.cuh) and the sums in FP64.
 //
 // Their bound is the integer and FP32 issue: about 75 instructions per kernel
 // value, of which one FP64 FMA per right-hand side; on the FP64 pipe alone a
@@ -31,14 +31,24 @@ __device__ __forceinline__ long long local_fx(long long q, long long cq, int shi
   return (q - cq + (1ll << (shift - 1))) >> shift;
 }
 
-// 1/|z| in FP64 where inv_fx refuses: points closer than 2^54 units.
-__device__ __noinline__ double inv_slow(double z0, double z1, double z2) {
-  return rsqrt(z0 * z0 + z1 * z1 + z2 * z2);
+// The kernel value of an integer difference; false where the integers do not
+// reach (points closer than 2^54 units).
+template <int KERN>
+__device__ __forceinline__ bool fx_value(long long dx, long long dy, long long dz, int kb, const FxConfig3& c3,
+                                         double* kv) {
+  if (KERN == EIFMM_KERNEL_CONFIG3) return config3_fx(dx, dy, dz, kb, c3, kv);
+  return inv_fx(dx, dy, dz, kb, kv);
+}
+// There, in FP64.
+template <int KERN>
+__device__ __noinline__ double fx_slow(double z0, double z1, double z2) {
+  return kern_f64(KERN, z0, z1, z2);
 }
 
 struct FxLeaf {
   double lo[3], lk;  // corner of the cube, half width of a leaf
   int depth, K, K2;  // units 2^-K of the points, 2^-K2 of box-relative coordinates
+  FxConfig3 c3, c32;  // constants of the config-3 kernel in units of the points and of the boxes
 };
 __device__ __forceinline__ void leaf_centre(const FxLeaf& f, int b, double* c) {
   int ic[3];
@@ -49,7 +59,7 @@ __device__ __forceinline__ void leaf_centre(const FxLeaf& f, int b, double* c) {
 // Step 1: W_m^I = sum_j sigma_j / |x_m - (y_j - c_I)|.  One CTA per non-empty
 // leaf, one thread per coefficient (in passes), the leaf's points staged as
 // integers; RCT right-hand sides share a kernel value.
-template <int RCT>
+template <int KERN, int RCT>
 __global__ void __launch_bounds__(256)
 k_p2m_fx(FxLeaf lf, const int32_t* __restrict__ leaves, const int32_t* __restrict__ off,
          const double* __restrict__ px, const double* __restrict__ py, const double* __restrict__ pz,
@@ -94,8 +104,8 @@ k_p2m_fx(FxLeaf lf, const int32_t* __restrict__ leaves, const int32_t* __restric
           for (int t = 0; t < cnt; ++t) {
             const longlong2 xy = s_xy[t];
             double kv;
-            if (!inv_fx(x0 - xy.x, x1 - xy.y, x2 - s_z[t], kb, &kv))
-              kv = inv_slow(X[3 * m] - (px[j0 + t] - c[0]), X[3 * m + 1] - (py[j0 + t] - c[1]),
+            if (!fx_value<KERN>(x0 - xy.x, x1 - xy.y, x2 - s_z[t], kb, lf.c32, &kv))
+              kv = fx_slow<KERN>(X[3 * m] - (px[j0 + t] - c[0]), X[3 * m + 1] - (py[j0 + t] - c[1]),
                             X[3 * m + 2] - (pz[j0 + t] - c[2]));
 #pragma unroll
             for (int rr = 0; rr < RCT; ++rr) acc[rr] += s_s[t][rr] * kv;
@@ -112,7 +122,7 @@ k_p2m_fx(FxLeaf lf, const int32_t* __restrict__ leaves, const int32_t* __restric
 // Step 7 + sum + un-permute.  One CTA per non-empty leaf; a thread takes one
 // point of the pass and one slice of the l (32 points: 4 slices), the slices are
 // added in order.
-template <int RCT>
+template <int KERN, int RCT>
 __global__ void __launch_bounds__(FX_THREADS)
 k_l2p_fx(FxLeaf lf, const int32_t* __restrict__ leaves, const int32_t* __restrict__ off,
          const int32_t* __restrict__ perm, const double* __restrict__ px, const double* __restrict__ py,
@@ -161,8 +171,8 @@ k_l2p_fx(FxLeaf lf, const int32_t* __restrict__ leaves, const int32_t* __restric
         for (int l = l0; l < l1; ++l) {
           const longlong2 xy = s_xy[l];
           double kv;
-          if (!inv_fx(z0 - xy.x, z1 - xy.y, z2 - s_z[l], kb, &kv))
-            kv = inv_slow((px[p] - c[0]) - X[3 * l], (py[p] - c[1]) - X[3 * l + 1], (pz[p] - c[2]) - X[3 * l + 2]);
+          if (!fx_value<KERN>(z0 - xy.x, z1 - xy.y, z2 - s_z[l], kb, lf.c32, &kv))
+            kv = fx_slow<KERN>((px[p] - c[0]) - X[3 * l], (py[p] - c[1]) - X[3 * l + 1], (pz[p] - c[2]) - X[3 * l + 2]);
 #pragma unroll
           for (int rr = 0; rr < RCT; ++rr) acc[rr] += kv * s_l[l * RCT + rr];
         }
@@ -189,7 +199,7 @@ k_l2p_fx(FxLeaf lf, const int32_t* __restrict__ leaves, const int32_t* __restric
 // chunks of FX_SRC as integers; a thread takes one target of the pass and one
 // slice of the chunk, and a target's slices are added in order.
 constexpr int FX_SRC = 512;
-template <int RCT>
+template <int KERN, int RCT>
 __global__ void __launch_bounds__(FX_THREADS)
 k_p2p_fx(FxLeaf lf, const int32_t* __restrict__ leaves, const int32_t* __restrict__ toff,
          const double* __restrict__ tx, const double* __restrict__ ty, const double* __restrict__ tz,
@@ -272,10 +282,10 @@ k_p2p_fx(FxLeaf lf, const int32_t* __restrict__ leaves, const int32_t* __restric
           for (int i = i0; i < i1; ++i) {
             const longlong2 xy = s_xy[i];
             double kv;
-            if (!inv_fx(x0 - xy.x, x1 - xy.y, x2 - s_z[i], kb, &kv)) {
+            if (!fx_value<KERN>(x0 - xy.x, x1 - xy.y, x2 - s_z[i], kb, lf.c3, &kv)) {
               const int j = s_j[i];
               if (exclude_self && j == p) continue;
-              kv = inv_slow(tx[p] - sx[j], ty[p] - sy[j], tz[p] - sz[j]);
+              kv = fx_slow<KERN>(tx[p] - sx[j], ty[p] - sy[j], tz[p] - sz[j]);
             }
 #pragma unroll
             for (int rr = 0; rr < RCT; ++rr) acc[rr] += s_s[i * RCT + rr] * kv;
@@ -304,6 +314,16 @@ FxLeaf fx_leaf(const Tree* t) {
   f.depth = t->depth;
   f.K = fx_point_exponent(t->L, t->depth);
   f.K2 = fx_box_exponent(t->L);
+  const FxConfig3* c[2] = {&f.c3, &f.c32};
+  for (int i = 0; i < 2; ++i) {
+    // 1e-3 (53 bits) times 2^(2 K), 2 K <= 134
+    int e = 0;
+    const double m = std::ldexp(std::frexp(1e-3, &e), 53);
+    const int sh = e - 53 + 2 * (i == 0 ? f.K : f.K2);
+    const unsigned __int128 v = sh >= 0 && sh < 75 ? (unsigned __int128)m << sh : sh < 0 && sh > -53 ? (unsigned __int128)m >> -sh : 0;
+    const_cast<FxConfig3*>(c[i])->e_hi = (unsigned long long)(v >> 64);
+    const_cast<FxConfig3*>(c[i])->e_lo = (unsigned long long)v;
+  }
   return f;
 }
 
@@ -321,11 +341,16 @@ int fx_box_exponent(double L) {
   std::frexp(L, &e);
   return 61 - e;
 }
-// The exponent field of the results stays in range (any L but extreme ones).
-bool fx_usable(int kern, double L) {
+// 1/r: the exponent field of the results stays in range (any L but extreme
+// ones).  config-3, whose constants set a scale: r below 700 and 1e-3 in the 126
+// bits of a square (depth 0: the box-relative coordinates alone).
+bool fx_usable(int kern, double L, int depth) {
   int e = 0;
   std::frexp(L, &e);
-  return kern == EIFMM_KERNEL_INV_R && e > -800 && e < 800;
+  if (kern == EIFMM_KERNEL_INV_R) return e > -800 && e < 800;
+  if (kern == EIFMM_KERNEL_CONFIG3)
+    return e <= 8 && fx_box_exponent(L) <= 67 && (depth == 0 || fx_point_exponent(L, depth) <= 67);
+  return false;
 }
 
 eifmm_status launch_to_fx(const double* x, int64_t n, int K, long long* q, cudaStream_t s) {
@@ -350,53 +375,62 @@ eifmm_status launch_fx_points(const Tree* t, cudaStream_t s) {
   return EIFMM_OK;
 }
 
-eifmm_status launch_p2m_fx(const Tree* t, const LevelOps& v, int R, double* W, cudaStream_t s) {
+eifmm_status launch_p2m_fx(const Tree* t, int kern, const LevelOps& v, int R, double* W, cudaStream_t s) {
   const PointSet& S = t->src;
   if (S.n_nonempty == 0) return EIFMM_OK;
   const FxLeaf f = fx_leaf(t);
   const long long* q = t->ws.fx_src;
   // passes of equal size over the coefficients, at most 256 threads
   const int passes = (v.d + 255) / 256, threads = (((v.d + passes - 1) / passes) + 31) / 32 * 32;
-#define EIFMM_P2M_FX(RCT)                                                                                           \
-  k_p2m_fx<RCT><<<S.n_nonempty, threads, 0, s>>>(f, S.nonempty, S.leaf_off, S.x, S.y, S.z, q, q + S.n, q + 2 * S.n, \
+#define EIFMM_P2M_FX(K, RCT)                                                                                           \
+  k_p2m_fx<K, RCT><<<S.n_nonempty, threads, 0, s>>>(f, S.nonempty, S.leaf_off, S.x, S.y, S.z, q, q + S.n, q + 2 * S.n, \
                                                  t->ws.sig, S.n, R, v.X, v.Xq, v.d, W)
-  if (R == 1) EIFMM_P2M_FX(1);
-  else if (R <= 4) EIFMM_P2M_FX(4);
-  else EIFMM_P2M_FX(8);
+  if (kern == EIFMM_KERNEL_CONFIG3) {
+    if (R == 1) EIFMM_P2M_FX(EIFMM_KERNEL_CONFIG3, 1);
+    else EIFMM_P2M_FX(EIFMM_KERNEL_CONFIG3, 4);
+  } else if (R == 1) EIFMM_P2M_FX(EIFMM_KERNEL_INV_R, 1);
+  else if (R <= 4) EIFMM_P2M_FX(EIFMM_KERNEL_INV_R, 4);
+  else EIFMM_P2M_FX(EIFMM_KERNEL_INV_R, 8);
 #undef EIFMM_P2M_FX
   EIFMM_CHECK_LAUNCH();
   return EIFMM_OK;
 }
 
-eifmm_status launch_l2p_fx(const Tree* t, const LevelOps& v, int R, double* f, int64_t ld_f, cudaStream_t s) {
+eifmm_status launch_l2p_fx(const Tree* t, int kern, const LevelOps& v, int R, double* f, int64_t ld_f, cudaStream_t s) {
   const PointSet& T = t->tgt;
   if (T.n_nonempty == 0) return EIFMM_OK;
   const FxLeaf lf = fx_leaf(t);
   const long long* q = t->same ? t->ws.fx_src : t->ws.fx_tgt;
   // d = 512 with 4 columns: 28 KB (8 columns would pass 48 KB with the sums)
-#define EIFMM_L2P_FX(RCT)                                                                                              \
-  k_l2p_fx<RCT><<<T.n_nonempty, FX_THREADS, (size_t)v.d * (24 + 8 * RCT), s>>>(                                        \
+#define EIFMM_L2P_FX(K, RCT)                                                                                              \
+  k_l2p_fx<K, RCT><<<T.n_nonempty, FX_THREADS, (size_t)v.d * (24 + 8 * RCT), s>>>(                                        \
       lf, T.nonempty, T.leaf_off, T.perm, T.x, T.y, T.z, q, q + T.n, q + 2 * T.n, T.n, R, v.X, v.Xq, v.d, t->ws.lh, \
       t->ws.fnear, t->ws.ffar, f, ld_f)
-  if (R == 1) EIFMM_L2P_FX(1);
-  else EIFMM_L2P_FX(4);
+  if (kern == EIFMM_KERNEL_CONFIG3) {
+    if (R == 1) EIFMM_L2P_FX(EIFMM_KERNEL_CONFIG3, 1);
+    else EIFMM_L2P_FX(EIFMM_KERNEL_CONFIG3, 4);
+  } else if (R == 1) EIFMM_L2P_FX(EIFMM_KERNEL_INV_R, 1);
+  else EIFMM_L2P_FX(EIFMM_KERNEL_INV_R, 4);
 #undef EIFMM_L2P_FX
   EIFMM_CHECK_LAUNCH();
   return EIFMM_OK;
 }
 
-eifmm_status launch_p2p_fx(const Tree* t, int R, double* fnear, cudaStream_t s) {
+eifmm_status launch_p2p_fx(const Tree* t, int kern, int R, double* fnear, cudaStream_t s) {
   const PointSet &T = t->tgt, &S = t->src;
   if (T.n_nonempty == 0) return EIFMM_OK;
   const FxLeaf f = fx_leaf(t);
   const long long* sq = t->ws.fx_src;
   const long long* tq = t->same ? sq : t->ws.fx_tgt;
-#define EIFMM_P2P_FX(RCT)                                                                                           \
-  k_p2p_fx<RCT><<<dim3(T.n_nonempty, near_split(T.max_leaf)), FX_THREADS, 0, s>>>(f, T.nonempty, T.leaf_off, T.x, T.y, T.z, tq, tq + T.n,         \
+#define EIFMM_P2P_FX(K, RCT)                                                                                           \
+  k_p2p_fx<K, RCT><<<dim3(T.n_nonempty, near_split(T.max_leaf)), FX_THREADS, 0, s>>>(f, T.nonempty, T.leaf_off, T.x, T.y, T.z, tq, tq + T.n,         \
                                                     tq + 2 * T.n, T.n, S.leaf_off, S.x, S.y, S.z, sq, sq + S.n,     \
                                                     sq + 2 * S.n, t->ws.sig, S.n, R, t->exclude_self, fnear)
-  if (R == 1) EIFMM_P2P_FX(1);
-  else EIFMM_P2P_FX(4);
+  if (kern == EIFMM_KERNEL_CONFIG3) {
+    if (R == 1) EIFMM_P2P_FX(EIFMM_KERNEL_CONFIG3, 1);
+    else EIFMM_P2P_FX(EIFMM_KERNEL_CONFIG3, 4);
+  } else if (R == 1) EIFMM_P2P_FX(EIFMM_KERNEL_INV_R, 1);
+  else EIFMM_P2P_FX(EIFMM_KERNEL_INV_R, 4);
 #undef EIFMM_P2P_FX
   EIFMM_CHECK_LAUNCH();
   return EIFMM_OK;
