@@ -5,8 +5,8 @@
 //   Delta v   : Gamma z = v (lower, forward), B^t w = z (upper, backward)
 //   Delta^t v : B z = v (lower, forward),     Gamma^t w = z (upper, backward)
 //
-// Both solves of one application run in one kernel.  A warp owns
-// kDeltaVpw = 16 vectors, kDeltaLpv = 2 lanes per vector, kept transposed in
+// Both solves of one application run in one kernel.  A warp owns 16 vectors
+// with 2 lanes per vector (or 4 with 8, DeltaShape), kept transposed in
 // shared memory ([entry][vector], row stride 17 so that both the transposing
 // copy and the lane-wise access are free of bank conflicts).  Each solve
 // walks 32-row blocks (blocked left-looking substitution): lane half h
@@ -31,11 +31,18 @@
 namespace eifmm {
 
 constexpr int kDeltaTile = 32;
-constexpr int kDeltaLpv = 2;                    // lanes per vector
-constexpr int kDeltaVpw = 32 / kDeltaLpv;       // vectors per warp
-constexpr int kDeltaRl = kDeltaTile / kDeltaLpv;  // rows of a block per lane
-constexpr int kDeltaLd = kDeltaVpw + 1;         // shared row stride (floats or doubles)
 constexpr int kDeltaMaxWarps = 8;               // warps per CTA
+// Shape of a solve by the lanes per vector: vectors per warp, rows of a block
+// per lane, shared row stride (floats or doubles).  2 lanes where the vectors
+// fill the GPU; 8 below that, where the chain of d dependent steps is what a
+// solve takes and a step costs its 16 or 4 row updates (512 vectors, d = 161:
+// 76 -> 33 us).  The order of every row's updates is the same: so is the result.
+template <int LPV>
+struct DeltaShape {
+  static constexpr int kVpw = 32 / LPV, kRl = kDeltaTile / LPV, kLd = kVpw + 1;
+};
+constexpr int64_t kDeltaFew = 4864;   // two warps of 16 vectors on each of 152 SMs
+constexpr int64_t kDeltaSpread = 152;  // CTAs wanted
 
 // Tiles of one solve: tile (J, K), K <= J, at (J(J+1)/2 + K) * 1024, entry
 // [k][i] = L'[32J + i][32K + k]; the diagonal tiles are zero on and above
@@ -68,11 +75,10 @@ __device__ __forceinline__ int64_t plane_row(int64_t v, int grid_level, int R) {
 // acc[i] -= col[i] * z for the lane's rows of one tile column (16-byte
 // loads of a half-warp-uniform address: shared memory when SH, else global
 // through L1).
-template <bool SH>
-__device__ __forceinline__ void tile_col_update(float (&acc)[kDeltaRl], const float* __restrict__ col,
-                                                float z) {
+template <bool SH, int RL>
+__device__ __forceinline__ void tile_col_update(float (&acc)[RL], const float* __restrict__ col, float z) {
 #pragma unroll
-  for (int q = 0; q < kDeltaRl / 4; ++q) {
+  for (int q = 0; q < RL / 4; ++q) {
     const float4 m = SH ? reinterpret_cast<const float4*>(col)[q] : __ldg(reinterpret_cast<const float4*>(col) + q);
     acc[4 * q + 0] -= m.x * z;
     acc[4 * q + 1] -= m.y * z;
@@ -80,11 +86,10 @@ __device__ __forceinline__ void tile_col_update(float (&acc)[kDeltaRl], const fl
     acc[4 * q + 3] -= m.w * z;
   }
 }
-template <bool SH>
-__device__ __forceinline__ void tile_col_update(double (&acc)[kDeltaRl], const double* __restrict__ col,
-                                                double z) {
+template <bool SH, int RL>
+__device__ __forceinline__ void tile_col_update(double (&acc)[RL], const double* __restrict__ col, double z) {
 #pragma unroll
-  for (int q = 0; q < kDeltaRl / 2; ++q) {
+  for (int q = 0; q < RL / 2; ++q) {
     const double2 m =
         SH ? reinterpret_cast<const double2*>(col)[q] : __ldg(reinterpret_cast<const double2*>(col) + q);
     acc[2 * q + 0] -= m.x * z;
@@ -95,30 +100,30 @@ __device__ __forceinline__ void tile_col_update(double (&acc)[kDeltaRl], const d
 __device__ __forceinline__ float apply_pivot(float v, float rp) { return v * rp; }
 __device__ __forceinline__ double apply_pivot(double v, double p) { return v / p; }
 
-// One forward solve L' x = v over the warp's kDeltaVpw vectors held in sz
-// (physical entry e of vector c at sz[e * kDeltaLd + c]); lane = c + kDeltaVpw h
-// works on rows kDeltaRl h .. of every block.  REV maps logical entry a to
+// One forward solve L' x = v over the warp's vectors held in sz
+// (physical entry e of vector c at sz[e * LD + c]); lane = c + VPW h works on
+// rows RL h .. of every block.  REV maps logical entry a to
 // physical dpad-1-a.  The solution overwrites sz.
-template <typename T, bool DIAG, bool REV, bool SH>
+template <typename T, bool DIAG, bool REV, bool SH, int LPV>
 __device__ __forceinline__ void tiled_solve(T* __restrict__ sz, int nb, const T* __restrict__ tiles,
                                             const T* __restrict__ piv, int lane) {
-  constexpr int TL = kDeltaTile, RL = kDeltaRl;
-  const int c = lane % kDeltaVpw, h = lane / kDeltaVpw;
+  constexpr int TL = kDeltaTile, RL = DeltaShape<LPV>::kRl, VPW = DeltaShape<LPV>::kVpw, LD = DeltaShape<LPV>::kLd;
+  const int c = lane % VPW, h = lane / VPW;
   for (int J = 0; J < nb; ++J) {
     const int pj = REV ? nb - 1 - J : J;
     T acc[RL];
 #pragma unroll
     for (int i = 0; i < RL; ++i) {
       const int row = h * RL + i;
-      acc[i] = sz[(pj * TL + (REV ? TL - 1 - row : row)) * kDeltaLd + c];
+      acc[i] = sz[(pj * TL + (REV ? TL - 1 - row : row)) * LD + c];
     }
     const T* tJ = tiles + (int64_t)(J * (J + 1) / 2) * TL * TL;
     for (int K = 0; K < J; ++K) {
       const T* tk = tJ + (int64_t)K * TL * TL + h * RL;
-      const T* zK = sz + (REV ? (nb - 1 - K) * TL + TL - 1 : K * TL) * kDeltaLd + c;
+      const T* zK = sz + (REV ? (nb - 1 - K) * TL + TL - 1 : K * TL) * LD + c;
 #pragma unroll
       for (int k = 0; k < TL; ++k) {
-        const T zk = zK[(REV ? -k : k) * kDeltaLd];
+        const T zk = zK[(REV ? -k : k) * LD];
         tile_col_update<SH>(acc, tk + k * TL, zk);
       }
     }
@@ -128,7 +133,7 @@ __device__ __forceinline__ void tiled_solve(T* __restrict__ sz, int nb, const T*
       const int owner = k / RL;  // the half that holds entry k
       T mine = acc[k % RL];
       if (DIAG && h == owner) mine = apply_pivot(mine, __ldg(piv + J * TL + k));
-      const T zk = kDeltaLpv == 1 ? mine : __shfl_sync(0xffffffffu, mine, c + owner * kDeltaVpw);
+      const T zk = __shfl_sync(0xffffffffu, mine, c + owner * VPW);
       if (h == owner) acc[k % RL] = zk;
       // the tile holds zeros on and above its diagonal, so the update of
       // every row leaves the rows up to k as they are
@@ -137,7 +142,7 @@ __device__ __forceinline__ void tiled_solve(T* __restrict__ sz, int nb, const T*
 #pragma unroll
     for (int i = 0; i < RL; ++i) {
       const int row = h * RL + i;
-      sz[(pj * TL + (REV ? TL - 1 - row : row)) * kDeltaLd + c] = acc[i];
+      sz[(pj * TL + (REV ? TL - 1 - row : row)) * LD + c] = acc[i];
     }
   }
 }
@@ -172,9 +177,11 @@ __device__ __forceinline__ void copy_tiles(void* dst, const void* src, int64_t b
 // out = M2^-1 M1^-1 in, both solves in one pass over the vectors.  SH: the
 // tiles of the running solve are staged in shared memory (one copy per CTA,
 // read by all its warps); otherwise they are read through L1.
-template <typename T, bool DIAG1, bool DIAG2, typename Ti, typename To, int PLANES, bool SH>
+// The first vwarps warps of a CTA own vectors; the others only help to stage.
+template <typename T, bool DIAG1, bool DIAG2, typename Ti, typename To, int PLANES, bool SH, int LPV>
 __global__ void __launch_bounds__(32 * kDeltaMaxWarps)
-k_delta(const __grid_constant__ DeltaBatch b) {
+k_delta(const __grid_constant__ DeltaBatch b, int vwarps) {
+  constexpr int kVpw = DeltaShape<LPV>::kVpw, kLd = DeltaShape<LPV>::kLd;
   extern __shared__ __align__(16) unsigned char s_raw[];
   int li = 0;
   while (li + 1 < b.nlev && (int)blockIdx.x >= b.lv[li + 1].block0) ++li;
@@ -184,15 +191,15 @@ k_delta(const __grid_constant__ DeltaBatch b) {
   const int dpad = nb * kDeltaTile;
   const int64_t tile_elems = (int64_t)nb * (nb + 1) / 2 * kDeltaTile * kDeltaTile;
   T* s_tiles = reinterpret_cast<T*>(s_raw);
-  T* sz = s_tiles + (SH ? tile_elems : 0) + (int64_t)w * dpad * kDeltaLd;
-  const int64_t v0 = ((int64_t)(blockIdx.x - L.block0) * (blockDim.x >> 5) + w) * kDeltaVpw;
+  T* sz = s_tiles + (SH ? tile_elems : 0) + (int64_t)w * dpad * kLd;
+  const int64_t v0 = ((int64_t)(blockIdx.x - L.block0) * vwarps + w) * kVpw;
   const int64_t nvec = L.nvec;
-  const bool live = v0 < nvec;
+  const bool live = w < vwarps && v0 < nvec;
   const Ti* __restrict__ in = (const Ti*)L.in;
   if (live) {
     // transposing load: row v0+vv -> column vv (four rows' loads in flight
     // before their shared stores)
-    for (int vv0 = 0; vv0 < kDeltaVpw; vv0 += 4) {
+    for (int vv0 = 0; vv0 < kVpw; vv0 += 4) {
       for (int j = lane; j < dpad; j += 32) {
         T x[4];
 #pragma unroll
@@ -202,7 +209,7 @@ k_delta(const __grid_constant__ DeltaBatch b) {
           x[u] = (v < nvec && j < d) ? (T)__ldg(in + row * L.ldi + j) : (T)0;
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) sz[j * kDeltaLd + vv0 + u] = x[u];
+        for (int u = 0; u < 4; ++u) sz[j * kLd + vv0 + u] = x[u];
       }
     }
   }
@@ -215,7 +222,7 @@ k_delta(const __grid_constant__ DeltaBatch b) {
   } else {
     __syncwarp();
   }
-  if (live) tiled_solve<T, DIAG1, false, SH>(sz, nb, t1, (const T*)L.p1, lane);
+  if (live) tiled_solve<T, DIAG1, false, SH, LPV>(sz, nb, t1, (const T*)L.p1, lane);
   if (SH) {
     __syncthreads();
     copy_tiles(s_tiles, t2, tile_elems * (int64_t)sizeof(T));
@@ -223,20 +230,20 @@ k_delta(const __grid_constant__ DeltaBatch b) {
     t2 = s_tiles;
   }
   if (!live) return;
-  tiled_solve<T, DIAG2, true, SH>(sz, nb, t2, (const T*)L.p2, lane);
+  tiled_solve<T, DIAG2, true, SH, LPV>(sz, nb, t2, (const T*)L.p2, lane);
   __syncwarp();
   To* out = (To*)L.out;
   const int ldo = L.ldo;
-  for (int vv = 0; vv < kDeltaVpw; ++vv) {
+  for (int vv = 0; vv < kVpw; ++vv) {
     const int64_t v = v0 + vv;
     if (v >= nvec) break;
     if (PLANES == 0) {
       const int64_t row = L.list ? L.list[v] : v;
-      for (int j = lane; j < ldo; j += 32) out[row * ldo + j] = j < d ? (To)sz[j * kDeltaLd + vv] : (To)0;
+      for (int j = lane; j < ldo; j += 32) out[row * ldo + j] = j < d ? (To)sz[j * kLd + vv] : (To)0;
     } else {
       const int64_t prow = plane_row(v, L.grid_level, L.R);
       for (int j = lane; j < ldo; j += 32) {
-        const T x = j < d ? sz[j * kDeltaLd + vv] : (T)0;
+        const T x = j < d ? sz[j * kLd + vv] : (T)0;
         if (PLANES == 1) {
           __nv_bfloat16* pl = (__nv_bfloat16*)L.planes;
           const __nv_bfloat16 hi = __float2bfloat16_rn((float)x);
@@ -286,7 +293,7 @@ DeltaLevel delta_level(int d, const DeltaOps<T>& op, bool transpose, const void*
 }
 
 template <auto KFN>
-eifmm_status delta_launch(const DeltaBatch& b, int blocks, int warps, size_t sm, cudaStream_t s) {
+eifmm_status delta_launch(const DeltaBatch& b, int blocks, int warps, int vwarps, size_t sm, cudaStream_t s) {
   constexpr int kDev = 64;
   static bool attr[kDev] = {};  // the attribute is per device
   int dev = 0;
@@ -295,9 +302,41 @@ eifmm_status delta_launch(const DeltaBatch& b, int blocks, int warps, size_t sm,
     EIFMM_CUDA(cudaFuncSetAttribute(KFN, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     if (dev >= 0 && dev < kDev) attr[dev] = true;
   }
-  KFN<<<(unsigned)blocks, 32 * warps, sm, s>>>(b);
+  KFN<<<(unsigned)blocks, 32 * warps, sm, s>>>(b, vwarps);
   EIFMM_CHECK_LAUNCH();
   return EIFMM_OK;
+}
+
+template <typename T, typename Ti, typename To, int PLANES, int LPV>
+eifmm_status launch_delta_shape(DeltaBatch& b, bool transpose, int nbmax, int64_t vectors, cudaStream_t s) {
+  constexpr int kVpw = DeltaShape<LPV>::kVpw;
+  const size_t per_warp = (size_t)nbmax * kDeltaTile * DeltaShape<LPV>::kLd * sizeof(T);
+  const size_t tiles = (size_t)nbmax * (nbmax + 1) / 2 * kDeltaTile * kDeltaTile * sizeof(T);
+  const size_t cap = 227 * 1024;
+  const bool sh = tiles + per_warp <= cap;
+  int vwarps = kDeltaMaxWarps;
+  while (vwarps > 1 && (sh ? tiles : 0) + vwarps * per_warp > cap) --vwarps;
+  if ((sh ? tiles : 0) + vwarps * per_warp > cap) {
+    set_error("Delta application: d too large for one warp's vectors in shared memory");
+    return EIFMM_EUNSUPPORTED;
+  }
+  // few vectors: a warp of them per CTA, spread over the SMs
+  if (LPV > 2)
+    while (vwarps > 1 && (vectors + (int64_t)vwarps * kVpw - 1) / ((int64_t)vwarps * kVpw) < kDeltaSpread) vwarps /= 2;
+  const int warps = LPV > 2 ? kDeltaMaxWarps : vwarps;
+  int blocks = 0;
+  for (int i = 0; i < b.nlev; ++i) {
+    b.lv[i].block0 = blocks;
+    const int64_t nw = (b.lv[i].nvec + kVpw - 1) / kVpw;
+    blocks += (int)((nw + vwarps - 1) / vwarps);
+  }
+  if (blocks == 0) return EIFMM_OK;
+  const size_t sm = (sh ? tiles : 0) + vwarps * per_warp;
+  if (!transpose)
+    return sh ? delta_launch<k_delta<T, true, false, Ti, To, PLANES, true, LPV>>(b, blocks, warps, vwarps, sm, s)
+              : delta_launch<k_delta<T, true, false, Ti, To, PLANES, false, LPV>>(b, blocks, warps, vwarps, sm, s);
+  return sh ? delta_launch<k_delta<T, false, true, Ti, To, PLANES, true, LPV>>(b, blocks, warps, vwarps, sm, s)
+            : delta_launch<k_delta<T, false, true, Ti, To, PLANES, false, LPV>>(b, blocks, warps, vwarps, sm, s);
 }
 
 // All levels of `b` in one launch (Delta if !transpose, else Delta^t).  The
@@ -305,31 +344,14 @@ eifmm_status delta_launch(const DeltaBatch& b, int blocks, int warps, size_t sm,
 template <typename T, typename Ti, typename To, int PLANES>
 eifmm_status launch_delta_batch(DeltaBatch& b, bool transpose, cudaStream_t s) {
   int nbmax = 0;
-  for (int i = 0; i < b.nlev; ++i) nbmax = b.lv[i].nvec > 0 && b.lv[i].nb > nbmax ? b.lv[i].nb : nbmax;
-  if (nbmax == 0) return EIFMM_OK;
-  const size_t per_warp = (size_t)nbmax * kDeltaTile * kDeltaLd * sizeof(T);
-  const size_t tiles = (size_t)nbmax * (nbmax + 1) / 2 * kDeltaTile * kDeltaTile * sizeof(T);
-  const size_t cap = 227 * 1024;
-  bool sh = tiles + per_warp <= cap;
-  int warps = kDeltaMaxWarps;
-  while (warps > 1 && (sh ? tiles : 0) + warps * per_warp > cap) --warps;
-  if ((sh ? tiles : 0) + warps * per_warp > cap) {
-    set_error("Delta application: d too large for one warp's vectors in shared memory");
-    return EIFMM_EUNSUPPORTED;
-  }
-  int blocks = 0;
+  int64_t vectors = 0;
   for (int i = 0; i < b.nlev; ++i) {
-    b.lv[i].block0 = blocks;
-    const int64_t nw = (b.lv[i].nvec + kDeltaVpw - 1) / kDeltaVpw;
-    blocks += (int)((nw + warps - 1) / warps);
+    nbmax = b.lv[i].nvec > 0 && b.lv[i].nb > nbmax ? b.lv[i].nb : nbmax;
+    vectors += b.lv[i].nvec;
   }
-  if (blocks == 0) return EIFMM_OK;
-  const size_t sm = (sh ? tiles : 0) + warps * per_warp;
-  if (!transpose)
-    return sh ? delta_launch<k_delta<T, true, false, Ti, To, PLANES, true>>(b, blocks, warps, sm, s)
-              : delta_launch<k_delta<T, true, false, Ti, To, PLANES, false>>(b, blocks, warps, sm, s);
-  return sh ? delta_launch<k_delta<T, false, true, Ti, To, PLANES, true>>(b, blocks, warps, sm, s)
-            : delta_launch<k_delta<T, false, true, Ti, To, PLANES, false>>(b, blocks, warps, sm, s);
+  if (nbmax == 0) return EIFMM_OK;
+  if (vectors < kDeltaFew) return launch_delta_shape<T, Ti, To, PLANES, 8>(b, transpose, nbmax, vectors, s);
+  return launch_delta_shape<T, Ti, To, PLANES, 2>(b, transpose, nbmax, vectors, s);
 }
 
 }  // namespace eifmm
