@@ -310,7 +310,7 @@ eifmm_status eifmm_tree_set_option(eifmm_tree* tree, eifmm_option opt, int value
  * the host, synchronises the stream and returns EINVAL if the count is not
  * zero. */
 #define EIFMM_STATIC_SORT_MAX_POINTS 1048576
-#define EIFMM_STATIC_SORT_SCRATCH_BYTES 8913296
+#define EIFMM_STATIC_SORT_SCRATCH_BYTES 8914176
 eifmm_status eifmm_tree_sort_static(const double* xyz, int64_t n,
                                     const double lo[3], double L, int depth,
                                     uint32_t* keys_out, int32_t* perm_out,
@@ -443,7 +443,9 @@ uint64_t eifmm_kernel_launches(void);
  * mixed path: [6] L2P of the far field + wait for the near field, [7] sum +
  * un-permute; FP64 path: [6] wait for the near field, [7] L2P + sum +
  * un-permute (7); [8] the near-field launch alone (on the library's side
- * stream); [9 + k] the M2L launch of level k alone. */
+ * stream); [9 + k] the M2L launch of level k alone (the residue products of the
+ * FP64 far field take all levels in the same launches: their time is in the
+ * leaf level's entry). */
 void eifmm_set_timing(int on);
 eifmm_status eifmm_last_step_times(const eifmm_tree* tree, float* ms20);
 

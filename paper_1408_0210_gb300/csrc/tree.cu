@@ -19,63 +19,77 @@ constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_ITEMS = 8;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;  // 2048 keys per block
 
-__global__ void k_keys(const double* __restrict__ xyz, int64_t n, double lo0,
-                       double lo1, double lo2, double hi0, double hi1,
-                       double hi2, double scale, int depth,
-                       uint32_t* __restrict__ keys, int32_t* __restrict__ idx,
-                       int* __restrict__ bad) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// The sort moves (key, index) pairs through LSD passes of at most 8 bits, the
+// 3 depth bits spread evenly.  A pass is three launches: digit counts per tile of
+// RS_TILE keys (the first pass's come with the keys), the scan of each digit's
+// row of counts, and the scatter, which ranks its tile in shared memory and
+// writes it in digit order (runs of neighbours instead of single words).
+// The passes alternate between an array of 8-byte pairs and the output arrays
+// (keys and indices apart), which the last one writes; the first takes the
+// indices as positions.  2^20 points, depth 5: the sort into kept arrays 174 ->
+// 153 us with its launches and its one read-back (separate words, 13 launches
+// before).
+constexpr int RS_DIGITS = 256;
+enum RsFormat { kRsKeys = 0, kRsPairs = 1, kRsSplit = 2 };
+
+// Keys of a tile of points and the tile's counts of the first digit.
+__global__ void __launch_bounds__(RS_THREADS)
+k_keys(const double* __restrict__ xyz, int64_t n, double lo0, double lo1, double lo2, double hi0, double hi1,
+       double hi2, double scale, int depth, uint32_t mask, uint32_t* __restrict__ keys,
+       uint32_t* __restrict__ counts, int nblocks, int* __restrict__ bad) {
+  __shared__ uint32_t h[RS_DIGITS];
+  h[threadIdx.x] = 0;
+  __syncthreads();
   const double lo[3] = {lo0, lo1, lo2};
   const double hi[3] = {hi0, hi1, hi2};
   const int nmax = (1 << depth) - 1;
-  int c[3];
-  bool out = false;
+#pragma unroll 4
+  for (int j = 0; j < RS_ITEMS; ++j) {
+    const int64_t i = (int64_t)blockIdx.x * RS_TILE + j * RS_THREADS + threadIdx.x;
+    if (i >= n) break;
+    int c[3];
+    bool out = false;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const double x = xyz[3 * i + a];
-    if (!(x >= lo[a] && x <= hi[a])) out = true;
-    // (x - lo) * scale: a subtraction then a product, never fused.  The
-    // conversion truncates toward zero and clamps to the int range (NaN gives
-    // 0); truncation equals floor wherever the clamp to [0, nmax] leaves the
-    // value unchanged.
-    const int v = __double2int_rz(__dmul_rn(__dsub_rn(x, lo[a]), scale));
-    c[a] = min(max(v, 0), nmax);
-  }
-  if (out) atomicAdd(bad, 1);
-  keys[i] = (uint32_t)morton_encode(c[0], c[1], c[2], depth);
-  idx[i] = (int32_t)i;
-}
-
-__global__ void k_rs_count(const uint32_t* __restrict__ keys, int64_t n,
-                           int shift, uint32_t* __restrict__ counts,
-                           int nblocks) {
-  __shared__ uint32_t h[256];
-  h[threadIdx.x] = 0;
-  __syncthreads();
-  const int64_t base = (int64_t)blockIdx.x * RS_TILE;
-  for (int i = threadIdx.x; i < RS_TILE; i += RS_THREADS) {
-    const int64_t p = base + i;
-    if (p < n) atomicAdd(&h[(keys[p] >> shift) & 255u], 1u);
+    for (int a = 0; a < 3; ++a) {
+      const double x = xyz[3 * i + a];
+      if (!(x >= lo[a] && x <= hi[a])) out = true;
+      // (x - lo) * scale: a subtraction then a product, never fused.  The
+      // conversion truncates toward zero and clamps to the int range (NaN gives
+      // 0); truncation equals floor wherever the clamp to [0, nmax] leaves the
+      // value unchanged.
+      const int v = __double2int_rz(__dmul_rn(__dsub_rn(x, lo[a]), scale));
+      c[a] = min(max(v, 0), nmax);
+    }
+    if (out) atomicAdd(bad, 1);
+    const uint32_t k = (uint32_t)morton_encode(c[0], c[1], c[2], depth);
+    keys[i] = k;
+    atomicAdd(&h[k & mask], 1u);
   }
   __syncthreads();
   counts[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
 }
 
-// Exclusive scan of the digit-major counts (256 x nblocks entries) in two
-// launches: per-tile totals, then each tile adds the totals of the tiles
-// before it to its own block-wide scan.  A tile is SC_TILE consecutive
-// entries, SC_ITEMS per thread.
-constexpr int SC_THREADS = 1024;
-constexpr int SC_ITEMS = 4;
-constexpr int SC_TILE = SC_THREADS * SC_ITEMS;
+template <int IN>
+__global__ void __launch_bounds__(RS_THREADS)
+k_rs_count(const uint32_t* __restrict__ kin, const uint2* __restrict__ pin, int64_t n, int shift, uint32_t mask, uint32_t* __restrict__ counts,
+           int nblocks) {
+  __shared__ uint32_t h[RS_DIGITS];
+  h[threadIdx.x] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < RS_ITEMS; ++j) {
+    const int64_t p = (int64_t)blockIdx.x * RS_TILE + j * RS_THREADS + threadIdx.x;
+    if (p < n) atomicAdd(&h[((IN == kRsPairs ? pin[p].x : kin[p]) >> shift) & mask], 1u);
+  }
+  __syncthreads();
+  counts[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
+}
 
-inline int64_t scan_tiles(int64_t len) { return (len + SC_TILE - 1) / SC_TILE; }
-
-// Exclusive scan of one value per thread over a block of SC_THREADS threads;
-// *total receives the block's sum.
+// Exclusive scan of one value per thread over the block; *total receives the
+// block's sum.
+template <int THREADS>
 __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* total) {
-  __shared__ uint32_t ws[SC_THREADS / 32];
+  __shared__ uint32_t ws[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   __syncthreads();  // ws may still be read by a previous call
   uint32_t x = v;
@@ -87,7 +101,7 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* total)
   if (lane == 31) ws[w] = x;
   __syncthreads();
   if (w == 0) {
-    uint32_t u = ws[lane];
+    uint32_t u = lane < THREADS / 32 ? ws[lane] : 0u;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xffffffffu, u, o);
@@ -96,72 +110,58 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* total)
     ws[lane] = u;
   }
   __syncthreads();
-  *total = ws[SC_THREADS / 32 - 1];
+  *total = ws[THREADS / 32 - 1];
   return x - v + (w > 0 ? ws[w - 1] : 0u);
 }
 
+// Exclusive scan of a digit's counts over the tiles, one block per digit; the
+// digit's total goes to total[digit] (the scatter scans the 256 totals itself).
+constexpr int SC_THREADS = 1024;
 __global__ void __launch_bounds__(SC_THREADS)
-k_scan_totals(const uint32_t* __restrict__ a, int64_t len, uint32_t* __restrict__ part) {
-  const int64_t base = (int64_t)blockIdx.x * SC_TILE + (int64_t)threadIdx.x * SC_ITEMS;
-  uint32_t s = 0;
-#pragma unroll
-  for (int j = 0; j < SC_ITEMS; ++j)
-    if (base + j < len) s += a[base + j];
-  uint32_t total;
-  block_excl_scan(s, &total);
-  if (threadIdx.x == 0) part[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(SC_THREADS)
-k_scan_apply(uint32_t* __restrict__ a, int64_t len, const uint32_t* __restrict__ part) {
-  uint32_t pre = 0;
-  for (int j = threadIdx.x; j < (int)blockIdx.x; j += SC_THREADS) pre += part[j];
-  uint32_t before;
-  block_excl_scan(pre, &before);
-  const int64_t base = (int64_t)blockIdx.x * SC_TILE + (int64_t)threadIdx.x * SC_ITEMS;
-  uint32_t v[SC_ITEMS], s = 0;
-#pragma unroll
-  for (int j = 0; j < SC_ITEMS; ++j) {
-    v[j] = base + j < len ? a[base + j] : 0u;
-    s += v[j];
+k_rs_rows(uint32_t* __restrict__ counts, int nblocks, uint32_t* __restrict__ total) {
+  uint32_t* row = counts + (int64_t)blockIdx.x * nblocks;
+  uint32_t run = 0;
+  for (int b0 = 0; b0 < nblocks; b0 += SC_THREADS) {
+    const int b = b0 + threadIdx.x;
+    const uint32_t v = b < nblocks ? row[b] : 0u;
+    uint32_t t;
+    const uint32_t x = block_excl_scan<SC_THREADS>(v, &t);
+    if (b < nblocks) row[b] = run + x;
+    run += t;
   }
-  uint32_t total;
-  uint32_t run = before + block_excl_scan(s, &total);
-#pragma unroll
-  for (int j = 0; j < SC_ITEMS; ++j) {
-    if (base + j < len) a[base + j] = run;
-    run += v[j];
-  }
+  if (threadIdx.x == 0) total[blockIdx.x] = run;
 }
 
-void launch_scan(uint32_t* counts, int64_t len, uint32_t* part, cudaStream_t s) {
-  const unsigned nt = (unsigned)scan_tiles(len);
-  k_scan_totals<<<nt, SC_THREADS, 0, s>>>(counts, len, part);
-  k_scan_apply<<<nt, SC_THREADS, 0, s>>>(counts, len, part);
-}
-
+template <int IN, int OUT>
 __global__ void __launch_bounds__(RS_THREADS)
-k_rs_scatter(const uint32_t* __restrict__ kin, const int32_t* __restrict__ vin,
-             uint32_t* __restrict__ kout, int32_t* __restrict__ vout, int64_t n,
-             int shift, const uint32_t* __restrict__ offsets, int nblocks) {
-  __shared__ uint32_t wc[RS_WARPS][257];
-  for (int i = threadIdx.x; i < RS_WARPS * 257; i += RS_THREADS) (&wc[0][0])[i] = 0;
+k_rs_scatter(const uint32_t* __restrict__ kin, const int32_t* __restrict__ vin, const uint2* __restrict__ pin,
+             uint2* __restrict__ pout,
+             uint32_t* __restrict__ kout, int32_t* __restrict__ vout, int64_t n, int shift, uint32_t mask,
+             const uint32_t* __restrict__ rows, const uint32_t* __restrict__ total, int nblocks) {
+  __shared__ uint32_t wc[RS_WARPS][RS_DIGITS + 1];
+  __shared__ uint32_t s_pos[RS_DIGITS];  // global position of the tile's position 0 in a digit's order
+  __shared__ uint32_t s_loc[RS_DIGITS];  // first tile position of a digit
+  __shared__ uint2 s_pair[RS_TILE];
+  for (int i = threadIdx.x; i < RS_WARPS * (RS_DIGITS + 1); i += RS_THREADS) (&wc[0][0])[i] = 0;
+  uint32_t all;
+  const uint32_t base = block_excl_scan<RS_THREADS>(total[threadIdx.x], &all);
+  const uint32_t row = rows[(int64_t)threadIdx.x * nblocks + blockIdx.x];
   __syncthreads();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const int64_t wbase = (int64_t)blockIdx.x * RS_TILE + (int64_t)w * (32 * RS_ITEMS);
-  uint32_t kk[RS_ITEMS];
-  int32_t vv[RS_ITEMS];
+  uint2 e[RS_ITEMS];
   uint32_t rank[RS_ITEMS];
-  int dig[RS_ITEMS];
 #pragma unroll
   for (int j = 0; j < RS_ITEMS; ++j) {
     const int64_t p = wbase + j * 32 + lane;
-    const bool valid = p < n;
-    kk[j] = valid ? kin[p] : 0u;
-    vv[j] = valid ? vin[p] : 0;
-    const int d = valid ? (int)((kk[j] >> shift) & 255u) : 256;
-    dig[j] = d;
+    e[j] = make_uint2(0u, 0u);
+    if (p < n) e[j] = IN == kRsPairs ? pin[p] : make_uint2(kin[p], IN == kRsSplit ? (uint32_t)vin[p] : (uint32_t)p);
+  }
+#pragma unroll
+  for (int j = 0; j < RS_ITEMS; ++j) {
+    const bool valid = wbase + j * 32 + lane < n;
+    const int d = valid ? (int)((e[j].x >> shift) & mask) : RS_DIGITS;
     const unsigned peers = __match_any_sync(0xffffffffu, d);
     const uint32_t old = wc[w][d];
     __syncwarp();
@@ -170,22 +170,88 @@ k_rs_scatter(const uint32_t* __restrict__ kin, const int32_t* __restrict__ vin,
     rank[j] = old + __popc(peers & lt);
   }
   __syncthreads();
-  for (int d = threadIdx.x; d < 256; d += RS_THREADS) {
+  {
+    const int d = threadIdx.x;
     uint32_t run = 0;
     for (int ww = 0; ww < RS_WARPS; ++ww) {
       const uint32_t t = wc[ww][d];
       wc[ww][d] = run;
       run += t;
     }
+    uint32_t cnt;
+    const uint32_t loc = block_excl_scan<RS_THREADS>(run, &cnt);
+    s_loc[d] = loc;
+    s_pos[d] = base + row - loc;
   }
   __syncthreads();
 #pragma unroll
-  for (int j = 0; j < RS_ITEMS; ++j) {
-    if (dig[j] == 256) continue;
-    const uint32_t pos = offsets[(int64_t)dig[j] * nblocks + blockIdx.x] + wc[w][dig[j]] + rank[j];
-    kout[pos] = kk[j];
-    vout[pos] = vv[j];
+  for (int j = 0; j < RS_ITEMS; ++j)
+    if (wbase + j * 32 + lane < n) {
+      const int d = (int)((e[j].x >> shift) & mask);
+      s_pair[s_loc[d] + wc[w][d] + rank[j]] = e[j];
+    }
+  __syncthreads();
+  const int64_t left = n - (int64_t)blockIdx.x * RS_TILE;
+  const int cnt = left < RS_TILE ? (int)left : RS_TILE;
+  for (int i = threadIdx.x; i < cnt; i += RS_THREADS) {
+    const uint2 q = s_pair[i];
+    const uint32_t pos = s_pos[(q.x >> shift) & mask] + (uint32_t)i;
+    if (OUT == kRsPairs) {
+      pout[pos] = q;
+    } else {
+      kout[pos] = q.x;
+      vout[pos] = (int32_t)q.y;
+    }
   }
+}
+
+// Scratch of the sort of n points: an array of pairs, counts, totals.
+struct SortBuffers {
+  uint2* pairs;
+  uint32_t* counts;
+  uint32_t* total;
+};
+
+// keys, perm: the sorted keys and input positions of the points xyz.
+eifmm_status sort_points(const double* xyz, int64_t n, const double lo[3], double L, int depth, uint32_t* keys,
+                         int32_t* perm, const SortBuffers& b, int* bad, cudaStream_t s) {
+  const int nb = (int)((n + RS_TILE - 1) / RS_TILE), T = RS_THREADS;
+  const int bits = 3 * depth, passes = (bits + 7) / 8;
+  // pass p writes the output arrays when an even number of passes follows it;
+  // the unsorted keys start where the first pass does not write
+  auto to_split = [&](int p) { return (passes - 1 - p) % 2 == 0; };
+  uint32_t* k0 = to_split(0) ? (uint32_t*)b.pairs : keys;
+  int shift = 0;
+  for (int p = 0; p < passes; ++p) {
+    const int w = bits / passes + (p < bits % passes ? 1 : 0);
+    const uint32_t mask = (1u << w) - 1u;
+    const bool split = to_split(p);
+    if (p == 0)
+      k_keys<<<nb, T, 0, s>>>(xyz, n, lo[0], lo[1], lo[2], lo[0] + L, lo[1] + L, lo[2] + L, ldexp(1.0, depth) / L,
+                              depth, mask, k0, b.counts, nb, bad);
+    else if (split)
+      k_rs_count<kRsPairs><<<nb, T, 0, s>>>(nullptr, b.pairs, n, shift, mask, b.counts, nb);
+    else
+      k_rs_count<kRsSplit><<<nb, T, 0, s>>>(keys, nullptr, n, shift, mask, b.counts, nb);
+    EIFMM_CHECK_LAUNCH();
+    k_rs_rows<<<RS_DIGITS, SC_THREADS, 0, s>>>(b.counts, nb, b.total);
+    EIFMM_CHECK_LAUNCH();
+    if (p == 0 && split)
+      k_rs_scatter<kRsKeys, kRsSplit><<<nb, T, 0, s>>>(k0, nullptr, nullptr, nullptr, keys, perm, n, shift, mask,
+                                                      b.counts, b.total, nb);
+    else if (p == 0)
+      k_rs_scatter<kRsKeys, kRsPairs><<<nb, T, 0, s>>>(k0, nullptr, nullptr, b.pairs, nullptr, nullptr, n, shift, mask,
+                                                      b.counts, b.total, nb);
+    else if (split)
+      k_rs_scatter<kRsPairs, kRsSplit><<<nb, T, 0, s>>>(nullptr, nullptr, b.pairs, nullptr, keys, perm, n, shift, mask,
+                                                       b.counts, b.total, nb);
+    else
+      k_rs_scatter<kRsSplit, kRsPairs><<<nb, T, 0, s>>>(keys, perm, nullptr, b.pairs, nullptr, nullptr, n, shift, mask,
+                                                       b.counts, b.total, nb);
+    EIFMM_CHECK_LAUNCH();
+    shift += w;
+  }
+  return EIFMM_OK;
 }
 
 // off[b] = first sorted position whose key is at least b (b = 0..nleaf;
@@ -287,8 +353,8 @@ eifmm_status build_pointset(const double* xyz, int64_t n, const double lo[3],
   const int nblocks = (int)((n + RS_TILE - 1) / RS_TILE);
   const int nb1 = nblocks > 0 ? nblocks : 1;
   size_t soff = 0;
-  const size_t o_k2 = take(soff, nn * 4), o_v2 = take(soff, nn * 4), o_cnt = take(soff, (size_t)256 * nb1 * 4),
-               o_part = take(soff, scan_tiles((int64_t)256 * nb1) * 4), o_bad = take(soff, 3 * sizeof(int));
+  const size_t o_pairs = take(soff, nn * 8), o_cnt = take(soff, (size_t)RS_DIGITS * nb1 * 4),
+               o_tot = take(soff, RS_DIGITS * 4), o_bad = take(soff, 3 * sizeof(int));
   // The sort's scratch is kept per device between builds (grown on demand,
   // held until the process exits); builds on one device take turns on it.
   int dev = 0;
@@ -303,40 +369,11 @@ eifmm_status build_pointset(const double* xyz, int64_t n, const double lo[3],
     sc.cap = soff;
   }
   unsigned char* scratch = sc.p;
-  uint32_t* k2 = (uint32_t*)(scratch + o_k2);
-  int32_t* v2 = (int32_t*)(scratch + o_v2);
-  uint32_t* counts = (uint32_t*)(scratch + o_cnt);
-  uint32_t* parts = (uint32_t*)(scratch + o_part);
+  const SortBuffers sb{(uint2*)(scratch + o_pairs), (uint32_t*)(scratch + o_cnt), (uint32_t*)(scratch + o_tot)};
   int* dbad = (int*)(scratch + o_bad);
   EIFMM_CUDA(cudaMemsetAsync(dbad, 0, 3 * sizeof(int), s));
 
-  const double scale = ldexp(1.0, depth) / L;
-  if (n > 0) {
-    k_keys<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(
-        xyz, n, lo[0], lo[1], lo[2], lo[0] + L, lo[1] + L, lo[2] + L, scale,
-        depth, ps->keys, ps->perm, dbad);
-    EIFMM_CHECK_LAUNCH();
-    uint32_t* kin = ps->keys;
-    int32_t* vin = ps->perm;
-    uint32_t* kout = k2;
-    int32_t* vout = v2;
-    const int bits = 3 * depth;
-    for (int shift = 0; shift < bits; shift += 8) {
-      k_rs_count<<<nblocks, RS_THREADS, 0, s>>>(kin, n, shift, counts, nblocks);
-      EIFMM_CHECK_LAUNCH();
-      launch_scan(counts, (int64_t)256 * nblocks, parts, s);
-      EIFMM_CHECK_LAUNCH();
-      k_rs_scatter<<<nblocks, RS_THREADS, 0, s>>>(kin, vin, kout, vout, n, shift,
-                                                   counts, nblocks);
-      EIFMM_CHECK_LAUNCH();
-      uint32_t* tk = kin; kin = kout; kout = tk;
-      int32_t* tv = vin; vin = vout; vout = tv;
-    }
-    if (kin != ps->keys) {
-      EIFMM_CUDA(cudaMemcpyAsync(ps->keys, kin, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
-      EIFMM_CUDA(cudaMemcpyAsync(ps->perm, vin, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-    }
-  }
+  if (n > 0) EIFMM_TRY(sort_points(xyz, n, lo, L, depth, ps->keys, ps->perm, sb, dbad, s));
   k_leaf_off<<<(unsigned)((nleaf + 1 + 255) / 256), 256, 0, s>>>(ps->keys, n, nleaf, ps->leaf_off);
   EIFMM_CHECK_LAUNCH();
   if (n > 0) {
@@ -370,19 +407,18 @@ void free_pointset(PointSet* ps) {
 
 // ---------------------------------------------------------------------------
 // Allocation-free variant of the bin/sort (eifmm_tree_sort_static).  Its
-// radix-sort scratch lives in a file-scope device array: keys and indices of
-// the other half of the ping-pong (4 + 4 bytes per point), the per-block
-// digit counts (256 x 4 bytes per 2048 points) and an error counter.
+// radix-sort scratch lives in a file-scope device array: the pairs of the
+// passes between (8 bytes per point), the digit counts of the tiles (256 x 4
+// bytes per 2048 points), their totals and an error counter.
 // ---------------------------------------------------------------------------
 namespace eifmm {
 namespace {
 constexpr int64_t kStaticMax = EIFMM_STATIC_SORT_MAX_POINTS;
 constexpr int64_t kStaticBlocks = (kStaticMax + RS_TILE - 1) / RS_TILE;
-constexpr size_t kOffKeys = 0;
-constexpr size_t kOffVals = kOffKeys + (size_t)kStaticMax * 4;
-constexpr size_t kOffCounts = kOffVals + (size_t)kStaticMax * 4;
-constexpr size_t kOffParts = kOffCounts + (size_t)256 * kStaticBlocks * 4;
-constexpr size_t kOffBad = kOffParts + (((size_t)256 * kStaticBlocks + SC_TILE - 1) / SC_TILE) * 4 + 16;
+constexpr size_t kOffPairs = 0;
+constexpr size_t kOffCounts = kOffPairs + (size_t)kStaticMax * 8;
+constexpr size_t kOffTotal = kOffCounts + (size_t)RS_DIGITS * kStaticBlocks * 4;
+constexpr size_t kOffBad = kOffTotal + RS_DIGITS * 4;
 constexpr size_t kStaticBytes = kOffBad + 256;
 static_assert(kStaticBytes == EIFMM_STATIC_SORT_SCRATCH_BYTES, "scratch size of the header");
 
@@ -437,39 +473,12 @@ extern "C" eifmm_status eifmm_tree_sort_static(const double* xyz, int64_t n, con
   unsigned char* base = nullptr;
   EIFMM_TRY(static_scratch(&base));
   cudaStream_t s = (cudaStream_t)stream;
-  uint32_t* k2 = (uint32_t*)(base + kOffKeys);
-  int32_t* v2 = (int32_t*)(base + kOffVals);
-  uint32_t* counts = (uint32_t*)(base + kOffCounts);
-  uint32_t* parts = (uint32_t*)(base + kOffParts);
+  const SortBuffers sb{(uint2*)(base + kOffPairs), (uint32_t*)(base + kOffCounts), (uint32_t*)(base + kOffTotal)};
   int* bad = (int*)(base + kOffBad);
   // the error counter must start at zero on every call
   EIFMM_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
   const int64_t nleaf = (int64_t)1 << (3 * depth);
-  const int nblocks = (int)((n + RS_TILE - 1) / RS_TILE);
-  if (n > 0) {
-    k_keys<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(xyz, n, lo[0], lo[1], lo[2], lo[0] + L, lo[1] + L,
-                                                        lo[2] + L, ldexp(1.0, depth) / L, depth, keys_out,
-                                                        perm_out, bad);
-    EIFMM_CHECK_LAUNCH();
-    uint32_t* kin = keys_out;
-    int32_t* vin = perm_out;
-    uint32_t* kout = k2;
-    int32_t* vout = v2;
-    for (int shift = 0; shift < 3 * depth; shift += 8) {
-      k_rs_count<<<nblocks, RS_THREADS, 0, s>>>(kin, n, shift, counts, nblocks);
-      EIFMM_CHECK_LAUNCH();
-      launch_scan(counts, (int64_t)256 * nblocks, parts, s);
-      EIFMM_CHECK_LAUNCH();
-      k_rs_scatter<<<nblocks, RS_THREADS, 0, s>>>(kin, vin, kout, vout, n, shift, counts, nblocks);
-      EIFMM_CHECK_LAUNCH();
-      uint32_t* tk = kin; kin = kout; kout = tk;
-      int32_t* tv = vin; vin = vout; vout = tv;
-    }
-    if (kin != keys_out) {
-      EIFMM_CUDA(cudaMemcpyAsync(keys_out, kin, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
-      EIFMM_CUDA(cudaMemcpyAsync(perm_out, vin, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-    }
-  }
+  if (n > 0) EIFMM_TRY(sort_points(xyz, n, lo, L, depth, keys_out, perm_out, sb, bad, s));
   k_leaf_off<<<(unsigned)((nleaf + 1 + 255) / 256), 256, 0, s>>>(keys_out, n, nleaf, leaf_off_out);
   EIFMM_CHECK_LAUNCH();
   int hbad = 0;
