@@ -95,6 +95,7 @@ struct CrtLv {
   int z0, nz, sz0, snz;      // planes of target boxes, planes of source boxes held
   int r0, Rc, R, G;          // columns r0 .. r0 + Rc of R, offset groups
   int nchunk, n0, ks0, ks1;  // chunks of K: n0 of ks0 k-steps, then ks1 k-steps each
+  unsigned pinv;             // 2^32 over the pairs of coefficients of a row, rounded up
   unsigned item0, pl0, rc0, mx0;  // first block of this level in each of the launches
   const double* W;
   double* g;
@@ -165,9 +166,6 @@ __device__ __forceinline__ Win window_of(const CrtLv& v, int ct, int w) {
   if (v.mode == kCrtM2L) {
     o.cs = w / 3;
     o.sy1 = w - 3 * o.cs;
-    o.mask = combo_mask(ct, o.cs, o.sy1);
-    o.slot = (2 * (o.sy1 - 1) + ((o.cs >> 1) & 1) - ((ct >> 1) & 1) + 3) * 7 + (o.cs & 1) - (ct & 1) + 3 +
-             ((o.cs >> 2) - (ct >> 2) + 3) * 49;
   } else {  // no shift: the 8 children of a box (M2M), its parent (L2L), itself (box)
     o.cs = v.mode == kCrtM2M ? w : (v.mode == kCrtL2L ? 0 : ct);
     o.slot = v.mode == kCrtM2M ? w : (v.mode == kCrtL2L ? ct : 0);
@@ -178,9 +176,9 @@ __device__ __forceinline__ Win window_of(const CrtLv& v, int ct, int w) {
 }
 
 // Morton key of box (x, y, z) of class c of nc
-__device__ __forceinline__ int64_t class_box(int nc, int c, int x, int y, int z, int level) {
-  if (nc == 1) return morton_encode(x, y, z, level);
-  return morton_encode(2 * x + (c & 1), 2 * y + ((c >> 1) & 1), 2 * z + (c >> 2), level);
+__device__ __forceinline__ int64_t class_box(int nc, int c, int x, int y, int z) {
+  const int64_t m = morton_encode(x, y, z, 0);
+  return nc == 1 ? m : 8 * m + c;
 }
 
 // scale exponent of a column from the bits of its largest |W|
@@ -191,15 +189,54 @@ __device__ __forceinline__ int w_exp(unsigned long long bits, int wbits) {
 }
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
-// v modulo crt_mod(i), in [-m/2, m/2]; |v| <= 2^60
-__device__ __forceinline__ int residue(long long v, int i) {
-  const int m = crt_mod(i);
-  const int c20 = (1 << 20) % m, c40 = (int)((1ll << 40) % m);
-  const int v2 = (int)(v >> 40), v1 = (int)(v >> 20) & 0xfffff, v0 = (int)v & 0xfffff;
-  // |v2 c40| < 2^29 and v1 c20 + v0 < 2^29 + 2^20: the offset keeps it positive
-  const unsigned u = (unsigned)(v2 * c40 + v1 * c20 + v0) + (unsigned)m * (unsigned)((1u << 30) / m);
-  int r = (int)(u % (unsigned)m);
-  return r > m / 2 ? r - m : r;
+// W 2^b rounded to an integer, |W| 2^b <= 2^58
+__device__ __forceinline__ long long w_int(double w, int b) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(w) & 0x7fffffffffffffffull;
+  const int e = (int)(u >> 52);
+  unsigned long long m = u & 0xfffffffffffffull;
+  if (e) m |= 1ull << 52;
+  const int sh = (e ? e : 1) - 1075 + b;  // at most 6
+  if (sh >= 0) m <<= sh;
+  else m = sh < -54 ? 0 : (m + (1ull << (-sh - 1))) >> -sh;
+  return w < 0.0 ? -(long long)m : (long long)m;
+}
+
+// 2^(12 j) modulo crt_mod(i), in [-m/2, m/2]
+__host__ __device__ constexpr int limb_res(int i, int j) {
+  int r = 1;
+  for (int k = 0; k < 12 * j; ++k) r = 2 * r % crt_mod(i);
+  return r > crt_mod(i) / 2 ? r - crt_mod(i) : r;
+}
+
+// Two integers, |v| <= 2^60, as FP32 limbs of 12 bits, the last one signed.
+struct Limbs {
+  float2 l[5];
+};
+__device__ __forceinline__ Limbs limbs_of(long long v0, long long v1) {
+  Limbs o;
+#pragma unroll
+  for (int j = 0; j < 5; ++j)
+    o.l[j] = j < 4 ? make_float2((float)((int)(v0 >> (12 * j)) & 0xfff), (float)((int)(v1 >> (12 * j)) & 0xfff))
+                   : make_float2((float)(int)(v0 >> 48), (float)(int)(v1 >> 48));
+  return o;
+}
+// Residues of both modulo crt_mod(I), in [-m/2, m/2], as two BF16.  The sum of
+// the limbs' residues is exact (below 2^22.1); its quotient by m is off by less
+// than 6e-4 before it is rounded, and a multiple of 1 / m for odd m comes no
+// nearer to a half than 1 / 2m >= 9.7e-4 (for m = 512 it is exact).  Residues up to
+// 256 are exact in BF16, whose bits are the upper half of FP32's.
+template <int I>
+__device__ __forceinline__ uint32_t residue2(const Limbs& v) {
+  constexpr float fm = (float)crt_mod(I), inv = 1.0f / fm;
+  float2 u = v.l[0];
+  u = __ffma2_rn(v.l[1], make_float2(limb_res(I, 1), limb_res(I, 1)), u);
+  u = __ffma2_rn(v.l[2], make_float2(limb_res(I, 2), limb_res(I, 2)), u);
+  u = __ffma2_rn(v.l[3], make_float2(limb_res(I, 3), limb_res(I, 3)), u);
+  u = __ffma2_rn(v.l[4], make_float2(limb_res(I, 4), limb_res(I, 4)), u);
+  const float2 k = __fadd2_rn(__ffma2_rn(u, make_float2(inv, inv), make_float2(12582912.0f, 12582912.0f)),
+                              make_float2(-12582912.0f, -12582912.0f));
+  const float2 r = __ffma2_rn(k, make_float2(-fm, -fm), u);
+  return __byte_perm(__float_as_uint(r.x), __float_as_uint(r.y), 0x7632);
 }
 
 __device__ __forceinline__ int find_level(const CrtArgs& a, unsigned CrtLv::*first, unsigned b) {
@@ -209,19 +246,28 @@ __device__ __forceinline__ int find_level(const CrtArgs& a, unsigned CrtLv::*fir
 }
 
 // ---------------------------------------------------------- largest |W| --
-constexpr int kMaxPer = 16384;  // entries per block
+// A block takes 32 boxes of a column, a warp four of them at once: the loads of
+// all four are in flight together (one box after the other took 34 us at any size).
+constexpr int kMaxBoxes = 32;
 __global__ void __launch_bounds__(256) k_crt_max(const __grid_constant__ CrtArgs a) {
   const CrtLv& v = a.lv[find_level(a, &CrtLv::mx0, blockIdx.x)];
-  const unsigned b = blockIdx.x - v.mx0;
-  const int r = v.r0 + (int)(b % v.Rc);
-  const int64_t n = ((int64_t)1 << (3 * v.slevel)) * v.ds;
-  const int64_t beg = (int64_t)(b / v.Rc) * kMaxPer, end = min(n, beg + kMaxPer);
+  const unsigned b = blockIdx.x - v.mx0, q = b / (unsigned)v.Rc;
+  const int r = v.r0 + (int)(b - q * v.Rc), ds = v.ds;
+  const int64_t box0 = (int64_t)q * kMaxBoxes + (threadIdx.x >> 5), n = (int64_t)1 << (3 * v.slevel);
+  const double* w[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int64_t box = box0 + 8 * j;
+    w[j] = v.W + ((box < n ? box : n - 1) * v.R + r) * ds;
+  }
   unsigned long long mx = 0;
-  for (int64_t i = beg + threadIdx.x; i < end; i += 256) {
-    const int64_t box = v.R == 1 ? 0 : i / v.ds;
-    const double w = v.R == 1 ? v.W[i] : v.W[(box * v.R + r) * v.ds + (i - box * v.ds)];
-    const unsigned long long x = (unsigned long long)__double_as_longlong(w) & 0x7fffffffffffffffull;
-    mx = x > mx ? x : mx;
+#pragma unroll 2
+  for (int l = threadIdx.x & 31; l < ds; l += 32) {
+    unsigned long long x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] = (unsigned long long)__double_as_longlong(w[j][l]) & 0x7fffffffffffffffull;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mx = x[j] > mx ? x[j] : mx;
   }
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long x = __shfl_xor_sync(0xffffffffu, mx, o);
@@ -232,14 +278,24 @@ __global__ void __launch_bounds__(256) k_crt_max(const __grid_constant__ CrtArgs
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 8; ++w) mx = sm[w] > mx ? sm[w] : mx;
-    atomicMax(v.wmax + r, mx);
+    if (mx > *(volatile unsigned long long*)(v.wmax + r)) atomicMax(v.wmax + r, mx);
   }
 }
 
 // ------------------------------------------------------- residue planes --
-// A block takes 8 boxes along x of one class, z, y and column: their W is
-// rounded to integers once, and every thread writes 8 terms of one box for
-// the 14 moduli (16-byte stores, 128 contiguous bytes per 8 threads).
+// A block takes 8 boxes along x of one class, z, y and column, a warp each: their
+// W is rounded to integers once, and every thread writes 8 terms of one box for
+// all moduli (16-byte stores, 128 contiguous bytes per 8 threads).  Both the
+// rounding and the residues stay off the FP64 and the conversion units: 262,144
+// points, 7 columns, d = 193, the leaf level 694 -> 455 us (3.5 TB/s).
+template <int I, int NM>
+__device__ __forceinline__ void store_residues(const Limbs (&v)[4], __nv_bfloat16* dst, int64_t step) {
+  if constexpr (I < NM) {
+    *reinterpret_cast<uint4*>(dst) =
+        make_uint4(residue2<I>(v[0]), residue2<I>(v[1]), residue2<I>(v[2]), residue2<I>(v[3]));
+    store_residues<I + 1, NM>(v, dst + step, step);
+  }
+}
 template <int NM>
 __global__ void __launch_bounds__(256) k_crt_planes(const __grid_constant__ CrtArgs a) {
   extern __shared__ long long s_w[];  // [8][K + 1]
@@ -256,15 +312,12 @@ __global__ void __launch_bounds__(256) k_crt_planes(const __grid_constant__ CrtA
   const int z = v.sz0 + zs, K = v.K, ld = K + 1;
   const unsigned long long bits = v.wmax[v.r0 + r];
   const bool fin = w_finite(bits);
-  const double sc = pow2(w_exp(fin ? bits : 0, v.wbits));
-  for (int i = threadIdx.x; i < 8 * K; i += 256) {
-    const int bx = i / K, l = i - bx * K, x = 8 * xs + bx;
-    long long q = 0;
-    if (l < v.ds && x < h && fin) {
-      const int64_t I = class_box(v.ncs, cls, x, y, z, v.slevel);
-      q = __double2ll_rn(v.W[(I * v.R + v.r0 + r) * v.ds + l] * sc);
-    }
-    s_w[bx * ld + l] = q;
+  const int e = w_exp(fin ? bits : 0, v.wbits);
+  {
+    const int bx = threadIdx.x >> 5, x = 8 * xs + bx;
+    const double* w = x < h && fin ? v.W + (class_box(v.ncs, cls, x, y, z) * v.R + v.r0 + r) * v.ds : nullptr;
+#pragma unroll 4
+    for (int l = threadIdx.x & 31; l < K; l += 32) s_w[bx * ld + l] = w && l < v.ds ? w_int(w[l], e) : 0;
   }
   __syncthreads();
   const int64_t plane = (int64_t)(K / 8) * v.snz * h * h * 8;  // elements of one (mod, r, class)
@@ -272,18 +325,11 @@ __global__ void __launch_bounds__(256) k_crt_planes(const __grid_constant__ CrtA
     const int bx = u & 7, k8 = u >> 3, x = 8 * xs + bx;
     if (x >= h) continue;
     const long long* q = s_w + bx * ld + 8 * k8;
-    long long w[8];
+    Limbs w[4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) w[j] = q[j];
+    for (int j = 0; j < 4; ++j) w[j] = limbs_of(q[2 * j], q[2 * j + 1]);
     __nv_bfloat16* dst = v.planes + (int64_t)(r * v.ncs + cls) * plane + ((((int64_t)k8 * v.snz + zs) * h + y) * h + x) * 8;
-#pragma unroll
-    for (int i = 0; i < NM; ++i) {
-      __nv_bfloat162 o[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        o[j] = __floats2bfloat162_rn((float)residue(w[2 * j], i), (float)residue(w[2 * j + 1], i));
-      *reinterpret_cast<uint4*>(dst + (int64_t)i * v.Rc * v.ncs * plane) = *reinterpret_cast<uint4*>(o);
-    }
+    store_residues<0, NM>(w, dst, (int64_t)v.Rc * v.ncs * plane);
   }
 }
 
@@ -571,68 +617,109 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
 // G / M modulo 1 = sum_i s_i y_i / m_i modulo 1, in fixed point of NW words (the
 // constants' rounding adds at most 2^(14 - 32 NW) of M; G itself is about 2^-10
 // of M, 2^-40 for Delta^t, whose terms cancel, with one word more).
-// A warp takes one (column, box) row, a lane two coefficients.
+// A thread takes two coefficients; the result is rounded in integers, once (the
+// FP64 pipe, at 1/64 of the integer rate, took two thirds of the time: the M2L's 45
+// million sums at 262,144 points, 7 columns 1,677 -> 626 us).
+constexpr int kRebuild = 128;
+
+// (H 2^64 + L) 2^(e - 128) times c, rounded to FP64; c normal and positive
+__device__ __forceinline__ double fixed_times(unsigned long long H, unsigned long long L, int e, double c) {
+  const bool neg = (long long)H < 0;
+  if (neg) {
+    L = ~L + 1;
+    H = ~H + (L == 0);
+  }
+  if (H == 0) {
+    H = L;
+    L = 0;
+    e -= 64;
+  }
+  if (H == 0) return 0.0;
+  const int z = __clzll((long long)H);
+  if (z) H = (H << z) | (L >> (64 - z));
+  const unsigned long long cb = (unsigned long long)__double_as_longlong(c);
+  unsigned long long P = __umul64hi(H, (cb << 11) | (1ull << 63));
+  // P 2^(e - z) (c's exponent in units of 2^-63): normalise its top bit
+  const int up = (long long)P >= 0;
+  P <<= up;
+  const unsigned long long m = (P >> 11) + ((P >> 10) & 1);
+  // value P 2^-64 2^(e - z - up) 2^(ec + 1), ec the exponent of c: P 2^-63 in [1, 2)
+  const int E = e - z - up + (int)(cb >> 52) - 1023;
+  double y;
+  if (E > -1022 && E < 1023) y = __longlong_as_double((long long)(((unsigned long long)(E + 1022) << 52) + m));
+  else y = scalbn((double)(long long)m, E - 52);
+  return neg ? -y : y;
+}
+
 template <int NM, int NW>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kRebuild)
 k_crt_rebuild(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK<NM, NW> kc) {
   const CrtLv& v = a.lv[find_level(a, &CrtLv::rc0, blockIdx.x)];
-  const int lane = threadIdx.x & 31;
-  const int64_t cells = (int64_t)v.nz * v.h * v.h, rows = cells * v.nct * v.Rc;
-  const int64_t row = (int64_t)(blockIdx.x - v.rc0) * 4 + (threadIdx.x >> 5);
+  const unsigned P = (unsigned)(v.d + 1) / 2;  // pairs of a row
+  const unsigned cells = (unsigned)(v.nz * v.h * v.h), rows = cells * (unsigned)(v.nct * v.Rc);
+  // the block's first pair, then a thread's within 2^16: one multiplication
+  const int64_t first = (int64_t)(blockIdx.x - v.rc0) * kRebuild;
+  const unsigned row0 = (unsigned)(first / P), t = (unsigned)(first - (int64_t)row0 * P) + threadIdx.x;
+  const unsigned dr = __umulhi(t, v.pinv), row = row0 + dr;
   if (row >= rows) return;
-  const int64_t cell = row % cells;
-  const int cls = (int)((row / cells) % v.nct), r = v.r0 + (int)(row / (cells * v.nct));
-  const int x = (int)(cell % v.h), y = (int)((cell / v.h) % v.h), z = v.z0 + (int)(cell / ((int64_t)v.h * v.h));
-  const int64_t I = class_box(v.nct, cls, x, y, z, v.tlevel);
+  const int c = 2 * (int)(t - dr * P);
   const int N = v.NT * v.Nt;
-  const int16_t* res = v.res + row * N;
-  double* g = v.g + (I * v.R + r) * v.d;
-  const double* add = v.add ? v.add + (I * v.R + r) * v.d : nullptr;
-  const unsigned long long bits = v.wmax[r];
-  const bool fin = w_finite(bits);
-  const double ws = fin ? pow2(-w_exp(bits, v.wbits)) : __longlong_as_double(0x7ff8000000000000ll);
-  for (int c = 2 * lane; c < v.d; c += 64) {
-    unsigned long long p[2][NW] = {};
+  const int64_t step = (int64_t)rows * N;
+  const int16_t* res = v.res + (int64_t)row * N + c;
+  int s0[NM], s1[NM];
+#pragma unroll
+  for (int i = 0; i < NM; ++i) {
+    const short2 u = *reinterpret_cast<const short2*>(res + i * v.G * step);
+    s0[i] = u.x;
+    s1[i] = u.y;
+  }
+  if (v.G > 1) {
+    for (int k = 1; k < v.G; ++k)
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        const short2 u = *reinterpret_cast<const short2*>(res + ((int64_t)i * v.G + k) * step);
+        s0[i] += u.x;
+        s1[i] += u.y;
+      }
 #pragma unroll
     for (int i = 0; i < NM; ++i) {
-      const int m = crt_mod(i);
-      const short2 t = *reinterpret_cast<const short2*>(res + (int64_t)i * v.G * rows * N + c);
-      int s0 = t.x, s1 = t.y;
-      if (v.G > 1) {
-        for (int k = 1; k < v.G; ++k) {
-          const short2 u = *reinterpret_cast<const short2*>(res + ((int64_t)i * v.G + k) * rows * N + c);
-          s0 += u.x;
-          s1 += u.y;
-        }
-        s0 %= m;
-        s1 %= m;
-      }
-      // non-negative, and zero for zero: a sum of nothing is exactly 0
-      s0 += s0 < 0 ? m : 0;
-      s1 += s1 < 0 ? m : 0;
-#pragma unroll
-      for (int w = 0; w < NW; ++w) {
-        p[0][w] += (unsigned long long)(unsigned)s0 * kc.k[i][w];
-        p[1][w] += (unsigned long long)(unsigned)s1 * kc.k[i][w];
-      }
+      s0[i] %= crt_mod(i);
+      s1[i] %= crt_mod(i);
     }
+  }
+  const unsigned rr = v.Rc == 1 ? 0u : row / (cells * (unsigned)v.nct), in = row - rr * cells * (unsigned)v.nct;
+  const int r = v.r0 + (int)rr;
+  const int lh = 31 - __clz(v.h);  // h is a power of two
+  const unsigned cz = in >> (2 * lh), cls = v.nct == 1 ? 0u : cz / (unsigned)v.nz;
+  const int64_t I = class_box(v.nct, (int)cls, (int)(in & (v.h - 1)), (int)((in >> lh) & (v.h - 1)),
+                              v.z0 + (int)(cz - cls * v.nz));
+  double* g = v.g + (I * v.R + r) * v.d + c;
+  const unsigned long long bits = v.wmax[r];
+  unsigned long long p[2][NW] = {};
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      if (c + e >= v.d) break;
+  for (int i = 0; i < NM; ++i) {
+    // non-negative, and zero for zero: a sum of nothing is exactly 0
+    const unsigned u0 = (unsigned)(s0[i] + (s0[i] < 0 ? crt_mod(i) : 0));
+    const unsigned u1 = (unsigned)(s1[i] + (s1[i] < 0 ? crt_mod(i) : 0));
 #pragma unroll
-      for (int w = 1; w < NW; ++w) p[e][w] += p[e][w - 1] >> 32;
-      // the signed top 64 bits and the words below
-      const long long hi = (long long)((p[e][NW - 1] << 32) | (p[e][NW - 2] & 0xffffffffull));
-      double G = fma((double)hi, 4294967296.0, (double)(unsigned)p[e][NW - 3]);
-      if (NW == 4) {
-        // the top words may hold little but the sign: add the last word exactly
-        // where the upper three fit a double, where they do not it is below
-        // its rounding
-        G = fma(G, 4294967296.0, (double)(unsigned)p[e][0]);
-      }
-      const double y = G * v.colscale[c + e] * ws;
-      g[c + e] = add ? add[c + e] + y : y;
+    for (int w = 0; w < NW; ++w) {
+      p[0][w] += (unsigned long long)u0 * kc.k[i][w];
+      p[1][w] += (unsigned long long)u1 * kc.k[i][w];
     }
+  }
+  const bool fin = w_finite(bits);
+  // colscale is in units of 2^(-32 NW)
+  const int e = 32 * NW - w_exp(bits, v.wbits);
+  const double* add = v.add ? v.add + (I * v.R + r) * v.d + c : nullptr;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    if (c + k >= v.d) break;
+#pragma unroll
+    for (int w = 1; w < NW; ++w) p[k][w] += p[k][w - 1] >> 32;
+    const unsigned long long H = (p[k][NW - 1] << 32) | (p[k][NW - 2] & 0xffffffffull);
+    const unsigned long long L = (p[k][NW - 3] << 32) | (NW == 4 ? p[k][0] & 0xffffffffull : 0ull);
+    double y = fin ? fixed_times(H, L, e, v.colscale[c + k]) : __longlong_as_double(0x7ff8000000000000ll);
+    g[k] = add ? add[k] + y : y;
   }
 }
 
@@ -705,14 +792,10 @@ __global__ void __launch_bounds__(256) k_crt_image(const double* __restrict__ kd
       w[j] = (mp < d && l < dl) ? __double2ll_rn(kdT[((int64_t)slot * dl + l) * d + mp] * up[mp]) : 0;
     }
     __nv_bfloat16* dst = img + ((int64_t)slot * NT + nt) * tile_e + ((int64_t)k8 * Nt + n) * 8;
+    Limbs q[4];
 #pragma unroll
-    for (int i = 0; i < kMods; ++i) {
-      __nv_bfloat162 o[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        o[j] = __floats2bfloat162_rn((float)residue(w[2 * j], i), (float)residue(w[2 * j + 1], i));
-      *reinterpret_cast<uint4*>(dst + (int64_t)i * nslots * NT * tile_e) = *reinterpret_cast<uint4*>(o);
-    }
+    for (int j = 0; j < 4; ++j) q[j] = limbs_of(w[2 * j], w[2 * j + 1]);
+    store_residues<0, kMods>(q, dst, (int64_t)nslots * NT * tile_e);
   }
 }
 
@@ -907,9 +990,11 @@ size_t res_bytes(CrtMode m, int N, int h, int nz, int Rc, int G) {
   return align256((size_t)mode_mods(m) * G * Rc * mode_nct(m) * nz * h * h * N * 2);
 }
 constexpr int kMaxGroups = 8;
-// offset groups are used only by M2L launches of few tiles: levels below this one
+// offset groups are used only by M2L and M2M launches of few tiles: levels below this one
 constexpr int kGroupLevel = 4;
-int max_groups(CrtMode m, int level) { return m == kCrtM2L && level < kGroupLevel ? kMaxGroups : 1; }
+int max_groups(CrtMode m, int level) {
+  return (m == kCrtM2L || m == kCrtM2M) && level < kGroupLevel ? kMaxGroups : 1;
+}
 size_t job_bytes(CrtMode m, const CrtImage& im, int level, int nz, int Rc) {
   const int h = mode_h(m, level);
   const int snz = std::min(h, nz + 2);
@@ -1131,9 +1216,12 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     for (int q = 0; q < a.nlev; ++q) {
       CrtLv& v = a.lv[q];
       // a launch of few tiles: the windows of the coarse levels' tiles are
-      // split into groups until the CTAs cover four waves
+      // split into groups until the CTAs cover four waves (M2L), or as long as
+      // they stay within one (M2M, whose CTAs have 8 short windows: 14 CTAs 29
+      // us, 112 CTAs 14 us; but 98 CTAs 31 us, 784 CTAs 51 us)
       v.G = 1;
-      while (v.G < max_groups(v.mode, v.tlevel) && items * v.G < 4 * (int64_t)nsm) v.G *= 2;
+      const int64_t most = (v.mode == kCrtM2M ? nsm : 8 * (int64_t)nsm - 1) / 2;
+      while (v.G < max_groups(v.mode, v.tlevel) && items * v.G <= most) v.G *= 2;
       v.planes = (__nv_bfloat16*)((char*)buf + off);
       off += planes_bytes(v.mode, v.K, v.h, v.snz, v.Rc);
       v.res = (int16_t*)((char*)buf + off);
@@ -1144,8 +1232,10 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
       v.mx0 = mx;
       it += (unsigned)(tiles(v) * v.G);
       pl += (unsigned)((int64_t)((v.h + 7) / 8) * v.h * v.snz * v.ncs * v.Rc);
-      rb += (unsigned)(((int64_t)v.nz * v.h * v.h * v.nct * v.Rc + 3) / 4);
-      mx += (unsigned)((((int64_t)1 << (3 * v.slevel)) * v.ds + kMaxPer - 1) / kMaxPer * v.Rc);
+      const unsigned pairs = (unsigned)(v.d + 1) / 2;
+      v.pinv = (unsigned)((0xffffffffull + pairs) / pairs);
+      rb += (unsigned)(((int64_t)v.nz * v.h * v.h * v.nct * v.Rc * pairs + kRebuild - 1) / kRebuild);
+      mx += (unsigned)((((int64_t)1 << (3 * v.slevel)) + kMaxBoxes - 1) / kMaxBoxes * v.Rc);
       const uint32_t ks = (uint32_t)std::max(v.ks0, v.nchunk > v.n0 ? v.ks1 : 0);
       stage = std::max(stage, ks * 32u * (uint32_t)v.Nt);
       win = std::max(win, ks * kWinStep);
@@ -1177,8 +1267,8 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     EIFMM_CHECK_LAUNCH();
     k_crt_gemm<<<it, kThreads, smem, s>>>(maps, a);
     EIFMM_CHECK_LAUNCH();
-    if (box) k_crt_rebuild<kBoxMods, 4><<<rb, 128, 0, s>>>(a, kcb);
-    else k_crt_rebuild<kMods, 3><<<rb, 128, 0, s>>>(a, kc);
+    if (box) k_crt_rebuild<kBoxMods, 4><<<rb, kRebuild, 0, s>>>(a, kcb);
+    else k_crt_rebuild<kMods, 3><<<rb, kRebuild, 0, s>>>(a, kc);
     EIFMM_CHECK_LAUNCH();
     i0 = i1;
   }
