@@ -20,9 +20,9 @@ def E():
     return eifmm
 
 
-def reference(x, depth):
+def reference(x, depth, lo=(0.0, 0.0, 0.0), L=1.0):
     side = 1 << depth
-    c = np.clip((x * side).astype(np.int64), 0, side - 1)
+    c = np.clip(((x - np.array(lo)) * (side / L)).astype(np.int64), 0, side - 1)
     key = np.zeros(len(x), dtype=np.int64)
     for b in range(depth):
         for a in range(3):
@@ -60,3 +60,22 @@ def test_sort_of_four_passes(E):
     perm = np.argsort(key, kind="stable")
     np.testing.assert_array_equal(ps, perm)
     np.testing.assert_array_equal(ks.view(np.uint32), key[perm])
+
+
+@pytest.mark.parametrize("lo,L", [((0.0, 0.0, 0.0), 0.75), ((-0.5, -0.0, 2.0), 4.0), ((-0.3, 10.7, 0.001), 3.7),
+                                  ((0.0, 0.0, 0.0), 2.0 ** -700), ((-1.0, -2.0, -3.0), 2.0 ** 20 / 3)])
+def test_keys_of_general_cubes(E, lo, L):
+    depth, n = 6, 5000
+    x = np.array(lo) + L * wl.uniform_cube(n, 9)
+    x[:4] = [lo, [a + L for a in lo], [lo[0] + L / 2, lo[1], lo[2] + L / 64], [-0.0 if a == 0 else a for a in lo]]
+    x = np.clip(x, np.array(lo), np.array(lo) + L)
+    keys, perm, off = reference(x, depth, lo, L)
+    ks, ps, os_ = (a.cpu().numpy() for a in E.eifmm_tree_sort_static(torch.from_numpy(x).cuda(), lo, L, depth))
+    np.testing.assert_array_equal(ks.view(np.uint32), keys)
+    np.testing.assert_array_equal(ps, perm)
+    np.testing.assert_array_equal(os_, off)
+    for bad in (np.nan, -np.nan, np.inf, -np.inf, np.nextafter(lo[1], -np.inf), np.nextafter(lo[1] + L, np.inf)):
+        y = x.copy()
+        y[77, 1] = bad
+        with pytest.raises(E.EifmmError, match="outside"):
+            E.eifmm_tree_sort_static(torch.from_numpy(y).cuda(), lo, L, depth)
