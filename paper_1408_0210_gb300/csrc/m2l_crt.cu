@@ -80,6 +80,7 @@ constexpr int kWins = 2;
 constexpr int kMaxStages = 8;
 constexpr int kDrainWarps = 8;
 constexpr int kThreads = 32 * (kDrainWarps + 3);
+constexpr int kAccCols = 256;  // TMEM columns of an accumulator
 constexpr uint32_t kSmemMax = 227u * 1024u;
 constexpr uint32_t kSmemBars = 512;
 
@@ -95,6 +96,7 @@ struct CrtLv {
   int z0, nz, sz0, snz;      // planes of target boxes, planes of source boxes held
   int r0, Rc, R, G;          // columns r0 .. r0 + Rc of R, offset groups
   int nchunk, n0, ks0, ks1;  // chunks of K: n0 of ks0 k-steps, then ks1 k-steps each
+  uint16_t ng[8][8];         // accumulations of a tile of class [ct], group [grp]
   unsigned pinv;             // 2^32 over the pairs of coefficients of a row, rounded up
   unsigned item0, pl0, rc0, mx0;  // first block of this level in each of the launches
   const double* W;
@@ -109,6 +111,7 @@ struct CrtLv {
 constexpr int kMaxLv = kMaxLevel - 1;
 struct CrtArgs {
   int nlev, stages;
+  unsigned items;
   uint32_t stage_b, win_b;
   int* err;
   CrtLv lv[kMaxLv];
@@ -141,15 +144,15 @@ void split_chunks(CrtLv* v) {
   v->n0 = a;
   v->nchunk = a + (n - 5 * a) / 3;
 }
-__device__ __forceinline__ int chunk_ksteps(const CrtLv& v, int c) { return c < v.n0 ? v.ks0 : v.ks1; }
+__host__ __device__ __forceinline__ int chunk_ksteps(const CrtLv& v, int c) { return c < v.n0 ? v.ks0 : v.ks1; }
 
 // bits of shifts s + 1 in {0, 1, 2} along one axis whose child offset
 // 2 s + cs - ct is at most one box (the near field)
-__device__ __forceinline__ int near_bits(int cs, int ct) { return cs == ct ? 2 : (cs > ct ? 3 : 6); }
+__host__ __device__ __forceinline__ int near_bits(int cs, int ct) { return cs == ct ? 2 : (cs > ct ? 3 : 6); }
 
 // The (sz, sx) shifts of class cs and y-shift sy + 1 that belong to the
 // interaction list of class ct: bit 3 (sz + 1) + sx + 1.
-__device__ __forceinline__ int combo_mask(int ct, int cs, int sy1) {
+__host__ __device__ __forceinline__ int combo_mask(int ct, int cs, int sy1) {
   if (!((near_bits((cs >> 1) & 1, (ct >> 1) & 1) >> sy1) & 1)) return 0x1ff;
   const int nx = near_bits(cs & 1, ct & 1), nz = near_bits((cs >> 2) & 1, (ct >> 2) & 1);
   const int m = ((nz & 1) ? nx : 0) | ((nz & 2) ? nx << 3 : 0) | ((nz & 4) ? nx << 6 : 0);
@@ -161,11 +164,16 @@ __device__ __forceinline__ int combo_mask(int ct, int cs, int sy1) {
 struct Win {
   int cs, sy1, mask, slot;
 };
-__device__ __forceinline__ Win window_of(const CrtLv& v, int ct, int w) {
+__host__ __device__ __forceinline__ Win window_of(const CrtLv& v, int ct, int w) {
   Win o;
   if (v.mode == kCrtM2L) {
-    o.cs = w / 3;
-    o.sy1 = w - 3 * o.cs;
+    // by the parity of the offset: the CTAs of all target classes read (nearly)
+    // the same operators at the same time
+    o.cs = ct ^ (w / 3);
+    o.sy1 = w % 3;
+    o.mask = combo_mask(ct, o.cs, o.sy1);
+    o.slot = (2 * (o.sy1 - 1) + ((o.cs >> 1) & 1) - ((ct >> 1) & 1) + 3) * 7 + (o.cs & 1) - (ct & 1) + 3 +
+             ((o.cs >> 2) - (ct >> 2) + 3) * 49;
   } else {  // no shift: the 8 children of a box (M2M), its parent (L2L), itself (box)
     o.cs = v.mode == kCrtM2M ? w : (v.mode == kCrtL2L ? 0 : ct);
     o.slot = v.mode == kCrtM2M ? w : (v.mode == kCrtL2L ? ct : 0);
@@ -173,6 +181,19 @@ __device__ __forceinline__ Win window_of(const CrtLv& v, int ct, int w) {
     o.mask = 0x10;
   }
   return o;
+}
+
+// Accumulations of kMaxSteps k-steps at most that the windows of a tile fill.
+int accumulations(const CrtLv& v, int ct, int grp) {
+  int n = 1, acc = 0;
+  for (int w = grp * v.nw / v.G; w < (grp + 1) * v.nw / v.G; ++w)
+    for (int c = 0; c < v.nchunk; ++c)
+      for (int m = window_of(v, ct, w).mask; m; m &= m - 1) {
+        const int ks = chunk_ksteps(v, c);
+        if (acc + ks > kMaxSteps) ++n, acc = 0;
+        acc += ks;
+      }
+  return n;
 }
 
 // Morton key of box (x, y, z) of class c of nc
@@ -353,8 +374,39 @@ __device__ __forceinline__ void mma_steps(uint32_t dst, uint32_t alo, uint32_t a
     mma_f16_el(dst, alo + kk * (kWinStep >> 4), ahi, blo + kk * n2, bhi, id, kk ? 1u : acc, el);
 }
 
-// One CTA: one modulus, one target tile (128 boxes of a class), one column
-// tile, one right-hand side, one group of (source class, y-shift) windows.
+struct Item {
+  int q, x0, y0, z0, ct, nt, r, grp, mod, w_beg, w_end;
+};
+__device__ __forceinline__ Item item_of(const CrtArgs& a, unsigned i) {
+  Item o;
+  o.q = find_level(a, &CrtLv::item0, i);
+  const CrtLv& v = a.lv[o.q];
+  unsigned b = i - v.item0;
+  auto digit = [&](int n) {
+    const unsigned q = b / (unsigned)n, r = b - q * (unsigned)n;
+    b = q;
+    return (int)r;
+  };
+  o.x0 = kTX * digit((v.h + kTX - 1) / kTX);
+  o.y0 = kTY * digit((v.h + kTY - 1) / kTY);
+  o.z0 = v.z0 + kTZ * digit((v.nz + kTZ - 1) / kTZ);
+  o.ct = digit(v.nct);
+  o.nt = digit(v.NT);
+  o.r = digit(v.Rc);
+  o.grp = digit(v.G);
+  o.mod = (int)b;
+  o.w_beg = o.grp * v.nw / v.G;
+  o.w_end = (o.grp + 1) * v.nw / v.G;
+  return o;
+}
+
+// One item: one modulus, one target tile (128 boxes of a class), one column
+// tile, one right-hand side, one group of (source class, y-shift) windows.  A
+// CTA per SM takes every gridDim-th; each role runs on into the next item, so
+// that its operands load and its first sums form while the last one's are
+// reduced and written.  2^20 points, d = 193, against a CTA per item: M2L 5.81 ->
+// 5.70 ms, L2L 0.39 -> 0.33, Delta^t 0.45 -> 0.36; d = 126: 3.80 -> 3.87, 0.32 -> 0.27,
+// 0.34 -> 0.28; 512 leaves, d = 193: M2L 0.40 -> 0.36.
 // Warps 0-7 drain the accumulators, warp 8 streams the operator residues
 // (K-chunk of one offset per stage), warp 9 issues the MMAs, warp 10 loads the
 // windows.  M = 128 boxes, N = Nt columns m', K in chunks of at most 64 terms.
@@ -379,26 +431,6 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
   auto aempty = [&](int i) { return smem_u32(&bars[2 * kMaxStages + 6 + i]); };
   uint32_t* tslot = (uint32_t*)(bars + 2 * kMaxStages + 8);
   volatile int* abort = (volatile int*)(tslot + 1);
-
-  const int q = find_level(a, &CrtLv::item0, blockIdx.x);
-  const CrtLv& v = a.lv[q];
-  const int h = v.h, K = v.K, Nt = v.Nt, nchunk = v.nchunk;
-  unsigned b = blockIdx.x - v.item0;
-  const int ntx = (h + kTX - 1) / kTX, nty = (h + kTY - 1) / kTY, ntz = (v.nz + kTZ - 1) / kTZ;
-  const int x0 = kTX * (int)(b % ntx);
-  b /= ntx;
-  const int y0 = kTY * (int)(b % nty);
-  b /= nty;
-  const int z0 = v.z0 + kTZ * (int)(b % ntz);
-  b /= ntz;
-  const int ct = (int)(b % v.nct);
-  b /= v.nct;
-  const int nt = (int)(b % v.NT);
-  b /= v.NT;
-  const int r = (int)(b % v.Rc);
-  b /= v.Rc;
-  const int grp = (int)(b % v.G), mod = (int)(b / v.G);
-  const int w_beg = grp * v.nw / v.G, w_end = (grp + 1) * v.nw / v.G;
 
   if (tid == 0) {
     for (int i = 0; i < kMaxStages; ++i) {
@@ -427,35 +459,39 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
   if (wu == 8) {
     // ----------------------------------------- operator residues (B) --
     const uint32_t el = elect_one();
-    const int64_t tile_b = (int64_t)K * Nt * 2, slot_b = v.NT * tile_b;  // bytes of a column tile, of a slot
-    const char* img = (const char*)v.img + (int64_t)mod * v.nslots * slot_b + nt * tile_b;
-    const int n0 = v.n0, ks0 = v.ks0, ks1 = v.ks1;
     const uint32_t stage_b = a.stage_b;
     int it = 0, st = 0;
     uint32_t ph = 0, dst = s_stage;
     bool ok = true;
-    for (int w = w_beg; w < w_end && ok; ++w) {
-      const Win wn = window_of(v, ct, w);
-      const int mask = wn.mask;
-      const char* src = img + wn.slot * slot_b;
-      for (int c = 0; c < nchunk && ok; ++c) {
-        const uint32_t bytes = (uint32_t)(c < n0 ? ks0 : ks1) * 32u * Nt;
+    for (unsigned i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
+      const Item t = item_of(a, i);
+      const CrtLv& v = a.lv[t.q];
+      const int64_t tile_b = (int64_t)v.K * v.Nt * 2, slot_b = v.NT * tile_b;  // bytes of a column tile, of a slot
+      const char* img = (const char*)v.img + (int64_t)t.mod * v.nslots * slot_b + t.nt * tile_b;
+      const int n0 = v.n0, ks0 = v.ks0, ks1 = v.ks1, nchunk = v.nchunk;
+      for (int w = t.w_beg; w < t.w_end && ok; ++w) {
+        const Win wn = window_of(v, t.ct, w);
+        const int mask = wn.mask;
+        const char* src = img + wn.slot * slot_b;
+        for (int c = 0; c < nchunk && ok; ++c) {
+          const uint32_t bytes = (uint32_t)(c < n0 ? ks0 : ks1) * 32u * (uint32_t)v.Nt;
 #pragma unroll
-        for (int m = 0; m < 9; ++m)
-          if (((mask >> m) & 1) && ok) {
-            if (it >= S) ok = mbar_wait_ab(bempty(st), ph ^ 1u, a.err, 11, abort);
-            if (ok) {
-              if (el) {
-                mbar_expect_tx(bfull(st), bytes);
-                bulk_g2s(dst, src + (2 * (m % 3 - 1) + 98 * (m / 3 - 1)) * slot_b, bytes, bfull(st));
+          for (int m = 0; m < 9; ++m)
+            if (((mask >> m) & 1) && ok) {
+              if (it >= S) ok = mbar_wait_ab(bempty(st), ph ^ 1u, a.err, 11, abort);
+              if (ok) {
+                if (el) {
+                  mbar_expect_tx(bfull(st), bytes);
+                  bulk_g2s(dst, src + (2 * (m % 3 - 1) + 98 * (m / 3 - 1)) * slot_b, bytes, bfull(st));
+                }
+                __syncwarp();
+                ++it;
+                dst += stage_b;
+                if (++st == S) st = 0, ph ^= 1u, dst = s_stage;
               }
-              __syncwarp();
-              ++it;
-              dst += stage_b;
-              if (++st == S) st = 0, ph ^= 1u, dst = s_stage;
             }
-          }
-        src += bytes;
+          src += bytes;
+        }
       }
     }
     drain_fills(it, S, bars, a.err);
@@ -464,39 +500,49 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     const uint32_t el = elect_one();
     int wi = 0;
     bool ok = true;
-    for (int w = w_beg; w < w_end && ok; ++w) {
-      const Win wn = window_of(v, ct, w);
-      int k0 = 0;
-      for (int c = 0; c < nchunk; ++c, ++wi) {
-        const int ks = chunk_ksteps(v, c);
-        const int s = wi & 1;
-        if (wi >= kWins && !mbar_wait_ab(wempty(s), ((wi >> 1) - 1) & 1, a.err, 12, abort)) {
-          ok = false;
-          break;
+    for (unsigned i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
+      const Item t = item_of(a, i);
+      const CrtLv& v = a.lv[t.q];
+      for (int w = t.w_beg; w < t.w_end && ok; ++w) {
+        const Win wn = window_of(v, t.ct, w);
+        int k0 = 0;
+        for (int c = 0; c < v.nchunk; ++c, ++wi) {
+          const int ks = chunk_ksteps(v, c);
+          const int s = wi & 1;
+          if (wi >= kWins && !mbar_wait_ab(wempty(s), ((wi >> 1) - 1) & 1, a.err, 12, abort)) {
+            ok = false;
+            break;
+          }
+          if (el) {
+            mbar_expect_tx(wfull(s), (uint32_t)ks * kWinStep);
+            for (int kk = 0; kk < ks; ++kk)
+              tma_load_5d(sbase + (uint32_t)s * a.win_b + (uint32_t)kk * kWinStep, &maps.m[t.q], 8 * (t.x0 - 1),
+                          t.y0 + wn.sy1 - 1, t.z0 - 1 - v.sz0, 2 * (k0 + kk), (t.mod * v.Rc + t.r) * v.ncs + wn.cs,
+                          wfull(s));
+          }
+          __syncwarp();
+          k0 += ks;
         }
-        if (el) {
-          mbar_expect_tx(wfull(s), (uint32_t)ks * kWinStep);
-          for (int kk = 0; kk < ks; ++kk)
-            tma_load_5d(sbase + (uint32_t)s * a.win_b + (uint32_t)kk * kWinStep, &maps.m[q], 8 * (x0 - 1),
-                        y0 + wn.sy1 - 1, z0 - 1 - v.sz0, 2 * (k0 + kk), (mod * v.Rc + r) * v.ncs + wn.cs, wfull(s));
-        }
-        __syncwarp();
-        k0 += ks;
       }
     }
     drain_fills(wi, kWins, bars + 2 * kMaxStages, a.err);
   } else if (wu == 9) {
     // ----------------------------------------------------- MMA issuer --
     const uint32_t el = elect_one();
-    const uint32_t id = idesc_bf16((uint32_t)Nt);
     const uint64_t dA = desc_k(sbase, kWinRows * 16u, (kTX + 2) * 16u);
-    const uint64_t dB = desc_k(s_stage, (uint32_t)Nt * 16u, 128u);
-    const uint32_t ahi = (uint32_t)(dA >> 32), bhi = (uint32_t)(dB >> 32), n2 = 2u * (uint32_t)Nt;
-    const uint32_t stage16 = a.stage_b >> 4, win16 = a.win_b >> 4;
-    const int n0 = v.n0, ks0 = v.ks0, ks1 = v.ks1;
+    const uint32_t ahi = (uint32_t)(dA >> 32), stage16 = a.stage_b >> 4, win16 = a.win_b >> 4;
     int st = 0, wi = 0, g = 0, acc = 0;
-    uint32_t ph = 0, blo = (uint32_t)dB, dst = tmem;
+    uint32_t ph = 0, dst = tmem, id = 0, n2 = 0, bhi = 0;
+    const uint32_t blo0 = (uint32_t)desc_k(s_stage, 0u, 128u);
+    uint32_t blo = blo0;  // with the item's LBO in the upper half
+    uint32_t lbo = 0;
     bool ok = true;
+    // accumulator g, when the sums of g - 2 have been taken from it
+    auto open_acc = [&]() {
+      acc = 0;
+      dst = tmem + (uint32_t)((g & 1) * kAccCols);
+      if (g >= 2) ok = ok && mbar_wait_ab(aempty(g & 1), ((g >> 1) - 1) & 1, a.err, 14, abort);
+    };
     // the steps of one window whose chunk has KS k-steps, unrolled over its
     // nine shifts: the start address of each is a constant offset
     auto window = [&](auto ksc, int mask, uint32_t awin) {
@@ -507,104 +553,108 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
           if (acc + KS > kMaxSteps) {  // this accumulator is full
             mma_commit_el(afull(g & 1), el);
             ++g;
-            acc = 0;
-            dst = tmem + (uint32_t)((g & 1) * Nt);
-            if (g >= 2) ok = ok && mbar_wait_ab(aempty(g & 1), ((g >> 1) - 1) & 1, a.err, 14, abort);
+            open_acc();
           }
           ok = ok && mbar_wait_ab(bfull(st), ph, a.err, 15, abort);
           if (!ok) return;
           tc_fence_after();
-          mma_steps<KS>(dst, awin + (uint32_t)((m / 3) * (kTX + 2) * kTY + m % 3), ahi, blo, bhi, n2, id,
+          mma_steps<KS>(dst, awin + (uint32_t)((m / 3) * (kTX + 2) * kTY + m % 3), ahi, blo | lbo, bhi, n2, id,
                         acc > 0 ? 1u : 0u, el);
           acc += KS;
           mma_commit_el(bempty(st), el);
           blo += stage16;
-          if (++st == S) st = 0, ph ^= 1u, blo = (uint32_t)dB;
+          if (++st == S) st = 0, ph ^= 1u, blo = blo0;
         }
     };
-    for (int w = w_beg; w < w_end && ok; ++w) {
-      const int mask = window_of(v, ct, w).mask;
-      for (int c = 0; c < nchunk && ok; ++c, ++wi) {
-        const int ks = c < n0 ? ks0 : ks1;
-        const int s = wi & 1;
-        ok = mbar_wait_ab(wfull(s), (wi >> 1) & 1, a.err, 13, abort);
-        if (!ok) break;
-        const uint32_t awin = (uint32_t)dA + (s ? win16 : 0u);
-        if (ks == 5) window(std::integral_constant<int, 5>(), mask, awin);
-        else if (ks == 4) window(std::integral_constant<int, 4>(), mask, awin);
-        else if (ks == 3) window(std::integral_constant<int, 3>(), mask, awin);
-        else if (ks == 2) window(std::integral_constant<int, 2>(), mask, awin);
-        else window(std::integral_constant<int, 1>(), mask, awin);
-        if (ok) mma_commit_el(wempty(s), el);
+    for (unsigned i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
+      const Item t = item_of(a, i);
+      const CrtLv& v = a.lv[t.q];
+      const int n0 = v.n0, ks0 = v.ks0, ks1 = v.ks1, nchunk = v.nchunk;
+      const uint64_t dB = desc_k(0, (uint32_t)v.Nt * 16u, 128u);
+      lbo = (uint32_t)dB;
+      bhi = (uint32_t)(dB >> 32);
+      n2 = 2u * (uint32_t)v.Nt;
+      id = idesc_bf16((uint32_t)v.Nt);
+      open_acc();
+      for (int w = t.w_beg; w < t.w_end && ok; ++w) {
+        const int mask = window_of(v, t.ct, w).mask;
+        for (int c = 0; c < nchunk && ok; ++c, ++wi) {
+          const int ks = c < n0 ? ks0 : ks1;
+          const int s = wi & 1;
+          ok = mbar_wait_ab(wfull(s), (wi >> 1) & 1, a.err, 13, abort);
+          if (!ok) break;
+          const uint32_t awin = (uint32_t)dA + (s ? win16 : 0u);
+          if (ks == 5) window(std::integral_constant<int, 5>(), mask, awin);
+          else if (ks == 4) window(std::integral_constant<int, 4>(), mask, awin);
+          else if (ks == 3) window(std::integral_constant<int, 3>(), mask, awin);
+          else if (ks == 2) window(std::integral_constant<int, 2>(), mask, awin);
+          else window(std::integral_constant<int, 1>(), mask, awin);
+          if (ok) mma_commit_el(wempty(s), el);
+        }
       }
+      if (ok) mma_commit_el(afull(g & 1), el);
+      ++g;
     }
-    if (ok) mma_commit_el(afull(g & 1), el);
   } else if (warp < kDrainWarps) {
     // -------------------------------------------------- residue sums --
     // warp w reads TMEM lanes 32 (w % 4) .. and half w / 4 of the columns
-    int ng = 1;
-    {
-      int acc = 0;
-      for (int w = w_beg; w < w_end; ++w) {
-        const int n = __popc(window_of(v, ct, w).mask);
-        for (int c = 0; c < nchunk; ++c) {
-          const int ks = chunk_ksteps(v, c);
-          for (int i = 0; i < n; ++i) {
-            if (acc + ks > kMaxSteps) ++ng, acc = 0;
-            acc += ks;
-          }
-        }
-      }
-    }
-    const int quad = warp & 3, half = warp >> 2, nh = Nt / 2;
-    const float fm = (float)crt_mod(mod);
-    const float2 inv2 = make_float2(1.0f / fm, 1.0f / fm), m2 = make_float2(-fm, -fm);
+    const int quad = warp & 3, half = warp >> 2;
     const float2 mg = make_float2(12582912.0f, 12582912.0f), ng2 = make_float2(-12582912.0f, -12582912.0f);
-    float2 sum[64];
+    int g = 0;
+    bool have = true;
+    for (unsigned it = blockIdx.x; it < a.items && have; it += gridDim.x) {
+      const Item t = item_of(a, it);
+      const CrtLv& v = a.lv[t.q];
+      const int Nt = v.Nt, nh = Nt / 2;
+      const float fm = (float)crt_mod(t.mod);
+      const float2 inv2 = make_float2(1.0f / fm, 1.0f / fm), m2 = make_float2(-fm, -fm);
+      float2 sum[64];
 #pragma unroll
-    for (int j = 0; j < 64; ++j) sum[j] = make_float2(0.f, 0.f);
-    for (int g = 0; g < ng; ++g) {
-      bool have = mbar_wait_ab(afull(g & 1), (g >> 1) & 1, a.err, 16, abort);
-      have = __all_sync(0xffffffffu, have);
-      if (!have) break;
-      tc_fence_after();
-      const uint32_t t0 = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)((g & 1) * Nt + half * nh);
+      for (int j = 0; j < 64; ++j) sum[j] = make_float2(0.f, 0.f);
+      for (int n = v.ng[t.ct][t.grp]; n > 0; --n, ++g) {
+        have = mbar_wait_ab(afull(g & 1), (g >> 1) & 1, a.err, 16, abort);
+        have = __all_sync(0xffffffffu, have);
+        if (!have) break;
+        tc_fence_after();
+        const uint32_t t0 = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)((g & 1) * kAccCols + half * nh);
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (16 * j < nh) {
-          float x[16];
-          tmem_ld16(t0 + 16u * j, x);
-          // |x| <= 240 2^16 and |sum| < 2^9: x + sum is an exact integer
-          // below 2^24; minus the nearest multiple of m (1.5 2^23 rounds to
-          // the nearest integer), again exact
+        for (int j = 0; j < 8; ++j)
+          if (16 * j < nh) {
+            float x[16];
+            tmem_ld16(t0 + 16u * j, x);
+            // |x| <= 240 2^16 and |sum| < 2^9: x + sum is an exact integer
+            // below 2^24; minus the nearest multiple of m (1.5 2^23 rounds to
+            // the nearest integer), again exact
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float2 u = __fadd2_rn(make_float2(x[2 * i], x[2 * i + 1]), sum[8 * j + i]);
-            const float2 k = __fadd2_rn(__ffma2_rn(u, inv2, mg), ng2);
-            sum[8 * j + i] = __ffma2_rn(k, m2, u);
+            for (int i = 0; i < 8; ++i) {
+              const float2 u = __fadd2_rn(make_float2(x[2 * i], x[2 * i + 1]), sum[8 * j + i]);
+              const float2 k = __fadd2_rn(__ffma2_rn(u, inv2, mg), ng2);
+              sum[8 * j + i] = __ffma2_rn(k, m2, u);
+            }
           }
-        }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(aempty(g & 1)) : "memory");
-    }
-    // row = (z, y, x) of the tile: TMEM lane 32 quad + lane
-    const int row = 32 * quad + lane;
-    const int x = x0 + (row & 7), y = y0 + ((row >> 3) & 3), z = z0 + (row >> 5);
-    if (x < h && y < h && z < v.z0 + v.nz) {
-      const int N = v.NT * Nt;
-      int16_t* out = v.res +
-                     ((((((int64_t)mod * v.G + grp) * v.Rc + r) * v.nct + ct) * v.nz + (z - v.z0)) * h + y) * (int64_t)h * N +
-                     (int64_t)x * N + nt * Nt + half * nh;
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(aempty(g & 1)) : "memory");
+      }
+      // row = (z, y, x) of the tile: TMEM lane 32 quad + lane
+      const int row = 32 * quad + lane, h = v.h;
+      const int x = t.x0 + (row & 7), y = t.y0 + ((row >> 3) & 3), z = t.z0 + (row >> 5);
+      if (have && x < h && y < h && z < v.z0 + v.nz) {
+        const int N = v.NT * Nt;
+        int16_t* out = v.res +
+                       ((((((int64_t)t.mod * v.G + t.grp) * v.Rc + t.r) * v.nct + t.ct) * v.nz + (z - v.z0)) * h + y) *
+                           (int64_t)h * N +
+                       (int64_t)x * N + t.nt * Nt + half * nh;
 #pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (8 * j < nh) {
-          uint32_t p[4];
+        for (int j = 0; j < 16; ++j)
+          if (8 * j < nh) {
+            uint32_t p[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            p[i] = ((uint32_t)(int)sum[4 * j + i].x & 0xffffu) | ((uint32_t)(int)sum[4 * j + i].y << 16);
-          *reinterpret_cast<uint4*>(out + 8 * j) = make_uint4(p[0], p[1], p[2], p[3]);
-        }
+            for (int i = 0; i < 4; ++i)
+              p[i] = ((uint32_t)(int)sum[4 * j + i].x & 0xffffu) | ((uint32_t)(int)sum[4 * j + i].y << 16);
+            *reinterpret_cast<uint4*>(out + 8 * j) = make_uint4(p[0], p[1], p[2], p[3]);
+          }
+      }
     }
   }
   tc_fence_before();
@@ -1222,6 +1272,8 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
       v.G = 1;
       const int64_t most = (v.mode == kCrtM2M ? nsm : 8 * (int64_t)nsm - 1) / 2;
       while (v.G < max_groups(v.mode, v.tlevel) && items * v.G <= most) v.G *= 2;
+      for (int ct = 0; ct < v.nct; ++ct)
+        for (int p = 0; p < v.G; ++p) v.ng[ct][p] = (uint16_t)accumulations(v, ct, p);
       v.planes = (__nv_bfloat16*)((char*)buf + off);
       off += planes_bytes(v.mode, v.K, v.h, v.snz, v.Rc);
       v.res = (int16_t*)((char*)buf + off);
@@ -1265,7 +1317,8 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     if (box) k_crt_planes<kBoxMods><<<pl, 256, pl_smem, s>>>(a);
     else k_crt_planes<kMods><<<pl, 256, pl_smem, s>>>(a);
     EIFMM_CHECK_LAUNCH();
-    k_crt_gemm<<<it, kThreads, smem, s>>>(maps, a);
+    a.items = it;
+    k_crt_gemm<<<std::min(it, (unsigned)nsm), kThreads, smem, s>>>(maps, a);
     EIFMM_CHECK_LAUNCH();
     if (box) k_crt_rebuild<kBoxMods, 4><<<rb, kRebuild, 0, s>>>(a, kcb);
     else k_crt_rebuild<kMods, 3><<<rb, kRebuild, 0, s>>>(a, kc);
