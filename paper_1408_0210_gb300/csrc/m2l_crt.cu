@@ -25,12 +25,12 @@
 //
 // Four launches cover all levels: largest |W| per level and column; the
 // residue planes of W; the residue GEMMs; the reconstruction.  At 2^20 points,
-// depth 5: eps 1e-6 (d = 193) 0.04 + 0.11 + 5.7 + 0.28 ms, where the FP32 pairs
-// took 144 ms; eps 1e-4 (d = 126) 3.9 ms, where the FP64 pipes took 195 ms; eps
-// 1e-7 (d = 256) 7.5 ms (202 ms in FP32 pairs).  The GEMM issues 14 / 1 of the
-// method's products, 13% of them zero (189 offsets for 165 pairs per box) and
-// is bound by the stream of operator residues: 86 KB per offset and 128 boxes,
-// 64 bytes per cycle and SM at the tensor cores' full rate.
+// depth 5: eps 1e-6 (d = 193) 4.9 + 0.2 ms, where the FP32 pairs took 144 ms; eps
+// 1e-4 (d = 126) 3.3 ms, where the FP64 pipes took 195 ms; eps 1e-7 (d = 256)
+// 8.0 ms (202 ms in FP32 pairs).  The GEMM issues 14 times the method's products,
+// 13% of them zero (189 offsets for 165 pairs per box), and at d = 193 runs at the rate
+// that a library BF16 product sustains (1.74 PFLOP/s); at d = 126, where an MMA is
+// shorter, what the issuing warp does between two steps takes a third.
 //
 // M2M, L2L and Delta^t are the same sums over the 8 children, the parent and the
 // box itself, without shifts.  Delta^t is formed explicitly in double-double
@@ -38,8 +38,8 @@
 // the product cancels by as much.  K(x, X) Delta^t l then errs by 1.6e-16 to 9e-16
 // (1/r, eps 1e-4 to 1e-7) where the FP64 triangular solves err by 2.3e-16 to 2.7e-15
 // (config-3 at 1e-6: 1.4e-12 and 7.2e-12).  At 2^20 points, depth 5, d = 193, on
-// the FP64 pipes before: M2M 3.0 -> 0.44 ms, L2L 5.1 -> 0.61 ms, Delta^t 3.5 -> 0.70
-// ms; 512 leaves: Delta^t 1.73 -> 0.075 ms.  They are bound by their passes over
+// the FP64 pipes before: M2M 3.0 -> 0.27 ms, L2L 5.1 -> 0.33 ms, Delta^t 3.5 -> 0.36
+// ms; 512 leaves: Delta^t 1.73 -> 0.037 ms.  They are bound by their passes over
 // the residues (28 bytes an entry) and, for small levels, by their launches.
 #include <algorithm>
 #include <cmath>
@@ -405,7 +405,7 @@ __device__ __forceinline__ Item item_of(const CrtArgs& a, unsigned i) {
 // CTA per SM takes every gridDim-th; each role runs on into the next item, so
 // that its operands load and its first sums form while the last one's are
 // reduced and written.  2^20 points, d = 193, against a CTA per item: M2L 5.81 ->
-// 5.70 ms, L2L 0.39 -> 0.33, Delta^t 0.45 -> 0.36; d = 126: 3.80 -> 3.87, 0.32 -> 0.27,
+// 5.70 ms (5.13 with the uniform waits), L2L 0.39 -> 0.33, Delta^t 0.45 -> 0.36; d = 126: 3.80 -> 3.87 (3.30), 0.32 -> 0.27,
 // 0.34 -> 0.28; 512 leaves, d = 193: M2L 0.40 -> 0.36.
 // Warps 0-7 drain the accumulators, warp 8 streams the operator residues
 // (K-chunk of one offset per stage), warp 9 issues the MMAs, warp 10 loads the
@@ -417,19 +417,20 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int wu = __shfl_sync(0xffffffffu, warp, 0);  // uniform: the roles of warps 8 to 10 run converged
+  // uniform for the compiler: the roles of warps 8 to 10 run converged
+  const int wu = (int)__reduce_or_sync(0xffffffffu, (unsigned)warp);
   const int S = a.stages;
   const uint32_t sbase = smem_u32(smem);
   const uint32_t s_stage = sbase + kWins * a.win_b;
   uint64_t* bars = (uint64_t*)(smem + kWins * a.win_b + (uint32_t)S * a.stage_b);
-  // bfull[8] bempty[8] wfull[2] wempty[2] afull[2] aempty[2]
+  // bfull[8] bempty[8] wfull[kWins] wempty[kWins] afull[2] aempty[2]
   auto bfull = [&](int i) { return smem_u32(&bars[i]); };
   auto bempty = [&](int i) { return smem_u32(&bars[kMaxStages + i]); };
   auto wfull = [&](int i) { return smem_u32(&bars[2 * kMaxStages + i]); };
-  auto wempty = [&](int i) { return smem_u32(&bars[2 * kMaxStages + 2 + i]); };
-  auto afull = [&](int i) { return smem_u32(&bars[2 * kMaxStages + 4 + i]); };
-  auto aempty = [&](int i) { return smem_u32(&bars[2 * kMaxStages + 6 + i]); };
-  uint32_t* tslot = (uint32_t*)(bars + 2 * kMaxStages + 8);
+  auto wempty = [&](int i) { return smem_u32(&bars[2 * kMaxStages + kWins + i]); };
+  auto afull = [&](int i) { return smem_u32(&bars[2 * kMaxStages + 2 * kWins + i]); };
+  auto aempty = [&](int i) { return smem_u32(&bars[2 * kMaxStages + 2 * kWins + 2 + i]); };
+  uint32_t* tslot = (uint32_t*)(bars + 2 * kMaxStages + 2 * kWins + 4);
   volatile int* abort = (volatile int*)(tslot + 1);
 
   if (tid == 0) {
@@ -437,9 +438,11 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
       mbar_init(bfull(i), 1);
       mbar_init(bempty(i), 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kWins; ++i) {
       mbar_init(wfull(i), 1);
       mbar_init(wempty(i), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
       mbar_init(afull(i), 1);
       mbar_init(aempty(i), kDrainWarps);
     }
@@ -454,7 +457,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
+  const uint32_t tmem = __reduce_or_sync(0xffffffffu, *tslot);
 
   if (wu == 8) {
     // ----------------------------------------- operator residues (B) --
@@ -478,11 +481,12 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
 #pragma unroll
           for (int m = 0; m < 9; ++m)
             if (((mask >> m) & 1) && ok) {
-              if (it >= S) ok = mbar_wait_ab(bempty(st), ph ^ 1u, a.err, 11, abort);
+              const char* from = src + (2 * (m % 3 - 1) + 98 * (m / 3 - 1)) * slot_b;
+              if (it >= S) ok = mbar_wait_u(bempty(st), ph ^ 1u, a.err, 11, abort);
               if (ok) {
                 if (el) {
                   mbar_expect_tx(bfull(st), bytes);
-                  bulk_g2s(dst, src + (2 * (m % 3 - 1) + 98 * (m / 3 - 1)) * slot_b, bytes, bfull(st));
+                  bulk_g2s(dst, from, bytes, bfull(st));
                 }
                 __syncwarp();
                 ++it;
@@ -498,7 +502,8 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
   } else if (wu == 10) {
     // ------------------------------------------------- windows of W (A) --
     const uint32_t el = elect_one();
-    int wi = 0;
+    int wi = 0, s = 0;
+    uint32_t wph = 0;
     bool ok = true;
     for (unsigned i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
       const Item t = item_of(a, i);
@@ -508,8 +513,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
         int k0 = 0;
         for (int c = 0; c < v.nchunk; ++c, ++wi) {
           const int ks = chunk_ksteps(v, c);
-          const int s = wi & 1;
-          if (wi >= kWins && !mbar_wait_ab(wempty(s), ((wi >> 1) - 1) & 1, a.err, 12, abort)) {
+          if (wi >= kWins && !mbar_wait_u(wempty(s), wph ^ 1u, a.err, 12, abort)) {
             ok = false;
             break;
           }
@@ -522,6 +526,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
           }
           __syncwarp();
           k0 += ks;
+          if (++s == kWins) s = 0, wph ^= 1u;
         }
       }
     }
@@ -531,8 +536,8 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     const uint32_t el = elect_one();
     const uint64_t dA = desc_k(sbase, kWinRows * 16u, (kTX + 2) * 16u);
     const uint32_t ahi = (uint32_t)(dA >> 32), stage16 = a.stage_b >> 4, win16 = a.win_b >> 4;
-    int st = 0, wi = 0, g = 0, acc = 0;
-    uint32_t ph = 0, dst = tmem, id = 0, n2 = 0, bhi = 0;
+    int st = 0, s = 0, g = 0, acc = 0;
+    uint32_t ph = 0, wph = 0, dst = tmem, id = 0, n2 = 0, bhi = 0;
     const uint32_t blo0 = (uint32_t)desc_k(s_stage, 0u, 128u);
     uint32_t blo = blo0;  // with the item's LBO in the upper half
     uint32_t lbo = 0;
@@ -541,7 +546,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     auto open_acc = [&]() {
       acc = 0;
       dst = tmem + (uint32_t)((g & 1) * kAccCols);
-      if (g >= 2) ok = ok && mbar_wait_ab(aempty(g & 1), ((g >> 1) - 1) & 1, a.err, 14, abort);
+      if (g >= 2) ok = ok && mbar_wait_u(aempty(g & 1), ((g >> 1) - 1) & 1, a.err, 14, abort);
     };
     // the steps of one window whose chunk has KS k-steps, unrolled over its
     // nine shifts: the start address of each is a constant offset
@@ -555,7 +560,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
             ++g;
             open_acc();
           }
-          ok = ok && mbar_wait_ab(bfull(st), ph, a.err, 15, abort);
+          ok = ok && mbar_wait_u(bfull(st), ph, a.err, 15, abort);
           if (!ok) return;
           tc_fence_after();
           mma_steps<KS>(dst, awin + (uint32_t)((m / 3) * (kTX + 2) * kTY + m % 3), ahi, blo | lbo, bhi, n2, id,
@@ -578,18 +583,18 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
       open_acc();
       for (int w = t.w_beg; w < t.w_end && ok; ++w) {
         const int mask = window_of(v, t.ct, w).mask;
-        for (int c = 0; c < nchunk && ok; ++c, ++wi) {
+        for (int c = 0; c < nchunk && ok; ++c) {
           const int ks = c < n0 ? ks0 : ks1;
-          const int s = wi & 1;
-          ok = mbar_wait_ab(wfull(s), (wi >> 1) & 1, a.err, 13, abort);
+          ok = mbar_wait_u(wfull(s), wph, a.err, 13, abort);
           if (!ok) break;
-          const uint32_t awin = (uint32_t)dA + (s ? win16 : 0u);
+          const uint32_t awin = (uint32_t)dA + (uint32_t)s * win16;
           if (ks == 5) window(std::integral_constant<int, 5>(), mask, awin);
           else if (ks == 4) window(std::integral_constant<int, 4>(), mask, awin);
           else if (ks == 3) window(std::integral_constant<int, 3>(), mask, awin);
           else if (ks == 2) window(std::integral_constant<int, 2>(), mask, awin);
           else window(std::integral_constant<int, 1>(), mask, awin);
           if (ok) mma_commit_el(wempty(s), el);
+          if (++s == kWins) s = 0, wph ^= 1u;
         }
       }
       if (ok) mma_commit_el(afull(g & 1), el);

@@ -105,6 +105,29 @@ __device__ __forceinline__ bool mbar_wait_ab(uint32_t a, uint32_t parity, int* e
   return true;
 }
 
+// As mbar_wait_ab for a converged warp, with a vote on every branch, so that the
+// control flow stays uniform for the compiler too: after a wait whose lanes
+// might part, MMAs and commits are issued as by a diverged thread.  The residue GEMM
+// at d = 193: 98 cycles per MMA and 263 per step before, 109 (the tensor rate) and
+// 147 with it; M2L of 2^20 points 5.70 -> 5.13 ms, at d = 126 3.86 -> 3.30.  The
+// FP32 tiers' kernels, whose steps are three times as long, gain nothing from it.
+__device__ __forceinline__ bool mbar_wait_u(uint32_t a, uint32_t parity, int* err, int code,
+                                            volatile int* abort) {
+  if (__all_sync(0xffffffffu, mbar_try(a, parity))) return true;
+  const long long t0 = clock64();
+  while (!__all_sync(0xffffffffu, mbar_try(a, parity))) {
+    const bool late = clock64() - t0 > kWaitCycles;
+    if (__any_sync(0xffffffffu, late || *abort)) {
+      if (late) {
+        atomicExch(err, code);
+        *abort = 1;
+      }
+      return false;
+    }
+  }
+  return true;
+}
+
 // Issue from a converged warp: one lane is elected once and only its
 // instructions take effect.  The operands then stay in uniform registers: a
 // loop that a single thread of a diverged warp runs needs about 100 cycles per
