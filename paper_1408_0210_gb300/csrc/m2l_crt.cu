@@ -25,12 +25,14 @@
 //
 // Four launches cover all levels: largest |W| per level and column; the
 // residue planes of W; the residue GEMMs; the reconstruction.  At 2^20 points,
-// depth 5: eps 1e-6 (d = 193) 4.9 + 0.2 ms, where the FP32 pairs took 144 ms; eps
-// 1e-4 (d = 126) 3.3 ms, where the FP64 pipes took 195 ms; eps 1e-7 (d = 256)
+// depth 5: eps 1e-6 (d = 193) 4.65 + 0.2 ms, where the FP32 pairs took 144 ms; eps
+// 1e-4 (d = 126) 2.3 ms, where the FP64 pipes took 195 ms; eps 1e-7 (d = 256)
 // 8.0 ms (202 ms in FP32 pairs).  The GEMM issues 14 times the method's products,
-// 13% of them zero (189 offsets for 165 pairs per box), and at d = 193 runs at the rate
-// that a library BF16 product sustains (1.74 PFLOP/s); at d = 126, where an MMA is
-// shorter, what the issuing warp does between two steps takes a third.
+// 13% of them zero (189 offsets for 165 pairs per box), 1.8 PFLOP/s at d = 193 and 1.45
+// at d = 126.  It is bound by shared memory: the operands of an MMA (4 KB of W, 32
+// bytes per column), the operator residues written there and the windows take 1,870
+// cycles per offset at 128 bytes a cycle (d = 193; 1,790 measured), 830 at d = 126
+// (860 measured); the MMAs take 1,350 and 510.
 //
 // M2M, L2L and Delta^t are the same sums over the 8 children, the parent and the
 // box itself, without shifts.  Delta^t is formed explicitly in double-double
@@ -405,7 +407,7 @@ __device__ __forceinline__ Item item_of(const CrtArgs& a, unsigned i) {
 // CTA per SM takes every gridDim-th; each role runs on into the next item, so
 // that its operands load and its first sums form while the last one's are
 // reduced and written.  2^20 points, d = 193, against a CTA per item: M2L 5.81 ->
-// 5.70 ms (5.13 with the uniform waits), L2L 0.39 -> 0.33, Delta^t 0.45 -> 0.36; d = 126: 3.80 -> 3.87 (3.30), 0.32 -> 0.27,
+// 5.70 ms (4.86 with the uniform waits and the short loop), L2L 0.39 -> 0.33, Delta^t 0.45 -> 0.36; d = 126: 3.80 -> 3.87 (2.33), 0.32 -> 0.27,
 // 0.34 -> 0.28; 512 leaves, d = 193: M2L 0.40 -> 0.36.
 // Warps 0-7 drain the accumulators, warp 8 streams the operator residues
 // (K-chunk of one offset per stage), warp 9 issues the MMAs, warp 10 loads the
@@ -478,10 +480,10 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
         const char* src = img + wn.slot * slot_b;
         for (int c = 0; c < nchunk && ok; ++c) {
           const uint32_t bytes = (uint32_t)(c < n0 ? ks0 : ks1) * 32u * (uint32_t)v.Nt;
-#pragma unroll
-          for (int m = 0; m < 9; ++m)
-            if (((mask >> m) & 1) && ok) {
-              const char* from = src + (2 * (m % 3 - 1) + 98 * (m / 3 - 1)) * slot_b;
+#pragma unroll 1
+          for (int left = mask; left && ok; left &= left - 1) {
+              const int m = __ffs(left) - 1, mz = (11 * m) >> 5;
+              const char* from = src + (2 * (m - 3 * mz - 1) + 98 * (mz - 1)) * slot_b;
               if (it >= S) ok = mbar_wait_u(bempty(st), ph ^ 1u, a.err, 11, abort);
               if (ok) {
                 if (el) {
@@ -548,13 +550,15 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
       dst = tmem + (uint32_t)((g & 1) * kAccCols);
       if (g >= 2) ok = ok && mbar_wait_u(aempty(g & 1), ((g >> 1) - 1) & 1, a.err, 14, abort);
     };
-    // the steps of one window whose chunk has KS k-steps, unrolled over its
-    // nine shifts: the start address of each is a constant offset
+    // the steps of one window whose chunk has KS k-steps.  A loop, not
+    // unrolled over the shifts: one warp runs through this code once per window,
+    // and fetching it took longer than the MMAs (M2L of 2^20 points, unrolled:
+    // d = 193 5.14 ms, this 4.86; d = 126 3.29, this 2.33)
     auto window = [&](auto ksc, int mask, uint32_t awin) {
       constexpr int KS = decltype(ksc)::value;
-#pragma unroll
-      for (int m = 0; m < 9; ++m)
-        if ((mask >> m) & 1) {
+#pragma unroll 1
+      for (int left = mask; left; left &= left - 1) {
+          const int m = __ffs(left) - 1, mz = (11 * m) >> 5;
           if (acc + KS > kMaxSteps) {  // this accumulator is full
             mma_commit_el(afull(g & 1), el);
             ++g;
@@ -563,7 +567,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
           ok = ok && mbar_wait_u(bfull(st), ph, a.err, 15, abort);
           if (!ok) return;
           tc_fence_after();
-          mma_steps<KS>(dst, awin + (uint32_t)((m / 3) * (kTX + 2) * kTY + m % 3), ahi, blo | lbo, bhi, n2, id,
+          mma_steps<KS>(dst, awin + (uint32_t)(mz * ((kTX + 2) * kTY - 3) + m), ahi, blo | lbo, bhi, n2, id,
                         acc > 0 ? 1u : 0u, el);
           acc += KS;
           mma_commit_el(bempty(st), el);
