@@ -19,6 +19,8 @@ namespace eifmm {
 
 static std::atomic<uint64_t> g_launches{0};
 static std::atomic<uint64_t> g_ops_uid{0};
+static std::atomic<uint64_t> g_generation{0};
+uint64_t next_generation() { return g_generation.fetch_add(1, std::memory_order_relaxed) + 1; }
 // ids of the operator sets not yet destroyed
 static std::mutex g_live_mu;
 static std::set<uint64_t> g_live_ops;
@@ -53,6 +55,7 @@ void dfree(void* p) {
 }
 
 void free_workspace(Workspace* ws) {
+  ws->gen = next_generation();
   for (int k = 0; k <= kMaxLevel; ++k) {
     dfree(ws->W[k]); dfree(ws->Wh[k]); dfree(ws->g[k]);
     if (k != 2) dfree(ws->l[k]);
@@ -157,6 +160,8 @@ eifmm_status alloc_wait_error(Workspace* ws) {
 // image does not fit the device's memory stays without one (the step runs on
 // the FP32 or FP64 pipes).  Several trees of one operator set may come here at the same time.
 static std::mutex g_crt_mu;
+static CrtImage LevelOps::* const kCrtImages[] = {&LevelOps::crt, &LevelOps::crtc, &LevelOps::crt_m2m,
+                                                  &LevelOps::crt_l2l, &LevelOps::crt_dt};
 eifmm_status ensure_crt_images(Ops* ops, int depth, bool m2l, cudaStream_t s) {
   std::lock_guard<std::mutex> lock(g_crt_mu);
   auto build = [&](CrtImage* im, const double* T, int nslots, int dl, int d) {
@@ -203,6 +208,7 @@ static eifmm_status ensure_crt(Tree* t, Ops* ops, int R, cudaStream_t s) {
   }
   const size_t need = n > 0 ? crt_scratch_bytes(n, jobs, R) : 0;
   if (need > ws.crt_bytes) {
+    ws.gen = next_generation();
     dfree(ws.crt_buf);
     ws.crt_buf = nullptr;
     ws.crt_bytes = 0;
@@ -660,6 +666,7 @@ extern "C" eifmm_status eifmm_ops_calibrate(eifmm_ops* ops, double eps, eifmm_st
   for (int64_t i = 0; i < n; ++i) hs[i] = 2.0 * next() - 1.0;
   double *dx = nullptr, *ds = nullptr, *fr = nullptr, *fm = nullptr;
   eifmm_tree* tree = nullptr;
+  Ops images;
   eifmm_status rc = EIFMM_OK;
   int best = 4;
   for (double& e : ops->o.calib_err) e = -1.0;
@@ -677,12 +684,23 @@ extern "C" eifmm_status eifmm_ops_calibrate(eifmm_ops* ops, double eps, eifmm_st
     }
     const double lo[3] = {0.0, 0.0, 0.0};
     if ((rc = eifmm_tree_build(dx, n, dx, n, lo, L, depth, 1, stream, &tree)) != EIFMM_OK) break;
-    // a view of the operators restricted to the calibration depth (with the
-    // images of the FP64 reference, which then belong to the set itself)
-    if ((rc = ensure_crt_images(&ops->o, depth, true, s)) != EIFMM_OK) break;
+    // a view of the operators restricted to the calibration depth, with the
+    // residue images of the FP64 reference: those that the set does not hold
+    // are built for the view alone
+    {
+      std::lock_guard<std::mutex> lock(g_crt_mu);
+      images = ops->o;
+    }
+    if ((rc = ensure_crt_images(&images, depth, true, s)) != EIFMM_OK) break;
     eifmm_ops view;
-    view.o = ops->o;
-    view.o.depth = depth;
+    auto set_view = [&](int tier) {
+      view.o = ops->o;
+      view.o.depth = depth;
+      view.o.tier = tier;
+      for (int k = 2; k <= depth; ++k)
+        for (CrtImage LevelOps::*im : kCrtImages) view.o.lv[k].*im = images.lv[k].*im;
+    };
+    set_view(ops->o.tier);
     if ((rc = evaluate_impl(tree, &view, ds, n, 1, fr, n, EIFMM_PREC_FP64, s)) != EIFMM_OK) break;
     std::vector<double> href(n), hm(n);
     if (cudaMemcpyAsync(href.data(), fr, n * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -702,9 +720,7 @@ extern "C" eifmm_status eifmm_ops_calibrate(eifmm_ops* ops, double eps, eifmm_st
       for (int k = 2; k <= depth; ++k)
         if (t == 0 && ops->o.lv[k].kd_img == nullptr) have_img = false;
       if (!have_img) continue;
-      view.o = ops->o;
-      view.o.depth = depth;
-      view.o.tier = t;
+      set_view(t);
       rc = evaluate_impl(tree, &view, ds, n, 1, fm, n, EIFMM_PREC_MIXED, s);
       if (rc == EIFMM_EUNSUPPORTED) {  // this tier cannot run these operators
         rc = EIFMM_OK;
@@ -732,11 +748,21 @@ extern "C" eifmm_status eifmm_ops_calibrate(eifmm_ops* ops, double eps, eifmm_st
   dfree(ds);
   dfree(fr);
   dfree(fm);
+  {
+    // The images built above go to the set where its tier uses them and it has
+    // none yet.  The set's own stay what they are: another thread or a recorded
+    // batch may be reading them.
+    std::lock_guard<std::mutex> lock(g_crt_mu);
+    for (int k = 2; k <= depth; ++k)
+      for (CrtImage LevelOps::*im : kCrtImages) {
+        CrtImage &mine = images.lv[k].*im, &sets = ops->o.lv[k].*im;
+        if (!mine.img || mine.img == sets.img) continue;
+        if (rc == EIFMM_OK && best >= 3 && !sets.img) sets = mine;
+        else free_crt_image(&mine);
+      }
+  }
   if (rc != EIFMM_OK) return rc;
   EIFMM_TRY(eifmm_ops_plan(ops, best, nullptr));
-  if (best < 3)  // only an evaluation in FP64 would use them, and it builds them again
-    for (int k = 2; k <= depth; ++k)
-      for (CrtImage* im : {&ops->o.lv[k].crt, &ops->o.lv[k].crt_m2m, &ops->o.lv[k].crt_l2l, &ops->o.lv[k].crt_dt}) free_crt_image(im);
   ops->o.calib_tier = best;
   if (tier_out) *tier_out = best;
   return EIFMM_OK;
@@ -820,6 +846,7 @@ extern "C" eifmm_status eifmm_autotune(eifmm_tree* tree, const eifmm_ops* ops, i
     cudaMemsetAsync(sg, 0, (size_t)ns * R * sizeof(double), s);
     if ((rc = evaluate_impl(tree, ops, sg, ns, R, fo, nt, (int)prec, s)) != EIFMM_OK) break;
     Workspace& ws = t.ws;
+    ws.gen = next_generation();  // a recorded batch holds the buffers and the choices from before
     for (int k = 0; k <= kMaxLevel; ++k) ws.m2l_kind[k] = ws.m2l_gshift[k] = 0;
     ws.p2p_sym = 0;
     // room for the partial sums of larger group counts, within 1 GiB per
@@ -967,7 +994,10 @@ extern "C" eifmm_status eifmm_evaluate_host(eifmm_tree* tree, const eifmm_ops* o
 
 // The batch is recorded once into a CUDA graph (after one direct pass that
 // sizes every workspace) and replayed by a single cudaGraphLaunch while the
-// same trees, operators, precision and array pointers are passed again.  The
+// same trees, operators, precision and array pointers are passed again and
+// nothing that the graph refers to has been replaced: the generations of the
+// workspaces and of the operators change with every buffer that a graph may
+// hold, and the trees' options are part of the key.  The
 // problems run on kBranches parallel branches (balanced by an estimated
 // cost, below), each tree on its own workspace and streams and the
 // operators only read, so the many small launches of uneven problems
@@ -986,8 +1016,8 @@ BatchGraph g_batch;
 std::mutex g_batch_mu;  // guards g_batch
 }  // namespace
 
-// A graph refers to the workspaces of its trees and operators: drop it when
-// one of them is destroyed.
+// Drop the graph when one of its trees or its operators are destroyed (the key
+// compares handles, whose addresses may come back).
 static void invalidate_batch(const void* h) {
   std::lock_guard<std::mutex> lock(g_batch_mu);
   if (!g_batch.exec) return;
@@ -1017,17 +1047,26 @@ extern "C" eifmm_status eifmm_evaluate_batched(eifmm_tree* const* trees, const d
   }
   cudaStream_t s = (cudaStream_t)stream;
   std::lock_guard<std::mutex> lock(g_batch_mu);
-  std::vector<const void*> key;
-  key.push_back(ops);
-  key.push_back((const void*)(intptr_t)prec);
-  key.push_back((const void*)(intptr_t)ops->o.tier);
-  key.push_back((const void*)s);
-  for (int p = 0; p < n_problems; ++p) {
-    key.push_back(trees[p]);
-    key.push_back(sigma[p]);
-    key.push_back(f[p]);
-  }
-  if (g_batch.exec && g_batch.key == key && !g_timing) {
+  auto make_key = [&]() {
+    std::vector<const void*> key;
+    key.push_back(ops);
+    key.push_back((const void*)(intptr_t)prec);
+    key.push_back((const void*)(intptr_t)ops->o.tier);
+    key.push_back((const void*)(uintptr_t)ops->o.gen);
+    key.push_back((const void*)s);
+    for (int p = 0; p < n_problems; ++p) {
+      const Tree& t = trees[p]->t;
+      key.push_back(trees[p]);
+      key.push_back(sigma[p]);
+      key.push_back(f[p]);
+      key.push_back((const void*)(uintptr_t)t.ws.gen);
+      uintptr_t options = 0;
+      for (int o = 0; o < kNumOptions; ++o) options = 2 * options + (uintptr_t)t.opt[o];
+      key.push_back((const void*)options);
+    }
+    return key;
+  };
+  if (g_batch.exec && !g_timing && g_batch.key == make_key()) {
     EIFMM_CUDA(cudaGraphLaunch(g_batch.exec, s));
     for (int p = 0; p < n_problems; ++p) trees[p]->t.ws.evaluated = true;
     return EIFMM_OK;
@@ -1124,7 +1163,7 @@ extern "C" eifmm_status eifmm_evaluate_batched(eifmm_tree* const* trees, const d
     set_error(std::string("eifmm_evaluate_batched: graph instantiation failed: ") + cudaGetErrorString(e));
     return EIFMM_ECUDA;
   }
-  g_batch.key = key;
+  g_batch.key = make_key();  // with the workspaces of the direct pass
   g_batch.stream = s;
   return EIFMM_OK;
 }

@@ -1237,6 +1237,7 @@ eifmm_status build_kd_image(Ops* ops, int fmt, cudaStream_t s) {
   for (int k = 2; k <= ops->depth; ++k) {
     LevelOps& v = ops->lv[k];
     if (v.kd_img_fmt == fmt) continue;
+    ops->gen = next_generation();
     dfree(v.kd_img);
     v.kd_img = nullptr;
     v.kd_img_fmt = -1;

@@ -121,6 +121,7 @@ struct Ops {
   double compress_eps = 0.0;
   uint64_t uid = 0;    // unique per loaded operator set: workspaces are keyed on it, not
                        // on the handle's address, which a later load may reuse
+  uint64_t gen = 0;    // changes when operands that an evaluation reads are replaced or freed
   LevelOps lv[kMaxLevel + 1];
   int* d_slot_lists = nullptr;  // [8][189] slot ids per parity class
 };
@@ -162,6 +163,7 @@ struct M2LSparse {
 eifmm_status wait_selftest(long long limit, int* code);  // m2l_tc.cu
 
 struct Workspace {
+  uint64_t gen = 0;  // changes when a buffer or a choice of kernels is replaced (recorded batches)
   const void* ops_id = nullptr;
   uint64_t ops_uid = 0;
   int nrhs = 0;
@@ -334,6 +336,7 @@ constexpr int kCrtMinRank = 8;
 // rounding is 1000 times smaller, takes the residues for all operators.
 constexpr double kCrtMaxKappa = 1e4;
 void free_workspace(Workspace* ws);
+uint64_t next_generation();  // unique in the process
 bool timing_enabled();
 
 // ----------------------------------------------------------- device util --

@@ -236,6 +236,7 @@ void free_compression(LevelOps& v) {
 }
 
 eifmm_status compress_ops(Ops* ops, double eps, cudaStream_t s) {
+  ops->gen = next_generation();
   for (int k = 2; k <= ops->depth; ++k) free_compression(ops->lv[k]);
   ops->compressed = false;
   if (!(eps > 0.0)) return EIFMM_OK;
