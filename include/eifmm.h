@@ -434,6 +434,12 @@ eifmm_status eifmm_wait_selftest(int64_t limit_cycles, int* code);
  * devices, all threads). */
 uint64_t eifmm_kernel_launches(void);
 
+/* For tests of the library's behaviour when memory is short: from now on
+ * allocations of more than `bytes` that a call of this thread makes fail as if
+ * the device had no room (`bytes` < 0: no limit, the default).  Returns how
+ * many the previous limit refused. */
+int64_t eifmm_debug_alloc_limit(int64_t bytes);
+
 /* Device times (ms) of the last evaluate on this tree, recorded with CUDA
  * events on the launching stream when timing is on (eifmm_set_timing(1);
  * the evaluate then waits for its last event).  ms[20]: [0] sigma gather +

@@ -36,9 +36,17 @@ static bool g_timing = false;
 void set_error(const std::string& msg) { g_err = msg; }
 bool timing_enabled() { return g_timing; }
 
+static thread_local size_t t_alloc_limit = SIZE_MAX;  // eifmm_debug_alloc_limit
+static thread_local int64_t t_alloc_refused = 0;
+
 eifmm_status dmalloc(void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
+  if (bytes > t_alloc_limit) {
+    ++t_alloc_refused;
+    set_error("device allocation of " + std::to_string(bytes) + " bytes refused by the limit of this thread");
+    return EIFMM_ENOMEM;
+  }
   cudaError_t e = cudaMalloc(p, bytes);
   if (e != cudaSuccess) {
     *p = nullptr;
@@ -82,7 +90,7 @@ void free_workspace(Workspace* ws) {
   dfree(ws->crt_max);
   ws->crt_buf = nullptr;
   ws->crt_max = nullptr;
-  ws->crt_bytes = 0;
+  ws->crt_bytes = ws->crt_refused = 0;
   dfree(ws->blas_ws);
   ws->blas_ws = nullptr;
   for (int k = 0; k <= kMaxLevel; ++k) ws->m2l_kind[k] = ws->m2l_gshift[k] = 0;
@@ -155,46 +163,64 @@ eifmm_status alloc_wait_error(Workspace* ws) {
   return EIFMM_OK;
 }
 
+// A stream that is being captured takes no allocation and no synchronisation.
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 // Residue images of the operators of levels 2..depth, built once per
 // operator set and ready for every stream on return.  An operator whose
-// image does not fit the device's memory stays without one (the step runs on
-// the FP32 or FP64 pipes).  Several trees of one operator set may come here at the same time.
+// image does not fit the device's memory stays without one for good (the step
+// runs on the FP32 or FP64 pipes): trying again would cost every later call its
+// allocations and the device-wide waits of their release.  While s is being
+// captured nothing is built; the steps without an image run on the pipes.
+// Several trees of one operator set may come here at the same time.
 static std::mutex g_crt_mu;
 static CrtImage LevelOps::* const kCrtImages[] = {&LevelOps::crt, &LevelOps::crtc, &LevelOps::crt_m2m,
                                                   &LevelOps::crt_l2l, &LevelOps::crt_dt};
 eifmm_status ensure_crt_images(Ops* ops, int depth, bool m2l, cudaStream_t s) {
   std::lock_guard<std::mutex> lock(g_crt_mu);
-  auto build = [&](CrtImage* im, const double* T, int nslots, int dl, int d) {
-    if (im->img || dl < kCrtMinRank || d < kCrtMinRank) return EIFMM_OK;
-    const eifmm_status rc = build_crt_image(T, nslots, dl, d, im, s);
-    return rc == EIFMM_ENOMEM ? EIFMM_OK : rc;
+  // builds an image that is neither there nor refused
+  auto ensure = [&](CrtImage* im, int dl, int d, auto&& build) -> eifmm_status {
+    if (im->img || im->refused || dl < kCrtMinRank || d < kCrtMinRank || capturing(s)) return EIFMM_OK;
+    const eifmm_status rc = build();
+    if (rc != EIFMM_ENOMEM) return rc;
+    im->refused = true;
+    return EIFMM_OK;
+  };
+  auto stack = [&](CrtImage* im, const double* T, int nslots, int dl, int d) {
+    return ensure(im, dl, d, [&] { return build_crt_image(T, nslots, dl, d, im, s); });
   };
   for (int k = 2; k <= depth; ++k) {
     LevelOps& v = ops->lv[k];
-    if (k < depth) EIFMM_TRY(build(&v.crt_m2m, v.m2mT, 8, ops->lv[k + 1].d, v.d));
-    if (k > 2) EIFMM_TRY(build(&v.crt_l2l, v.l2lT, 8, ops->lv[k - 1].d, v.d));
-    if (k == depth && v.d >= kCrtMinRank && !v.crt_dt.img && !v.crt_dt.refused) {
-      const eifmm_status rc = build_crt_delta_image(v, &v.crt_dt, s);
-      if (rc != EIFMM_OK && rc != EIFMM_ENOMEM) return rc;
-    }
+    if (k < depth) EIFMM_TRY(stack(&v.crt_m2m, v.m2mT, 8, ops->lv[k + 1].d, v.d));
+    if (k > 2) EIFMM_TRY(stack(&v.crt_l2l, v.l2lT, 8, ops->lv[k - 1].d, v.d));
+    if (k == depth)
+      EIFMM_TRY(ensure(&v.crt_dt, v.d, v.d, [&] { return build_crt_delta_image(v, &v.crt_dt, s); }));
     if (!m2l) continue;
     if (ops->compressed && v.r > 0) {
-      EIFMM_TRY(build(&v.crtc, v.Ct, kNumSlots, v.r, v.r));
-    } else if (!v.crt.img) {
-      EIFMM_TRY(build(&v.crt, v.kdT, kNumSlots, v.d, v.d));
-      if (v.crt.img) EIFMM_TRY(crt_kappa((int)ops->kern, v, ops->L * ldexp(1.0, -(k + 1)), &v.crt.kappa, s));
+      EIFMM_TRY(stack(&v.crtc, v.Ct, kNumSlots, v.r, v.r));
+    } else {
+      EIFMM_TRY(stack(&v.crt, v.kdT, kNumSlots, v.d, v.d));
+      if (v.crt.kappa < 0.0 && v.d >= kCrtMinRank && !capturing(s))
+        EIFMM_TRY(crt_kappa((int)ops->kern, v, ops->L * ldexp(1.0, -(k + 1)), &v.crt.kappa, s));
     }
   }
   return EIFMM_OK;
 }
 
 // Images and scratch of the residue products for an evaluation with the FP64
-// far field.  Without room for the scratch crt_bytes stays 0 and those steps
-// run on the FP32 or FP64 pipes.
+// far field.  A step whose scratch there is no room for runs on the FP32 or FP64
+// pipes (crt_ready); a size that did not fit is not asked for again.
 static eifmm_status ensure_crt(Tree* t, Ops* ops, int R, cudaStream_t s) {
   Workspace& ws = t->ws;
   EIFMM_TRY(ensure_crt_images(ops, t->depth, !t->opt[EIFMM_OPT_M2L_FP64], s));
-  CrtJob jobs[3 * kMaxLevel];
+  CrtJob jobs[4 * kMaxLevel];
   int n = 0;
   auto add = [&](CrtMode m, int k, const CrtImage& im) {
     if (im.img) jobs[n++] = CrtJob{m, k, &im, nullptr, nullptr, nullptr};
@@ -207,14 +233,15 @@ static eifmm_status ensure_crt(Tree* t, Ops* ops, int R, cudaStream_t s) {
     if (k == t->depth) add(kCrtBox, k, v.crt_dt);
   }
   const size_t need = n > 0 ? crt_scratch_bytes(n, jobs, R) : 0;
-  if (need > ws.crt_bytes) {
+  if (need > ws.crt_bytes && (ws.crt_refused == 0 || need < ws.crt_refused) && !capturing(s)) {
     ws.gen = next_generation();
     dfree(ws.crt_buf);
     ws.crt_buf = nullptr;
     ws.crt_bytes = 0;
     const eifmm_status rc = dmalloc(&ws.crt_buf, need);
     if (rc == EIFMM_OK) ws.crt_bytes = need;
-    else if (rc != EIFMM_ENOMEM) return rc;
+    else if (rc == EIFMM_ENOMEM) ws.crt_refused = need;
+    else return rc;
   }
   return EIFMM_OK;
 }
@@ -307,6 +334,12 @@ extern "C" const char* eifmm_last_error(void) { return g_err.c_str(); }
 extern "C" const char* eifmm_version(void) { return "eifmm-gb300 0.1 (sm_103a)"; }
 extern "C" void eifmm_set_timing(int on) { g_timing = on != 0; }
 extern "C" uint64_t eifmm_kernel_launches(void) { return g_launches.load(); }
+extern "C" int64_t eifmm_debug_alloc_limit(int64_t bytes) {
+  const int64_t refused = t_alloc_refused;
+  t_alloc_refused = 0;
+  t_alloc_limit = bytes < 0 ? SIZE_MAX : (size_t)bytes;
+  return refused;
+}
 
 namespace eifmm {
 eifmm_status launch_direct_sum(int kern, const double* tgt, const double* src, int64_t n_src,

@@ -536,8 +536,8 @@ eifmm_status launch_m2l64(int level, int d, int R, const double* kdT, const int*
 // M2M and L2L of np parents by residues on the tensor cores: four launches of
 // about 30 us together at least, which the warp kernels on the FP64 pipes take
 // at 4e6 products per column (64 parents at d = 90; d = 193: 52 us).
-static bool crt_transfer(const Workspace& ws, const CrtImage& im, int64_t np, int R) {
-  return im.img && ws.crt_bytes > 0 && (double)np * R * 8.0 * im.d * im.dl >= 4e6;
+static bool crt_transfer(const Workspace& ws, CrtMode mode, int level, const CrtImage& im, int64_t np, int R) {
+  return crt_ready(mode, level, im, R, ws.crt_bytes) && (double)np * R * 8.0 * im.d * im.dl >= 4e6;
 }
 
 eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_sigma, int R,
@@ -582,7 +582,7 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   for (int k = kap - 1; k >= 2; --k) {
     const int dk = ops->lv[k].d, dc = ops->lv[k + 1].d;
     const int64_t np = (int64_t)1 << (3 * k);
-    if (!pairs && crt_transfer(ws, ops->lv[k].crt_m2m, np, R)) {
+    if (!pairs && crt_transfer(ws, kCrtM2M, k, ops->lv[k].crt_m2m, np, R)) {
       const CrtJob job{kCrtM2M, k, &ops->lv[k].crt_m2m, ws.W[k + 1], ws.W[k], nullptr};
       EIFMM_TRY(launch_crt(1, &job, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
       continue;
@@ -609,7 +609,7 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
       if (timing_enabled()) cudaEventRecord(ws.ev_m2l[k], s);
       if (ops->compressed && v.r > 0)
         EIFMM_TRY(m2l_compressed(ws, ops, k, R, fp64, pair, s));
-      else if (!fp64 && v.crt.img && ws.crt_bytes > 0 && !(pair && v.crt.kappa > kCrtMaxKappa))
+      else if (!fp64 && crt_ready(kCrtM2L, k, v.crt, R, ws.crt_bytes) && !(pair && v.crt.kappa > kCrtMaxKappa))
         jobs[nj++] = CrtJob{kCrtM2L, k, &v.crt, ws.W[k], ws.g[k], nullptr};
       else if (pair)
         EIFMM_TRY(launch_m2l_df(k, v.d, R, v.kdT, ops->d_slot_lists, ws.W[k], ws.g[k], ws.part64, ws.part64_cap,
@@ -627,7 +627,7 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   for (int k = 3; k <= kap; ++k) {
     const int dk = ops->lv[k].d, dp = ops->lv[k - 1].d;
     const int64_t nb = (int64_t)1 << (3 * k);
-    if (crt_transfer(ws, ops->lv[k].crt_l2l, nb / 8, R)) {
+    if (crt_transfer(ws, kCrtL2L, k, ops->lv[k].crt_l2l, nb / 8, R)) {
       const CrtJob job{kCrtL2L, k, &ops->lv[k].crt_l2l, ws.l[k - 1], ws.l[k], ws.g[k]};
       EIFMM_TRY(launch_crt(1, &job, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
       continue;
@@ -638,7 +638,7 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   }
   record(ws, 5, s);
   // step 6: the explicit Delta^t in residues, or the triangular solves
-  if (vl.crt_dt.img && ws.crt_bytes > 0) {
+  if (crt_ready(kCrtBox, kap, vl.crt_dt, R, ws.crt_bytes)) {
     const CrtJob job{kCrtBox, kap, &vl.crt_dt, ws.l[kap], ws.lh, nullptr};
     EIFMM_TRY(launch_crt(1, &job, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
   } else {

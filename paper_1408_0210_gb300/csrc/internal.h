@@ -58,8 +58,8 @@ __host__ __device__ inline double kern_f64(int kern, double z0, double z1, doubl
 struct CrtImage {
   void* img = nullptr;         // BF16
   double* colscale = nullptr;  // [d] scale of column m' in the reconstruction
-  double kappa = 0.0;          // amplification of rounding by the operators (crt_kappa)
-  bool refused = false;        // the operators cannot be represented
+  double kappa = -1.0;         // amplification of rounding by the operators (crt_kappa); -1: not known
+  bool refused = false;        // the operators cannot be represented, or their image did not fit
   int nslots = 0, dl = 0, d = 0;     // operators, rank of the source and of the target
   int K = 0, Nt = 0, NT = 0;         // terms padded to 16, columns of a tile, tiles
 };
@@ -201,7 +201,7 @@ struct Workspace {
   double* part64 = nullptr;     // the same for the FP64 far field (FP64 and FP32-pair M2L)
   size_t part64_cap = 0;        // doubles in part64
   void* crt_buf = nullptr;      // residue planes and sums of the FP64 M2L on the tensor cores
-  size_t crt_bytes = 0;
+  size_t crt_bytes = 0, crt_refused = 0;  // its size; the last size that did not fit (0: none)
   unsigned long long* crt_max = nullptr;  // [kMaxLevel + 1][R] bits of the largest |W|
   int nsm = 0;                  // SMs of the workspace's device
   uint32_t* wmax = nullptr;     // [kMaxLevel + 1] bits of max |W| per level (FP16 planes)

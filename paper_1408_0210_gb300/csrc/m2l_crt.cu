@@ -1081,6 +1081,12 @@ size_t crt_scratch_bytes(int njobs, const CrtJob* jobs, int R) {
   return std::max(most, std::min(total, kScratchLimit));
 }
 
+bool crt_ready(CrtMode mode, int level, const CrtImage& im, int R, size_t bytes) {
+  if (!im.img || bytes == 0) return false;
+  const CrtJob job{mode, level, &im, nullptr, nullptr, nullptr};
+  return crt_scratch_bytes(1, &job, R) <= bytes;
+}
+
 void free_crt_image(CrtImage* im) {
   dfree(im->img);
   dfree(im->colscale);

@@ -23,6 +23,8 @@ struct CrtJob {
 // Scratch for the jobs of one call (M2L jobs run together, others one by one);
 // jobs beyond the library's limit run in slabs and columns.
 size_t crt_scratch_bytes(int njobs, const CrtJob* jobs, int R);
+// Whether a job of this image can run in `bytes` of scratch.
+bool crt_ready(CrtMode mode, int level, const CrtImage& img, int R, size_t bytes);
 // All jobs on stream s, in `buf` (buf_bytes from crt_scratch_bytes); wmax:
 // [kMaxLevel + 1][R] words; err: error word of the bounded waits.
 eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t buf_bytes, unsigned long long* wmax,

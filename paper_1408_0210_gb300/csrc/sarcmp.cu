@@ -326,7 +326,7 @@ eifmm_status m2l_compressed(Workspace& ws, const Ops* ops, int k, int R, bool fp
   EIFMM_TRY((launch_delta_batch<double, double, double, 0>(b, false, s)));
   double* wt = (double*)ws.tmp;  // rows x r
   EIFMM_TRY(gemm64(false, rows, r, d, ws.Wh[k], d, v.U, r, wt, r, s));
-  if (!fp64 && v.crtc.img && ws.crt_bytes > 0) {
+  if (!fp64 && crt_ready(kCrtM2L, k, v.crtc, R, ws.crt_bytes)) {
     const CrtJob job{kCrtM2L, k, &v.crtc, wt, ws.Wh[k], nullptr};
     EIFMM_TRY(launch_crt(1, &job, R, ws.crt_buf, ws.crt_bytes, ws.crt_max, ws.nsm, ws.err, s));
   } else if (pair) {

@@ -27,7 +27,7 @@ EXPORTS = [
     "eifmm_set_timing", "eifmm_last_step_times", "eifmm_direct_sum", "eifmm_kernel_launches",
     "eifmm_tree_sort_static", "eifmm_ops_calibrate", "eifmm_autotune", "eifmm_measure_rates",
     "eifmm_ops_calibration", "eifmm_tree_set_option", "eifmm_ops_compress", "eifmm_ops_basis",
-    "eifmm_wait_selftest",
+    "eifmm_wait_selftest", "eifmm_debug_alloc_limit",
 ]
 OPTIONS = {"m2l_128row": 0, "p2p_pair_symmetric": 1, "single_stream": 2, "m2l_fp64": 3,
            "m2l_stream_k": 4, "near_field_late": 5}
@@ -86,6 +86,7 @@ def lib() -> C.CDLL:
         "eifmm_tree_set_option": (i32, [vp, i32, i32]),
         "eifmm_ops_compress": (i32, [vp, dbl, vp, vp]),
         "eifmm_wait_selftest": (i32, [i64, vp]),
+        "eifmm_debug_alloc_limit": (i64, [i64]),
         "eifmm_ops_basis": (i32, [vp, i32, vp, vp, vp, vp]),
     }
     for name, (res, args) in sig.items():
@@ -419,6 +420,12 @@ def eifmm_wait_selftest(limit_cycles: int) -> tuple[int, int]:
     code = C.c_int(-1)
     st = lib().eifmm_wait_selftest(int(limit_cycles), C.byref(code))
     return st, code.value
+
+
+def eifmm_debug_alloc_limit(n_bytes: int) -> int:
+    """From now on this thread's allocations above n_bytes fail as if the device
+    had no room (negative: no limit).  Returns how many the last limit refused."""
+    return int(lib().eifmm_debug_alloc_limit(int(n_bytes)))
 
 
 def eifmm_kernel_launches() -> int:
