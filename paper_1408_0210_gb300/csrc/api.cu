@@ -203,6 +203,9 @@ eifmm_status ensure_crt_images(Ops* ops, int depth, bool m2l, cudaStream_t s) {
     if (k == depth)
       EIFMM_TRY(ensure(&v.crt_dt, v.d, v.d, [&] { return build_crt_delta_image(v, &v.crt_dt, s); }));
     if (!m2l) continue;
+    const bool steep = crt_steep((int)ops->kern, ops->L, k);
+    if (!v.crt.img) v.crt.refused = v.crt.refused || steep;
+    if (!v.crtc.img) v.crtc.refused = v.crtc.refused || steep;
     if (ops->compressed && v.r > 0) {
       EIFMM_TRY(stack(&v.crtc, v.Ct, kNumSlots, v.r, v.r));
     } else {
@@ -293,7 +296,7 @@ eifmm_status ensure_workspace(Tree* t, const Ops* ops, int R, int prec) {
     }
     if (need) EIFMM_TRY(dalloc(&ws.part64, need));
     ws.part64_cap = need;
-    EIFMM_TRY(dalloc(&ws.crt_max, (size_t)(kMaxLevel + 1) * R));
+    EIFMM_TRY(dalloc(&ws.crt_max, crt_max_words(kap, R)));
     EIFMM_TRY(alloc_wait_error(&ws));
     if (fx_usable((int)ops->kern, t->L, t->depth)) {
       EIFMM_TRY(dalloc(&ws.fx_src, (size_t)3 * std::max<int64_t>(t->src.n, 1)));

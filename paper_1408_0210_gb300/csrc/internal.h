@@ -202,7 +202,7 @@ struct Workspace {
   size_t part64_cap = 0;        // doubles in part64
   void* crt_buf = nullptr;      // residue planes and sums of the FP64 M2L on the tensor cores
   size_t crt_bytes = 0, crt_refused = 0;  // its size; the last size that did not fit (0: none)
-  unsigned long long* crt_max = nullptr;  // [kMaxLevel + 1][R] bits of the largest |W|
+  unsigned long long* crt_max = nullptr;  // bits of the largest |W| of the units (crt_max_words)
   int nsm = 0;                  // SMs of the workspace's device
   uint32_t* wmax = nullptr;     // [kMaxLevel + 1] bits of max |W| per level (FP16 planes)
   M2LSparse sparse[kMaxLevel + 1];  // levels most of whose boxes hold no targets (tier 0, one right-hand side)

@@ -6,8 +6,8 @@
 // The FP64 pipes of this GPU run at 1/72 of the FP32 rate, the tensor cores
 // 25 times above the latter.  The sum is therefore formed exactly in integers by
 // residues (K. Ozaki, Y. Uchino, T. Imamura, "Ozaki Scheme II", 2025): W is
-// rounded to 59-bit integers with one power-of-two scale per level and
-// right-hand side, row m' of every T^delta with one scale per row, chosen so
+// rounded to 59-bit integers with a power-of-two scale (M2L: one per level and
+// right-hand side), row m' of every T^delta with one scale per row, chosen so
 // that the whole sum over offsets and l stays below M / 2 in magnitude, M the
 // product of 14 pairwise coprime moduli up to 513 (125.2 bits).  Modulo m_i
 // both operands are integers in [-256, 256], exact in BF16; a product is at
@@ -22,9 +22,13 @@
 // 2 to 4, uniform and clustered points), the FP64 sum on the FP64 pipes by
 // 1.2e-15 to 6.8e-15 and the FP32 pairs by about 2e-12; for the config-3 kernel
 // (eps 1e-6) 4.2e-13 against 6.6e-12 in FP64.
+// Uneven problems (kWeakBits) keep their digits by a second part: 1/r, 2,000 charges
+// of order 1 that cancel in one corner and 1e-12 elsewhere, depth 7: f differs from
+// the FP64 pipes' by 4e-16 in the median; with one part by 1.8e-14.
 //
-// Four launches cover all levels: largest |W| per level and column; the
-// residue planes of W; the residue GEMMs; the reconstruction.  At 2^20 points,
+// Six launches cover all levels: largest |W| per level, box and column; the
+// residue planes of W; those of the second part (kWeakBits), if any; the residue
+// GEMMs; the reconstruction; that of the targets with a second part.  At 2^20 points,
 // depth 5: eps 1e-6 (d = 193) 4.65 + 0.2 ms, where the FP32 pairs took 144 ms; eps
 // 1e-4 (d = 126) 2.3 ms, where the FP64 pipes took 195 ms; eps 1e-7 (d = 256)
 // 8.0 ms (202 ms in FP32 pairs).  The GEMM issues 14 times the method's products,
@@ -35,7 +39,8 @@
 // (860 measured); the MMAs take 1,350 and 510.
 //
 // M2M, L2L and Delta^t are the same sums over the 8 children, the parent and the
-// box itself, without shifts.  Delta^t is formed explicitly in double-double
+// box itself, without shifts.  A sum stays within one parent or box, and so does
+// its scale: a weak box next to strong ones keeps all its bits.  Delta^t is formed explicitly in double-double
 // and takes 18 moduli (160.5 bits): its entries reach 2^34 / |A| at eps 1e-7, and
 // the product cancels by as much.  K(x, X) Delta^t l then errs by 1.6e-16 to 9e-16
 // (1/r, eps 1e-4 to 1e-7) where the FP64 triangular solves err by 2.3e-16 to 2.7e-15
@@ -64,6 +69,15 @@ __host__ __device__ constexpr int crt_mod(int i) {
 // |W| 2^b < 2^wbits; sum over offsets and l of |T| 2^a < 2^rowbits; wbits +
 // rowbits + 1 (the sign) is the size of the product of the moduli.
 constexpr int kWBits = 58, kRowBits = 66, kEntryBits = 60;  // |T| 2^a < 2^60
+// The M2L's scale is the level's, so a target box all of whose sources are far
+// weaker than the level's strongest box would get them in few bits.  Such a box
+// (the exponent of the largest |W| of its interaction list more than kWeakBits
+// below that of the level's: nearer, the rounding is at most half a unit in the
+// last place of its strongest source) also takes a second part, the same sum over
+// what the rounding left of W, in units 2^-59 times smaller, added in FP64: 53
+// bits down to 2^-64 of the level's largest.  Even problems have no such box; the
+// items of the second part then do not exist, and its two kernels end at once.
+constexpr int kWeakBits = 5, kRestBits = 59;
 constexpr int kBoxWBits = 55, kBoxRowBits = 104;
 constexpr int kMaxSteps = 15;  // k-steps of 16 terms in one accumulation: 240 terms
 
@@ -108,12 +122,22 @@ struct CrtLv {
   int16_t* res;              // [mod][group][r][class][z][y][x][NT Nt]
   const __nv_bfloat16* img;  // [mod][slot][column tile][k8][Nt][8]
   const double* colscale;    // per column m': M 2^(-96 - a)
-  unsigned long long* wmax;  // [R] bits of the largest |W|
+  // [unit][R] bits of the largest |W| of a unit, the boxes that share a scale:
+  // source box J is in unit J >> sshift, target box I takes unit I >> tshift
+  unsigned long long* wmax;
+  int sshift, tshift;
+  // second part of the M2L (kWeakBits): null elsewhere
+  unsigned long long* bmax;  // [box][R] bits of the largest |W| of a box
+  unsigned char* weak;       // [box][R] target boxes that take the second part
+  unsigned char* need;       // [r][class][tile z, y, x] tiles that hold some
+  int pstep;                 // class grids of the first part in `planes`
+  int64_t rstep;             // entries of the first part in `res`
 };
 constexpr int kMaxLv = kMaxLevel - 1;
 struct CrtArgs {
   int nlev, stages;
-  unsigned items;
+  unsigned items, plane_blocks, rebuild_blocks;
+  unsigned* any;  // set when some target takes the second part (null: never)
   uint32_t stage_b, win_b;
   int* err;
   CrtLv lv[kMaxLv];
@@ -207,8 +231,7 @@ __device__ __forceinline__ int64_t class_box(int nc, int c, int x, int y, int z)
 // scale exponent of a column from the bits of its largest |W|
 __device__ __forceinline__ bool w_finite(unsigned long long bits) { return bits < 0x7ff0000000000000ull; }
 __device__ __forceinline__ int w_exp(unsigned long long bits, int wbits) {
-  const int b = wbits - ((int)(bits >> 52) - 1022);
-  return b > 1020 ? 1020 : b;
+  return wbits - ((int)(bits >> 52) - 1022);
 }
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
@@ -222,6 +245,19 @@ __device__ __forceinline__ long long w_int(double w, int b) {
   if (sh >= 0) m <<= sh;
   else m = sh < -54 ? 0 : (m + (1ull << (-sh - 1))) >> -sh;
   return w < 0.0 ? -(long long)m : (long long)m;
+}
+
+// What the rounding left, (w 2^b - v) 2^kRestBits rounded to an integer, at most
+// 2^58 in magnitude; the terms are formed modulo 2^64.
+__device__ __forceinline__ long long w_rest(double w, int b, long long v) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(w) & 0x7fffffffffffffffull;
+  const int e = (int)(u >> 52);
+  unsigned long long m = u & 0xfffffffffffffull;
+  if (e) m |= 1ull << 52;
+  const int sh = (e ? e : 1) - 1075 + b + kRestBits;  // at most 65
+  if (sh >= 0) m = sh < 64 ? m << sh : 0;
+  else m = sh < -54 ? 0 : (m + (1ull << (-sh - 1))) >> -sh;
+  return (long long)((w < 0.0 ? 0 - m : m) - ((unsigned long long)v << kRestBits));
 }
 
 // 2^(12 j) modulo crt_mod(i), in [-m/2, m/2]
@@ -269,40 +305,42 @@ __device__ __forceinline__ int find_level(const CrtArgs& a, unsigned CrtLv::*fir
 }
 
 // ---------------------------------------------------------- largest |W| --
-// A block takes 32 boxes of a column, a warp four of them at once: the loads of
-// all four are in flight together (one box after the other took 34 us at any size).
+// A block takes 32 boxes of a column, eight lanes a box with eight loads in flight
+// (one box after the other by a warp took 34 us at any size).  One maximum per
+// unit: the whole level (M2L, and each box), eight children or one box.
 constexpr int kMaxBoxes = 32;
+__device__ __forceinline__ unsigned long long max_over(unsigned long long m, int lanes) {
+  for (int o = 1; o < lanes; o <<= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xffffffffu, m, o);
+    m = x > m ? x : m;
+  }
+  return m;
+}
 __global__ void __launch_bounds__(256) k_crt_max(const __grid_constant__ CrtArgs a) {
   const CrtLv& v = a.lv[find_level(a, &CrtLv::mx0, blockIdx.x)];
   const unsigned b = blockIdx.x - v.mx0, q = b / (unsigned)v.Rc;
-  const int r = v.r0 + (int)(b - q * v.Rc), ds = v.ds;
-  const int64_t box0 = (int64_t)q * kMaxBoxes + (threadIdx.x >> 5), n = (int64_t)1 << (3 * v.slevel);
-  const double* w[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int64_t box = box0 + 8 * j;
-    w[j] = v.W + ((box < n ? box : n - 1) * v.R + r) * ds;
+  const int r = v.r0 + (int)(b - q * v.Rc), ds = v.ds, t = threadIdx.x;
+  const int64_t first = (int64_t)q * kMaxBoxes;  // the boxes of a level are a multiple of 32
+  const double* w = v.W + ((first + (t >> 3)) * v.R + r) * ds;
+  unsigned long long m = 0;
+#pragma unroll 8
+  for (int l = t & 7; l < ds; l += 8) {
+    const unsigned long long x = (unsigned long long)__double_as_longlong(w[l]) & 0x7fffffffffffffffull;
+    m = x > m ? x : m;
   }
-  unsigned long long mx = 0;
-#pragma unroll 2
-  for (int l = threadIdx.x & 31; l < ds; l += 32) {
-    unsigned long long x[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) x[j] = (unsigned long long)__double_as_longlong(w[j][l]) & 0x7fffffffffffffffull;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) mx = x[j] > mx ? x[j] : mx;
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long x = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = x > mx ? x : mx;
-  }
-  __shared__ unsigned long long sm[8];
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = mx;
+  m = max_over(m, 8);
+  __shared__ unsigned long long sm[kMaxBoxes];
+  if ((t & 7) == 0) sm[t >> 3] = m;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) mx = sm[w] > mx ? sm[w] : mx;
-    if (mx > *(volatile unsigned long long*)(v.wmax + r)) atomicMax(v.wmax + r, mx);
-  }
+  if (t >= kMaxBoxes) return;
+  m = sm[t];
+  if (v.bmax) v.bmax[(first + t) * v.R + r] = m;
+  const int per = v.sshift >= 5 ? kMaxBoxes : 1 << v.sshift;
+  m = max_over(m, per);
+  if (t % per != 0) return;
+  unsigned long long* out = v.wmax + ((first + t) >> v.sshift) * v.R + r;
+  if (v.sshift <= 5) *out = m;
+  else if (m > *(volatile unsigned long long*)out) atomicMax(out, m);
 }
 
 // ------------------------------------------------------- residue planes --
@@ -319,11 +357,44 @@ __device__ __forceinline__ void store_residues(const Limbs (&v)[4], __nv_bfloat1
     store_residues<I + 1, NM>(v, dst + step, step);
   }
 }
-template <int NM>
-__global__ void __launch_bounds__(256) k_crt_planes(const __grid_constant__ CrtArgs a) {
-  extern __shared__ long long s_w[];  // [8][K + 1]
-  const CrtLv& v = a.lv[find_level(a, &CrtLv::pl0, blockIdx.x)];
-  unsigned b = blockIdx.x - v.pl0;
+// Index in `need` of the tile of target box (x, y, z) of class ct, column r.
+__device__ __forceinline__ int need_index(const CrtLv& v, int r, int ct, int z, int y, int x) {
+  const int nx = (v.h + kTX - 1) / kTX, ny = (v.h + kTY - 1) / kTY, nz = (v.nz + kTZ - 1) / kTZ;
+  return (((r * v.nct + ct) * nz + (z - v.z0) / kTZ) * ny + y / kTY) * nx + x / kTX;
+}
+// Whether box (x, y, z) of class ct takes the second part, by its warp.  The
+// boxes of its interaction list are the children of the 27 neighbours of its
+// parent (x, y, z) but its own neighbours.
+__device__ __forceinline__ void mark_weak(const CrtArgs& a, const CrtLv& v, int r, int ct, int z, int y, int x,
+                                          int64_t box, unsigned long long level) {
+  // by the exponents (subnormals count as the smallest one); most boxes have a
+  // strong source among the first 32 looked at
+  const int enough = (int)(level >> 52) - kWeakBits;
+  bool some = false, strong = !w_finite(level);
+  for (int i = threadIdx.x & 31; i < 224 && !strong; i += 32) {
+    const int n = i >> 3, c = i & 7, dx = n % 3 - 1, dy = n / 3 % 3 - 1, dz = n / 9 - 1;
+    const bool in = i < 216 && x + dx >= 0 && y + dy >= 0 && z + dz >= 0 && x + dx < v.h && y + dy < v.h && z + dz < v.h;
+    const int ox = 2 * dx + (c & 1) - (ct & 1), oy = 2 * dy + ((c >> 1) & 1) - ((ct >> 1) & 1),
+              oz = 2 * dz + (c >> 2) - (ct >> 2);
+    unsigned long long m = 0;
+    if (in && (abs(ox) > 1 || abs(oy) > 1 || abs(oz) > 1))
+      m = v.bmax[class_box(8, c, x + dx, y + dy, z + dz) * v.R + r];
+    some = some || m > 0;
+    strong = __any_sync(0xffffffffu, m > 0 && (int)(m >> 52) >= enough);
+  }
+  const bool weak = __any_sync(0xffffffffu, some) && !strong;
+  if ((threadIdx.x & 31) != 0) return;
+  v.weak[box * v.R + r] = weak;
+  if (weak) {
+    v.need[need_index(v, r - v.r0, ct, z, y, x)] = 1;
+    *a.any = 1;
+  }
+}
+// One block of the planes; REST: of the second part.
+template <int NM, bool REST>
+__device__ __forceinline__ void planes_block(const CrtArgs& a, unsigned block, long long* s_w) {
+  const CrtLv& v = a.lv[find_level(a, &CrtLv::pl0, block)];
+  unsigned b = block - v.pl0;
   const int h = v.h, nxs = (h + 7) / 8;
   const int xs = (int)(b % nxs);
   b /= nxs;
@@ -333,14 +404,19 @@ __global__ void __launch_bounds__(256) k_crt_planes(const __grid_constant__ CrtA
   b /= v.snz;
   const int cls = (int)(b % v.ncs), r = (int)(b / v.ncs);
   const int z = v.sz0 + zs, K = v.K, ld = K + 1;
-  const unsigned long long bits = v.wmax[v.r0 + r];
-  const bool fin = w_finite(bits);
-  const int e = w_exp(fin ? bits : 0, v.wbits);
   {
     const int bx = threadIdx.x >> 5, x = 8 * xs + bx;
-    const double* w = x < h && fin ? v.W + (class_box(v.ncs, cls, x, y, z) * v.R + v.r0 + r) * v.ds : nullptr;
+    const int64_t box = x < h ? class_box(v.ncs, cls, x, y, z) : 0;
+    const unsigned long long bits = v.wmax[(box >> v.sshift) * v.R + v.r0 + r];
+    const bool fin = w_finite(bits);
+    const int e = w_exp(fin ? bits : 0, v.wbits);
+    const double* w = x < h && fin ? v.W + (box * v.R + v.r0 + r) * v.ds : nullptr;
 #pragma unroll 4
-    for (int l = threadIdx.x & 31; l < K; l += 32) s_w[bx * ld + l] = w && l < v.ds ? w_int(w[l], e) : 0;
+    for (int l = threadIdx.x & 31; l < K; l += 32) {
+      const long long q = w && l < v.ds ? w_int(w[l], e) : 0;
+      s_w[bx * ld + l] = REST && w && l < v.ds ? w_rest(w[l], e, q) : q;
+    }
+    if (!REST && v.bmax && x < h && z >= v.z0 && z < v.z0 + v.nz) mark_weak(a, v, v.r0 + r, cls, z, y, x, box, bits);
   }
   __syncthreads();
   const int64_t plane = (int64_t)(K / 8) * v.snz * h * h * 8;  // elements of one (mod, r, class)
@@ -351,8 +427,23 @@ __global__ void __launch_bounds__(256) k_crt_planes(const __grid_constant__ CrtA
     Limbs w[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) w[j] = limbs_of(q[2 * j], q[2 * j + 1]);
-    __nv_bfloat16* dst = v.planes + (int64_t)(r * v.ncs + cls) * plane + ((((int64_t)k8 * v.snz + zs) * h + y) * h + x) * 8;
+    __nv_bfloat16* dst = v.planes + (int64_t)((REST ? v.pstep : 0) + r * v.ncs + cls) * plane +
+                         ((((int64_t)k8 * v.snz + zs) * h + y) * h + x) * 8;
     store_residues<0, NM>(w, dst, (int64_t)v.Rc * v.ncs * plane);
+  }
+}
+template <int NM>
+__global__ void __launch_bounds__(256) k_crt_planes(const __grid_constant__ CrtArgs a) {
+  extern __shared__ long long s_w[];  // [8][K + 1]
+  planes_block<NM, false>(a, blockIdx.x, s_w);
+}
+template <int NM>
+__global__ void __launch_bounds__(256) k_crt_planes_rest(const __grid_constant__ CrtArgs a) {
+  extern __shared__ long long s_w[];
+  if (*a.any == 0) return;
+  for (unsigned b = blockIdx.x; b < a.plane_blocks; b += gridDim.x) {
+    planes_block<NM, true>(a, b, s_w);
+    __syncthreads();
   }
 }
 
@@ -377,10 +468,12 @@ __device__ __forceinline__ void mma_steps(uint32_t dst, uint32_t alo, uint32_t a
 }
 
 struct Item {
-  int q, x0, y0, z0, ct, nt, r, grp, mod, w_beg, w_end;
+  int q, x0, y0, z0, ct, nt, r, grp, mod, w_beg, w_end, part;
 };
 __device__ __forceinline__ Item item_of(const CrtArgs& a, unsigned i) {
   Item o;
+  o.part = i >= a.items ? 1 : 0;
+  if (o.part) i -= a.items;
   o.q = find_level(a, &CrtLv::item0, i);
   const CrtLv& v = a.lv[o.q];
   unsigned b = i - v.item0;
@@ -400,6 +493,11 @@ __device__ __forceinline__ Item item_of(const CrtArgs& a, unsigned i) {
   o.w_beg = o.grp * v.nw / v.G;
   o.w_end = (o.grp + 1) * v.nw / v.G;
   return o;
+}
+
+// An item of the second part whose tile holds no weak target is left out.
+__device__ __forceinline__ bool left_out(const CrtLv& v, const Item& t) {
+  return t.part && !__any_sync(0xffffffffu, v.need[need_index(v, t.r, t.ct, t.z0, t.y0, t.x0)] != 0);
 }
 
 // One item: one modulus, one target tile (128 boxes of a class), one column
@@ -422,6 +520,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
   // uniform for the compiler: the roles of warps 8 to 10 run converged
   const int wu = (int)__reduce_or_sync(0xffffffffu, (unsigned)warp);
   const int S = a.stages;
+  const unsigned items = __reduce_or_sync(0xffffffffu, a.any && *a.any ? 2u * a.items : a.items);
   const uint32_t sbase = smem_u32(smem);
   const uint32_t s_stage = sbase + kWins * a.win_b;
   uint64_t* bars = (uint64_t*)(smem + kWins * a.win_b + (uint32_t)S * a.stage_b);
@@ -468,9 +567,10 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     int it = 0, st = 0;
     uint32_t ph = 0, dst = s_stage;
     bool ok = true;
-    for (unsigned i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
+    for (unsigned i = blockIdx.x; i < items && ok; i += gridDim.x) {
       const Item t = item_of(a, i);
       const CrtLv& v = a.lv[t.q];
+      if (left_out(v, t)) continue;
       const int64_t tile_b = (int64_t)v.K * v.Nt * 2, slot_b = v.NT * tile_b;  // bytes of a column tile, of a slot
       const char* img = (const char*)v.img + (int64_t)t.mod * v.nslots * slot_b + t.nt * tile_b;
       const int n0 = v.n0, ks0 = v.ks0, ks1 = v.ks1, nchunk = v.nchunk;
@@ -507,9 +607,10 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     int wi = 0, s = 0;
     uint32_t wph = 0;
     bool ok = true;
-    for (unsigned i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
+    for (unsigned i = blockIdx.x; i < items && ok; i += gridDim.x) {
       const Item t = item_of(a, i);
       const CrtLv& v = a.lv[t.q];
+      if (left_out(v, t)) continue;
       for (int w = t.w_beg; w < t.w_end && ok; ++w) {
         const Win wn = window_of(v, t.ct, w);
         int k0 = 0;
@@ -523,8 +624,8 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
             mbar_expect_tx(wfull(s), (uint32_t)ks * kWinStep);
             for (int kk = 0; kk < ks; ++kk)
               tma_load_5d(sbase + (uint32_t)s * a.win_b + (uint32_t)kk * kWinStep, &maps.m[t.q], 8 * (t.x0 - 1),
-                          t.y0 + wn.sy1 - 1, t.z0 - 1 - v.sz0, 2 * (k0 + kk), (t.mod * v.Rc + t.r) * v.ncs + wn.cs,
-                          wfull(s));
+                          t.y0 + wn.sy1 - 1, t.z0 - 1 - v.sz0, 2 * (k0 + kk),
+                          t.part * v.pstep + (t.mod * v.Rc + t.r) * v.ncs + wn.cs, wfull(s));
           }
           __syncwarp();
           k0 += ks;
@@ -575,9 +676,10 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
           if (++st == S) st = 0, ph ^= 1u, blo = blo0;
         }
     };
-    for (unsigned i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
+    for (unsigned i = blockIdx.x; i < items && ok; i += gridDim.x) {
       const Item t = item_of(a, i);
       const CrtLv& v = a.lv[t.q];
+      if (left_out(v, t)) continue;
       const int n0 = v.n0, ks0 = v.ks0, ks1 = v.ks1, nchunk = v.nchunk;
       const uint64_t dB = desc_k(0, (uint32_t)v.Nt * 16u, 128u);
       lbo = (uint32_t)dB;
@@ -611,9 +713,10 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     const float2 mg = make_float2(12582912.0f, 12582912.0f), ng2 = make_float2(-12582912.0f, -12582912.0f);
     int g = 0;
     bool have = true;
-    for (unsigned it = blockIdx.x; it < a.items && have; it += gridDim.x) {
+    for (unsigned it = blockIdx.x; it < items && have; it += gridDim.x) {
       const Item t = item_of(a, it);
       const CrtLv& v = a.lv[t.q];
+      if (left_out(v, t)) continue;
       const int Nt = v.Nt, nh = Nt / 2;
       const float fm = (float)crt_mod(t.mod);
       const float2 inv2 = make_float2(1.0f / fm, 1.0f / fm), m2 = make_float2(-fm, -fm);
@@ -650,7 +753,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
       const int x = t.x0 + (row & 7), y = t.y0 + ((row >> 3) & 3), z = t.z0 + (row >> 5);
       if (have && x < h && y < h && z < v.z0 + v.nz) {
         const int N = v.NT * Nt;
-        int16_t* out = v.res +
+        int16_t* out = v.res + t.part * v.rstep +
                        ((((((int64_t)t.mod * v.G + t.grp) * v.Rc + t.r) * v.nct + t.ct) * v.nz + (z - v.z0)) * h + y) *
                            (int64_t)h * N +
                        (int64_t)x * N + t.nt * Nt + half * nh;
@@ -675,19 +778,15 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
 // -------------------------------------------------------- reconstruction --
 // G / M modulo 1 = sum_i s_i y_i / m_i modulo 1, in fixed point of NW words (the
 // constants' rounding adds at most 2^(14 - 32 NW) of M; G itself is about 2^-10
-// of M, 2^-40 for Delta^t, whose terms cancel, with one word more).
+// of M, 2^-40 for Delta^t, whose terms cancel, with one word more, and down to
+// 2^-74 for the first part of a weak target, with two more).
 // A thread takes two coefficients; the result is rounded in integers, once (the
 // FP64 pipe, at 1/64 of the integer rate, took two thirds of the time: the M2L's 45
 // million sums at 262,144 points, 7 columns 1,677 -> 626 us).
 constexpr int kRebuild = 128;
 
-// (H 2^64 + L) 2^(e - 128) times c, rounded to FP64; c normal and positive
-__device__ __forceinline__ double fixed_times(unsigned long long H, unsigned long long L, int e, double c) {
-  const bool neg = (long long)H < 0;
-  if (neg) {
-    L = ~L + 1;
-    H = ~H + (L == 0);
-  }
+// +-(H 2^64 + L) 2^(e - 128) times c, rounded to FP64; c normal and positive
+__device__ __forceinline__ double fixed_times(bool neg, unsigned long long H, unsigned long long L, int e, double c) {
   if (H == 0) {
     H = L;
     L = 0;
@@ -710,29 +809,54 @@ __device__ __forceinline__ double fixed_times(unsigned long long H, unsigned lon
   return neg ? -y : y;
 }
 
-template <int NM, int NW>
-__global__ void __launch_bounds__(kRebuild)
-k_crt_rebuild(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK<NM, NW> kc) {
-  const CrtLv& v = a.lv[find_level(a, &CrtLv::rc0, blockIdx.x)];
-  const unsigned P = (unsigned)(v.d + 1) / 2;  // pairs of a row
-  const unsigned cells = (unsigned)(v.nz * v.h * v.h), rows = cells * (unsigned)(v.nct * v.Rc);
-  // the block's first pair, then a thread's within 2^16: one multiplication
-  const int64_t first = (int64_t)(blockIdx.x - v.rc0) * kRebuild;
-  const unsigned row0 = (unsigned)(first / P), t = (unsigned)(first - (int64_t)row0 * P) + threadIdx.x;
-  const unsigned dr = __umulhi(t, v.pinv), row = row0 + dr;
-  if (row >= rows) return;
-  const int c = 2 * (int)(t - dr * P);
-  const int N = v.NT * v.Nt;
-  const int64_t step = (int64_t)rows * N;
-  const int16_t* res = v.res + (int64_t)row * N + c;
-  int s0[NM], s1[NM];
+// The signed fraction p (NW words of 32 bits, the lowest first) times 2^e c.
+template <int NW>
+__device__ __forceinline__ double fraction_times(const unsigned long long (&p)[NW], int e, double c) {
+  if constexpr (NW <= 4) {
+    unsigned long long H = (p[NW - 1] << 32) | (p[NW - 2] & 0xffffffffull);
+    unsigned long long L = (p[NW - 3] << 32) | (NW == 4 ? p[0] & 0xffffffffull : 0ull);
+    const bool neg = (long long)H < 0;
+    if (neg) {
+      L = ~L + 1;
+      H = ~H + (L == 0);
+    }
+    return fixed_times(neg, H, L, e, c);
+  } else {  // the four words from the first one that counts
+    const bool neg = (p[NW - 1] >> 31) & 1;
+    unsigned w[NW + 3] = {};  // w[3] the lowest
+    unsigned long long carry = neg ? 1 : 0;
+    int t = 3;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+      carry += neg ? ~(unsigned)p[i] : (unsigned)p[i];
+      w[i + 3] = (unsigned)carry;
+      carry >>= 32;
+      if (w[i + 3]) t = i + 3;
+    }
+    unsigned long long H = 0, L = 0;
+#pragma unroll
+    for (int i = 3; i < NW + 3; ++i)
+      if (i == t) {
+        H = (unsigned long long)w[i] << 32 | w[i - 1];
+        L = (unsigned long long)w[i - 2] << 32 | w[i - 3];
+      }
+    return fixed_times(neg, H, L, e + 32 * (t - (NW + 2)), c);
+  }
+}
+
+constexpr int kMaxGroups = 8;
+// Residues of coefficients c and c + 1, the offset groups added.
+template <int NM, bool GROUPS>
+__device__ __forceinline__ void load_pair(const CrtLv& v, const int16_t* __restrict__ res, int64_t step, int (&s0)[NM],
+                                          int (&s1)[NM]) {
+  const int64_t mod = GROUPS ? v.G * step : step;
 #pragma unroll
   for (int i = 0; i < NM; ++i) {
-    const short2 u = *reinterpret_cast<const short2*>(res + i * v.G * step);
+    const short2 u = *reinterpret_cast<const short2*>(res + i * mod);
     s0[i] = u.x;
     s1[i] = u.y;
   }
-  if (v.G > 1) {
+  if (GROUPS && v.G > 1) {
     for (int k = 1; k < v.G; ++k)
 #pragma unroll
       for (int i = 0; i < NM; ++i) {
@@ -746,14 +870,11 @@ k_crt_rebuild(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK<NM
       s1[i] %= crt_mod(i);
     }
   }
-  const unsigned rr = v.Rc == 1 ? 0u : row / (cells * (unsigned)v.nct), in = row - rr * cells * (unsigned)v.nct;
-  const int r = v.r0 + (int)rr;
-  const int lh = 31 - __clz(v.h);  // h is a power of two
-  const unsigned cz = in >> (2 * lh), cls = v.nct == 1 ? 0u : cz / (unsigned)v.nz;
-  const int64_t I = class_box(v.nct, (int)cls, (int)(in & (v.h - 1)), (int)((in >> lh) & (v.h - 1)),
-                              v.z0 + (int)(cz - cls * v.nz));
-  double* g = v.g + (I * v.R + r) * v.d + c;
-  const unsigned long long bits = v.wmax[r];
+}
+// The sums from their residues.
+template <int NM, int NW>
+__device__ __forceinline__ void rebuild_pair(const CrtLv& v, const CrtK<NM, NW>& kc, const int (&s0)[NM],
+                                             const int (&s1)[NM], int c, int e, bool fin, double* y) {
   unsigned long long p[2][NW] = {};
 #pragma unroll
   for (int i = 0; i < NM; ++i) {
@@ -766,20 +887,69 @@ k_crt_rebuild(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK<NM
       p[1][w] += (unsigned long long)u1 * kc.k[i][w];
     }
   }
-  const bool fin = w_finite(bits);
-  // colscale is in units of 2^(-32 NW)
-  const int e = 32 * NW - w_exp(bits, v.wbits);
-  const double* add = v.add ? v.add + (I * v.R + r) * v.d + c : nullptr;
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
+    y[k] = 0.0;
     if (c + k >= v.d) break;
 #pragma unroll
     for (int w = 1; w < NW; ++w) p[k][w] += p[k][w - 1] >> 32;
-    const unsigned long long H = (p[k][NW - 1] << 32) | (p[k][NW - 2] & 0xffffffffull);
-    const unsigned long long L = (p[k][NW - 3] << 32) | (NW == 4 ? p[k][0] & 0xffffffffull : 0ull);
-    double y = fin ? fixed_times(H, L, e, v.colscale[c + k]) : __longlong_as_double(0x7ff8000000000000ll);
-    g[k] = add ? add[k] + y : y;
+    y[k] = fin ? fraction_times<NW>(p[k], e, v.colscale[c + k]) : __longlong_as_double(0x7ff8000000000000ll);
   }
+}
+
+// One block of coefficient pairs; WEAK: both parts of the weak targets among them.
+template <int NM, int NW, bool GROUPS, bool WEAK>
+__device__ __forceinline__ void rebuild_block(const CrtArgs& a, const CrtK<NM, NW>& kc, unsigned block) {
+  const CrtLv& v = a.lv[find_level(a, &CrtLv::rc0, block)];
+  const unsigned P = (unsigned)(v.d + 1) / 2;  // pairs of a row
+  const unsigned cells = (unsigned)(v.nz * v.h * v.h), rows = cells * (unsigned)(v.nct * v.Rc);
+  // the block's first pair, then a thread's within 2^16: one multiplication
+  const int64_t first = (int64_t)(block - v.rc0) * kRebuild;
+  const unsigned row0 = (unsigned)(first / P), t = (unsigned)(first - (int64_t)row0 * P) + threadIdx.x;
+  const unsigned dr = __umulhi(t, v.pinv), row = row0 + dr;
+  if (row >= rows) return;
+  const int c = 2 * (int)(t - dr * P);
+  const int N = v.NT * v.Nt;
+  const int64_t step = (int64_t)rows * N;
+  const int16_t* res = v.res + (int64_t)row * N + c;
+  int s0[NM], s1[NM];
+  if (!GROUPS) load_pair<NM, GROUPS>(v, res, step, s0, s1);
+  const unsigned rr = v.Rc == 1 ? 0u : row / (cells * (unsigned)v.nct), in = row - rr * cells * (unsigned)v.nct;
+  const int r = v.r0 + (int)rr;
+  const int lh = 31 - __clz(v.h);  // h is a power of two
+  const unsigned cz = in >> (2 * lh), cls = v.nct == 1 ? 0u : cz / (unsigned)v.nz;
+  const int64_t I = class_box(v.nct, (int)cls, (int)(in & (v.h - 1)), (int)((in >> lh) & (v.h - 1)),
+                              v.z0 + (int)(cz - cls * v.nz));
+  if (WEAK && !v.weak[I * v.R + r]) return;
+  double* g = v.g + (I * v.R + r) * v.d + c;
+  const unsigned long long bits = v.wmax[(I >> v.tshift) * v.R + r];
+  const bool fin = w_finite(bits);
+  // colscale is in units of 2^(-32 NW), NW of the mode
+  const int e = (NM == kMods ? 96 : 128) - w_exp(bits, v.wbits);
+  const double* add = v.add ? v.add + (I * v.R + r) * v.d + c : nullptr;
+  double y[2];
+  if (GROUPS) load_pair<NM, GROUPS>(v, res, step, s0, s1);
+  rebuild_pair<NM, NW>(v, kc, s0, s1, c, e, fin, y);
+  if (WEAK) {
+    double z[2];
+    load_pair<NM, GROUPS>(v, res + v.rstep, step, s0, s1);
+    rebuild_pair<NM, NW>(v, kc, s0, s1, c, e - kRestBits, fin, z);
+    y[0] += z[0];
+    y[1] += z[1];
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+    if (c + k < v.d) g[k] = add ? add[k] + y[k] : y[k];
+}
+template <int NM, int NW, bool GROUPS>
+__global__ void __launch_bounds__(kRebuild)
+k_crt_rebuild(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK<NM, NW> kc) {
+  rebuild_block<NM, NW, GROUPS, false>(a, kc, blockIdx.x);
+}
+__global__ void __launch_bounds__(kRebuild)
+k_crt_rebuild_weak(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK<kMods, 5> kc) {
+  if (*a.any == 0) return;
+  for (unsigned b = blockIdx.x; b < a.rebuild_blocks; b += gridDim.x) rebuild_block<kMods, 5, true, true>(a, kc, b);
 }
 
 // ---------------------------------------------------------- the images --
@@ -1042,13 +1212,13 @@ int mode_mods(CrtMode m) { return m == kCrtBox ? kBoxMods : kMods; }
 int mode_ncs(CrtMode m) { return m == kCrtL2L ? 1 : 8; }
 int mode_nct(CrtMode m) { return m == kCrtM2M ? 1 : 8; }
 int mode_h(CrtMode m, int level) { return m == kCrtM2M ? 1 << level : 1 << (level - 1); }
+int mode_parts(CrtMode m) { return m == kCrtM2L ? 2 : 1; }
 size_t planes_bytes(CrtMode m, int K, int h, int snz, int Rc) {
-  return align256((size_t)mode_mods(m) * Rc * mode_ncs(m) * snz * h * h * K * 2);
+  return align256((size_t)mode_parts(m) * mode_mods(m) * Rc * mode_ncs(m) * snz * h * h * K * 2);
 }
 size_t res_bytes(CrtMode m, int N, int h, int nz, int Rc, int G) {
-  return align256((size_t)mode_mods(m) * G * Rc * mode_nct(m) * nz * h * h * N * 2);
+  return align256((size_t)mode_parts(m) * mode_mods(m) * G * Rc * mode_nct(m) * nz * h * h * N * 2);
 }
-constexpr int kMaxGroups = 8;
 // offset groups are used only by M2L and M2M launches of few tiles: levels below this one
 constexpr int kGroupLevel = 4;
 int max_groups(CrtMode m, int level) {
@@ -1058,6 +1228,9 @@ size_t job_bytes(CrtMode m, const CrtImage& im, int level, int nz, int Rc) {
   const int h = mode_h(m, level);
   const int snz = std::min(h, nz + 2);
   return planes_bytes(m, im.K, h, snz, Rc) + res_bytes(m, im.NT * im.Nt, h, nz, Rc, max_groups(m, level));
+}
+int64_t need_tiles(int h, int nz, int Rc) {
+  return (int64_t)((h + kTX - 1) / kTX) * ((h + kTY - 1) / kTY) * ((nz + kTZ - 1) / kTZ) * 8 * Rc;
 }
 // columns and planes of one slab of a level within `limit` bytes
 void slab_shape(CrtMode m, const CrtImage& im, int level, int R, size_t limit, int* Rc, int* nz) {
@@ -1081,10 +1254,33 @@ size_t crt_scratch_bytes(int njobs, const CrtJob* jobs, int R) {
   return std::max(most, std::min(total, kScratchLimit));
 }
 
+bool crt_steep(int kern, double L, int level) {
+  const double w = L * std::ldexp(1.0, -level);
+  double near = 0.0, far = 0.0;
+  for (int a = 0; a < 3; ++a)
+    near = std::max(near, std::fabs(kern_f64(kern, a == 0 ? w : 0.0, a == 1 ? w : 0.0, a == 2 ? w : 0.0)));
+  for (int i = 0; i < 32; ++i) {  // several distances: the kernel may oscillate
+    const double z = 4.0 * w * (0.9 + 0.1 * i / 31.0);
+    far = std::max(far, std::fabs(kern_f64(kern, z, z, z)));
+  }
+  return !(near > 0.0 && far >= 0x1p-7 * near);
+}
+
 bool crt_ready(CrtMode mode, int level, const CrtImage& im, int R, size_t bytes) {
   if (!im.img || bytes == 0) return false;
   const CrtJob job{mode, level, &im, nullptr, nullptr, nullptr};
   return crt_scratch_bytes(1, &job, R) <= bytes;
+}
+
+// [kMaxLevel + 1][R] maxima of the M2L's levels, the word `any`, the tiles' `need`,
+// the boxes' maxima, their `weak`; or the maxima of another mode's units
+size_t crt_max_words(int depth, int R) {
+  size_t boxes = 0, tiles = 0;
+  for (int k = 2; k <= depth; ++k) {
+    boxes += (size_t)1 << (3 * k);
+    tiles += need_tiles(1 << (k - 1), 1 << (k - 1), R);
+  }
+  return (size_t)(kMaxLevel + 1) * R + 1 + (tiles + 7) / 8 + boxes * R + (boxes * R + 7) / 8;
 }
 
 void free_crt_image(CrtImage* im) {
@@ -1200,6 +1396,7 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     return EIFMM_ECUDA;
   }
   static const CrtK<kMods, 3> kc = crt_constants<kMods, 3>();
+  static const CrtK<kMods, 5> kweak = crt_constants<kMods, 5>();
   static const CrtK<kBoxMods, 4> kcb = crt_constants<kBoxMods, 4>();
   static bool attr[64] = {};
   int dev = 0;
@@ -1208,7 +1405,28 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     EIFMM_CUDA(cudaFuncSetAttribute(k_crt_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
     if (dev < 64) attr[dev] = true;
   }
-  EIFMM_CUDA(cudaMemsetAsync(wmax, 0, sizeof(unsigned long long) * (kMaxLevel + 1) * R, s));
+  const bool m2l = njobs > 0 && jobs[0].mode == kCrtM2L;
+  unsigned* any = nullptr;
+  unsigned char *need = nullptr, *weak[kMaxLevel + 1] = {};
+  unsigned long long* bmax[kMaxLevel + 1] = {};
+  if (m2l) {
+    unsigned long long* p = wmax + (size_t)(kMaxLevel + 1) * R;
+    any = (unsigned*)p++;
+    need = (unsigned char*)p;
+    size_t boxes = 0, tiles = 0;
+    for (int j = 0; j < njobs; ++j) tiles += need_tiles(1 << (jobs[j].level - 1), 1 << (jobs[j].level - 1), R);
+    p += (tiles + 7) / 8;
+    EIFMM_CUDA(cudaMemsetAsync(wmax, 0, (char*)p - (char*)wmax, s));
+    for (int j = 0; j < njobs; ++j) {
+      bmax[jobs[j].level] = p + boxes * R;
+      boxes += (size_t)1 << (3 * jobs[j].level);
+    }
+    unsigned char* c = (unsigned char*)(p + boxes * R);
+    for (int j = 0; j < njobs; ++j) {
+      weak[jobs[j].level] = c;
+      c += ((size_t)1 << (3 * jobs[j].level)) * R;
+    }
+  }
   // slabs of all jobs, largest levels first; consecutive ones that fit the
   // scratch together share their launches
   std::vector<CrtLv> todo;
@@ -1247,7 +1465,15 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
         v.add = b.add;
         v.img = (const __nv_bfloat16*)b.img->img;
         v.colscale = b.img->colscale;
-        v.wmax = wmax + (size_t)b.level * R;
+        v.sshift = b.mode == kCrtM2L ? 3 * b.level : b.mode == kCrtM2M ? 3 : 0;
+        v.tshift = b.mode == kCrtM2L ? 3 * b.level : b.mode == kCrtL2L ? 3 : 0;
+        v.wmax = b.mode == kCrtM2L ? wmax + (size_t)b.level * R : wmax;
+        if (m2l) {
+          v.bmax = bmax[b.level];
+          v.weak = weak[b.level];
+          v.need = need;
+          need += need_tiles(h, v.nz, v.Rc);
+        }
         todo.push_back(v);
       }
   }
@@ -1255,6 +1481,7 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     CrtArgs a = {};
     CrtMaps maps = {};
     a.err = err;
+    a.any = any;
     size_t off = 0, i1 = i0;
     int64_t items = 0;
     auto tiles = [](const CrtLv& v) {
@@ -1278,6 +1505,7 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     unsigned it = 0, pl = 0, rb = 0, mx = 0;
     uint32_t stage = 0, win = 0;
     size_t pl_smem = 0;
+    bool groups = false;
     for (int q = 0; q < a.nlev; ++q) {
       CrtLv& v = a.lv[q];
       // a launch of few tiles: the windows of the coarse levels' tiles are
@@ -1287,8 +1515,11 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
       v.G = 1;
       const int64_t most = (v.mode == kCrtM2M ? nsm : 8 * (int64_t)nsm - 1) / 2;
       while (v.G < max_groups(v.mode, v.tlevel) && items * v.G <= most) v.G *= 2;
+      groups = groups || v.G > 1;
       for (int ct = 0; ct < v.nct; ++ct)
         for (int p = 0; p < v.G; ++p) v.ng[ct][p] = (uint16_t)accumulations(v, ct, p);
+      v.pstep = mode_mods(v.mode) * v.Rc * v.ncs;
+      v.rstep = (int64_t)mode_mods(v.mode) * v.G * v.Rc * v.nct * v.nz * v.h * v.h * v.NT * v.Nt;
       v.planes = (__nv_bfloat16*)((char*)buf + off);
       off += planes_bytes(v.mode, v.K, v.h, v.snz, v.Rc);
       v.res = (int16_t*)((char*)buf + off);
@@ -1308,7 +1539,7 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
       win = std::max(win, ks * kWinStep);
       pl_smem = std::max(pl_smem, (size_t)8 * (v.K + 1) * sizeof(long long));
       const cuuint64_t hh = (cuuint64_t)v.h;
-      cuuint64_t dims[5] = {8 * hh, hh, (cuuint64_t)v.snz, (cuuint64_t)v.K / 8, (cuuint64_t)mode_mods(v.mode) * v.Rc * v.ncs};
+      cuuint64_t dims[5] = {8 * hh, hh, (cuuint64_t)v.snz, (cuuint64_t)v.K / 8, (cuuint64_t)mode_parts(v.mode) * v.pstep};
       cuuint64_t strides[4] = {16 * hh, 16 * hh * hh, 16 * hh * hh * v.snz, 16 * hh * hh * v.snz * (v.K / 8)};
       cuuint32_t box[5] = {8 * (kTX + 2), kTY, kTZ + 2, 2, 1};
       cuuint32_t estr[5] = {1, 1, 1, 1, 1};
@@ -1333,11 +1564,22 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     else k_crt_planes<kMods><<<pl, 256, pl_smem, s>>>(a);
     EIFMM_CHECK_LAUNCH();
     a.items = it;
+    a.plane_blocks = pl;
+    a.rebuild_blocks = rb;
+    if (m2l) {
+      k_crt_planes_rest<kMods><<<std::min(pl, 4 * (unsigned)nsm), 256, pl_smem, s>>>(a);
+      EIFMM_CHECK_LAUNCH();
+    }
     k_crt_gemm<<<std::min(it, (unsigned)nsm), kThreads, smem, s>>>(maps, a);
     EIFMM_CHECK_LAUNCH();
-    if (box) k_crt_rebuild<kBoxMods, 4><<<rb, kRebuild, 0, s>>>(a, kcb);
-    else k_crt_rebuild<kMods, 3><<<rb, kRebuild, 0, s>>>(a, kc);
+    if (box) k_crt_rebuild<kBoxMods, 4, false><<<rb, kRebuild, 0, s>>>(a, kcb);
+    else if (groups) k_crt_rebuild<kMods, 3, true><<<rb, kRebuild, 0, s>>>(a, kc);
+    else k_crt_rebuild<kMods, 3, false><<<rb, kRebuild, 0, s>>>(a, kc);
     EIFMM_CHECK_LAUNCH();
+    if (m2l) {
+      k_crt_rebuild_weak<<<std::min(rb, 8 * (unsigned)nsm), kRebuild, 0, s>>>(a, kweak);
+      EIFMM_CHECK_LAUNCH();
+    }
     i0 = i1;
   }
   return EIFMM_OK;

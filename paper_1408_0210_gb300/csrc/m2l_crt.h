@@ -20,13 +20,25 @@ struct CrtJob {
   double* g;
   const double* add;
 };
+// Words for the largest |W| of the units that share a scale (a level of the M2L
+// and its boxes, a box of a tree of this depth elsewhere) and the marks of the
+// M2L's second part.
+size_t crt_max_words(int depth, int R);
 // Scratch for the jobs of one call (M2L jobs run together, others one by one);
 // jobs beyond the library's limit run in slabs and columns.
 size_t crt_scratch_bytes(int njobs, const CrtJob* jobs, int R);
+// Whether the kernel falls off so steeply within an interaction list that the M2L
+// of this level stays on the FP32 or FP64 pipes.  The operators of all offsets
+// share one scale per row, 60 bits for its largest entry; between the closest
+// separated points, a box width w apart, and the farthest, 4 sqrt(3) w, 1/r falls
+// to 2^-2.8 and an entry keeps 57 bits, exp(-r^2) at w = 1/2 to 2^-17.  53 bits
+// are left down to 2^-7.
+bool crt_steep(int kern, double L, int level);
 // Whether a job of this image can run in `bytes` of scratch.
 bool crt_ready(CrtMode mode, int level, const CrtImage& img, int R, size_t bytes);
-// All jobs on stream s, in `buf` (buf_bytes from crt_scratch_bytes); wmax:
-// [kMaxLevel + 1][R] words; err: error word of the bounded waits.
+// M2L jobs, or one job of another mode, on stream s, in `buf` (buf_bytes from
+// crt_scratch_bytes); wmax: crt_max_words(depth, R) words; err: error word of the
+// bounded waits.
 eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t buf_bytes, unsigned long long* wmax,
                         int nsm, int* err, cudaStream_t s);
 // The residue image of an operator stack [nslots][l < dl][m' < d].

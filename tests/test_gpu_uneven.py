@@ -3,13 +3,16 @@ cube and 1e-14 in the opposite one, every step compared with the CPU EIFMM box b
 box, so that a weak box has to keep its own digits.
 
 exp(-r^2) on a cube of edge 8 leaves the weak corner to its own charges (the strong
-ones are at e^-48 there); 1/r carries the strong ones everywhere.
+ones are at e^-48 there) and the M2L to the FP64 pipes or FP32 pairs; 1/r carries the
+strong ones everywhere, and its M2L runs in residues.
 
 Tolerances: W, l and f are sums of at most 8 d and 189 d products in FP64 on both
 sides, each sum with errors of 189 d 2^-53 (8e-12 at d = 340) of its absolute terms;
 these exceed the results by 7 (exp) and 19 (1/r) at level 4, positive charges: 1e-9
 for a box or a target.  g: 10 * 189 d 2^-53 of the absolute terms, summed here.
 FP32 pairs (tier 4): 2^-46 a product instead."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -90,3 +93,50 @@ def test_weak_boxes_keep_their_digits(E, orc, kern, L, prec):
     A = orc.kernel(kern, (X[:, None] - Y[None]).reshape(-1, 3)).reshape(d, d)
     lh, ll = (E.eifmm_debug_export(tree, w, DEPTH, d)[:, 0] for w in (4, 3))
     assert (np.abs(lh @ A - ll).max(1) <= 1e-12 * (np.abs(lh) @ np.abs(A)).max(1)).all()
+
+
+
+def ints(a, e):
+    """a 2^e as exact integers."""
+    return np.array([int(Fraction(float(v)) * 2 ** e) for v in a.ravel()], dtype=object).reshape(a.shape)
+
+
+# Operators without rounding: Gamma = B = 1 (Delta = 1), K(z) = |z|^2 and nodes on a
+# grid, so that T^delta = K^delta is exact.  The exported W then gives g exactly, and
+# the residue M2L's error is the rounding of W, at most 2^-53 of the largest W of the
+# interaction list for every term, and one or two of the sum (each 2^-53 of the
+# absolute terms): together below 2^-51 of that W times the row sums of |T|.
+@pytest.mark.parametrize("depth,d,weak", [(4, 8, (1.0,)), (4, 17, (1.0,)), (4, 8, (2.0 ** -30,)), (4, 17, (2.0 ** -30,)),
+                                          (4, 8, (2.0 ** -55,)), (4, 17, (2.0 ** -55,)),
+                                          (5, 17, (2.0 ** -55, 1.0, 2.0 ** -20))])  # several tiles and columns
+def test_residue_m2l_is_exact_to_its_rounding(E, orc, depth, d, weak):
+    rng = np.random.default_rng(7)
+    lv = {}
+    for k in range(2, depth + 1):
+        p = rng.integers(-128, 128, (2, d, 3)) / 256.0 * 2.0 ** -k
+        lv[k] = dict(d=d, X=p[0], Y=p[1], Gamma=np.eye(d), B=np.eye(d), eps_est=1e-6)
+    x = np.concatenate([0.25 * wl.uniform_cube(N // 2, 35), 0.75 + 0.25 * wl.uniform_cube(N // 2, 36)])
+    R = len(weak)
+    s = wl.sigma_uniform(N, R, 37)
+    s[N // 2:] *= np.array(weak)
+    ops = E.eifmm_ops_load("quad", 1.0, depth, lv)
+    tree = E.eifmm_tree_build(dev(x), None, (0, 0, 0), 1.0, depth, True)
+    f = torch.zeros(R, N, dtype=torch.float64, device="cuda")
+    E.eifmm_evaluate(tree, ops, dev(s.T).T if R > 1 else dev(s[:, 0]), f.T if R > 1 else f[0], "fp64")
+    for k in (2, depth):
+        Ws, gs = (E.eifmm_debug_export(tree, w, k, d, R) for w in (0, 2))
+        Kd = orc.m2l_operators("quad", 1.0, k, lv[k])
+        boxes = np.flatnonzero(Ws[:, 0].any(1))
+        for r in range(R):
+            W, g = Ws[:, r], gs[:, r]
+            for b in (int(boxes[0]), int(boxes[1]), int(boxes[-2]), int(boxes[-1])):
+                total, largest, rows = np.zeros(d, dtype=object), 0.0, np.zeros(d)
+                for J in orc.interaction_list(k, b):
+                    if J < 0 or not W[J].any():
+                        continue
+                    t = [p - q for p, q in zip(coords(int(J), k), coords(b, k))]
+                    T = Kd[t[0] + 3 + 7 * (t[1] + 3) + 49 * (t[2] + 3)]
+                    total += ints(T, 60) @ ints(W[J], 200)
+                    largest, rows = max(largest, np.abs(W[J]).max()), rows + np.abs(T).sum(1)
+                err = [abs(float(Fraction(int(v), 2 ** 260) - Fraction(float(w)))) for v, w in zip(total, g[b])]
+                assert (np.array(err) <= 2.0 ** -51 * largest * rows).all(), (k, r, b)
