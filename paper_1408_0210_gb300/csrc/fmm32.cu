@@ -1400,7 +1400,13 @@ eifmm_status alloc_mixed_workspace(Tree* t, const Ops* ops, int R) {
         EIFMM_TRY(build_m2l_sparse(t->tgt.leaf_off, k, kap, &sp, nullptr));
         int64_t n = 0;
         for (int c : sp.cnt) n += c;
-        if (4 * n > nboxes(k)) {  // the dense tiles are cheaper to load
+        // the dense tiles are cheaper to load: a sparse one takes 1.6 times as
+        // long in many waves and three times in one (20,000 to 300,000 points on
+        // a sphere: level 5, 16 tiles 1,130 us, 128 dense ones, a wave as well,
+        // 360 us; level 6, one wave 1,170 us, seven dense ones 2,550 us)
+        const int sms = sm_count();
+        const int64_t sparse_waves = (sp.tile0[8] + sms - 1) / sms, waves = (m2l_t256_ctas(k, 1) + sms - 1) / sms;
+        if (4 * n > nboxes(k) || 3 * sparse_waves > waves) {
           dfree(sp.list);
           continue;
         }

@@ -51,3 +51,31 @@ def test_sparse_matches_dense(E, kind, n, depth, tier):
     a, b = out["sparse"][0], out["dense"][0]
     assert np.abs(a - b).max() <= 2e-5 * np.abs(b).max()
     assert np.abs(out["sparse"][2] - out["dense"][2]).max() <= 2e-5 * np.abs(out["dense"][2]).max()
+
+
+# One wave of tiles either way at level 5, seven against two at level 6: the M2L of
+# a few occupied boxes takes no longer than that of all of them.
+@pytest.mark.parametrize("depth", [5, 6])
+def test_sparse_m2l_is_not_slower(E, depth):
+    n, m = 20000, 2 ** depth
+    x = wl.sphere_surface(n, 64)
+    c = (np.arange(m) + 0.5) / m
+    fill = np.stack(np.meshgrid(c, c, c, indexing="ij"), -1).reshape(-1, 3)
+    s = dev(wl.sigma_uniform(n, 1, 65)[:, 0])
+    ops = E.eifmm_ops_build("inv_r", 1.0, depth, 1e-4)
+    ops.plan(0)
+    ms = {}
+    for name, t in (("sparse", x), ("dense", fill)):
+        tree = E.eifmm_tree_build(dev(x), dev(t), (0, 0, 0), 1.0, depth, False)
+        tree.set_option("single_stream", True)
+        f = torch.zeros(len(t), dtype=torch.float64, device="cuda")
+        E.eifmm_set_timing(True)
+        try:
+            runs = []
+            for _ in range(6):
+                E.eifmm_evaluate(tree, ops, s, f, "mixed")
+                runs.append(E.eifmm_last_step_times(tree)[9 + depth])
+        finally:
+            E.eifmm_set_timing(False)
+        ms[name] = min(runs)
+    assert ms["sparse"] <= 1.25 * ms["dense"], ms
