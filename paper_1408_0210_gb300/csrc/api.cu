@@ -100,6 +100,7 @@ void free_workspace(Workspace* ws) {
     dfree(sp.list);
     sp = M2LSparse();
   }
+  for (bool& b : ws->sparse_ran) b = false;
   ws->p2m_sparse = false;
   dfree(ws->fnear); dfree(ws->ffar); dfree(ws->tmp); dfree(ws->gsym); dfree(ws->wmax);
   ws->gsym = nullptr;

@@ -1730,7 +1730,8 @@ eifmm_status launch_m2l_level(Tree* t, const Ops* ops, int k, int R, int kind, i
     return launch_m2l_h16(a, ws.tmap[k][0], ws.tmap[k][1], ws.wmax, v.kscale, s);
   }
   const bool rule = kind == 0;
-  if (rule && ws.sparse[k].list && !t->opt[EIFMM_OPT_M2L_128ROW]) return launch_m2l_t256g(a, ws.sparse[k], s);
+  ws.sparse_ran[k] = rule && ws.sparse[k].list && !t->opt[EIFMM_OPT_M2L_128ROW];
+  if (ws.sparse_ran[k]) return launch_m2l_t256g(a, ws.sparse[k], s);
   if (rule) {
     // the transposed kernel where a parity class fills at least one of its
     // 256-row tiles; the 128-row kernel at the coarse levels
@@ -2016,15 +2017,18 @@ eifmm_status eval_mixed(Tree* t, const Ops* ops, const double* sigma, int64_t ld
 }
 
 // Steps 4 to 6 of the last evaluation again over all boxes, up to `level`, where
-// the evaluation left out boxes without targets (the values of the others stay
-// what they were, to the bit).
+// that evaluation left out boxes without targets: an export may cost a far field
+// and fail as an evaluation does.  The sparse M2L forms its sums as the dense
+// kernel with one offset group does, so that the other boxes' values stay what
+// they were, to the bit.
 static eifmm_status complete_sparse(Tree* t, const Ops* o, int level, bool lhat) {
   Workspace& ws = t->ws;
   bool any = false;
   for (int k = 5; k <= level; ++k)
-    if (ws.sparse[k].list) {
+    if (ws.sparse_ran[k]) {
       any = true;
-      EIFMM_TRY(launch_m2l_level(t, o, k, 1, 1, 0, nullptr));
+      EIFMM_TRY(launch_m2l_level(t, o, k, 1, 1, -4, nullptr));
+      ws.sparse_ran[k] = true;  // a replay of a recorded batch runs the sparse form again
     }
   for (int k = 3; any && k <= level; ++k)
     if (!xfer_blas(false, o->lv[k], o->lv[k - 1], nboxes(k - 1), 1, ws.l32[k - 1], ws.g32[k], ws.l32[k], ws.blas_ws,

@@ -206,6 +206,7 @@ struct Workspace {
   int nsm = 0;                  // SMs of the workspace's device
   uint32_t* wmax = nullptr;     // [kMaxLevel + 1] bits of max |W| per level (FP16 planes)
   M2LSparse sparse[kMaxLevel + 1];  // levels most of whose boxes hold no targets (tier 0, one right-hand side)
+  bool sparse_ran[kMaxLevel + 1] = {};  // levels whose last M2L left boxes out
   bool p2m_sparse = false;      // few leaves hold sources: rows of the others are zero from the start
   SkPlanDev sk;                 // stream-K plan of the leaf level (tier 0), when it pays
   int* err = nullptr;           // device error word of bounded waits

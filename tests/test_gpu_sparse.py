@@ -79,3 +79,31 @@ def test_sparse_m2l_is_not_slower(E, depth):
             E.eifmm_set_timing(False)
         ms[name] = min(runs)
     assert ms["sparse"] <= 1.25 * ms["dense"], ms
+
+
+def test_export_gives_what_the_evaluation_used(E):
+    """With another M2L kernel (option m2l_128row) nothing is left out and nothing is
+    run again for an export: every box's steps are those of that kernel, as on the
+    same sources with a target in every leaf; and so they are again afterwards."""
+    n, depth = 20000, 6
+    x, m = wl.sphere_surface(n, 66), 2 ** depth
+    c = (np.arange(m) + 0.5) / m
+    fill = np.stack(np.meshgrid(c, c, c, indexing="ij"), -1).reshape(-1, 3)
+    s = dev(wl.sigma_uniform(n, 1, 67)[:, 0])
+    ops = E.eifmm_ops_build("inv_r", 1.0, depth, 1e-4)
+    ops.plan(0)
+    d = ops.error_estimate(depth)[1]
+    out = {}
+    for name, t in (("sparse", x), ("dense", fill)):
+        tree = E.eifmm_tree_build(dev(x), dev(t), (0, 0, 0), 1.0, depth, False)
+        f = torch.zeros(len(t), dtype=torch.float64, device="cuda")
+        for row in (True, False, True):
+            tree.set_option("m2l_128row", row)
+            E.eifmm_evaluate(tree, ops, s, f, "mixed")
+            for again in range(2):  # an export changes nothing for the next one
+                out[name, row, again] = [E.eifmm_debug_export(tree, w, depth, d) for w in (2, 3, 4)]
+    for row in (True, False):
+        for again in range(2):
+            for a, b in zip(out["sparse", row, again], out["dense", row, 0]):
+                assert np.array_equal(a, b), (row, again)
+    assert not np.array_equal(out["dense", True, 0][0], out["dense", False, 0][0])
