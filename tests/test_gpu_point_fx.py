@@ -100,3 +100,10 @@ def test_point_kernels(E, kern, n, lo, L, depth, R, tiny, two):
         K = kernel(kern, y[i], x[j])
         ref, mag = K @ s[j].astype(LD), K @ np.abs(s[j]).astype(LD)
         assert (np.abs(near[i] - ref) <= (len(j) + ulps) * u * mag).all()
+
+
+# From depth 7 on the nearest nodes lie closer than the integers of box-relative
+# coordinates reach (L / 64 here): one warp takes both forms.
+@pytest.mark.parametrize("kern", ["inv_r", "config3"])
+def test_point_kernels_on_a_deep_tree(E, kern):
+    test_point_kernels(E, kern, 300, (0.0, 0.0, 0.0), 1.0, 7, 1, 0.02, False)

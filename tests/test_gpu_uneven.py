@@ -96,6 +96,25 @@ def test_weak_boxes_keep_their_digits(E, orc, kern, L, prec):
 
 
 
+def test_pair_arithmetic_m2l(E):
+    """A steep kernel's M2L in tiers 3 and 4 runs in FP32 pairs: against the FP64 pipes
+    (option m2l_fp64) 1e-10 of the leaf level's largest g (a product is good to 2^-47,
+    the absolute terms are 7 times the result, 22,000 terms), and not the same bits."""
+    x, s = 8.0 * wl.uniform_cube(N, 38), dev(wl.sigma_uniform(N, 1, 39)[:, 0])
+    ops = E.eifmm_ops_build("exp_r2", 8.0, DEPTH, 1e-6)
+    tree = E.eifmm_tree_build(dev(x), None, (0, 0, 0), 8.0, DEPTH, True)
+    d = ops.error_estimate(DEPTH)[1]
+    for tier in (3, 4):
+        ops.plan(tier)
+        g = {}
+        for fp64 in (True, False):
+            tree.set_option("m2l_fp64", fp64)
+            E.eifmm_evaluate(tree, ops, s, torch.zeros(N, dtype=torch.float64, device="cuda"), "mixed")
+            g[fp64] = E.eifmm_debug_export(tree, 2, DEPTH, d)
+        diff = np.abs(g[True] - g[False]).max()
+        assert 0.0 < diff <= 1e-10 * np.abs(g[True]).max()
+
+
 def ints(a, e):
     """a 2^e as exact integers."""
     return np.array([int(Fraction(float(v)) * 2 ** e) for v in a.ravel()], dtype=object).reshape(a.shape)
