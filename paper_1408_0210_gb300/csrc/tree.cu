@@ -343,14 +343,19 @@ __global__ void k_gather_points(const double* __restrict__ xyz,
   lz[p] = (float)(pz - s_ctr[2 * nc + c[2]]);
 }
 
-// cnt[0]: their number, cnt[1]: the points of the fullest
+// cnt[0]: their number, cnt[kFullest]: the points of the fullest, in a cache line of
+// its own, which an SM reads from L1; next to the counter every read went to L2
+// between the additions.  Tree build of 2^20 points in 2^27 leaves: 3.75 ms; next to
+// the counter 4.18, with a reduction in every warp, empty ones too, 4.69.
+constexpr int kFullest = 32;
+constexpr int kCounters = 2 + kFullest;  // points outside the cube, then cnt
 __global__ void k_nonempty(const int32_t* __restrict__ off, int64_t nleaf,
                            int32_t* __restrict__ list, int32_t* __restrict__ cnt) {
   const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int n = b < nleaf ? off[b + 1] - off[b] : 0;
-  if (n > 0) list[atomicAdd(cnt, 1)] = (int32_t)b;
-  const int most = __reduce_max_sync(0xffffffffu, n);
-  if ((threadIdx.x & 31) == 0 && most > cnt[1]) atomicMax(cnt + 1, most);
+  if (n == 0) return;
+  list[atomicAdd(cnt, 1)] = (int32_t)b;
+  if (n > cnt[kFullest]) atomicMax(cnt + kFullest, n);  // an old count only costs an atomic more
 }
 
 struct SortScratch {
@@ -395,7 +400,7 @@ eifmm_status build_pointset(const double* xyz, int64_t n, const double lo[3],
   const int nb1 = nblocks > 0 ? nblocks : 1;
   size_t soff = 0;
   const size_t o_pairs = take(soff, nn * 8), o_cnt = take(soff, (size_t)RS_DIGITS * nb1 * 4),
-               o_tot = take(soff, RS_DIGITS * 4), o_bad = take(soff, 3 * sizeof(int));
+               o_tot = take(soff, RS_DIGITS * 4), o_bad = take(soff, kCounters * sizeof(int));
   // The sort's scratch is kept per device between builds (grown on demand,
   // held until the process exits); builds on one device take turns on it.
   int dev = 0;
@@ -412,7 +417,7 @@ eifmm_status build_pointset(const double* xyz, int64_t n, const double lo[3],
   unsigned char* scratch = sc.p;
   const SortBuffers sb{(uint2*)(scratch + o_pairs), (uint32_t*)(scratch + o_cnt), (uint32_t*)(scratch + o_tot)};
   int* dbad = (int*)(scratch + o_bad);
-  EIFMM_CUDA(cudaMemsetAsync(dbad, 0, 3 * sizeof(int), s));
+  EIFMM_CUDA(cudaMemsetAsync(dbad, 0, kCounters * sizeof(int), s));
 
   if (n > 0) EIFMM_TRY(sort_points(xyz, n, lo, L, depth, ps->keys, ps->perm, sb, dbad, s));
   k_leaf_off<<<(unsigned)((nleaf + 1 + 255) / 256), 256, 0, s>>>(ps->keys, n, nleaf, ps->leaf_off);
@@ -426,11 +431,11 @@ eifmm_status build_pointset(const double* xyz, int64_t n, const double lo[3],
   }
   k_nonempty<<<(unsigned)((nleaf + 255) / 256), 256, 0, s>>>(ps->leaf_off, nleaf, ps->nonempty, dbad + 1);
   EIFMM_CHECK_LAUNCH();
-  int hb[3] = {0, 0, 0};
-  EIFMM_CUDA(cudaMemcpyAsync(hb, dbad, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  int hb[kCounters] = {};
+  EIFMM_CUDA(cudaMemcpyAsync(hb, dbad, kCounters * sizeof(int), cudaMemcpyDeviceToHost, s));
   EIFMM_CUDA(cudaStreamSynchronize(s));
   ps->n_nonempty = hb[1];
-  ps->max_leaf = hb[2];
+  ps->max_leaf = hb[1 + kFullest];
   if (hb[0] != 0) {
     set_error("eifmm_tree_build: " + std::to_string(hb[0]) +
               " coordinates lie outside the cube [lo, lo + L]^3");
