@@ -1850,11 +1850,11 @@ eifmm_status eval_mixed(Tree* t, const Ops* ops, const double* sigma, int64_t ld
       if (g == 0) {
         // no sources: every row is zero
       } else if (acc)
-        k_p2m32x<true><<<g, 32 * PT_WARPS, 0, s>>>(list, nl, S.leaf_off, nboxes(kap), S.lx, S.ly, S.lz, ws.sig32, vl.X32,
-                                                   vl.d, vl.dp, ws.W32[kap], lp, gl, sigma, S.perm);
+        k_p2m32x<true><<<g, 32 * PT_WARPS, 0, s>>>(list, nl, S.leaf_off, nboxes(kap), S.lx, S.ly, S.lz, ws.sig32,
+                                                   vl.X32, vl.d, vl.dp, ws.W32[kap], lp, gl, sigma, S.perm);
       else
-        k_p2m32x<false><<<g, 32 * PT_WARPS, 0, s>>>(list, nl, S.leaf_off, nboxes(kap), S.lx, S.ly, S.lz, ws.sig32, vl.X32,
-                                                    vl.d, vl.dp, ws.W32[kap], lp, gl, sigma, S.perm);
+        k_p2m32x<false><<<g, 32 * PT_WARPS, 0, s>>>(list, nl, S.leaf_off, nboxes(kap), S.lx, S.ly, S.lz, ws.sig32,
+                                                    vl.X32, vl.d, vl.dp, ws.W32[kap], lp, gl, sigma, S.perm);
     } else {
       EIFMM_POINT_DISPATCH(EIFMM_P2M);
     }

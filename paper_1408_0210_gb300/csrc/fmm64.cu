@@ -162,8 +162,9 @@ k_m2l64(int level, int d, int R, const double* __restrict__ kdT,
 }
 
 
-// Step 4 of tiers 3 and 4 for operators that amplify rounding
-// (kCrtMaxKappa in internal.h), with the FP64 numbers carried as unevaluated sums of two FP32 numbers (hi + lo, about 46
+// Step 4 of tiers 3 and 4 where the residue M2L does not run (operators that amplify
+// rounding, kCrtMaxKappa in internal.h, or fall off steeply, crt_steep; no room for its
+// image), with the FP64 numbers carried as unevaluated sums of two FP32 numbers (hi + lo, about 46
 // significant bits) on the FP32 pipes, which run 72 times faster than the
 // FP64 ones on this GPU.  Each product hi_a hi_b is split exactly with an
 // FMA (p + e), the cross terms hi_a lo_b + lo_a hi_b are added in FP32, and
@@ -569,7 +570,8 @@ eifmm_status eval_fp64(Tree* t, const Ops* ops, const double* sigma, int64_t ld_
   // last bits of W: there W comes from the FP64 pipes as before.
   bool pairs = false;
   for (int k = 2; k <= kap; ++k)
-    pairs = pairs || (pair_m2l && !t->opt[EIFMM_OPT_M2L_FP64] && !ops->compressed && ops->lv[k].crt.kappa > kCrtMaxKappa);
+    pairs = pairs || (pair_m2l && !t->opt[EIFMM_OPT_M2L_FP64] && !ops->compressed &&
+                      ops->lv[k].crt.kappa > kCrtMaxKappa);
   if (ws.fx_src && !pairs) {
     EIFMM_TRY(launch_p2m_fx(t, kern, vl, R, ws.W[kap], s));
   } else if (S.n_nonempty > 0) {

@@ -330,11 +330,12 @@ eifmm_status launch_m2l64(int level, int d, int R, const double* kdT, const int*
 eifmm_status m2l_compressed(Workspace& ws, const Ops* ops, int k, int R, bool fp64, bool pair, cudaStream_t s);
 // Smallest rank that runs on the tensor cores.
 constexpr int kCrtMinRank = 8;
-// Operators with a larger crt_kappa keep FP32 pairs in tiers 3 and 4: there the
+// Operators with a larger crt_kappa keep FP32 pairs in tiers 3 and 4.  A choice,
+// not a bound: the residues would be faster and more accurate there too, but the
 // pairs' own rounding shows in the result (measured 1.3e-14 kappa of f: 1e-8 for
 // the config-3 kernel at eps 1e-6, kappa 7.7e5, and 3.5e-12 for 1/r at 1e-7,
-// kappa 1.2e3), and those results stay what they were.  The FP64 path, whose
-// rounding is 1000 times smaller, takes the residues for all operators.
+// kappa 1.2e3), so that f would move by as much (config-3: 1e-8, a hundredth of
+// eps).  The FP64 path takes the residues for all operators.
 constexpr double kCrtMaxKappa = 1e4;
 void free_workspace(Workspace* ws);
 uint64_t next_generation();  // unique in the process

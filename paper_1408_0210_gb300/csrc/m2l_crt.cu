@@ -373,7 +373,8 @@ __device__ __forceinline__ void mark_weak(const CrtArgs& a, const CrtLv& v, int 
   bool some = false, strong = !w_finite(level);
   for (int i = threadIdx.x & 31; i < 224 && !strong; i += 32) {
     const int n = i >> 3, c = i & 7, dx = n % 3 - 1, dy = n / 3 % 3 - 1, dz = n / 9 - 1;
-    const bool in = i < 216 && x + dx >= 0 && y + dy >= 0 && z + dz >= 0 && x + dx < v.h && y + dy < v.h && z + dz < v.h;
+    const bool in = i < 216 && x + dx >= 0 && y + dy >= 0 && z + dz >= 0 && x + dx < v.h && y + dy < v.h &&
+                    z + dz < v.h;
     const int ox = 2 * dx + (c & 1) - (ct & 1), oy = 2 * dy + ((c >> 1) & 1) - ((ct >> 1) & 1),
               oz = 2 * dz + (c >> 2) - (ct >> 2);
     unsigned long long m = 0;
@@ -504,9 +505,9 @@ __device__ __forceinline__ bool left_out(const CrtLv& v, const Item& t) {
 // tile, one right-hand side, one group of (source class, y-shift) windows.  A
 // CTA per SM takes every gridDim-th; each role runs on into the next item, so
 // that its operands load and its first sums form while the last one's are
-// reduced and written.  2^20 points, d = 193, against a CTA per item: M2L 5.81 ->
-// 5.70 ms (4.86 with the uniform waits and the short loop), L2L 0.39 -> 0.33, Delta^t 0.45 -> 0.36; d = 126: 3.80 -> 3.87 (2.33), 0.32 -> 0.27,
-// 0.34 -> 0.28; 512 leaves, d = 193: M2L 0.40 -> 0.36.
+// reduced and written.  Against a CTA per item, 2^20 points: L2L 0.39 -> 0.33 and
+// Delta^t 0.45 -> 0.36 ms at d = 193, 0.32 -> 0.27 and 0.34 -> 0.28 at d = 126; the M2L
+// about the same there, 0.40 -> 0.36 with 512 leaves.
 // Warps 0-7 drain the accumulators, warp 8 streams the operator residues
 // (K-chunk of one offset per stage), warp 9 issues the MMAs, warp 10 loads the
 // windows.  M = 128 boxes, N = Nt columns m', K in chunks of at most 64 terms.
@@ -582,20 +583,20 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
           const uint32_t bytes = (uint32_t)(c < n0 ? ks0 : ks1) * 32u * (uint32_t)v.Nt;
 #pragma unroll 1
           for (int left = mask; left && ok; left &= left - 1) {
-              const int m = __ffs(left) - 1, mz = (11 * m) >> 5;
-              const char* from = src + (2 * (m - 3 * mz - 1) + 98 * (mz - 1)) * slot_b;
-              if (it >= S) ok = mbar_wait_u(bempty(st), ph ^ 1u, a.err, 11, abort);
-              if (ok) {
-                if (el) {
-                  mbar_expect_tx(bfull(st), bytes);
-                  bulk_g2s(dst, from, bytes, bfull(st));
-                }
-                __syncwarp();
-                ++it;
-                dst += stage_b;
-                if (++st == S) st = 0, ph ^= 1u, dst = s_stage;
+            const int m = __ffs(left) - 1, mz = (11 * m) >> 5;
+            const char* from = src + (2 * (m - 3 * mz - 1) + 98 * (mz - 1)) * slot_b;
+            if (it >= S) ok = mbar_wait_u(bempty(st), ph ^ 1u, a.err, 11, abort);
+            if (ok) {
+              if (el) {
+                mbar_expect_tx(bfull(st), bytes);
+                bulk_g2s(dst, from, bytes, bfull(st));
               }
+              __syncwarp();
+              ++it;
+              dst += stage_b;
+              if (++st == S) st = 0, ph ^= 1u, dst = s_stage;
             }
+          }
           src += bytes;
         }
       }
@@ -653,28 +654,28 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     };
     // the steps of one window whose chunk has KS k-steps.  A loop, not
     // unrolled over the shifts: one warp runs through this code once per window,
-    // and fetching it took longer than the MMAs (M2L of 2^20 points, unrolled:
-    // d = 193 5.14 ms, this 4.86; d = 126 3.29, this 2.33)
+    // and fetching it took longer than the MMAs (M2L of 2^20 points, unrolled and
+    // so: d = 193 5.14 and 4.86 ms, d = 126 3.29 and 2.33)
     auto window = [&](auto ksc, int mask, uint32_t awin) {
       constexpr int KS = decltype(ksc)::value;
 #pragma unroll 1
       for (int left = mask; left; left &= left - 1) {
-          const int m = __ffs(left) - 1, mz = (11 * m) >> 5;
-          if (acc + KS > kMaxSteps) {  // this accumulator is full
-            mma_commit_el(afull(g & 1), el);
-            ++g;
-            open_acc();
-          }
-          ok = ok && mbar_wait_u(bfull(st), ph, a.err, 15, abort);
-          if (!ok) return;
-          tc_fence_after();
-          mma_steps<KS>(dst, awin + (uint32_t)(mz * ((kTX + 2) * kTY - 3) + m), ahi, blo | lbo, bhi, n2, id,
-                        acc > 0 ? 1u : 0u, el);
-          acc += KS;
-          mma_commit_el(bempty(st), el);
-          blo += stage16;
-          if (++st == S) st = 0, ph ^= 1u, blo = blo0;
+        const int m = __ffs(left) - 1, mz = (11 * m) >> 5;
+        if (acc + KS > kMaxSteps) {  // this accumulator is full
+          mma_commit_el(afull(g & 1), el);
+          ++g;
+          open_acc();
         }
+        ok = ok && mbar_wait_u(bfull(st), ph, a.err, 15, abort);
+        if (!ok) return;
+        tc_fence_after();
+        mma_steps<KS>(dst, awin + (uint32_t)(mz * ((kTX + 2) * kTY - 3) + m), ahi, blo | lbo, bhi, n2, id,
+                      acc > 0 ? 1u : 0u, el);
+        acc += KS;
+        mma_commit_el(bempty(st), el);
+        blo += stage16;
+        if (++st == S) st = 0, ph ^= 1u, blo = blo0;
+      }
     };
     for (unsigned i = blockIdx.x; i < items && ok; i += gridDim.x) {
       const Item t = item_of(a, i);
@@ -1485,8 +1486,8 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     size_t off = 0, i1 = i0;
     int64_t items = 0;
     auto tiles = [](const CrtLv& v) {
-      return (int64_t)((v.h + kTX - 1) / kTX) * ((v.h + kTY - 1) / kTY) * ((v.nz + kTZ - 1) / kTZ) * v.nct * v.NT * v.Rc *
-             mode_mods(v.mode);
+      return (int64_t)((v.h + kTX - 1) / kTX) * ((v.h + kTY - 1) / kTY) * ((v.nz + kTZ - 1) / kTZ) * v.nct * v.NT *
+             v.Rc * mode_mods(v.mode);
     };
     for (; i1 < todo.size() && a.nlev < kMaxLv; ++i1) {
       const CrtLv& v = todo[i1];
@@ -1539,7 +1540,8 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
       win = std::max(win, ks * kWinStep);
       pl_smem = std::max(pl_smem, (size_t)8 * (v.K + 1) * sizeof(long long));
       const cuuint64_t hh = (cuuint64_t)v.h;
-      cuuint64_t dims[5] = {8 * hh, hh, (cuuint64_t)v.snz, (cuuint64_t)v.K / 8, (cuuint64_t)mode_parts(v.mode) * v.pstep};
+      cuuint64_t dims[5] = {8 * hh, hh, (cuuint64_t)v.snz, (cuuint64_t)v.K / 8,
+                            (cuuint64_t)mode_parts(v.mode) * v.pstep};
       cuuint64_t strides[4] = {16 * hh, 16 * hh * hh, 16 * hh * hh * v.snz, 16 * hh * hh * v.snz * (v.K / 8)};
       cuuint32_t box[5] = {8 * (kTX + 2), kTY, kTZ + 2, 2, 1};
       cuuint32_t estr[5] = {1, 1, 1, 1, 1};

@@ -327,7 +327,8 @@ FxLeaf fx_leaf(const Tree* t) {
     int e = 0;
     const double m = std::ldexp(std::frexp(1e-3, &e), 53);
     const int sh = e - 53 + 2 * (i == 0 ? f.K : f.K2);
-    const unsigned __int128 v = sh >= 0 && sh < 75 ? (unsigned __int128)m << sh : sh < 0 && sh > -53 ? (unsigned __int128)m >> -sh : 0;
+    const unsigned __int128 m128 = (unsigned __int128)m;
+    const unsigned __int128 v = sh >= 0 && sh < 75 ? m128 << sh : sh < 0 && sh > -53 ? m128 >> -sh : 0;
     const_cast<FxConfig3*>(c[i])->e_hi = (unsigned long long)(v >> 64);
     const_cast<FxConfig3*>(c[i])->e_lo = (unsigned long long)v;
   }
@@ -409,8 +410,8 @@ eifmm_status launch_l2p_fx(const Tree* t, int kern, const LevelOps& v, int R, do
   const FxLeaf lf = fx_leaf(t);
   const long long* q = t->same ? t->ws.fx_src : t->ws.fx_tgt;
   // d = 512 with 4 columns: 28 KB (8 columns would pass 48 KB with the sums)
-#define EIFMM_L2P_FX(K, RCT)                                                                                              \
-  k_l2p_fx<K, RCT><<<T.n_nonempty, FX_THREADS, (size_t)v.d * (24 + 8 * RCT), s>>>(                                        \
+#define EIFMM_L2P_FX(K, RCT)                                                                                        \
+  k_l2p_fx<K, RCT><<<T.n_nonempty, FX_THREADS, (size_t)v.d * (24 + 8 * RCT), s>>>(                                  \
       lf, T.nonempty, T.leaf_off, T.perm, T.x, T.y, T.z, q, q + T.n, q + 2 * T.n, T.n, R, v.X, v.Xq, v.d, t->ws.lh, \
       t->ws.fnear, t->ws.ffar, f, ld_f)
   if (kern == EIFMM_KERNEL_CONFIG3) {
@@ -429,10 +430,10 @@ eifmm_status launch_p2p_fx(const Tree* t, int kern, int R, double* fnear, cudaSt
   const FxLeaf f = fx_leaf(t);
   const long long* sq = t->ws.fx_src;
   const long long* tq = t->same ? sq : t->ws.fx_tgt;
-#define EIFMM_P2P_FX(K, RCT)                                                                                           \
-  k_p2p_fx<K, RCT><<<dim3(T.n_nonempty, near_split(T.max_leaf)), FX_THREADS, 0, s>>>(f, T.nonempty, T.leaf_off, T.x, T.y, T.z, tq, tq + T.n,         \
-                                                    tq + 2 * T.n, T.n, S.leaf_off, S.x, S.y, S.z, sq, sq + S.n,     \
-                                                    sq + 2 * S.n, t->ws.sig, S.n, R, t->exclude_self, fnear)
+#define EIFMM_P2P_FX(K, RCT)                                                                                      \
+  k_p2p_fx<K, RCT><<<dim3(T.n_nonempty, near_split(T.max_leaf)), FX_THREADS, 0, s>>>(                             \
+      f, T.nonempty, T.leaf_off, T.x, T.y, T.z, tq, tq + T.n, tq + 2 * T.n, T.n, S.leaf_off, S.x, S.y, S.z, sq, \
+      sq + S.n, sq + 2 * S.n, t->ws.sig, S.n, R, t->exclude_self, fnear)
   if (kern == EIFMM_KERNEL_CONFIG3) {
     if (R == 1) EIFMM_P2P_FX(EIFMM_KERNEL_CONFIG3, 1);
     else EIFMM_P2P_FX(EIFMM_KERNEL_CONFIG3, 4);

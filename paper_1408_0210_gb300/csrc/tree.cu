@@ -113,8 +113,8 @@ k_keys(const double* __restrict__ xyz, int64_t n, const __grid_constant__ KeyBox
 
 template <int IN>
 __global__ void __launch_bounds__(RS_THREADS)
-k_rs_count(const uint32_t* __restrict__ kin, const uint2* __restrict__ pin, int64_t n, int shift, uint32_t mask, uint32_t* __restrict__ counts,
-           int nblocks) {
+k_rs_count(const uint32_t* __restrict__ kin, const uint2* __restrict__ pin, int64_t n, int shift, uint32_t mask,
+           uint32_t* __restrict__ counts, int nblocks) {
   __shared__ uint32_t h[RS_DIGITS];
   h[threadIdx.x] = 0;
   __syncthreads();
