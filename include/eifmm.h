@@ -77,14 +77,16 @@ typedef enum {
  *            tier 3: far field in FP64, near field in FP32 (Kahan sums);
  *            tier 4: FP64 everywhere (near field too), as FP64.
  *          The FP64 far field sums its products in integer residues on the
- *          tensor cores and rounds each sum once to FP64 (M2L: twice where a
- *          box is far weaker than its level).  W enters a box's M2L sum with
- *          53 bits or more relative to the largest of its interaction list,
- *          as long as that is above 2^-64 of the largest |W| of the level and
- *          column; what lies below 2^-117 of the latter is cut off.  M2M,
- *          L2L and step 6 have no such limit, nor has the M2L of a kernel
- *          that falls off steeply within an interaction list (exp(-r^2) on a
- *          large cube), which runs on the FP64 pipes or in FP32 pairs.
+ *          tensor cores and rounds each sum once to FP64.  M2M, L2L and step
+ *          6 round their operand to 56 bits or more of the largest entry of
+ *          a parent or box, the M2L to 58 bits of the largest |W| of a level
+ *          and column.  A box whose interaction list holds only values far
+ *          below that (2^-5 to 2^-8 of it, by the rank) takes its terms in
+ *          full, from a second residue part or on the FP64 pipes: no box is
+ *          less precise than in FP64.  The M2L of a kernel that
+ *          falls off steeply within an interaction list (exp(-r^2) on a
+ *          large cube) runs on the FP64 pipes (FP64) or in FP32 pairs (tiers
+ *          3 and 4).
  *          In every tier the M2L applies K^delta Delta (built once with
  *          FP64 solves) to W, so step 3 needs no solve.
  */

@@ -57,6 +57,7 @@ __host__ __device__ inline double kern_f64(int kern, double z0, double z1, doubl
 // (m2l_crt.cu): [modulus][slot][column tile][k8][Nt columns m'][8 terms l].
 struct CrtImage {
   void* img = nullptr;         // BF16
+  const double* T = nullptr;   // the operators themselves, [slot][l][m']
   double* colscale = nullptr;  // [d] scale of column m' in the reconstruction
   double kappa = -1.0;         // amplification of rounding by the operators (crt_kappa); -1: not known
   bool refused = false;        // the operators cannot be represented, or their image did not fit

@@ -22,13 +22,13 @@
 // 2 to 4, uniform and clustered points), the FP64 sum on the FP64 pipes by
 // 1.2e-15 to 6.8e-15 and the FP32 pairs by about 2e-12; for the config-3 kernel
 // (eps 1e-6) 4.2e-13 against 6.6e-12 in FP64.
-// Uneven problems (kWeakBits) keep their digits by a second part: 1/r, 2,000 charges
+// Uneven problems keep their digits (weak_bits): 1/r, 2,000 charges
 // of order 1 that cancel in one corner and 1e-12 elsewhere, depth 7: f differs from
 // the FP64 pipes' by 4e-16 in the median; with one part by 1.8e-14.
 //
 // Six launches cover all levels: largest |W| per level, box and column; the
-// residue planes of W; those of the second part (kWeakBits), if any; the residue
-// GEMMs; the reconstruction; that of the targets with a second part.  At 2^20 points,
+// residue planes of W; those of the second part (weak_bits), if any; the residue
+// GEMMs; the reconstruction; the weak boxes.  At 2^20 points,
 // depth 5: eps 1e-6 (d = 193) 4.65 + 0.2 ms, where the FP32 pairs took 144 ms; eps
 // 1e-4 (d = 126) 2.3 ms, where the FP64 pipes took 195 ms; eps 1e-7 (d = 256)
 // 8.0 ms (202 ms in FP32 pairs).  The GEMM issues 14 times the method's products,
@@ -70,14 +70,27 @@ __host__ __device__ constexpr int crt_mod(int i) {
 // rowbits + 1 (the sign) is the size of the product of the moduli.
 constexpr int kWBits = 58, kRowBits = 66, kEntryBits = 60;  // |T| 2^a < 2^60
 // The M2L's scale is the level's, so a target box all of whose sources are far
-// weaker than the level's strongest box would get them in few bits.  Such a box
-// (the exponent of the largest |W| of its interaction list more than kWeakBits
-// below that of the level's: nearer, the rounding is at most half a unit in the
-// last place of its strongest source) also takes a second part, the same sum over
-// what the rounding left of W, in units 2^-59 times smaller, added in FP64: 53
-// bits down to 2^-64 of the level's largest.  Even problems have no such box; the
-// items of the second part then do not exist, and its two kernels end at once.
-constexpr int kWeakBits = 5, kRestBits = 59;
+// weaker than the level's strongest box would get them in few bits.  A box is weak
+// where the exponent of the largest |W| of its interaction list lies more than
+// weak_bits(d) below that of the level's.  Up to there the rounding of W, 2^-58 of
+// the level's largest, adds less to the sum than FP64 rounds its d terms and more to
+// (exact sums, clustered points, lists of one or two occupied boxes: 0.76 of the FP64
+// pipes' error at the limit for d = 17, 0.44 for d = 64, 0.21 for d = 128).
+//
+// The weak boxes of a tile with kTileWork or more occupied sources take a second
+// part: the same sum over what the rounding left of W, in units 2^-kRestBits times
+// smaller, added in FP64.  Fewer sources, and boxes weaker than kMaxWeak, are summed
+// on the FP64 pipes source by source: most weak boxes lie at the rim of a cluster
+// and have one or two (2^20 points of a mixture of 8 Gaussians, d = 193: 308 boxes on 112 of
+// the 256 tiles of level 5).  Even problems have no weak box; the second part then
+// has no items, and its two kernels end at once.
+__host__ __device__ __forceinline__ int weak_bits(int d) {
+  int b = 4;
+  while (d >= 4) ++b, d >>= 2;
+  return b;
+}
+constexpr int kRestBits = 59, kMaxWeak = 60;
+constexpr unsigned kTileWork = 128;
 constexpr int kBoxWBits = 55, kBoxRowBits = 104;
 constexpr int kMaxSteps = 15;  // k-steps of 16 terms in one accumulation: 240 terms
 
@@ -126,10 +139,11 @@ struct CrtLv {
   // source box J is in unit J >> sshift, target box I takes unit I >> tshift
   unsigned long long* wmax;
   int sshift, tshift;
-  // second part of the M2L (kWeakBits): null elsewhere
+  // weak boxes of the M2L: null elsewhere
   unsigned long long* bmax;  // [box][R] bits of the largest |W| of a box
-  unsigned char* weak;       // [box][R] target boxes that take the second part
-  unsigned char* need;       // [r][class][tile z, y, x] tiles that hold some
+  unsigned char* weak;       // [box][R] 1 or, beyond kMaxWeak, 2 for a weak target box
+  unsigned* need;            // [r][class][tile z, y, x] occupied sources of the tile's weak boxes (1)
+  const double* T;           // the operators, [slot][l < ds][m' < d]
   int pstep;                 // class grids of the first part in `planes`
   int64_t rstep;             // entries of the first part in `res`
 };
@@ -137,7 +151,9 @@ constexpr int kMaxLv = kMaxLevel - 1;
 struct CrtArgs {
   int nlev, stages;
   unsigned items, plane_blocks, rebuild_blocks;
-  unsigned* any;  // set when some target takes the second part (null: never)
+  // [0] some tile takes the second part, [1] weak boxes in `list` (null: not the M2L)
+  unsigned* any;
+  uint2* list;  // (level << 16 | column, box)
   uint32_t stage_b, win_b;
   int* err;
   CrtLv lv[kMaxLv];
@@ -362,15 +378,17 @@ __device__ __forceinline__ int need_index(const CrtLv& v, int r, int ct, int z, 
   const int nx = (v.h + kTX - 1) / kTX, ny = (v.h + kTY - 1) / kTY, nz = (v.nz + kTZ - 1) / kTZ;
   return (((r * v.nct + ct) * nz + (z - v.z0) / kTZ) * ny + y / kTY) * nx + x / kTX;
 }
-// Whether box (x, y, z) of class ct takes the second part, by its warp.  The
+// Whether box (x, y, z) of class ct is weak, by its warp.  The
 // boxes of its interaction list are the children of the 27 neighbours of its
 // parent (x, y, z) but its own neighbours.
 __device__ __forceinline__ void mark_weak(const CrtArgs& a, const CrtLv& v, int r, int ct, int z, int y, int x,
                                           int64_t box, unsigned long long level) {
   // by the exponents (subnormals count as the smallest one); most boxes have a
   // strong source among the first 32 looked at
-  const int enough = (int)(level >> 52) - kWeakBits;
-  bool some = false, strong = !w_finite(level);
+  const int top = (int)(level >> 52), enough = top - weak_bits(v.ds);
+  int most = -1;
+  unsigned occupied = 0;
+  bool strong = !w_finite(level);
   for (int i = threadIdx.x & 31; i < 224 && !strong; i += 32) {
     const int n = i >> 3, c = i & 7, dx = n % 3 - 1, dy = n / 3 % 3 - 1, dz = n / 9 - 1;
     const bool in = i < 216 && x + dx >= 0 && y + dy >= 0 && z + dz >= 0 && x + dx < v.h && y + dy < v.h &&
@@ -380,16 +398,19 @@ __device__ __forceinline__ void mark_weak(const CrtArgs& a, const CrtLv& v, int 
     unsigned long long m = 0;
     if (in && (abs(ox) > 1 || abs(oy) > 1 || abs(oz) > 1))
       m = v.bmax[class_box(8, c, x + dx, y + dy, z + dz) * v.R + r];
-    some = some || m > 0;
-    strong = __any_sync(0xffffffffu, m > 0 && (int)(m >> 52) >= enough);
+    occupied += __popc(__ballot_sync(0xffffffffu, m > 0));
+    if (m > 0) most = max(most, (int)(m >> 52));
+    strong = __any_sync(0xffffffffu, most >= enough);
   }
-  const bool weak = __any_sync(0xffffffffu, some) && !strong;
+  most = __reduce_max_sync(0xffffffffu, most);
   if ((threadIdx.x & 31) != 0) return;
-  v.weak[box * v.R + r] = weak;
-  if (weak) {
-    v.need[need_index(v, r - v.r0, ct, z, y, x)] = 1;
-    *a.any = 1;
-  }
+  const bool weak = !strong && occupied > 0;
+  v.weak[box * v.R + r] = !weak ? 0 : top - most > kMaxWeak ? 2 : 1;
+  if (!weak) return;
+  a.list[atomicAdd(a.any + 1, 1u)] = make_uint2((unsigned)(&v - a.lv) << 16 | (unsigned)r, (unsigned)box);
+  if (top - most > kMaxWeak) return;
+  const unsigned old = atomicAdd(v.need + need_index(v, r - v.r0, ct, z, y, x), occupied);
+  if (old < kTileWork && old + occupied >= kTileWork) *a.any = 1;
 }
 // One block of the planes; REST: of the second part.
 template <int NM, bool REST>
@@ -496,9 +517,9 @@ __device__ __forceinline__ Item item_of(const CrtArgs& a, unsigned i) {
   return o;
 }
 
-// An item of the second part whose tile holds no weak target is left out.
+// An item of the second part is left out where its tile does not take that.
 __device__ __forceinline__ bool left_out(const CrtLv& v, const Item& t) {
-  return t.part && !__any_sync(0xffffffffu, v.need[need_index(v, t.r, t.ct, t.z0, t.y0, t.x0)] != 0);
+  return t.part && !__any_sync(0xffffffffu, v.need[need_index(v, t.r, t.ct, t.z0, t.y0, t.x0)] >= kTileWork);
 }
 
 // One item: one modulus, one target tile (128 boxes of a class), one column
@@ -921,7 +942,10 @@ __device__ __forceinline__ void rebuild_block(const CrtArgs& a, const CrtK<NM, N
   const unsigned cz = in >> (2 * lh), cls = v.nct == 1 ? 0u : cz / (unsigned)v.nz;
   const int64_t I = class_box(v.nct, (int)cls, (int)(in & (v.h - 1)), (int)((in >> lh) & (v.h - 1)),
                               v.z0 + (int)(cz - cls * v.nz));
-  if (WEAK && !v.weak[I * v.R + r]) return;
+  if (WEAK) {
+    const int x = (int)(in & (v.h - 1)), y = (int)((in >> lh) & (v.h - 1)), z = v.z0 + (int)(cz - cls * v.nz);
+    if (v.weak[I * v.R + r] != 1 || v.need[need_index(v, (int)rr, (int)cls, z, y, x)] < kTileWork) return;
+  }
   double* g = v.g + (I * v.R + r) * v.d + c;
   const unsigned long long bits = v.wmax[(I >> v.tshift) * v.R + r];
   const bool fin = w_finite(bits);
@@ -947,10 +971,61 @@ __global__ void __launch_bounds__(kRebuild)
 k_crt_rebuild(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK<NM, NW> kc) {
   rebuild_block<NM, NW, GROUPS, false>(a, kc, blockIdx.x);
 }
+// A weak box on the FP64 pipes: a block takes 32 coefficients, a warp every fourth
+// occupied source; the warps' sums are added in order.
+__device__ __forceinline__ void weak_box(const CrtLv& v, int r, int64_t box, int c0, double* s_sum) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, mp = c0 + lane;
+  int b[3];
+  morton_decode(box, v.tlevel, b);
+  const int n = 1 << v.tlevel;
+  double sum = 0.0;
+  int turn = 0;
+  for (int k = 0; k < 224; k += 32) {  // the children of the 27 neighbours of its parent
+    const int i = k + lane, x = (b[0] & ~1) - 2 + i % 6, y = (b[1] & ~1) - 2 + i / 6 % 6, z = (b[2] & ~1) - 2 + i / 36;
+    const int dx = x - b[0], dy = y - b[1], dz = z - b[2];
+    const bool in = i < 216 && x >= 0 && y >= 0 && z >= 0 && x < n && y < n && z < n &&
+                    (abs(dx) > 1 || abs(dy) > 1 || abs(dz) > 1);
+    const int J = in ? (int)morton_encode(x, y, z, v.tlevel) : 0, slot = (dz + 3) * 49 + (dy + 3) * 7 + dx + 3;
+    for (unsigned left = __ballot_sync(0xffffffffu, in && v.bmax[(int64_t)J * v.R + r] != 0); left; left &= left - 1) {
+      const int from = __ffs(left) - 1;
+      const int64_t Js = __shfl_sync(0xffffffffu, J, from);
+      const int sl = __shfl_sync(0xffffffffu, slot, from);
+      if ((turn++ & 3) != warp || mp >= v.d) continue;
+      const double* T = v.T + (int64_t)sl * v.ds * v.d + mp;
+      const double* w = v.W + (Js * v.R + r) * v.ds;
+#pragma unroll 8
+      for (int l = 0; l < v.ds; ++l) sum = fma(T[(int64_t)l * v.d], w[l], sum);
+    }
+  }
+  __syncthreads();
+  s_sum[threadIdx.x] = sum;
+  __syncthreads();
+  if (warp == 0 && mp < v.d)
+    v.g[(box * v.R + r) * v.d + mp] = s_sum[lane] + s_sum[32 + lane] + s_sum[64 + lane] + s_sum[96 + lane];
+}
+// The weak boxes: by the second part, or on the FP64 pipes.
 __global__ void __launch_bounds__(kRebuild)
-k_crt_rebuild_weak(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK<kMods, 5> kc) {
-  if (*a.any == 0) return;
-  for (unsigned b = blockIdx.x; b < a.rebuild_blocks; b += gridDim.x) rebuild_block<kMods, 5, true, true>(a, kc, b);
+k_crt_weak(const __grid_constant__ CrtArgs a, const __grid_constant__ CrtK<kMods, 5> kc) {
+  __shared__ double s_sum[kRebuild];
+  const unsigned n = a.any[1];
+  if (n == 0) return;
+  if (a.any[0])
+    for (unsigned b = blockIdx.x; b < a.rebuild_blocks; b += gridDim.x) rebuild_block<kMods, 5, true, true>(a, kc, b);
+  const unsigned chunks = (kMaxD + 31) / 32;
+  for (unsigned u = blockIdx.x; u < n * chunks; u += gridDim.x) {
+    const uint2 e = a.list[u / chunks];
+    const CrtLv& v = a.lv[e.x >> 16];
+    const int r = (int)(e.x & 0xffffu), c0 = 32 * (int)(u % chunks);
+    if (c0 >= v.d) continue;
+    const int64_t box = e.y;
+    int b[3];
+    morton_decode(box, v.tlevel, b);
+    const int ct = (b[0] & 1) | (b[1] & 1) << 1 | (b[2] & 1) << 2;
+    if (v.weak[box * v.R + r] == 1 &&
+        v.need[need_index(v, r - v.r0, ct, b[2] >> 1, b[1] >> 1, b[0] >> 1)] >= kTileWork)
+      continue;
+    weak_box(v, r, box, c0, s_sum);
+  }
 }
 
 // ---------------------------------------------------------- the images --
@@ -1274,14 +1349,14 @@ bool crt_ready(CrtMode mode, int level, const CrtImage& im, int R, size_t bytes)
 }
 
 // [kMaxLevel + 1][R] maxima of the M2L's levels, the word `any`, the tiles' `need`,
-// the boxes' maxima, their `weak`; or the maxima of another mode's units
+// the boxes' maxima, their list, their `weak`; or the maxima of another mode's units
 size_t crt_max_words(int depth, int R) {
   size_t boxes = 0, tiles = 0;
   for (int k = 2; k <= depth; ++k) {
     boxes += (size_t)1 << (3 * k);
     tiles += need_tiles(1 << (k - 1), 1 << (k - 1), R);
   }
-  return (size_t)(kMaxLevel + 1) * R + 1 + (tiles + 7) / 8 + boxes * R + (boxes * R + 7) / 8;
+  return (size_t)(kMaxLevel + 1) * R + 1 + (tiles + 1) / 2 + 2 * boxes * R + (boxes * R + 7) / 8;
 }
 
 void free_crt_image(CrtImage* im) {
@@ -1291,6 +1366,7 @@ void free_crt_image(CrtImage* im) {
 }
 
 eifmm_status build_crt_image(const double* kdT, int nslots, int dl, int d, CrtImage* im, cudaStream_t s) {
+  im->T = kdT;
   im->d = d;
   im->dl = dl;
   im->nslots = nslots;
@@ -1407,22 +1483,24 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     if (dev < 64) attr[dev] = true;
   }
   const bool m2l = njobs > 0 && jobs[0].mode == kCrtM2L;
-  unsigned* any = nullptr;
-  unsigned char *need = nullptr, *weak[kMaxLevel + 1] = {};
+  unsigned *any = nullptr, *need = nullptr;
+  uint2* list = nullptr;
+  unsigned char* weak[kMaxLevel + 1] = {};
   unsigned long long* bmax[kMaxLevel + 1] = {};
   if (m2l) {
     unsigned long long* p = wmax + (size_t)(kMaxLevel + 1) * R;
     any = (unsigned*)p++;
-    need = (unsigned char*)p;
+    need = (unsigned*)p;
     size_t boxes = 0, tiles = 0;
     for (int j = 0; j < njobs; ++j) tiles += need_tiles(1 << (jobs[j].level - 1), 1 << (jobs[j].level - 1), R);
-    p += (tiles + 7) / 8;
+    p += (tiles + 1) / 2;
     EIFMM_CUDA(cudaMemsetAsync(wmax, 0, (char*)p - (char*)wmax, s));
     for (int j = 0; j < njobs; ++j) {
       bmax[jobs[j].level] = p + boxes * R;
       boxes += (size_t)1 << (3 * jobs[j].level);
     }
-    unsigned char* c = (unsigned char*)(p + boxes * R);
+    list = (uint2*)(p + boxes * R);
+    unsigned char* c = (unsigned char*)(p + 2 * boxes * R);
     for (int j = 0; j < njobs; ++j) {
       weak[jobs[j].level] = c;
       c += ((size_t)1 << (3 * jobs[j].level)) * R;
@@ -1473,6 +1551,7 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
           v.bmax = bmax[b.level];
           v.weak = weak[b.level];
           v.need = need;
+          v.T = b.img->T;
           need += need_tiles(h, v.nz, v.Rc);
         }
         todo.push_back(v);
@@ -1483,6 +1562,8 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     CrtMaps maps = {};
     a.err = err;
     a.any = any;
+    a.list = list;
+    if (m2l && i0 > 0) EIFMM_CUDA(cudaMemsetAsync(any, 0, 2 * sizeof(unsigned), s));
     size_t off = 0, i1 = i0;
     int64_t items = 0;
     auto tiles = [](const CrtLv& v) {
@@ -1579,7 +1660,7 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
     else k_crt_rebuild<kMods, 3, false><<<rb, kRebuild, 0, s>>>(a, kc);
     EIFMM_CHECK_LAUNCH();
     if (m2l) {
-      k_crt_rebuild_weak<<<std::min(rb, 8 * (unsigned)nsm), kRebuild, 0, s>>>(a, kweak);
+      k_crt_weak<<<8 * (unsigned)nsm, kRebuild, 0, s>>>(a, kweak);
       EIFMM_CHECK_LAUNCH();
     }
     i0 = i1;

@@ -122,9 +122,10 @@ def ints(a, e):
 
 # Operators without rounding: Gamma = B = 1 (Delta = 1), K(z) = |z|^2 and nodes on a
 # grid, so that T^delta = K^delta is exact.  The exported W then gives g exactly, and
-# the residue M2L's error is the rounding of W, at most 2^-53 of the largest W of the
-# interaction list for every term, and one or two of the sum (each 2^-53 of the
-# absolute terms): together below 2^-51 of that W times the row sums of |T|.
+# the residue M2L's error is the rounding of W, for these boxes (even ones and weak
+# ones) at most 2^-53 of the largest W of the interaction list for every term, and one
+# or two of the sum (each 2^-53 of the absolute terms): together below 2^-51 of that W
+# times the row sums of |T|.
 @pytest.mark.parametrize("depth,d,weak", [(4, 8, (1.0,)), (4, 17, (1.0,)), (4, 8, (2.0 ** -30,)), (4, 17, (2.0 ** -30,)),
                                           (4, 8, (2.0 ** -55,)), (4, 17, (2.0 ** -55,)),
                                           (5, 17, (2.0 ** -55, 1.0, 2.0 ** -20))])  # several tiles and columns
@@ -159,3 +160,52 @@ def test_residue_m2l_is_exact_to_its_rounding(E, orc, depth, d, weak):
                     largest, rows = max(largest, np.abs(W[J]).max()), rows + np.abs(T).sum(1)
                 err = [abs(float(Fraction(int(v), 2 ** 260) - Fraction(float(w)))) for v, w in zip(total, g[b])]
                 assert (np.array(err) <= 2.0 ** -51 * largest * rows).all(), (k, r, b)
+
+
+# A kernel's weak boxes with few sources run on the FP64 pipes, those of a crowded
+# tile take a second residue part, boxes beyond 2^-60 the pipes again, boxes up to the
+# limit neither: over clustered points no group's error exceeds that of the M2L on the
+# FP64 pipes (option m2l_fp64), against exact sums as above.
+@pytest.mark.parametrize("d", [8, 17, 64])
+@pytest.mark.parametrize("points,weak", [("mixture", 1.0), ("corners", 2.0 ** -6), ("corners", 2.0 ** -12),
+                                         ("corners", 2.0 ** -70)])
+def test_no_less_precise_than_the_fp64_pipes(E, orc, d, points, weak):
+    rng = np.random.default_rng(8)
+    lv = {}
+    for k in range(2, DEPTH + 1):
+        p = rng.integers(-128, 128, (2, d, 3)) / 256.0 * 2.0 ** -k
+        lv[k] = dict(d=d, X=p[0], Y=p[1], Gamma=np.eye(d), B=np.eye(d), eps_est=1e-6)
+    if points == "mixture":
+        n = 40000
+        x, s = wl.gaussian_mixture(n, 3), wl.sigma_uniform(n, 1, 40)[:, 0]
+    else:  # the strong corner, a crowded weak one, single points between
+        n = N
+        x = np.concatenate([0.25 * wl.uniform_cube(n // 2, 41), 0.75 + 0.25 * wl.uniform_cube(n // 2 - 40, 42),
+                            0.3 + 0.4 * wl.uniform_cube(40, 43)])
+        s = wl.sigma_uniform(n, 1, 44)[:, 0]
+        s[n // 2:] *= weak
+    ops = E.eifmm_ops_load("quad", 1.0, DEPTH, lv)
+    g = {}
+    for fp64 in (True, False):
+        tree = E.eifmm_tree_build(dev(x), None, (0, 0, 0), 1.0, DEPTH, True)
+        tree.set_option("m2l_fp64", fp64)
+        E.eifmm_evaluate(tree, ops, dev(s), torch.zeros(n, dtype=torch.float64, device="cuda"), "fp64")
+        W, g[fp64] = (E.eifmm_debug_export(tree, w, DEPTH, d)[:, 0] for w in (0, 2))
+    Kd = orc.m2l_operators("quad", 1.0, DEPTH, lv[DEPTH]).astype(np.longdouble)
+    err = {}  # binary exponents below the level's largest -> [(pipes, residues)]
+    for b in rng.choice(8 ** DEPTH, 400, replace=False):
+        total, largest, rows = np.zeros(d, np.longdouble), 0.0, np.zeros(d)
+        for J in orc.interaction_list(DEPTH, int(b)):
+            if J >= 0 and W[J].any():
+                t = [p - q for p, q in zip(coords(int(J), DEPTH), coords(int(b), DEPTH))]
+                T = Kd[t[0] + 3 + 7 * (t[1] + 3) + 49 * (t[2] + 3)]
+                total += T @ W[J].astype(np.longdouble)
+                largest, rows = max(largest, np.abs(W[J]).max()), rows + np.abs(T).sum(1).astype(float)
+        if largest > 0.0:
+            e = [np.sqrt((((g[f][b] - total) / (largest * rows)).astype(float) ** 2).mean()) for f in (True, False)]
+            err.setdefault(int(np.log2(np.abs(W).max() / largest)) // 3, []).append(e)
+    assert sum(len(e) for e in err.values()) >= 60
+    for below, e in err.items():
+        pipes, residues = np.mean(e, axis=0)
+        # single boxes scatter by a factor; 20 are a mean.  1.1 where the pipes run
+        assert len(e) < 20 or residues <= 1.1 * pipes, (below, len(e), pipes, residues)
