@@ -207,7 +207,10 @@ eifmm_status eifmm_ops_calibration(const eifmm_ops* ops, double* err4, int* tier
  * whose sum reaches (1 - eps) of the total.  C^delta = U^t K^delta U (r x r)
  * replaces K^delta: step 4 becomes w~ = U^t What (What = Delta W by the FP64
  * solves), g~ = sum_J C^delta w~, g = U g~.  eps = 0 removes the
- * compression.  ranks (may be NULL): int[11], entry k = r of level k (0
+ * compression.  Its projections and Delta run on the FP64 pipes, the
+ * uncompressed M2L on the tensor cores: on this GPU the compression makes an
+ * evaluation slower (64 columns at eps 1e-6: 0.84 s with it, 0.41 s without).
+ * ranks (may be NULL): int[11], entry k = r of level k (0
  * outside 2..depth).  Synchronises `stream`.  Errors: EINVAL (null, eps
  * outside [0, 1), all-zero operators), ENOMEM, ECUDA. */
 eifmm_status eifmm_ops_compress(eifmm_ops* ops, double eps, eifmm_stream stream,
@@ -335,9 +338,15 @@ eifmm_status eifmm_tree_sort_static(const double* xyz, int64_t n,
  * r*ld_f] (n_tgt x n_rhs), both FP64 and in the caller's original point
  * order.  The ops must cover the tree's levels (ops depth >= tree depth;
  * levels deeper than the tree are not used) and have the tree's L.  The
- * tree owns the workspace; the first call for a given (ops, n_rhs) allocates
- * it and later calls allocate nothing.  Calls that share a tree must not
- * overlap.  sigma must be finite: the mixed path's library GEMMs (M2M,
+ * tree owns the workspace; the first call for a given (ops, n_rhs, prec, tier,
+ * options) allocates it and later calls allocate nothing.  For the FP64 far
+ * field (FP64, tiers 3 and 4) the operator set grows at its first use by the
+ * residues of its operators (415 MB a level at rank 193, 2.5 GB at rank 512),
+ * and a tree by up to 4 GiB of scratch; where one of them does not fit, its
+ * steps run on the FP64 or FP32 pipes from then on.  While `stream` is being
+ * captured nothing is allocated or built: capture after a first call with
+ * the same arguments, or such steps are captured on the pipes.  Calls that
+ * share a tree must not overlap.  sigma must be finite: the mixed path's library GEMMs (M2M,
  * L2L) do not carry infinities or NaNs through, so a non-finite sigma gives
  * an unspecified f.  Errors: EINVAL (null, n_rhs < 1 or > 256, ld < n, ops
  * depth below the tree's, L mismatch), ENOMEM, ECUDA. */
@@ -383,10 +392,12 @@ eifmm_status eifmm_evaluate_host(eifmm_tree* tree, const eifmm_ops* ops,
  * boxes x d^2, plus the near field, targets x 27 x sources per leaf).
  * The first call evaluates them directly and records them into a CUDA
  * graph; a later call with the same trees, arrays, operators, precision,
- * tier and stream replays that graph with one launch.  The
- * library keeps one such graph per process (a call with other arguments
- * records a new one; destroying one of its trees or its operators drops
- * it).  The legacy default stream (NULL) is never captured: every call on it
+ * tier and stream replays that graph with one launch, as long as no other
+ * call has replaced what it refers to (a tree's options, its workspace by
+ * another n_rhs or precision, tuned variants, the operators' compression or
+ * tier); otherwise it records anew.  The library keeps one such graph per
+ * process (a call with other arguments records a new one; destroying one of
+ * its trees or its operators drops it).  The legacy default stream (NULL) is never captured: every call on it
  * evaluates directly.  Calls from several host threads are serialised.
  * Errors as eifmm_evaluate. */
 eifmm_status eifmm_evaluate_batched(eifmm_tree* const* trees,
@@ -401,7 +412,9 @@ eifmm_status eifmm_evaluate_batched(eifmm_tree* const* trees,
  *   what = 0 W (step 1-2), 1 What (step 3), 2 g (step 4), 3 l (step 5),
  *          4 lhat (step 6, level = depth), 5 f_far, 6 f_near (n_tgt x n_rhs
  *          column-major, original target order).
- * `n` is the capacity of `out` in doubles.  Synchronous.  Errors: EINVAL
+ * `n` is the capacity of `out` in doubles.  Synchronous.  Where the
+ * evaluation left out boxes without targets (tier 0, few occupied leaves)
+ * steps 4 to 6 are run for them first.  Errors: EINVAL
  * when nothing was evaluated, the level is out of range, n is too small, or
  * (what 0-4) the operator set of that evaluation has been destroyed since. */
 eifmm_status eifmm_debug_export(const eifmm_tree* tree, int what, int level,

@@ -204,10 +204,11 @@ eifmm_status ensure_crt_images(Ops* ops, int depth, bool m2l, cudaStream_t s) {
     if (k == depth)
       EIFMM_TRY(ensure(&v.crt_dt, v.d, v.d, [&] { return build_crt_delta_image(v, &v.crt_dt, s); }));
     if (!m2l) continue;
-    const bool steep = crt_steep((int)ops->kern, ops->L, k);
-    if (!v.crt.img) v.crt.refused = v.crt.refused || steep;
-    if (!v.crtc.img) v.crtc.refused = v.crtc.refused || steep;
-    if (ops->compressed && v.r > 0) {
+    const bool comp = ops->compressed && v.r > 0;
+    CrtImage& im = comp ? v.crtc : v.crt;
+    if (!im.img && !im.refused && (comp ? v.r : v.d) >= kCrtMinRank)
+      im.refused = crt_steep((int)ops->kern, ops->L, k);
+    if (comp) {
       EIFMM_TRY(stack(&v.crtc, v.Ct, kNumSlots, v.r, v.r));
     } else {
       EIFMM_TRY(stack(&v.crt, v.kdT, kNumSlots, v.d, v.d));
