@@ -26,9 +26,9 @@
 // of order 1 that cancel in one corner and 1e-12 elsewhere, depth 7: f differs from
 // the FP64 pipes' by 4e-16 in the median; with one part by 1.8e-14.
 //
-// Six launches cover all levels: largest |W| per level, box and column; the
+// Seven launches cover all levels: largest |W| per level, box and column; the
 // residue planes of W; those of the second part (weak_bits), if any; the residue
-// GEMMs; the reconstruction; the weak boxes.  At 2^20 points,
+// GEMMs; those of the second part; the reconstruction; the weak boxes.  At 2^20 points,
 // depth 5: eps 1e-6 (d = 193) 4.65 + 0.2 ms, where the FP32 pairs took 144 ms; eps
 // 1e-4 (d = 126) 2.3 ms, where the FP64 pipes took 195 ms; eps 1e-7 (d = 256)
 // 8.0 ms (202 ms in FP32 pairs).  The GEMM issues 14 times the method's products,
@@ -83,7 +83,7 @@ constexpr int kWBits = 58, kRowBits = 66, kEntryBits = 60;  // |T| 2^a < 2^60
 // on the FP64 pipes source by source: most weak boxes lie at the rim of a cluster
 // and have one or two (2^20 points of a mixture of 8 Gaussians, d = 193: 308 boxes on 112 of
 // the 256 tiles of level 5).  Even problems have no weak box; the second part then
-// has no items, and its two kernels end at once.
+// has no items, and its three kernels end at once.
 __host__ __device__ __forceinline__ int weak_bits(int d) {
   int b = 4;
   while (d >= 4) ++b, d >>= 2;
@@ -490,12 +490,10 @@ __device__ __forceinline__ void mma_steps(uint32_t dst, uint32_t alo, uint32_t a
 }
 
 struct Item {
-  int q, x0, y0, z0, ct, nt, r, grp, mod, w_beg, w_end, part;
+  int q, x0, y0, z0, ct, nt, r, grp, mod, w_beg, w_end;
 };
 __device__ __forceinline__ Item item_of(const CrtArgs& a, unsigned i) {
   Item o;
-  o.part = i >= a.items ? 1 : 0;
-  if (o.part) i -= a.items;
   o.q = find_level(a, &CrtLv::item0, i);
   const CrtLv& v = a.lv[o.q];
   unsigned b = i - v.item0;
@@ -519,7 +517,7 @@ __device__ __forceinline__ Item item_of(const CrtArgs& a, unsigned i) {
 
 // An item of the second part is left out where its tile does not take that.
 __device__ __forceinline__ bool left_out(const CrtLv& v, const Item& t) {
-  return t.part && !__any_sync(0xffffffffu, v.need[need_index(v, t.r, t.ct, t.z0, t.y0, t.x0)] >= kTileWork);
+  return !__any_sync(0xffffffffu, v.need[need_index(v, t.r, t.ct, t.z0, t.y0, t.x0)] >= kTileWork);
 }
 
 // One item: one modulus, one target tile (128 boxes of a class), one column
@@ -534,6 +532,10 @@ __device__ __forceinline__ bool left_out(const CrtLv& v, const Item& t) {
 // windows.  M = 128 boxes, N = Nt columns m', K in chunks of at most 64 terms.
 // Two TMEM accumulators of Nt columns: while one is filled (15 k-steps at
 // most), the other is added to the register sums modulo m.
+// REST: the second part of the M2L, for the tiles that take it (a launch of its own,
+// which ends at once where none does; as more items of one launch their checks took
+// 1.2% of the M2L and 6% of the L2L).
+template <bool REST>
 __global__ void __launch_bounds__(kThreads, 1)
 k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -542,7 +544,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
   // uniform for the compiler: the roles of warps 8 to 10 run converged
   const int wu = (int)__reduce_or_sync(0xffffffffu, (unsigned)warp);
   const int S = a.stages;
-  const unsigned items = __reduce_or_sync(0xffffffffu, a.any && *a.any ? 2u * a.items : a.items);
+  if (REST && *a.any == 0) return;
   const uint32_t sbase = smem_u32(smem);
   const uint32_t s_stage = sbase + kWins * a.win_b;
   uint64_t* bars = (uint64_t*)(smem + kWins * a.win_b + (uint32_t)S * a.stage_b);
@@ -589,10 +591,10 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     int it = 0, st = 0;
     uint32_t ph = 0, dst = s_stage;
     bool ok = true;
-    for (unsigned i = blockIdx.x; i < items && ok; i += gridDim.x) {
+    for (unsigned i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
       const Item t = item_of(a, i);
       const CrtLv& v = a.lv[t.q];
-      if (left_out(v, t)) continue;
+      if (REST && left_out(v, t)) continue;
       const int64_t tile_b = (int64_t)v.K * v.Nt * 2, slot_b = v.NT * tile_b;  // bytes of a column tile, of a slot
       const char* img = (const char*)v.img + (int64_t)t.mod * v.nslots * slot_b + t.nt * tile_b;
       const int n0 = v.n0, ks0 = v.ks0, ks1 = v.ks1, nchunk = v.nchunk;
@@ -629,10 +631,10 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     int wi = 0, s = 0;
     uint32_t wph = 0;
     bool ok = true;
-    for (unsigned i = blockIdx.x; i < items && ok; i += gridDim.x) {
+    for (unsigned i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
       const Item t = item_of(a, i);
       const CrtLv& v = a.lv[t.q];
-      if (left_out(v, t)) continue;
+      if (REST && left_out(v, t)) continue;
       for (int w = t.w_beg; w < t.w_end && ok; ++w) {
         const Win wn = window_of(v, t.ct, w);
         int k0 = 0;
@@ -647,7 +649,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
             for (int kk = 0; kk < ks; ++kk)
               tma_load_5d(sbase + (uint32_t)s * a.win_b + (uint32_t)kk * kWinStep, &maps.m[t.q], 8 * (t.x0 - 1),
                           t.y0 + wn.sy1 - 1, t.z0 - 1 - v.sz0, 2 * (k0 + kk),
-                          t.part * v.pstep + (t.mod * v.Rc + t.r) * v.ncs + wn.cs, wfull(s));
+                          (REST ? v.pstep : 0) + (t.mod * v.Rc + t.r) * v.ncs + wn.cs, wfull(s));
           }
           __syncwarp();
           k0 += ks;
@@ -698,10 +700,10 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
         if (++st == S) st = 0, ph ^= 1u, blo = blo0;
       }
     };
-    for (unsigned i = blockIdx.x; i < items && ok; i += gridDim.x) {
+    for (unsigned i = blockIdx.x; i < a.items && ok; i += gridDim.x) {
       const Item t = item_of(a, i);
       const CrtLv& v = a.lv[t.q];
-      if (left_out(v, t)) continue;
+      if (REST && left_out(v, t)) continue;
       const int n0 = v.n0, ks0 = v.ks0, ks1 = v.ks1, nchunk = v.nchunk;
       const uint64_t dB = desc_k(0, (uint32_t)v.Nt * 16u, 128u);
       lbo = (uint32_t)dB;
@@ -735,10 +737,10 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
     const float2 mg = make_float2(12582912.0f, 12582912.0f), ng2 = make_float2(-12582912.0f, -12582912.0f);
     int g = 0;
     bool have = true;
-    for (unsigned it = blockIdx.x; it < items && have; it += gridDim.x) {
+    for (unsigned it = blockIdx.x; it < a.items && have; it += gridDim.x) {
       const Item t = item_of(a, it);
       const CrtLv& v = a.lv[t.q];
-      if (left_out(v, t)) continue;
+      if (REST && left_out(v, t)) continue;
       const int Nt = v.Nt, nh = Nt / 2;
       const float fm = (float)crt_mod(t.mod);
       const float2 inv2 = make_float2(1.0f / fm, 1.0f / fm), m2 = make_float2(-fm, -fm);
@@ -775,7 +777,7 @@ k_crt_gemm(const __grid_constant__ CrtMaps maps, const __grid_constant__ CrtArgs
       const int x = t.x0 + (row & 7), y = t.y0 + ((row >> 3) & 3), z = t.z0 + (row >> 5);
       if (have && x < h && y < h && z < v.z0 + v.nz) {
         const int N = v.NT * Nt;
-        int16_t* out = v.res + t.part * v.rstep +
+        int16_t* out = v.res + (REST ? v.rstep : 0) +
                        ((((((int64_t)t.mod * v.G + t.grp) * v.Rc + t.r) * v.nct + t.ct) * v.nz + (z - v.z0)) * h + y) *
                            (int64_t)h * N +
                        (int64_t)x * N + t.nt * Nt + half * nh;
@@ -872,11 +874,15 @@ template <int NM, bool GROUPS>
 __device__ __forceinline__ void load_pair(const CrtLv& v, const int16_t* __restrict__ res, int64_t step, int (&s0)[NM],
                                           int (&s1)[NM]) {
   const int64_t mod = GROUPS ? v.G * step : step;
+  int u[NM];
+#pragma unroll
+  for (int i = 0; i < NM; ++i) u[i] = *reinterpret_cast<const int*>(res + i * mod);
+#pragma unroll
+  for (int i = 0; i < NM; ++i) asm volatile("" : "+r"(u[i]));  // every load is on its way before the first use
 #pragma unroll
   for (int i = 0; i < NM; ++i) {
-    const short2 u = *reinterpret_cast<const short2*>(res + i * mod);
-    s0[i] = u.x;
-    s1[i] = u.y;
+    s0[i] = (int16_t)u[i];
+    s1[i] = u[i] >> 16;
   }
   if (GROUPS && v.G > 1) {
     for (int k = 1; k < v.G; ++k)
@@ -1479,7 +1485,8 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
   int dev = 0;
   EIFMM_CUDA(cudaGetDevice(&dev));
   if (dev >= 64 || !attr[dev]) {
-    EIFMM_CUDA(cudaFuncSetAttribute(k_crt_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
+    EIFMM_CUDA(cudaFuncSetAttribute(k_crt_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
+    EIFMM_CUDA(cudaFuncSetAttribute(k_crt_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
     if (dev < 64) attr[dev] = true;
   }
   const bool m2l = njobs > 0 && jobs[0].mode == kCrtM2L;
@@ -1653,7 +1660,11 @@ eifmm_status launch_crt(int njobs, const CrtJob* jobs, int R, void* buf, size_t 
       k_crt_planes_rest<kMods><<<std::min(pl, 4 * (unsigned)nsm), 256, pl_smem, s>>>(a);
       EIFMM_CHECK_LAUNCH();
     }
-    k_crt_gemm<<<std::min(it, (unsigned)nsm), kThreads, smem, s>>>(maps, a);
+    k_crt_gemm<false><<<std::min(it, (unsigned)nsm), kThreads, smem, s>>>(maps, a);
+    if (m2l) {
+      EIFMM_CHECK_LAUNCH();
+      k_crt_gemm<true><<<std::min(it, (unsigned)nsm), kThreads, smem, s>>>(maps, a);
+    }
     EIFMM_CHECK_LAUNCH();
     if (box) k_crt_rebuild<kBoxMods, 4, false><<<rb, kRebuild, 0, s>>>(a, kcb);
     else if (groups) k_crt_rebuild<kMods, 3, true><<<rb, kRebuild, 0, s>>>(a, kc);
