@@ -209,7 +209,7 @@ eifmm_status eifmm_ops_calibration(const eifmm_ops* ops, double* err4, int* tier
  * solves), g~ = sum_J C^delta w~, g = U g~.  eps = 0 removes the
  * compression.  Its projections and Delta run on the FP64 pipes, the
  * uncompressed M2L on the tensor cores: on this GPU the compression makes an
- * evaluation slower (64 columns at eps 1e-6: 0.83 s with it, 0.39 s without).
+ * evaluation slower (64 columns at eps 1e-6: 0.82 s with it, 0.38 s without).
  * ranks (may be NULL): int[11], entry k = r of level k (0
  * outside 2..depth).  Synchronises `stream`.  Errors: EINVAL (null, eps
  * outside [0, 1), all-zero operators), ENOMEM, ECUDA. */
