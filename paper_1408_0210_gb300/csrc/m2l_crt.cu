@@ -40,9 +40,9 @@
 //
 // M2M, L2L and Delta^t are the same sums over the 8 children, the parent and the
 // box itself, without shifts.  A sum stays within one parent or box, and so does
-// its scale: a weak box next to strong ones keeps all its bits.  Delta^t is formed explicitly in double-double
-// and takes 18 moduli (160.5 bits): its entries reach 2^34 / |A| at eps 1e-7, and
-// the product cancels by as much.  K(x, X) Delta^t l then errs by 1.6e-16 to 9e-16
+// its scale: a weak box next to strong ones keeps all its bits.  Delta^t is formed
+// explicitly in double-double and takes 18 moduli (160.5 bits): its entries reach
+// 2^34 / |A| at eps 1e-7, and the product cancels by as much.  K(x, X) Delta^t l then errs by 1.6e-16 to 9e-16
 // (1/r, eps 1e-4 to 1e-7) where the FP64 triangular solves err by 2.3e-16 to 2.7e-15
 // (config-3 at 1e-6: 1.4e-12 and 7.2e-12).  At 2^20 points, depth 5, d = 193, on
 // the FP64 pipes before: M2M 3.0 -> 0.27 ms, L2L 5.1 -> 0.33 ms, Delta^t 3.5 -> 0.36
